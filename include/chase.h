@@ -63,15 +63,18 @@ typedef struct {
 #define CHASE_EIGENSOLVER_ERROR 8 /* the projected eigensolve (Alg. 2 line 3) failed */
 
 /* ---- arithmetic of the filter products (Alg. 4) ---- */
-#define CHASE_FP64 0 /* complex128 products on the FP64 tensor pipe (mma.sync f64, ~1 TFLOP/s) */
-/* Split-BF16: both operands cut into seven 7-bit integer slices (one power-
- * of-two scale per row of H without its diagonal and per column of the
- * block), slice products on the BF16 tensor cores (tcgen05) with exactly
- * accumulated leading levels; the diagonal of H and the recurrence's
- * shift/scale/axpby are applied in FP64.  Each entry of a product is
- * accurate to about 2^-49 max|off-diagonal row of H| max|column| per term.
- * Reads H through its Hermitian symmetry.  QR, Rayleigh-Ritz, residuals
- * and Lanczos stay FP64. */
+/* FP64 accuracy.  Products with H of more than 6 columns and N >= 128 run on
+ * the BF16 tensor cores in residue arithmetic (exact products of the operands
+ * rounded to 2^-60 of the 2-norm of a row of H or a column of the block, put
+ * together and finished in FP64: no further from the exact product than an
+ * FP64 GEMM); smaller ones, and the batched entry points, on the FP64 pipes. */
+#define CHASE_FP64 0
+/* Split: the same residue products with the operands rounded to 2^-48 of
+ * those norms (the batched entry points: both operands cut into seven 7-bit
+ * digits, each entry accurate to about 2^-49 max|off-diagonal row of H|
+ * max|column| per term).  The diagonal of H and the recurrence's
+ * shift/scale/axpby are applied in FP64.  Reads H through its Hermitian
+ * symmetry.  QR, Rayleigh-Ritz, residuals and Lanczos keep FP64 accuracy. */
 #define CHASE_SPLIT_BF16 1
 /* Split-BF16 filter as above, and the product H Q of Rayleigh-Ritz (Alg. 2
  * line 2, reused for the residuals) on the same split product: each entry
@@ -199,12 +202,12 @@ long long chase_device_allocations(void);
 /* Kernel timing, for benchmarks (the paper has no counterpart).  While
  * timing is on, the library records a pair of CUDA events on the launching
  * stream around the launches of its products with H:
- *   CHASE_TIMED_SPLIT_PRODUCT  the split-BF16 tensor-core product kernel
- *                              (zgemm_split_kernel; the slicing of the block
- *                              and the K-segment combine are outside);
- *   CHASE_TIMED_FP64_PRODUCT   the FP64 product with H of the filter and of
- *                              Rayleigh-Ritz (DMMA tile kernel, or the
- *                              few-column kernel for at most 6 columns).
+ *   CHASE_TIMED_SPLIT_PRODUCT  the tensor-core product of a split filter (the
+ *                              residue GEMM; making the residues of the block
+ *                              and putting the product together are outside);
+ *   CHASE_TIMED_FP64_PRODUCT   the product with H at FP64 accuracy, of the
+ *                              filter and of Rayleigh-Ritz (the residue GEMM,
+ *                              or the FP64 kernels for small products).
  * chase_kernel_timing(1) clears the record and starts; (0) stops.
  * chase_kernel_timing_read waits for the recorded events of one kind and
  * returns their summed duration (seconds), the kernel launches they cover,

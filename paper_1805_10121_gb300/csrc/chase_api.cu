@@ -135,14 +135,33 @@ int timed_h_product(Dev& d, const T* H, int64_t N, int64_t ldh, const T* X, int6
 // is the second buffer of the double buffering.  start[i] = number of
 // columns with degree < i for i = 0 .. maxdeg + 1 (columns with degree < i
 // have retired before step i).  Returns the column-product count.
-// One filter product: the FP64 DMMA kernel, or the split-BF16 tensor-core
-// kernel when slices of H are given.
+// H prepared for residue products (rns.cu): `full` for products in the
+// caller's precision, `low` for the reduced precisions of the split filter
+// (nullptr: not prepared), and the workspace they share.
+struct RnsSet {
+  const RnsH* full = nullptr;
+  const RnsH* low = nullptr;
+  RnsX* x = nullptr;
+};
+
+// Products with H take the residue path from this size on; below it, a few
+// columns or rows, the FP64 kernels are done sooner than its three launches.
+bool rns_pays(int64_t N, int b) { return N >= 128 && b > kFewColMax; }
+
+// Bytes that a call may still allocate after the residue planes of H.
+size_t rns_reserve(int64_t N, int b) {
+  return (size_t(2) << 30) + static_cast<size_t>(N) * b * 16 * 4;
+}
+
+// One filter product: in residue arithmetic when H is prepared for it, else
+// the FP64 DMMA kernel (FP32 kernel in single precision).
 template <class T>
-int filter_product(Dev& d, const T* H, int64_t N, int64_t ldh, const SplitH* sh, SplitX* sx,
-                   const T* X, int64_t ldx, int b, T* Y, int64_t ldy, int j0,
-                   double alpha, double beta, double shift, int nslices = 7) {
-  if constexpr (!is_single<T>) {
-    if (sh) return zgemm_split(d, *sh, *sx, X, ldx, j0, b, Y, ldy, alpha, beta, shift, nslices);
+int filter_product(Dev& d, const T* H, int64_t N, int64_t ldh, const RnsSet* rs, const T* X,
+                   int64_t ldx, int b, T* Y, int64_t ldy, int j0, double alpha, double beta,
+                   double shift, int nslices = 7) {
+  if (rs) {
+    const RnsH* h = nslices < 7 || !rs->full ? rs->low : rs->full;
+    return rns_product(d, *h, *rs->x, X, ldx, j0, b, Y, ldy, alpha, beta, shift);
   }
   return timed_h_product(d, H, N, ldh, X, ldx, b, Y, ldy, j0, alpha, beta, shift);
 }
@@ -166,8 +185,8 @@ struct FilterGroup {
 template <class T>
 int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx, T* Wk,
                   int64_t ldw, const std::vector<FilterGroup>& groups, int maxdeg, double b_sup,
-                  double mu1, double mu_nn, long long* matvecs, const SplitH* sh = nullptr,
-                  SplitX* sx = nullptr, long long* matvecs_low = nullptr) {
+                  double mu1, double mu_nn, long long* matvecs, const RnsSet* rs = nullptr,
+                  long long* matvecs_low = nullptr) {
   const double c = 0.5 * (b_sup + mu_nn);  // Alg. 4 line 2
   const double e = 0.5 * (b_sup - mu_nn);
   const double sigma1 = e / (mu1 - c);     // line 3
@@ -176,10 +195,10 @@ int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx,
                      double alpha, double beta) -> int {
     const int j0 = g.col0 + s, j1 = g.col0 + g.ncols;
     if (j0 >= j1) return CHASE_OK;
-    CHASE_TRY(filter_product(d, H, N, ldh, sh, sx, src, lds, j1, dst, ldd, j0, alpha, beta, c,
+    CHASE_TRY(filter_product(d, H, N, ldh, rs, src, lds, j1, dst, ldd, j0, alpha, beta, c,
                              g.nslices));
     mv += j1 - j0;
-    if (sh && g.nslices < 7) low += j1 - j0;
+    if (rs && g.nslices < 7) low += j1 - j0;
     return CHASE_OK;
   };
   // line 4: W = (sigma_1 / e) (H - c I) V
@@ -213,14 +232,14 @@ int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx,
 template <class T>
 int filter_sorted(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx,
                   T* Wk, int64_t ldw, int b, const int* start, int maxdeg, double b_sup,
-                  double mu1, double mu_nn, long long* matvecs, const SplitH* sh = nullptr,
-                  SplitX* sx = nullptr, int nslices = 7) {
+                  double mu1, double mu_nn, long long* matvecs, const RnsSet* rs = nullptr,
+                  int nslices = 7) {
   std::vector<FilterGroup> one(1);
   one[0].ncols = b;
   one[0].nslices = nslices;
   one[0].start.assign(start, start + maxdeg + 2);
   return filter_groups(d, H, N, ldh, X, ldx, Wk, ldw, one, maxdeg, b_sup, mu1, mu_nn, matvecs,
-                       sh, sx);
+                       rs);
 }
 
 void starts_from_sorted(const int* m, int b, int maxdeg, std::vector<int>& start) {
@@ -381,7 +400,7 @@ int rr_alloc(Dev& d, int64_t N, int b, RRWork<T>& w) {
 template <class T>
 int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, int b,
            RRWork<T>& w, const SplitH* sh = nullptr, SplitX* sx = nullptr,
-           double* t_hq = nullptr) {
+           double* t_hq = nullptr, const RnsSet* rs = nullptr) {
   const int64_t lN = ld_pad<T>(N), lg = ld_pad<T>(b);
   PhaseTimer tq(d.st);  // the product alone (synchronises only when timed)
   if (t_hq) tq.begin(t_hq);
@@ -392,7 +411,8 @@ int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, 
       on_split = true;
     }
   }
-  if (!on_split) CHASE_TRY(timed_h_product(d, H, N, ldh, Q, ldq, b, w.HQ, lN, 0, 1.0, 0.0, 0.0));
+  if (!on_split)
+    CHASE_TRY(filter_product(d, H, N, ldh, rs, Q, ldq, b, w.HQ, lN, 0, 1.0, 0.0, 0.0));
   if (t_hq) tq.end();
   // G = Q^H H Q is Hermitian up to rounding: form its lower triangle (the one
   // the eigensolver reads) and take the upper one from it
@@ -418,10 +438,10 @@ int rr_post(Dev& d, int64_t N, T* Q, int64_t ldq, int b, const double* w_dev, do
 template <class T>
 int rr_core(Dev& d, const T* H, int64_t N, int64_t ldh, T* Q, int64_t ldq, int b,
             double* w_dev, double* res_dev, RRWork<T>& w, double* t_eigh, double* flops,
-            const SplitH* sh = nullptr, SplitX* sx = nullptr, double* t_hq = nullptr) {
+            double* t_hq = nullptr, const RnsSet* rs = nullptr) {
   if (b == 0) return CHASE_OK;
   const int64_t lg = ld_pad<T>(b);
-  CHASE_TRY(rr_pre(d, H, N, ldh, Q, ldq, b, w, sh, sx, t_hq));
+  CHASE_TRY(rr_pre<T>(d, H, N, ldh, Q, ldq, b, w, nullptr, nullptr, t_hq, rs));
   PhaseTimer tm(d.st);
   tm.begin(t_eigh);
   CHASE_TRY(eigh_device(d, w.G, lg, b, w_dev));  // (W, Lambda) = TSOLVE(G)
@@ -622,16 +642,22 @@ struct Solver {
   int64_t lh = 0, lv = 0, ls = 0, lw = 0;
   OrthWork<T> ow;
   RRWork<T> rw;
-  SplitH sh;
+  SplitH sh;  // digit slices of the batched solve's split filter
   SplitX sx;
+  // H in residue planes: FP64 accuracy (FP64 filter, Rayleigh-Ritz), the split
+  // filter's, and its reduced precisions / single precision
+  RnsH h64, hsplit, hlow;
+  RnsX rx;
+  RnsSet filter_set, rr_set;
+  bool rns = false;
   // single precision with CHASE_SPLIT_BF16: the filter runs on widened FP64
   // copies of the active block (Dv, Dw), the product with 4 slices
   using Wide = typename std::conditional<is_cplx<T>, chase_c64, double>::type;
   Wide *Dv = nullptr, *Dw = nullptr;
   int64_t lD = 0;
   bool split = false;
-  bool split_rr = false;            // H Q of Rayleigh-Ritz on the split product too
-  const SplitH* rr_slices = nullptr;  // the slices of H used there
+  bool split_rr = false;              // H Q of Rayleigh-Ritz on the split product too
+  const SplitH* rr_slices = nullptr;  // batched solve: the slices of H used there
   SplitX* rr_sx = nullptr;
   double *dw = nullptr, *dres = nullptr;
   int* dperm = nullptr;
@@ -687,17 +713,7 @@ struct Solver {
                          : (o.precision == CHASE_SPLIT_BF16 || o.precision == CHASE_SPLIT_BF16_RR ||
                             o.precision == CHASE_SPLIT_BF16_ADAPT);
     split_rr = !is_single<T> && o.precision == CHASE_SPLIT_BF16_RR;
-    if (split && !grouped_split) {  // slices of H once per solve, slice workspace for the block
-      CHASE_TRY(split_prepare_h(d, dH, N, lh, sh));
-      CHASE_TRY(split_alloc_x(d, N, nx, sx, is_cplx<T>));
-      rr_slices = &sh;
-      rr_sx = &sx;
-      if constexpr (is_single<T>) {
-        lD = ld_pad<Wide>(N);
-        CHASE_TRY(d.alloc(&Dv, static_cast<size_t>(lD) * nx));
-        CHASE_TRY(d.alloc(&Dw, static_cast<size_t>(lD) * nx));
-      }
-    }
+    if (!grouped_split) CHASE_TRY(prepare_rns(d));
     CHASE_TRY(d.alloc(&dw, nx));
     CHASE_TRY(d.alloc(&dres, nx));
     CHASE_TRY(d.alloc(&dperm, nx));
@@ -742,6 +758,38 @@ struct Solver {
     order.assign(nx, 0);
     perm.assign(nx, 0);
     tol_eff = o.conv_mode == CHASE_CONV_REL ? tol * h : tol;
+    return CHASE_OK;
+  }
+
+  // H in residue planes, once per solve, and their workspace: the FP64
+  // solver's filter and Rayleigh-Ritz share one set; a split filter has its
+  // own (with CHASE_SPLIT_BF16_ADAPT a second one for its reduced precisions)
+  // beside Rayleigh-Ritz's FP64 one; single precision needs the low set only.
+  int prepare_rns(Dev& d) {
+    rns = split || rns_pays(N, nx);
+    if (!rns) return CHASE_OK;
+    const bool want64 = !is_single<T> && !split_rr && rns_pays(N, nx);
+    const bool want_split = !is_single<T> && split;
+    const bool want_low = is_single<T> || o.precision == CHASE_SPLIT_BF16_ADAPT;
+    const int low = rns_low_moduli(N);
+    const size_t reserve = rns_reserve(N, nx);
+    CHASE_TRY(rns_alloc_x(d, N, nx, want64 ? kRnsFp64 : want_split ? rns_split_moduli(N) : low, is_cplx<T>, rx));
+    if constexpr (is_single<T>) {
+      if (split) {
+        lD = ld_pad<Wide>(N);
+        CHASE_TRY(d.alloc(&Dv, static_cast<size_t>(lD) * nx));
+        CHASE_TRY(d.alloc(&Dw, static_cast<size_t>(lD) * nx));
+      }
+    }
+    if (want_split) CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), reserve, hsplit));
+    if (want_low) CHASE_TRY(rns_prepare_h(d, dH, N, lh, low, reserve, hlow));
+    if (want64) CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, reserve, h64));
+    filter_set.full = want_split ? &hsplit : want64 ? &h64 : nullptr;
+    filter_set.low = want_low ? &hlow : nullptr;
+    filter_set.x = &rx;
+    rr_set.full = want64 ? &h64 : split_rr ? &hsplit : nullptr;
+    rr_set.low = want_low ? &hlow : nullptr;
+    rr_set.x = &rx;
     return CHASE_OK;
   }
 
@@ -812,15 +860,15 @@ struct Solver {
       if (split) {  // widen, filter on the split product, round back
         CHASE_TRY(launch_convert(d, Va(), lv, Dv, lD, N, b()));
         CHASE_TRY(filter_groups(d, static_cast<const Wide*>(nullptr), N, lD, Dv, lD, Dw, lD,
-                                groups, maxdeg, b_sup, mu1, mu_nn, &fm, &sh, &sx, &low));
+                                groups, maxdeg, b_sup, mu1, mu_nn, &fm, &filter_set, &low));
         CHASE_TRY(launch_convert(d, Dv, lD, Va(), lv, N, b()));
       } else {
         CHASE_TRY(filter_groups(d, dH, N, lh, Va(), lv, Wk, lw, groups, maxdeg, b_sup, mu1, mu_nn,
-                                &fm, nullptr, &sx));
+                                &fm, rns ? &filter_set : nullptr));
       }
     } else {
       CHASE_TRY(filter_groups(d, dH, N, lh, Va(), lv, Wk, lw, groups, maxdeg, b_sup, mu1, mu_nn,
-                              &fm, split ? &sh : nullptr, &sx, &low));
+                              &fm, rns ? &filter_set : nullptr, &low));
     }
     tm.end();
     S.filter_slices_low += low > 0 ? 1 : 0;
@@ -873,8 +921,7 @@ struct Solver {
     // lines 7-8: Rayleigh-Ritz on the active block, residuals
     tm.begin(&S.t_rr);
     CHASE_TRY(rr_core(d, dH, N, lh, va, lv, nb, dw, dres, rw, &S.t_eigh, &S.flops_total,
-                      split_rr ? rr_slices : nullptr, split_rr ? rr_sx : nullptr,
-                      &S.t_rr_product));
+                      &S.t_rr_product, rns && (rr_set.full || rr_set.low) ? &rr_set : nullptr));
     S.flops_rr_product += kMv * N2 * nb;
     CHASE_CUDA(cudaMemcpyAsync(ra.data(), dw, sizeof(double) * nb, cudaMemcpyDeviceToHost, d.st));
     CHASE_CUDA(cudaMemcpyAsync(rr.data(), dres, sizeof(double) * nb, cudaMemcpyDeviceToHost, d.st));
@@ -1191,20 +1238,23 @@ int filter_impl(const T* H, int64_t N, int64_t ldh, T* V, int64_t ldv, int b, co
   CHASE_CUDA(cudaMemcpyAsync(start.data(), dstart, sizeof(int) * start.size(), cudaMemcpyDeviceToHost, d.st));
   CHASE_CUDA(cudaMemcpyAsync(&maxdeg, dinfo, sizeof(int), cudaMemcpyDeviceToHost, d.st));
   CHASE_TRY(d.sync_check("chase_filter plan"));
-  SplitH sh;
-  SplitX sx;
-  const bool split = precision != CHASE_FP64;
-  const int nslices = precision == CHASE_SPLIT_BF16_4 ? 4 : precision == CHASE_SPLIT_BF16_3 ? 3 : 7;
-  if constexpr (!is_single<T>) {
-    if (split) {
-      CHASE_TRY(split_prepare_h(d, dH, N, lh, sh));
-      CHASE_TRY(split_alloc_x(d, N, b, sx, is_cplx<T>));
-    }
+  const bool rns = precision != CHASE_FP64 || rns_pays(N, b);
+  RnsH rh;
+  RnsX rx;
+  RnsSet rs;
+  if (rns) {
+    const int nmod = is_single<T> || precision == CHASE_SPLIT_BF16_4 || precision == CHASE_SPLIT_BF16_3
+                         ? rns_low_moduli(N)
+                         : precision == CHASE_FP64 ? kRnsFp64 : rns_split_moduli(N);
+    CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), rh));
+    rs.full = &rh;
+    rs.x = &rx;
   }
   // sorted copy into the workspace; V becomes the second buffer
   CHASE_TRY(launch_permute_cols(d, dV, lv, wk, lw, N, b, dperm, false));
   CHASE_TRY(filter_sorted(d, dH, N, lh, wk, lw, dV, lv, b, start.data(), maxdeg, b_sup, mu1,
-                          mu_nevnex, nullptr, split ? &sh : nullptr, &sx, nslices));
+                          mu_nevnex, nullptr, rns ? &rs : nullptr));
   CHASE_TRY(launch_permute_cols(d, wk, lw, dV, lv, N, b, dperm, true));
   if (dV != V)
     CHASE_TRY(copy_block(d, V, ldv, dV, lv, N, b,
@@ -1316,13 +1366,25 @@ extern "C" int chase_filter_mixed(const chase_c64* H, int64_t N, int64_t ldh, ch
   int* dperm = nullptr;
   CHASE_TRY(d.alloc(&dperm, b));
   CHASE_CUDA(cudaMemcpyAsync(dperm, order.data(), sizeof(int) * b, cudaMemcpyHostToDevice, d.st));
-  SplitH sh;
-  SplitX sx;
-  CHASE_TRY(split_prepare_h(d, dH, N, lh, sh));
-  CHASE_TRY(split_alloc_x(d, N, b, sx, true));
+  RnsH full, low;
+  RnsX rx;
+  RnsSet rs;
+  rs.x = &rx;
+  const bool any_low = *std::min_element(ns.begin(), ns.end()) < 7;
+  const bool any_full = *std::max_element(ns.begin(), ns.end()) == 7;
+  const int nlow = rns_low_moduli(N);
+  CHASE_TRY(rns_alloc_x(d, N, b, any_full ? rns_split_moduli(N) : nlow, true, rx));
+  if (any_full) {
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), rns_reserve(N, b), full));
+    rs.full = &full;
+  }
+  if (any_low) {
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nlow, rns_reserve(N, b), low));
+    rs.low = &low;
+  }
   CHASE_TRY(launch_permute_cols(d, dV, lv, wk, lw, N, b, dperm, false));
   CHASE_TRY(filter_groups(d, dH, N, lh, wk, lw, dV, lv, groups, maxdeg, b_sup, mu1, mu_nevnex,
-                          nullptr, &sh, &sx));
+                          nullptr, &rs));
   CHASE_TRY(launch_permute_cols(d, wk, lw, dV, lv, N, b, dperm, true));
   if (dV != V)
     CHASE_TRY(copy_block(d, V, ldv, dV, lv, N, b,
@@ -1419,8 +1481,18 @@ extern "C" int chase_rayleigh_ritz(const chase_c64* H, int64_t N, int64_t ldh, c
   double *dw = nullptr, *dr = nullptr;
   CHASE_TRY(d.alloc(&dw, b));
   if (resid) CHASE_TRY(d.alloc(&dr, b));
+  RnsH rh;
+  RnsX rx;
+  RnsSet rs;
+  const bool rns = rns_pays(N, b);
+  if (rns) {
+    CHASE_TRY(rns_alloc_x(d, N, b, kRnsFp64, true, rx));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, rns_reserve(N, b), rh));
+    rs.full = &rh;
+    rs.x = &rx;
+  }
   double te = 0.0, fl = 0.0;
-  CHASE_TRY(rr_core(d, dH, N, lh, dQ, lq, b, dw, dr, w, &te, &fl));
+  CHASE_TRY(rr_core(d, dH, N, lh, dQ, lq, b, dw, dr, w, &te, &fl, nullptr, rns ? &rs : nullptr));
   if (!dev) CHASE_TRY(copy_block(d, Q, ldq, dQ, lq, N, b, cudaMemcpyDeviceToHost));
   CHASE_CUDA(cudaMemcpyAsync(ritz, dw, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
   if (resid) CHASE_CUDA(cudaMemcpyAsync(resid, dr, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
@@ -1455,7 +1527,16 @@ int residuals_impl(const T* H, int64_t N, int64_t ldh, const T* V, int64_t ldv, 
   CHASE_TRY(d.alloc(&dl, b));
   CHASE_TRY(d.alloc(&dr, b));
   CHASE_CUDA(cudaMemcpyAsync(dl, lambda, sizeof(double) * b, cudaMemcpyHostToDevice, d.st));
-  CHASE_TRY(gemm(d, N, N, dH, lh, dV, lv, b, HV, lw, 0, b, 1.0, 0.0, 0.0));
+  if (rns_pays(N, b)) {
+    RnsH rh;
+    RnsX rx;
+    const int nmod = is_single<T> ? rns_low_moduli(N) : kRnsFp64;
+    CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), rh));
+    CHASE_TRY(rns_product(d, rh, rx, dV, lv, 0, b, HV, lw, 1.0, 0.0, 0.0));
+  } else {
+    CHASE_TRY(gemm(d, N, N, dH, lh, dV, lv, b, HV, lw, 0, b, 1.0, 0.0, 0.0));
+  }
   CHASE_TRY(launch_resid_norms(d, HV, lw, dV, lv, N, b, dl, dr));
   CHASE_CUDA(cudaMemcpyAsync(resid, dr, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
   return d.sync_check("chase_residuals");

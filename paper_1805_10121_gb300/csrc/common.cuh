@@ -129,7 +129,7 @@ int make_tmap_c64(CUtensorMap* map, const void* base, int64_t rows, int64_t cols
 int make_tmap_f64(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld,
                   int box_rows, int box_cols);
 // A 3-D bf16 tensor {d0, d1, d2} with byte strides s1 (dim 1) and s2 (dim 2),
-// box {b0, b1, b2}, 32-byte swizzle (b0 * 2 must be 32).
+// box {b0, b1, b2}; swizzle as wide as the box row (b0 * 2 = 32, 64 or 128).
 int make_tmap_bf16_3d(CUtensorMap* map, const void* base, int64_t d0, int64_t d1, int64_t d2,
                       int64_t s1, int64_t s2, int b0, int b1, int b2);
 

@@ -32,6 +32,8 @@ struct Dev {
   int alloc(T** p, size_t count) {
     return alloc_bytes(reinterpret_cast<void**>(p), count * sizeof(T));
   }
+  // Give an allocation of this context back before the context ends.
+  void release(void* p);
   // Synchronise the stream and turn the device error flag into a status.
   int sync_check(const char* where);
 };
@@ -190,6 +192,47 @@ int zgemm_split(Dev& d, const SplitH& h, SplitX& x, const chase_c64* X, int64_t 
                 int nslices = 7);
 int zgemm_split(Dev& d, const SplitH& h, SplitX& x, const double* X, int64_t ldx, int j0, int j1,
                 double* C, int64_t ldc, double alpha, double beta, double shift, int nslices = 7);
+
+// ---- rns.cu: products with H in residue arithmetic on the tensor cores -----
+// Moduli per accuracy: kRnsFp64 stands in for FP64 GEMMs (operands rounded to
+// 2^-60 of a row's or column's 2-norm), rns_split_moduli(N) for the split
+// filter (2^-48), rns_low_moduli(N) for its reduced precisions and for single
+// precision (2^-30).
+constexpr int kRnsMaxModuli = 14;
+constexpr int kRnsFp64 = 14;
+int rns_split_moduli(int64_t N);
+int rns_low_moduli(int64_t N);
+// Residue planes of H (per modulus two planes of N x Kp bf16 for complex H,
+// one for real), row exponents and the real diagonal, which the epilogue
+// applies in FP64.  resident < nmod: memory holds only that many moduli at a
+// time, and every product slices H anew (src, lds) for each group of them.
+struct RnsH {
+  void* A = nullptr;
+  int* E = nullptr;
+  double* Dg = nullptr;
+  int64_t N = 0, Kp = 0;
+  int cplx = 1, nmod = 0, resident = 0;
+  const void* src = nullptr;
+  int64_t lds = 0;
+  int src_kind = 0;  // 0 complex128, 1 float64, 2 complex64, 3 float32
+};
+// Workspace for up to cap_cols columns at a time: residue planes of the block
+// (B), of the product (G), column exponents.
+struct RnsX {
+  void* B = nullptr;
+  int16_t* G = nullptr;
+  int* F = nullptr;
+  int cap_cols = 0, planes = 0;
+  int64_t Kp = 0, ldg = 0;
+};
+// reserve: bytes to leave free when the planes are large
+template <class T>
+int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, RnsH& out);
+int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX& out);
+// C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1]
+template <class T>
+int rns_product(Dev& d, const RnsH& h, RnsX& x, const T* X, int64_t ldx, int j0, int j1, T* C,
+                int64_t ldc, double alpha, double beta, double shift);
 
 // ---- grouped filter: many independent problems per launch ----------------
 // One problem of a grouped filter, in device memory.  buf0 holds the block

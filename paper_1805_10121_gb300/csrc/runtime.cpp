@@ -112,7 +112,7 @@ int make_tmap_bf16_3d(CUtensorMap* map, const void* base, int64_t d0, int64_t d1
     return CHASE_CUDA_ERROR;
   }
   if ((reinterpret_cast<uintptr_t>(base) & 15) != 0 || (s1 & 15) != 0 || (s2 & 15) != 0 ||
-      (b0 * 2 != 32 && b0 * 2 != 64)) {
+      (b0 * 2 != 32 && b0 * 2 != 64 && b0 * 2 != 128)) {
     set_error("bf16 tensor map: misaligned base/stride or box");
     return CHASE_INVALID_ARG;
   }
@@ -124,7 +124,9 @@ int make_tmap_bf16_3d(CUtensorMap* map, const void* base, int64_t d0, int64_t d1
   cuuint32_t estride[3] = {1, 1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), gdim, gstride,
                    box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   b0 * 2 == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+                   b0 * 2 == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
+                   : b0 * 2 == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
+                                  : CU_TENSOR_MAP_SWIZZLE_32B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     set_error("cuTensorMapEncodeTiled (bf16 3-D) failed (%d)", (int)r);
@@ -164,6 +166,15 @@ int Dev::alloc_bytes(void** p, size_t bytes) {
   }
   bufs.push_back(*p);
   return CHASE_OK;
+}
+
+void Dev::release(void* p) {
+  for (auto it = bufs.begin(); it != bufs.end(); ++it)
+    if (*it == p) {
+      bufs.erase(it);
+      cudaFreeAsync(p, st);
+      return;
+    }
 }
 
 int Dev::sync_check(const char* where) {

@@ -91,13 +91,16 @@ def poisson_trace(n_requests: int, rate: float, seed: int,
 
 def footprint_bytes(n: int, nev: int, nex: int, split: bool) -> int:
     """Device bytes a request holds while it runs: the current and next H
-    (complex128), the FFT generator's temporaries, the split slices of H,
+    (complex128), the FFT generator's temporaries, the residue planes of H,
     the resident block and the solver's N x (nev+nex) workspaces."""
     nx = nev + nex
     h = 16 * n * n
     gen = 3 * h                                   # construction temporaries
-    slices = 28 * n * n if split else 0          # 7 BF16 slice planes of [Re H | Im H]
-    blocks = 16 * n * nx * 10                    # V, filter buffer, RR/QR work, slices of V
+    # BF16 residue planes of H, two per modulus: 14 moduli for products at FP64
+    # accuracy, 11 more for a split filter
+    slices = (56 + (44 if split else 0)) * n * n
+    # V, filter buffer, RR/QR work; residue planes of the block and of the product
+    blocks = 16 * n * nx * 10 + 2 * 56 * n * nx
     return int(2 * h + gen + slices + blocks)
 
 
