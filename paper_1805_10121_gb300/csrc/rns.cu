@@ -36,7 +36,7 @@
 // both CTAs' warp 0 load their half of the operands by TMA (64-wide K,
 // 128-byte swizzle) into a ring of stages whose barriers live in the even
 // CTA; its warp 1 issues tcgen05.mma.cta_group::2 (M = 256, N = BN), so each
-// CTA reads only half of B from shared memory; warps 2-9 of each CTA reduce
+// CTA reads only half of B from shared memory; warps 2-17 of each CTA reduce
 // and store its 128 rows.  Persistent pairs walk the tiles of all residue
 // planes.  Every wait is bounded.
 #include <cuda_bf16.h>
@@ -56,7 +56,7 @@ constexpr int kModuli[kRnsMaxModuli] = {509, 505, 493, 481, 461, 457, 449,
                                         433, 421, 409, 401, 397, 389, 373};
 constexpr int BM = 128;          // rows per CTA (256 per pair)
 constexpr int BK = 64;           // K per stage: one 128-byte swizzle row
-constexpr int kEpiWarps = 8;     // two per TMEM lane quarter
+constexpr int kEpiWarps = 16;    // four per TMEM lane quarter
 constexpr int kThreads = (2 + kEpiWarps) * 32;
 constexpr int kLimbBits = 13;
 constexpr int kNonFinite = 0x7fffffff;  // exponent of a row or column with an Inf or NaN
@@ -74,21 +74,34 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::
                    : "memory");
 }
+// True in one lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t e;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(e));
+  return e != 0;
+}
 // Address, in the cluster's shared window, of the same variable in CTA `rank`.
 __device__ __forceinline__ uint32_t map_to_rank(const void* p, uint32_t rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
   return r;
 }
+// The barriers of a pair order TMA writes, MMAs and TMEM reads, all of which
+// complete before the arrival that announces them (complete_tx, commit,
+// tcgen05.wait::ld); no generic-proxy data passes between the CTAs.  So CTA
+// scope is enough: at cluster scope every wait and arrival drained the warp's
+// memory pipe first, the largest stall of the GEMM (N = 4096, 788 columns, 22
+// planes: 701 -> 669 us).
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(bar)
-               : "memory");
+  asm volatile("mbarrier.arrive.release.cta.shared::cluster.b64 _, [%0];\n" ::"r"(bar) : "memory");
 }
 __device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity) {
   uint32_t done;
   asm volatile(
       "{\n .reg .pred p;\n"
-      " mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+      " mbarrier.try_wait.parity.acquire.cta.shared::cta.b64 p, [%1], %2;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(done)
       : "r"(smem_u32(bar)), "r"(parity)
@@ -141,14 +154,40 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
-#define RNS_TMEM_LD16(taddr, r)                                                                      \
-  asm volatile(                                                                                      \
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}," \
-      " [%16];\n"                                                                                    \
-      : "=r"((r)[0]), "=r"((r)[1]), "=r"((r)[2]), "=r"((r)[3]), "=r"((r)[4]), "=r"((r)[5]),          \
-        "=r"((r)[6]), "=r"((r)[7]), "=r"((r)[8]), "=r"((r)[9]), "=r"((r)[10]), "=r"((r)[11]),        \
-        "=r"((r)[12]), "=r"((r)[13]), "=r"((r)[14]), "=r"((r)[15])                                   \
-      : "r"(taddr))
+// 8 columns of this thread's row of an accumulator, as 4 column pairs.  The
+// loads are complete after tmem_wait_ld, through which their registers pass so
+// that no use of them can be scheduled before it.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, unsigned long long (&r)[4]) {
+  uint32_t u[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+               : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
+                 "=r"(u[7])
+               : "r"(taddr));
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    r[i] = static_cast<unsigned long long>(u[2 * i]) |
+           static_cast<unsigned long long>(u[2 * i + 1]) << 32;
+}
+__device__ __forceinline__ void tmem_wait_ld(unsigned long long (&r)[4]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+l"(r[0]), "+l"(r[1]), "+l"(r[2]), "+l"(r[3])::"memory");
+}
+// Two FP32 operations in one instruction, each rounded as its scalar form.
+__device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
+  return static_cast<unsigned long long>(__float_as_uint(lo)) |
+         static_cast<unsigned long long>(__float_as_uint(hi)) << 32;
+}
+__device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b,
+                                                        unsigned long long c) {
+  unsigned long long d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, unsigned long long b) {
+  unsigned long long d;
+  asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 
 // 2^e as a double from its exponent bits, for -1022 <= e <= 1023.
 __device__ __forceinline__ double pow2_normal(int e) {
@@ -168,7 +207,7 @@ struct Cfg {
   static constexpr int NSTAGE = 196608 / STAGE > 8 ? 8 : 196608 / STAGE;
   static constexpr int BUF = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;
   static constexpr int TMEM = 2 * BUF;  // two accumulators
-  static constexpr int HC = BN / 2;     // columns per epilogue warp
+  static constexpr int HC = BN / 4;     // columns per epilogue warp
   // more than half an SM's shared memory: one CTA per SM, so the pairs of
   // concurrent kernels never wait for one another's TMEM
   static constexpr int SMEM = 1024 + NSTAGE * STAGE + 256;
@@ -245,8 +284,13 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
 
+  // Warps 0 and 1 run their loops with all lanes, and one elected lane issues:
+  // with only lane 0 in the loop the operands of every TMA and MMA went
+  // through per-instruction transfers to uniform registers, and the tensor
+  // pipe idled between the MMAs of a stage (same product: 669 -> 528 us).
+  const bool leader = elect_one();
   if (warp == 0) {
-    if (lane == 0) {  // ---------------- TMA producer (both CTAs)
+    {  // ---------------- TMA producer (both CTAs)
       long long g = 0;  // stages issued by this CTA
       bool ok = true;
       const CUtensorMap* last = nullptr;
@@ -254,14 +298,16 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
         Tile T;
         tile(t, T);
         if (T.mapA != last) {
-          if (maps_in_global) {
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(T.mapA)
-                         : "memory");
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(T.mapB)
-                         : "memory");
+          if (leader) {
+            if (maps_in_global) {
+              asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(T.mapA)
+                           : "memory");
+              asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;\n" ::"l"(T.mapB)
+                           : "memory");
+            }
+            prefetch_tmap(T.mapA);
+            prefetch_tmap(T.mapB);
           }
-          prefetch_tmap(T.mapA);
-          prefetch_tmap(T.mapB);
           last = T.mapA;
         }
         const int ra = T.row0 + static_cast<int>(rank) * BM;
@@ -270,25 +316,29 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
           const int st = static_cast<int>(g % NSTAGE);
           if (g >= NSTAGE &&
               !wait_cluster_bounded(&empty[st], static_cast<uint32_t>((g / NSTAGE) & 1) ^ 1u)) {
-            atomicOr(err, KERR_TIMEOUT_EMPTY);
+            if (leader) atomicOr(err, KERR_TIMEOUT_EMPTY);
             ok = false;
             break;
           }
-          if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * C::STAGE);
           const uint32_t bar = map_to_rank(&full[st], 0);
-          tma_load_pair(smem_u32(sA + st * C::A_BYTES), T.mapA, ks * BK, ra, T.planeA, bar);
-          tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
+          if (leader) {
+            if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * C::STAGE);
+            tma_load_pair(smem_u32(sA + st * C::A_BYTES), T.mapA, ks * BK, ra, T.planeA, bar);
+            tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
+          }
+          __syncwarp();
         }
       }
       // no copy may be in flight when the pair ends (the even CTA's barriers
       // count the copies of both; the odd CTA waits at the cluster barrier)
       if (rank == 0)
         for (long long k = (g > NSTAGE ? g - NSTAGE : 0); k < g; ++k)
-          if (!wait_cluster_bounded(&full[k % NSTAGE], static_cast<uint32_t>((k / NSTAGE) & 1)))
+          if (!wait_cluster_bounded(&full[k % NSTAGE], static_cast<uint32_t>((k / NSTAGE) & 1)) &&
+              leader)
             atomicOr(err, KERR_TIMEOUT_FULL);
     }
   } else if (warp == 1) {
-    if (rank == 0 && lane == 0) {  // ---------------- MMA issuer
+    if (rank == 0) {  // ---------------- MMA issuer
       // kind::f16: FP32 D, BF16 A and B, K-major, M = 256, N = BN
       constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
                                  ((uint32_t)(2 * BM >> 4) << 24);
@@ -305,38 +355,41 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
             ++c;
             if (c >= 2 && !wait_cluster_bounded(&acc_empty[c & 1],
                                                 static_cast<uint32_t>((c >> 1) & 1) ^ 1u)) {
-              atomicOr(err, KERR_TIMEOUT_FULL);
+              if (leader) atomicOr(err, KERR_TIMEOUT_FULL);
               ok = false;
               break;
             }
           }
           const int st = static_cast<int>(g % NSTAGE);
           if (!wait_cluster_bounded(&full[st], static_cast<uint32_t>((g / NSTAGE) & 1))) {
-            atomicOr(err, KERR_TIMEOUT_FULL);
+            if (leader) atomicOr(err, KERR_TIMEOUT_FULL);
             ok = false;
             break;
           }
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           const uint32_t a0 = smem_u32(sA + st * C::A_BYTES), b0 = smem_u32(sB + st * C::B_BYTES);
           const uint32_t d = tmem + static_cast<uint32_t>(c & 1) * C::BUF;
+          const bool last = in + 1 == cs || ks == T.nst - 1;
+          if (leader) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k)
-            umma_pair(d, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc,
-                      (in == 0 && k == 0) ? 0u : 1u);
-          commit_pair(&empty[st]);
-          if (++in == cs || ks == T.nst - 1) {
-            commit_pair(&acc_full[c & 1]);
-            in = 0;
+            for (int k = 0; k < BK / 16; ++k)
+              umma_pair(d, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc,
+                        (in == 0 && k == 0) ? 0u : 1u);
+            commit_pair(&empty[st]);
+            if (last) commit_pair(&acc_full[c & 1]);
           }
+          __syncwarp();
+          in = last ? 0 : in + 1;
         }
       }
       // every MMA of this pair has completed when this fires
-      commit_pair(done);
-      if (!wait_cluster_bounded(done, 0)) atomicOr(err, KERR_TIMEOUT_FULL);
+      if (leader) commit_pair(done);
+      __syncwarp();
+      if (!wait_cluster_bounded(done, 0) && leader) atomicOr(err, KERR_TIMEOUT_FULL);
     }
   } else {
-    // ---------------- reduction (warps 2..9): lanes 32 (w % 4) .. +31 (one
-    // row each), half hf of the columns
+    // ---------------- reduction (warps 2..17): lanes 32 (w % 4) .. +31 (one
+    // row each), quarter hf of the columns
     const int q = warp & 3;
     const int hf = (warp - 2) >> 2;
     const int rit = static_cast<int>(rank) * BM + q * 32 + lane;  // row in the tile
@@ -348,9 +401,15 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
       Tile T;
       tile(t, T);
       const Modulus m = tab.m[T.modulus];
-      float acc[C::HC];
+      // column pairs: packed FP32 arithmetic halves the instructions of what
+      // bounded the kernel then (same product: 528 -> 442 us; four warps per
+      // lane quarter instead of two, a load ahead: 426 us, 1.36 PFLOP/s)
+      unsigned long long acc[C::HC / 2];
 #pragma unroll
-      for (int j = 0; j < C::HC; ++j) acc[j] = 0.f;
+      for (int j = 0; j < C::HC / 2; ++j) acc[j] = 0ull;
+      const unsigned long long invp2 = pack_f32x2(m.invp, m.invp), mp2 = pack_f32x2(-m.p, -m.p),
+                               rnd2 = pack_f32x2(kRound, kRound),
+                               mrnd2 = pack_f32x2(-kRound, -kRound);
       for (int left = T.nst; left > 0; left -= m.chunk, ++c) {
         if (!wait_cluster_bounded(&acc_full[c & 1], static_cast<uint32_t>((c >> 1) & 1))) {
           if (lane == 0) atomicOr(err, KERR_TIMEOUT_FULL);
@@ -359,20 +418,19 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
         }
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const uint32_t tb = tbase + static_cast<uint32_t>(c & 1) * C::BUF;
+        // the load of the next 8 columns is in flight while these are reduced
+        unsigned long long r[2][4];
+        tmem_ld8(tb, r[0]);
 #pragma unroll
-        for (int j0 = 0; j0 < C::HC; j0 += 32) {
-          constexpr int kMost = C::HC < 32 ? C::HC : 32;
-          uint32_t r[32];
-          RNS_TMEM_LD16(tb + j0, r);
-          if (j0 + 16 < C::HC) RNS_TMEM_LD16(tb + j0 + 16, r + 16);
-          asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+        for (int j0 = 0; j0 < C::HC; j0 += 8) {
+          tmem_wait_ld(r[(j0 / 8) & 1]);
+          if (j0 + 8 < C::HC) tmem_ld8(tb + j0 + 8, r[(j0 / 8 + 1) & 1]);
 #pragma unroll
-          for (int j = 0; j < kMost; ++j) {
-            if (j0 + j >= C::HC) break;
+          for (int j = 0; j < 4; ++j) {
             // |v| <= 2^24, an integer; v - p rint(v / p), exact
-            const float v = __uint_as_float(r[j]);
-            const float k = __fadd_rn(fmaf(v, m.invp, kRound), -kRound);
-            acc[j0 + j] += fmaf(-k, m.p, v);
+            const unsigned long long v = r[(j0 / 8) & 1][j];
+            const unsigned long long k = add_f32x2(fma_f32x2(v, invp2, rnd2), mrnd2);
+            acc[j0 / 2 + j] = add_f32x2(acc[j0 / 2 + j], fma_f32x2(k, mp2, v));
           }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -387,8 +445,10 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
 #pragma unroll
         for (int j = 0; j < C::HC; ++j) {
           if (cb + j < T.ncols) {
-            const float k = __fadd_rn(fmaf(acc[j], m.invp, kRound), -kRound);
-            const float x = fmaf(-k, m.p, acc[j]);
+            const float a = __uint_as_float(
+                static_cast<uint32_t>(j % 2 ? acc[j / 2] >> 32 : acc[j / 2]));
+            const float k = __fadd_rn(fmaf(a, m.invp, kRound), -kRound);
+            const float x = fmaf(-k, m.p, a);
             // the low bits of x + 1.5 * 2^23 are x as a two's complement integer
             gp[j * T.ldg] = static_cast<int16_t>(__float_as_uint(__fadd_rn(x, kRound)) & 0xffffu);
           }
