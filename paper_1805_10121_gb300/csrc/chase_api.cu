@@ -260,7 +260,6 @@ template <class T>
 struct OrthWork {
   T* P = nullptr;     // nconv x b, leading dimension ld_pad(nconv)
   T* G = nullptr;     // b x b, leading dimension ld_pad(b)
-  T* Rinv = nullptr;  // panel workspace of the blocked Cholesky / solve, >= 32 b
   double* nrm = nullptr;  // b
 };
 
@@ -269,32 +268,101 @@ int orth_alloc(Dev& d, int64_t N, int nconv, int b, OrthWork<T>& w) {
   (void)N;
   CHASE_TRY(d.alloc(&w.P, static_cast<size_t>(ld_pad<T>(std::max(nconv, 1))) * b));
   CHASE_TRY(d.alloc(&w.G, static_cast<size_t>(ld_pad<T>(b)) * b));
-  CHASE_TRY(d.alloc(&w.Rinv, static_cast<size_t>(std::max(b, 32)) * b));
   CHASE_TRY(d.alloc(&w.nrm, static_cast<size_t>(b)));
   return CHASE_OK;
 }
 
+// Products of tall blocks: in residue arithmetic from the size on that products
+// with H take it (N = 1000, 70 columns: V^H V in 40 us, 357 us on the FP64
+// pipe, whose grid a product this small does not fill), else, or where the
+// planes do not fit the memory, on the FP64 pipe.
+template <class T>
+bool dense_pays(int64_t N, int b) {
+  return !is_single<T> && rns_pays(N, b);
+}
+
+// C (p x q) = X^H Y; lower: at least the lower triangle.  X == Y slices once.
+template <class T>
+int tall_gram(Dev& d, int64_t N, const T* X, int64_t ldx, int p, const T* Y, int64_t ldy, int q,
+              T* C, int64_t ldc, bool lower = false) {
+  if constexpr (!is_single<T>) {
+    if (dense_pays<T>(N, q)) {
+      RnsBlock x, y;
+      const bool same = X == Y && p == q && ldx == ldy;
+      int st = rns_columns(d, Y, ldy, N, q, y);
+      if (st == CHASE_OK && !same) st = rns_columns(d, X, ldx, N, p, x);
+      if (st == CHASE_OK) st = rns_dense(d, same ? y : x, true, y, C, ldc, 1.0, 0.0);
+      rns_release(d, x);
+      rns_release(d, y);
+      if (st != CHASE_OUT_OF_MEMORY) return st;
+    }
+  }
+  return gram(d, N, X, ldx, p, Y, ldy, q, C, ldc, lower);
+}
+
+// C (N x b) = alpha A (N x k) B (k x b) + beta C, C apart from A and B.
+template <class T>
+int tall_gemm(Dev& d, int64_t N, int k, const T* A, int64_t lda, const T* B, int64_t ldb, int b,
+              T* C, int64_t ldc, double alpha, double beta) {
+  if constexpr (!is_single<T>) {
+    if (dense_pays<T>(N, b)) {
+      RnsBlock x, y;
+      int st = rns_columns(d, B, ldb, k, b, y);
+      if (st == CHASE_OK) st = rns_rows(d, A, lda, N, k, x);
+      if (st == CHASE_OK) st = rns_dense(d, x, false, y, C, ldc, alpha, beta);
+      rns_release(d, x);
+      rns_release(d, y);
+      if (st != CHASE_OUT_OF_MEMORY) return st;
+    }
+  }
+  return gemm(d, N, k, A, lda, B, ldb, b, C, ldc, 0, b, alpha, beta, 0.0);
+}
+
+// V (N x b) <- V R (b x b) in place.
+template <class T>
+int tall_update(Dev& d, int64_t N, T* V, int64_t ldv, const T* R, int64_t ldr, int b) {
+  if (dense_pays<T>(N, b)) {  // the residue planes of V are its copy
+    RnsBlock x, y;
+    int st = rns_columns(d, R, ldr, b, b, y);
+    if (st == CHASE_OK) st = rns_rows(d, V, ldv, N, b, x);
+    if (st == CHASE_OK) st = rns_dense(d, x, false, y, V, ldv, 1.0, 0.0);
+    rns_release(d, x);
+    rns_release(d, y);
+    if (st != CHASE_OUT_OF_MEMORY) return st;
+  }
+  // panels of rows through a small buffer
+  const int64_t rows = std::min<int64_t>(N, 4096), ldt = ld_pad<T>(rows);
+  T* t = nullptr;
+  CHASE_TRY(d.alloc(&t, static_cast<size_t>(ldt) * b));
+  for (int64_t r0 = 0; r0 < N; r0 += rows) {
+    const int64_t n = std::min(rows, N - r0);
+    CHASE_TRY(gemm(d, n, b, V + r0, ldv, R, ldr, b, t, ldt, 0, b, 1.0, 0.0, 0.0));
+    CHASE_TRY(copy_block(d, V + r0, ldv, t, ldt, n, b, cudaMemcpyDeviceToDevice));
+  }
+  d.release(t);
+  return CHASE_OK;
+}
+
 // One Cholesky QR pass in two halves: cholqr_launch projects V against Y
-// and factors its Gram matrix (a breakdown sets KERR_CHOL_BREAKDOWN in d.err,
-// read at the caller's next synchronisation); cholqr_finish applies the
-// factor, V <- V L^-H.
+// and turns its Gram matrix L L^H into L^-H (a breakdown sets
+// KERR_CHOL_BREAKDOWN in d.err, read at the caller's next synchronisation);
+// cholqr_finish applies it, V <- V L^-H.
 template <class T>
 int cholqr_launch(Dev& d, int64_t N, const T* Y, int64_t ldy, int nconv, T* V, int64_t ldv,
                   int b, OrthWork<T>& w, double shift, double* flops) {
   const int64_t ldp = ld_pad<T>(nconv), ldg = ld_pad<T>(b);
   if (nconv > 0) {  // V <- V - Y (Y^H V)
-    CHASE_TRY(gram(d, N, Y, ldy, nconv, V, ldv, b, w.P, ldp));
-    CHASE_TRY(gemm(d, N, nconv, Y, ldy, w.P, ldp, b, V, ldv, 0, b, -1.0, 1.0, 0.0));
+    CHASE_TRY(tall_gram(d, N, Y, ldy, nconv, V, ldv, b, w.P, ldp));
+    CHASE_TRY(tall_gemm(d, N, nconv, Y, ldy, w.P, ldp, b, V, ldv, -1.0, 1.0));
     *flops += (is_cplx<T> ? 16.0 : 4.0) * N * nconv * b;
   }
-  CHASE_TRY(gram(d, N, V, ldv, b, V, ldv, b, w.G, ldg, /*lower=*/true));  // the factor reads only it
-  return cholesky_blocked(d, w.G, ldg, b, Prec<T>::chol_tol, shift, w.nrm, w.Rinv);
+  CHASE_TRY(tall_gram(d, N, V, ldv, b, V, ldv, b, w.G, ldg, /*lower=*/true));
+  return cholesky_inverse(d, w.G, ldg, b, Prec<T>::chol_tol, shift, w.nrm);
 }
 
 template <class T>
 int cholqr_finish(Dev& d, int64_t N, T* V, int64_t ldv, int b, OrthWork<T>& w, double* flops) {
-  // V <- V L^-H (= V R^-1 with R = L^H), in place
-  CHASE_TRY(trsm_right_lh(d, V, ldv, N, w.G, ld_pad<T>(b), b, w.Rinv));
+  CHASE_TRY(tall_update(d, N, V, ldv, w.G, ld_pad<T>(b), b));
   *flops += (is_cplx<T> ? 1.0 : 0.25) *
             (8.0 * N * b * b + 4.0 * N * b * b + 8.0 * b * b * b / 3.0);
   return CHASE_OK;
@@ -416,7 +484,7 @@ int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, 
   if (t_hq) tq.end();
   // G = Q^H H Q is Hermitian up to rounding: form its lower triangle (the one
   // the eigensolver reads) and take the upper one from it
-  CHASE_TRY(gram(d, N, Q, ldq, b, w.HQ, lN, b, w.G, lg, /*lower=*/true));
+  CHASE_TRY(tall_gram(d, N, Q, ldq, b, w.HQ, lN, b, w.G, lg, /*lower=*/true));
   return launch_fill_upper_hermitian(d, w.G, lg, b);
 }
 
@@ -424,10 +492,10 @@ template <class T>
 int rr_post(Dev& d, int64_t N, T* Q, int64_t ldq, int b, const double* w_dev, double* res_dev,
             RRWork<T>& w, double* flops) {
   const int64_t lN = ld_pad<T>(N), lg = ld_pad<T>(b);
-  CHASE_TRY(gemm(d, N, b, Q, ldq, w.G, lg, b, w.T2, lN, 0, b, 1.0, 0.0, 0.0));  // Q W
+  CHASE_TRY(tall_gemm(d, N, b, Q, ldq, w.G, lg, b, w.T2, lN, 1.0, 0.0));  // Q W
   if (res_dev) {
     // H (Q W) = (H Q) W: the residual reuses the product with H
-    CHASE_TRY(gemm(d, N, b, w.HQ, lN, w.G, lg, b, w.T3, lN, 0, b, 1.0, 0.0, 0.0));
+    CHASE_TRY(tall_gemm(d, N, b, w.HQ, lN, w.G, lg, b, w.T3, lN, 1.0, 0.0));
     CHASE_TRY(launch_resid_norms(d, w.T3, lN, w.T2, lN, N, b, w_dev, res_dev));
   }
   CHASE_TRY(copy_block(d, Q, ldq, w.T2, lN, N, b, cudaMemcpyDeviceToDevice));

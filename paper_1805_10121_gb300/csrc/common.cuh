@@ -107,6 +107,14 @@ __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
   asm volatile("prefetch.tensormap [%0];\n" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
 }
 
+// Programmatic dependent launch: a kernel launched with launch_pdl starts its
+// blocks as the kernel before it drains, and must call pdl_wait before it
+// reads or writes what that one touched.  pdl_next lets the next one start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+}
+
 // D = A(8x4, row) * B(4x8, col) + D on the FP64 tensor pipe.
 // Fragment layout: a = A[lane/4][lane%4], b = B[lane%4][lane/4],
 // d = {D[lane/4][2*(lane%4)], D[lane/4][2*(lane%4)+1]}.
@@ -116,6 +124,24 @@ __device__ __forceinline__ void dmma_8x8x4(double& d0, double& d1, double a, dou
                : "d"(a), "d"(b));
 }
 #endif  // __CUDACC__
+
+#ifdef __CUDACC__
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
 
 // ----------------------------------------------------------------------------
 // Host: tensor maps

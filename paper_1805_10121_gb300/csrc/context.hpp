@@ -95,19 +95,13 @@ int launch_resid_norms(Dev& d, const T* HV, int64_t ldhv, const T* V, int64_t ld
 // diagonal made real: the Hermitian matrix that G's lower triangle defines.
 template <class T>
 int launch_fill_upper_hermitian(Dev& d, T* G, int64_t ldg, int p);
-// In-place lower Cholesky G = L L^H (one CTA); sets KERR_CHOL_BREAKDOWN when a
-// pivot is not above rel_tol * G_jj.  `shift` is added to the diagonal first.
+// G (p x p, its lower triangle) = L L^H becomes L^-H: upper triangular, zeros
+// below the diagonal.  Sets KERR_CHOL_BREAKDOWN when a pivot is not above
+// rel_tol * G_jj.  `shift` is added to the diagonal first; diag_ref: p doubles
+// of workspace.
 template <class T>
-int launch_cholesky(Dev& d, T* G, int64_t ldg, int p, double rel_tol, double shift);
-// Blocked Cholesky (32-wide panels, trailing updates on the FP64 GEMM); the
-// pivot test uses the diagonal of G + shift before any update (diag_ref, p
-// doubles of workspace); work holds >= 32 p entries.
-template <class T>
-int cholesky_blocked(Dev& d, T* G, int64_t ldg, int p, double rel_tol, double shift,
-                     double* diag_ref, T* work);
-// X (N x p) <- X L^-H (blocked right-side triangular solve); work >= 32 p entries.
-template <class T>
-int trsm_right_lh(Dev& d, T* X, int64_t ldx, int64_t N, const T* L, int64_t ldl, int p, T* work);
+int cholesky_inverse(Dev& d, T* G, int64_t ldg, int p, double rel_tol, double shift,
+                     double* diag_ref);
 // One Lanczos three-term step on r independent runs (one CTA per run, run c
 // in column c of each N x r block, leading dimension ld):
 // alpha = Re(v^H w); w -= alpha v + beta_prev v_prev; beta = ||w||;
@@ -233,6 +227,25 @@ int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX
 template <class T>
 int rns_product(Dev& d, const RnsH& h, RnsX& x, const T* X, int64_t ldx, int j0, int j1, T* C,
                 int64_t ldc, double alpha, double beta, double shift);
+
+// Products of tall blocks (orthogonalisation, Rayleigh-Ritz) at FP64 accuracy.
+// n vectors of K entries in residue planes: the columns of a block, or its rows.
+// Memory comes with the vectors and goes with rns_release; CHASE_OUT_OF_MEMORY
+// leaves nothing behind and nothing changed.
+struct RnsBlock {
+  void* P = nullptr;
+  int* E = nullptr;
+  int64_t n = 0, K = 0, Kp = 0;
+};
+template <class T>
+int rns_columns(Dev& d, const T* X, int64_t ldx, int64_t K, int n, RnsBlock& out);
+template <class T>
+int rns_rows(Dev& d, const T* X, int64_t ldx, int64_t M, int K, RnsBlock& out);
+void rns_release(Dev& d, RnsBlock& b);
+// C[r, c] = alpha sum_k (a_r or conj(a_r))[k] b_c[k] + beta C[r, c]
+template <class T>
+int rns_dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, T* C, int64_t ldc,
+              double alpha, double beta);
 
 // ---- grouped filter: many independent problems per launch ----------------
 // One problem of a grouped filter, in device memory.  buf0 holds the block

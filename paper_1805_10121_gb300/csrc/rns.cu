@@ -465,7 +465,7 @@ __device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const 
 struct OneProduct {
   const CUtensorMap* mapA;
   const CUtensorMap* mapB;
-  int rtiles, ctiles, plane0, per_modulus, bn, nst, M, ncols;
+  int rtiles, ctiles, plane0, per_modulus, swap_a, bn, nst, M, ncols;
   int16_t* G;
   long long ldg, gplane;
   __device__ __forceinline__ void operator()(int t, Tile& T) const {
@@ -475,7 +475,7 @@ struct OneProduct {
     T.mapB = mapB;
     T.row0 = rt * 2 * BM;
     T.col0 = ct * bn;
-    T.planeA = pl;
+    T.planeA = pl ^ swap_a;
     T.planeB = plane0 + pl;
     T.modulus = T.planeB / per_modulus;
     T.nst = nst;
@@ -490,9 +490,11 @@ template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmTab tab, int rtiles, int ctiles, int nplanes,
-                    int plane0, int per_modulus, int nst, int M, int ncols, int16_t* __restrict__ G,
+                    int plane0, int per_modulus, int swap_a, int nst, int M, int ncols,
+                    int16_t* __restrict__ G,
                     long long ldg, long long gplane, int* __restrict__ err) {
-  OneProduct p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, BN, nst, M, ncols, G, ldg, gplane};
+  OneProduct p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, BN, nst, M, ncols,
+               G, ldg, gplane};
   gemm_body<BN>(p, rtiles * ctiles * nplanes, tab, 0, err);
 }
 
@@ -667,6 +669,45 @@ __device__ __forceinline__ int scale_exponent(float ss, uint32_t mb, int off, fl
   return static_cast<int>(floorf(L - margin - 0.5f * log2f(ss))) - off;
 }
 
+// Residues in planes [m0, m1) of two neighbouring integers (xr + i xi).
+template <int NM, int NL, bool CP>
+__device__ __forceinline__ void store_residues(const long long (&xr)[2], const long long (&xi)[2],
+                                               __nv_bfloat16* __restrict__ o, long long stride,
+                                               const SliceTab& tab, int m0, int m1) {
+  float lr[2][NL], li[2][NL];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    limbs<NL>(xr[h], lr[h]);
+    if constexpr (CP) limbs<NL>(xi[h], li[h]);
+  }
+  unsigned long long pr[NL], pi[NL];
+#pragma unroll
+  for (int i = 0; i < NL; ++i) {
+    pr[i] = pack_f32x2(lr[0][i], lr[1][i]);
+    if constexpr (CP) pi[i] = pack_f32x2(li[0][i], li[1][i]);
+  }
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+    if (m < m0 || m >= m1) continue;
+    const SliceMod& t = tab.m[m];
+    unsigned long long nr = pr[0];
+#pragma unroll
+    for (int i = 1; i < NL; ++i) nr = fma_f32x2(pr[i], t.c[i], nr);
+    if constexpr (CP) {
+      unsigned long long ni = fma_f32x2(pi[0], t.jc[0], 0ull);
+#pragma unroll
+      for (int i = 1; i < NL; ++i) ni = fma_f32x2(pi[i], t.jc[i], ni);
+      *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(add_f32x2(nr, ni), t));
+      *reinterpret_cast<uint32_t*>(o + stride) =
+          pack2(reduce2(fma_f32x2(ni, pack_f32x2(-1.f, -1.f), nr), t));
+      o += 2 * stride;
+    } else {
+      *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(nr, t));
+      o += stride;
+    }
+  }
+}
+
 // One vector of n entries (a column of X, or column r of the Hermitian H as
 // row r conjugated) to its residues in planes [m0, m1): element k of plane
 // (m - m0) goes to out[plane * stride + k].  skip: index left out (set to
@@ -718,49 +759,20 @@ __device__ __forceinline__ void slice_vector(const E* __restrict__ v, int n, boo
   if (threadIdx.x == 0) *exponent = s;
   const bool zero = s == kNonFinite;
   for (int k = 2 * threadIdx.x; k < n; k += 2 * kSliceThreads) {
-    float lr[2][NL], li[2][NL];
+    long long xr[2] = {}, xi[2] = {};
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      long long xr = 0, xi = 0;
       if (k + h < n && k + h != skip && !zero) {
         const E e = v[k + h];
-        xr = scaled_int(re_in(e), s);
+        xr[h] = scaled_int(re_in(e), s);
         if constexpr (CP) {
-          xi = scaled_int(im_in(e), s);
-          if (conj) xi = -xi;
+          xi[h] = scaled_int(im_in(e), s);
+          if (conj) xi[h] = -xi[h];
         }
       }
-      limbs<NL>(xr, lr[h]);
-      if constexpr (CP) limbs<NL>(xi, li[h]);
-    }
-    unsigned long long pr[NL], pi[NL];
-#pragma unroll
-    for (int i = 0; i < NL; ++i) {
-      pr[i] = pack_f32x2(lr[0][i], lr[1][i]);
-      if constexpr (CP) pi[i] = pack_f32x2(li[0][i], li[1][i]);
     }
     // rows are padded to 64 entries, so the second of a pair is inside
-    __nv_bfloat16* o = out + k;
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      if (m < m0 || m >= m1) continue;
-      const SliceMod& t = tab.m[m];
-      unsigned long long nr = pr[0];
-#pragma unroll
-      for (int i = 1; i < NL; ++i) nr = fma_f32x2(pr[i], t.c[i], nr);
-      if constexpr (CP) {
-        unsigned long long ni = fma_f32x2(pi[0], t.jc[0], 0ull);
-#pragma unroll
-        for (int i = 1; i < NL; ++i) ni = fma_f32x2(pi[i], t.jc[i], ni);
-        *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(add_f32x2(nr, ni), t));
-        *reinterpret_cast<uint32_t*>(o + stride) =
-            pack2(reduce2(fma_f32x2(ni, pack_f32x2(-1.f, -1.f), nr), t));
-        o += 2 * stride;
-      } else {
-        *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(nr, t));
-        o += stride;
-      }
-    }
+    store_residues<NM, NL, CP>(xr, xi, out + k, stride, tab, m0, m1);
   }
 }
 
@@ -789,6 +801,95 @@ __global__ void __launch_bounds__(kSliceThreads)
   const int c = blockIdx.x;
   slice_vector<NM, NL, E>(X + static_cast<long long>(j0 + c) * ldx, N, false, -1, B + c * Kp, plane,
                           Fx + c, tab, 0, NM);
+}
+
+// Rows of a column-major X (M x K) as vectors: row r of plane q goes to
+// out[q * plane + r * Kp]. A block takes 32 rows; reads are coalesced along
+// the rows, and a 32 x 64 tile of scaled integers in shared memory turns them
+// into stores along K.  Bound by the 2 bytes per plane and entry it writes.
+constexpr int kRowBlock = 32;
+template <int NM, int NL, class E>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_slice_rows_kernel(const E* __restrict__ X, long long ldx, int M, int K,
+                          const __grid_constant__ SliceTab tab, __nv_bfloat16* __restrict__ out,
+                          long long Kp, long long plane, int* __restrict__ Ex) {
+  constexpr bool CP = is_complex<E>;
+  constexpr int W = CP ? 2 : 1;
+  constexpr int G = kSliceThreads / kRowBlock;  // threads per row
+  __shared__ float sf[G][kRowBlock];
+  __shared__ uint32_t su[G][kRowBlock];
+  __shared__ long long tile[W][kRowBlock][65];
+  const int row = threadIdx.x % kRowBlock, grp = threadIdx.x / kRowBlock;
+  const int r0 = blockIdx.x * kRowBlock;
+  const bool in = r0 + row < M;
+  const E* x = X + r0 + row;
+  float ss = 0.f;
+  uint32_t mb = 0, any = 0;
+  if (in)
+    for (int k = grp; k < K; k += G) {
+      const E e = x[k * ldx];
+      const float fa = abs_f32(re_in(e), 0), fb = CP ? abs_f32(im_in(e), 0) : 0.f;
+      ss = fmaf(fa, fa, fmaf(fb, fb, ss));
+      mb = max(mb, max(abs_hi(re_in(e)), abs_hi(im_in(e))));
+      any |= low_word(re_in(e)) | low_word(im_in(e));
+    }
+  if (mb == 0 && any != 0) mb = 1;
+  auto reduce_rows = [&]() {
+    __syncthreads();
+    sf[grp][row] = ss;
+    su[grp][row] = mb;
+    __syncthreads();
+    ss = 0.f;
+    mb = 0;
+#pragma unroll
+    for (int g = 0; g < G; ++g) {
+      ss += sf[g][row];
+      mb = max(mb, su[g][row]);
+    }
+  };
+  reduce_rows();
+  int off = 0;
+  const bool again = (mb < kSafeLo || mb >= kSafeHi) && mb >= (1u << 20) && mb < 0x7FF00000u;
+  if (__syncthreads_or(again)) {
+    const float before = ss;
+    if (again) off = static_cast<int>(mb >> 20) - 1023;
+    ss = 0.f;
+    if (in && again)
+      for (int k = grp; k < K; k += G) {
+        const E e = x[k * ldx];
+        const float fa = abs_f32(re_in(e), off), fb = CP ? abs_f32(im_in(e), off) : 0.f;
+        ss = fmaf(fa, fa, fmaf(fb, fb, ss));
+      }
+    reduce_rows();
+    if (!again) ss = before;
+  }
+  const int s = scale_exponent(ss, mb, off, (CP ? 2.f : 1.f) * K, tab.log2_norm);
+  if (grp == 0 && in) Ex[r0 + row] = s;
+  const bool zero = s == kNonFinite;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int k0 = 0; k0 < K; k0 += 64) {
+    __syncthreads();
+    for (int kk = grp; kk < 64; kk += G) {
+      long long a = 0, b = 0;
+      if (in && k0 + kk < K && !zero) {
+        const E e = x[(k0 + kk) * ldx];
+        a = scaled_int(re_in(e), s);
+        if constexpr (CP) b = scaled_int(im_in(e), s);
+      }
+      tile[0][row][kk] = a;
+      if constexpr (CP) tile[W - 1][row][kk] = b;
+    }
+    __syncthreads();
+    for (int q = warp; q < kRowBlock && r0 + q < M; q += kSliceThreads / 32) {
+      long long xr[2], xi[2] = {};
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        xr[h] = tile[0][q][2 * lane + h];
+        if constexpr (CP) xi[h] = tile[W - 1][q][2 * lane + h];
+      }
+      store_residues<NM, NL, CP>(xr, xi, out + (r0 + q) * Kp + k0 + 2 * lane, plane, tab, 0, NM);
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1117,6 +1218,7 @@ struct GemmArgs {
   const void* B;
   int64_t b_rows, b_planes;  // B: b_planes of b_rows x Kp (plane stride), ncols rows used
   int ncols, nplanes, plane0, per_modulus;
+  int swap_a = 0;  // 1: A conjugated (the two planes of a modulus change places)
   int16_t* G;
   int64_t ldg, gplane;
   const GemmTab* tab;
@@ -1139,7 +1241,7 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
   const int64_t tiles = static_cast<int64_t>(rt) * ct * a.nplanes;
   const unsigned grid = 2 * static_cast<unsigned>(std::min<int64_t>(tiles, pairs));
   rns_gemm_kernel<BN><<<grid, kThreads, C::SMEM, d.st>>>(
-      tmA, tmB, *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus,
+      tmA, tmB, *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a,
       static_cast<int>((a.K + BK - 1) / BK), static_cast<int>(a.M), a.ncols, a.G, a.ldg, a.gplane,
       d.err);
   note_launch();
@@ -1290,6 +1392,67 @@ int product_any(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0,
   set_error("residue product: %d moduli", h.nmod);
   return CHASE_INVALID_ARG;
 }
+
+template <class E>
+int slice_columns(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
+  rns_slice_x_kernel<kRnsFp64, limbs_of(kRnsFp64), E>
+      <<<static_cast<unsigned>(b.n), kSliceThreads, 0, d.st>>>(
+          X, ldx, static_cast<int>(b.K), 0, tables(kRnsFp64, is_complex<E>).slice,
+          static_cast<__nv_bfloat16*>(b.P), b.Kp, b.n * b.Kp, b.E);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+template <class E>
+int slice_rows(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
+  rns_slice_rows_kernel<kRnsFp64, limbs_of(kRnsFp64), E>
+      <<<static_cast<unsigned>((b.n + kRowBlock - 1) / kRowBlock), kSliceThreads, 0, d.st>>>(
+          X, ldx, static_cast<int>(b.n), static_cast<int>(b.K),
+          tables(kRnsFp64, is_complex<E>).slice, static_cast<__nv_bfloat16*>(b.P), b.Kp,
+          b.n * b.Kp, b.E);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+template <class E>
+int dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, E* C, int64_t ldc,
+          double alpha, double beta) {
+  constexpr bool CP = is_complex<E>;
+  constexpr int PP = CP ? 2 : 1;
+  const Tables& t = tables(kRnsFp64, CP);
+  const int64_t ldg = (a.n + 7) / 8 * 8, gplane = ldg * b.n;
+  int16_t* G = nullptr;
+  CHASE_TRY(d.alloc(&G, static_cast<size_t>(gplane) * kRnsFp64 * PP));
+  GemmArgs g;
+  g.A = a.P;
+  g.K = a.K;
+  g.M = a.n;
+  g.Kp = a.Kp;
+  g.a_planes = kRnsFp64 * PP;
+  g.B = b.P;
+  g.b_rows = b.n;
+  g.b_planes = kRnsFp64 * PP;
+  g.ncols = static_cast<int>(b.n);
+  g.nplanes = kRnsFp64 * PP;
+  g.plane0 = 0;
+  g.per_modulus = PP;
+  g.swap_a = CP && conj_a ? 1 : 0;
+  g.G = G;
+  g.ldg = ldg;
+  g.gplane = gplane;
+  g.tab = &t.gemm;
+  CHASE_TRY(run_gemm(d, g));
+  const int gx = static_cast<int>((a.n + 255) / 256);
+  const dim3 grid(static_cast<unsigned>(gx),
+                  static_cast<unsigned>(std::min<int64_t>(b.n, std::max(1, 16 * 152 / gx))));
+  rns_crt_kernel<kRnsFp64, E><<<grid, 128, 0, d.st>>>(
+      G, ldg, gplane, t.crt, a.E, b.E, nullptr, static_cast<int>(a.n), static_cast<int>(b.n), 0,
+      nullptr, 0, C, ldc, crt_scale(t.crt, alpha, beta, 0.0));
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  d.release(G);
+  return CHASE_OK;
+}
 }  // namespace
 }  // namespace rns
 
@@ -1384,6 +1547,56 @@ int rns_product(Dev& d, const RnsH& h, RnsX& x, const T* X, int64_t ldx, int j0,
   return rns::product_any<D>(d, h, x, reinterpret_cast<const D*>(X), ldx, j0, j1,
                              reinterpret_cast<D*>(C), ldc, alpha, beta, shift);
 }
+
+namespace {
+template <class T>
+int alloc_block(Dev& d, int64_t n, int64_t K, RnsBlock& out) {
+  out.n = n;
+  out.K = K;
+  out.Kp = (K + rns::BK - 1) / rns::BK * rns::BK;
+  const size_t planes = kRnsFp64 * (rns::is_complex<typename Kind<T>::D> ? 2 : 1);
+  CHASE_TRY(d.alloc_bytes(&out.P, planes * n * out.Kp * 2));
+  const int st = d.alloc(&out.E, static_cast<size_t>(n));
+  if (st != CHASE_OK) rns_release(d, out);
+  return st;
+}
+}  // namespace
+
+template <class T>
+int rns_columns(Dev& d, const T* X, int64_t ldx, int64_t K, int n, RnsBlock& out) {
+  using D = typename Kind<T>::D;
+  CHASE_TRY(alloc_block<T>(d, n, K, out));
+  return rns::slice_columns<D>(d, reinterpret_cast<const D*>(X), ldx, out);
+}
+
+template <class T>
+int rns_rows(Dev& d, const T* X, int64_t ldx, int64_t M, int K, RnsBlock& out) {
+  using D = typename Kind<T>::D;
+  CHASE_TRY(alloc_block<T>(d, M, K, out));
+  return rns::slice_rows<D>(d, reinterpret_cast<const D*>(X), ldx, out);
+}
+
+void rns_release(Dev& d, RnsBlock& b) {
+  if (b.P) d.release(b.P);
+  if (b.E) d.release(b.E);
+  b = RnsBlock{};
+}
+
+template <class T>
+int rns_dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, T* C, int64_t ldc,
+              double alpha, double beta) {
+  using D = typename Kind<T>::D;
+  return rns::dense<D>(d, a, conj_a, b, reinterpret_cast<D*>(C), ldc, alpha, beta);
+}
+
+#define CHASE_INSTANTIATE_DENSE(T)                                                                 \
+  template int rns_columns<T>(Dev&, const T*, int64_t, int64_t, int, RnsBlock&);                   \
+  template int rns_rows<T>(Dev&, const T*, int64_t, int64_t, int, RnsBlock&);                      \
+  template int rns_dense<T>(Dev&, const RnsBlock&, bool, const RnsBlock&, T*, int64_t, double,     \
+                            double);
+CHASE_INSTANTIATE_DENSE(chase_c64)
+CHASE_INSTANTIATE_DENSE(double)
+#undef CHASE_INSTANTIATE_DENSE
 
 #define CHASE_INSTANTIATE_RNS(T)                                                                 \
   template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, RnsH&);           \
