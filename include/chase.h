@@ -199,6 +199,12 @@ long long chase_kernel_launches(void);
  * Instrumentation (the paper has no counterpart); never fails. */
 long long chase_device_allocations(void);
 
+/* Workspace comes from a stream-ordered memory pool that the library keeps per
+ * device; between calls it holds at most 1/16 of the device's memory for the
+ * next ones.  This hands all that is not in use back to the driver (after the
+ * calling program has synchronised; a call in flight keeps what it uses). */
+int chase_release_workspace(void);
+
 /* Kernel timing, for benchmarks (the paper has no counterpart).  While
  * timing is on, the library records a pair of CUDA events on the launching
  * stream around the launches of its products with H:

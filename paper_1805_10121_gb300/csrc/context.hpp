@@ -40,6 +40,10 @@ struct Dev {
 
 bool is_device_ptr(const void* p);
 
+// Bytes that the library's pool on the current device holds but does not use:
+// free memory to the library although cudaMemGetInfo counts it as taken.
+size_t pool_idle_bytes();
+
 // Records a CUDA event pair on stream `s` around product launches while
 // chase_kernel_timing is on (a no-op otherwise).  end() gives the launches
 // the range covered and their algorithmic (FP64-equivalent) and executed

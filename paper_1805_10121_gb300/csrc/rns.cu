@@ -1505,6 +1505,7 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
   if (per * nmod > (size_t(16) << 30)) {
     size_t free_b = 0, total_b = 0;
     CHASE_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    free_b += pool_idle_bytes();
     while (out.resident > 1 && per * out.resident + reserve > free_b) out.resident /= 2;
   }
   int st = CHASE_OUT_OF_MEMORY;

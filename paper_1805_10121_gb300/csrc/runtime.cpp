@@ -144,10 +144,81 @@ Dev::~Dev() {
   if (sync_on_exit) cudaStreamSynchronize(st);
 }
 
+// ---------------------------------------------------------------------------
+// Workspace memory.  CUDA's default pool hands everything back to the driver
+// at each synchronisation, so every call mapped its workspace anew, about 2.4
+// ms per GB (filter N = 4096, 1.1 GB of residue planes: 2.4 of 9.8 ms).  The
+// library has a pool of its own per device, which keeps at most 1/16 of the
+// device's memory between calls, hands it back when an allocation fails and on
+// chase_release_workspace, and leaves the default pool's settings alone.
+// Stream-ordered like the default pool: safe with several threads and streams.
+// ---------------------------------------------------------------------------
+namespace {
+constexpr int kMaxPoolDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pool[kMaxPoolDevices] = {};
+bool g_pool_tried[kMaxPoolDevices] = {};
+
+// The current device's pool; nullptr (the default pool serves) if it has none.
+cudaMemPool_t device_pool() {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxPoolDevices) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (!g_pool_tried[dev]) {
+    g_pool_tried[dev] = true;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    size_t free_b = 0, total_b = 0;
+    cudaMemPool_t p = nullptr;
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+        cudaMemPoolCreate(&p, &props) == cudaSuccess) {
+      uint64_t keep = total_b / 16;
+      if (cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess)
+        g_pool[dev] = p;
+      else
+        cudaMemPoolDestroy(p);
+    }
+    cudaGetLastError();
+  }
+  return g_pool[dev];
+}
+
+cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t st) {
+  cudaMemPool_t pool = device_pool();
+  if (!pool) return cudaMallocAsync(p, bytes, st);
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  if (e == cudaErrorMemoryAllocation) {  // idle blocks of other sizes may be in the way
+    cudaGetLastError();
+    cudaStreamSynchronize(st);
+    cudaMemPoolTrimTo(pool, 0);
+    e = cudaMallocFromPoolAsync(p, bytes, pool, st);
+  }
+  return e;
+}
+}  // namespace
+
+size_t pool_idle_bytes() {
+  cudaMemPool_t pool = device_pool();
+  uint64_t reserved = 0, used = 0;
+  if (!pool ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return reserved > used ? static_cast<size_t>(reserved - used) : 0;
+}
+
 int Dev::init() {
   void* p = nullptr;
   g_allocs.fetch_add(1, std::memory_order_relaxed);
-  CHASE_CUDA(cudaMallocAsync(&p, sizeof(int), st));
+  CHASE_CUDA(pool_malloc(&p, sizeof(int), st));
   err = static_cast<int*>(p);
   CHASE_CUDA(cudaMemsetAsync(err, 0, sizeof(int), st));
   return CHASE_OK;
@@ -157,7 +228,7 @@ int Dev::alloc_bytes(void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return CHASE_OK;
   g_allocs.fetch_add(1, std::memory_order_relaxed);
-  cudaError_t e = cudaMallocAsync(p, bytes, st);
+  cudaError_t e = pool_malloc(p, bytes, st);
   if (e != cudaSuccess) {
     cudaGetLastError();
     set_error("device workspace allocation of %zu bytes failed: %s", bytes, cudaGetErrorString(e));
@@ -325,6 +396,16 @@ extern "C" int chase_kernel_timing_read(int kind, double* seconds, long long* la
   *launches = n;
   if (flops) *flops = f;
   if (tensor_flops) *tensor_flops = tf;
+  return CHASE_OK;
+}
+
+extern "C" int chase_release_workspace(void) {
+  std::lock_guard<std::mutex> lk(chase::g_pool_mu);
+  for (cudaMemPool_t p : chase::g_pool)
+    if (p) {
+      const cudaError_t e = cudaMemPoolTrimTo(p, 0);
+      if (e != cudaSuccess) return chase::cuda_status(e, "chase_release_workspace");
+    }
   return CHASE_OK;
 }
 
