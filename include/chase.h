@@ -67,13 +67,12 @@ typedef struct {
  * the BF16 tensor cores in residue arithmetic (exact products of the operands
  * rounded to 2^-60 of the 2-norm of a row of H or a column of the block, put
  * together and finished in FP64: no further from the exact product than an
- * FP64 GEMM); smaller ones, and the batched entry points, on the FP64 pipes. */
+ * FP64 GEMM); smaller ones on the FP64 pipes.  The batched entry points do the
+ * same for batches of 2e7 FLOPs and more per degree step. */
 #define CHASE_FP64 0
 /* Split: the same residue products with the operands rounded to 2^-48 of
- * those norms (the batched entry points: both operands cut into seven 7-bit
- * digits, each entry accurate to about 2^-49 max|off-diagonal row of H|
- * max|column| per term).  The diagonal of H and the recurrence's
- * shift/scale/axpby are applied in FP64.  Reads H through its Hermitian
+ * those norms.  The diagonal of H and the recurrence's shift/scale/axpby are
+ * applied in FP64.  Reads H through its Hermitian
  * symmetry.  QR, Rayleigh-Ritz, residuals and Lanczos keep FP64 accuracy. */
 #define CHASE_SPLIT_BF16 1
 /* Split-BF16 filter as above, and the product H Q of Rayleigh-Ritz (Alg. 2
@@ -152,8 +151,9 @@ typedef struct {
   long long filter_matvecs_low; /* filter column products made with fewer than 7 slices */
 } chase_stats;
 
-/* Tile choice of the grouped FP64 filter: time the candidates on the first
- * degree step (result cached per batch shape), or 0..3 for a fixed shape
+/* Tile choice of the grouped FP64 filter: residue products for batches of 2e7
+ * FLOPs and more per degree step, below that the candidates timed on the first
+ * degree step (result cached per batch shape); or 0..3 for a fixed shape
  * (0: 64 x 16, 1: 64 x 32, 2: 128 x 16, 3: 64 x 8 rows x complex columns). */
 #define CHASE_TILE_AUTO (-1)
 
@@ -162,7 +162,8 @@ typedef struct {
   int problems;            /* problems with work (N > 0 and b > 0) */
   int steps;               /* degree steps (the largest degree of the batch; summed over
                               the iterations of chase_solve_batched) */
-  int tile_config;         /* FP64 tile shape used (see CHASE_TILE_AUTO); -1 for split */
+  int tile_config;         /* FP64 tile shape used (see CHASE_TILE_AUTO); -1 for residue
+                              products (split, and FP64 batches of some size) */
   int launches;            /* kernel launches of the call (graph nodes counted once) */
   long long matvecs;       /* column products with H over all problems (sum of the degrees) */
   double flops;            /* 8 N^2 per column product, summed over problems */
@@ -475,8 +476,9 @@ int chase_solve_f32(const float* H, int64_t N, int64_t ldh, int nev, int nex, do
  * precision CHASE_FP64 or CHASE_SPLIT_BF16.
  * tile      CHASE_TILE_AUTO or a fixed FP64 tile shape (ignored for split).
  * stats     out, or NULL.
- * Workspace: N[p] x b[p] per problem (FP64), plus the slices of every H
- * (28 N[p]^2 bytes) for split; released before return.
+ * Workspace: N[p] x b[p] per problem, plus the residue planes of every H (44
+ * N[p]^2 bytes for split, 56 for FP64); where these do not all fit, parts of
+ * the batch are filtered in turn.  Released before return.
  * Errors: CHASE_INVALID_ARG (sizes, bounds, degrees, host H or V),
  * CHASE_OUT_OF_MEMORY, CHASE_CUDA_ERROR, CHASE_TIMEOUT.  On error V may hold
  * partial results. */

@@ -13,11 +13,12 @@
 // computed on the host once per call, and the whole sequence of step
 // launches is captured into a CUDA graph and launched once.
 //
-// FP64 products run on the DMMA kernel with one of four tile shapes chosen
-// by timing the first step (which only writes the second buffer, so it can
-// be repeated); the choice is cached per batch shape.  Split-BF16 products
-// slice the active columns of every problem in one launch per step and run
-// the tensor-core kernel with its fixed 128 x 32 complex tile.
+// Products run as residue GEMMs (rns.cu): per step one launch slices the
+// active columns of every problem, one multiplies, one puts the products
+// together.  FP64 batches that are too small for that, and those for which the
+// caller names a tile shape, run on the DMMA kernel; its shape is chosen by
+// timing the first step (which only writes the second buffer, so it can be
+// repeated), and the choice is cached per batch shape.
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -43,25 +44,28 @@ struct Coef {
   double c, e, sigma1;
 };
 
-// Step list of degree step i (1-based) for a tile shape bm x bn, where bn
-// counts B-map columns (complex columns for FP64, real ones for split);
-// real_cols = 2 for split, 1 for FP64.  sigma_prev[k] is sigma after step
-// i - 1 of problem k (Alg. 4 line 11).
+// Step list of degree step i (1-based): FP64 tiles of bm x bn complex columns,
+// or (nmod > 0) residue products with tiles bn columns wide.  sigma_prev[k] is
+// sigma after step i - 1 of problem k (Alg. 4 line 11).
+struct StepTotals {
+  int tiles = 0, cols = 0, blocks = 0;
+};
 void build_step(const std::vector<GroupedFilterInput>& in, const std::vector<Coef>& co, int i,
-                int bm, int bn, int real_cols, const std::vector<double>& sigma_prev,
-                std::vector<GroupedStep>& out, int* ntiles, int* ncols) {
+                int bm, int bn, int nmod, const std::vector<double>& sigma_prev,
+                std::vector<GroupedStep>& out, StepTotals* totals) {
   out.clear();
-  int tiles = 0, cols = 0;
+  StepTotals t;
   for (size_t k = 0; k < co.size(); ++k) {
     const GroupedFilterInput& pi = in[co[k].q];
     if (i > pi.maxdeg) continue;
     const int s = pi.start[i];
     if (s >= pi.b) continue;
-    GroupedStep g;
+    GroupedStep g{};
     g.prob = static_cast<int>(k);
     g.s = s;
-    g.tile0 = tiles;
-    g.col0 = cols;
+    g.tile0 = t.tiles;
+    g.col0 = t.cols;
+    g.blk0 = t.blocks;
     if (i == 1) {  // Alg. 4 line 4
       g.alpha = co[k].sigma1 / co[k].e;
       g.beta = 0.0;
@@ -72,19 +76,47 @@ void build_step(const std::vector<GroupedFilterInput>& in, const std::vector<Coe
       g.beta = -tau * sigma;
     }
     g.shift = co[k].c;
+    const int cols = pi.b - s;
+    if (nmod > 0) {
+      g.sc = rns_scale(nmod, g.alpha, g.beta, g.shift);
+      t.tiles += rns_grouped_tiles(nmod, bn, pi.n, cols);
+      t.blocks += rns_grouped_crt_blocks(pi.n, cols);
+    } else {
+      t.tiles += (pi.n + bm - 1) / bm * ((cols + bn - 1) / bn);
+    }
+    t.cols += cols;
     out.push_back(g);
-    const int rt = (pi.n + bm - 1) / bm;
-    const int ct = (real_cols * (pi.b - s) + bn - 1) / bn;
-    tiles += rt * ct;
-    cols += pi.b - s;
   }
   GroupedStep sentinel{};
   sentinel.prob = -1;
-  sentinel.tile0 = tiles;
-  sentinel.col0 = cols;
+  sentinel.tile0 = t.tiles;
+  sentinel.col0 = t.cols;
+  sentinel.blk0 = t.blocks;
   out.push_back(sentinel);
-  *ntiles = tiles;
-  *ncols = cols;
+  *totals = t;
+}
+
+// Width of the residue tiles of degree step i: the one with the least work,
+// counting a tile's padding columns.
+int residue_tile_width(const std::vector<GroupedFilterInput>& in, const std::vector<Coef>& co,
+                       int i, int nmod) {
+  int best = 32;
+  double best_cost = 0.0;
+  for (int bn = 32; bn <= 256; bn += 32) {
+    double cost = 0.0;
+    for (const Coef& c : co) {
+      const GroupedFilterInput& pi = in[c.q];
+      if (i > pi.maxdeg || pi.start[i] >= pi.b) continue;
+      // two stages' time for the start and the end of a tile
+      cost += rns_grouped_tiles(nmod, bn, pi.n, pi.b - pi.start[i]) * ((pi.n + 63) / 64 + 2.0) *
+              rns_stage_cost(bn);
+    }
+    if (best_cost == 0.0 || cost < 0.995 * best_cost) {
+      best_cost = cost;
+      best = bn;
+    }
+  }
+  return best;
 }
 
 std::mutex g_tune_mu;
@@ -126,26 +158,64 @@ float elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
 
 }  // namespace
 
-int grouped_split_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap) {
+// Residue products from 2e7 FLOPs a degree step on: below that the FP64 tiles
+// take less time than the three launches (about 20 us).
+int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile) {
+  int64_t most = 0;
+  double step = 0.0;
+  for (const GroupedFilterInput& g : in) {
+    most = std::max<int64_t>(most, g.n);
+    step += 8.0 * g.n * static_cast<double>(g.n) * g.b;
+  }
+  if (split) return rns_split_moduli(most);
+  return tile == CHASE_TILE_AUTO && step >= 2e7 ? kRnsFp64 : 0;
+}
+
+void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in) {
+  for (GroupedFilterInput& g : in) {
+    for (void* p : {g.A, static_cast<void*>(g.E), static_cast<void*>(g.Dg), g.Bsl, g.G,
+                    static_cast<void*>(g.F)})
+      if (p) d.release(p);
+    g.A = g.Bsl = g.G = nullptr;
+    g.E = g.F = nullptr;
+    g.Dg = nullptr;
+    g.bcap = 0;
+  }
+}
+
+namespace {
+int alloc_planes(Dev& d, GroupedFilterInput& g, int bcap, int nmod) {
+  const int64_t Kp = rns_k_padded(g.n);
+  g.bcap = std::max(bcap, 1);
+  const size_t block = static_cast<size_t>(2 * nmod) * g.bcap * Kp * 2;
+  CHASE_TRY(d.alloc_bytes(&g.A, static_cast<size_t>(2 * nmod) * g.n * Kp * 2));
+  CHASE_TRY(d.alloc(&g.E, static_cast<size_t>(g.n)));
+  CHASE_TRY(d.alloc(&g.Dg, static_cast<size_t>(g.n)));
+  CHASE_TRY(d.alloc_bytes(&g.Bsl, block));
+  CHASE_TRY(d.alloc_bytes(&g.G, block));
+  return d.alloc(&g.F, static_cast<size_t>(g.bcap));
+}
+}  // namespace
+
+int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
+                        int nmod) {
   std::vector<GroupedSliceH> hs;
   int rows = 0;
   for (size_t q = 0; q < in.size(); ++q) {
     GroupedFilterInput& g = in[q];
     if (g.n == 0) continue;
-    const int64_t Kp = split_k_padded(g.n);
-    CHASE_TRY(d.alloc_bytes(&g.A, static_cast<size_t>(kSplitSlices) * g.n * Kp * 2));
-    CHASE_TRY(d.alloc(&g.E, static_cast<size_t>(g.n)));
-    CHASE_TRY(d.alloc(&g.Dg, static_cast<size_t>(g.n)));
-    g.bcap = std::max(bcap[q], 1);
-    CHASE_TRY(d.alloc_bytes(&g.Bsl, static_cast<size_t>(kSplitSlices) * 2 * g.bcap * Kp * 2));
-    CHASE_TRY(d.alloc(&g.F, static_cast<size_t>(g.bcap)));
+    const int st = alloc_planes(d, g, bcap[q], nmod);
+    if (st != CHASE_OK) {
+      grouped_rns_release(d, in);
+      return st;
+    }
     GroupedSliceH sh;
     sh.H = reinterpret_cast<const double2*>(g.H);
     sh.ldh = g.ldh;
     sh.A = g.A;
     sh.E = g.E;
     sh.Dg = g.Dg;
-    sh.Kp = Kp;
+    sh.Kp = rns_k_padded(g.n);
     sh.n = g.n;
     sh.row0 = rows;
     hs.push_back(sh);
@@ -156,13 +226,16 @@ int grouped_split_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std
   CHASE_TRY(d.alloc(&dsl, hs.size()));
   CHASE_CUDA(cudaMemcpyAsync(dsl, hs.data(), sizeof(GroupedSliceH) * hs.size(),
                              cudaMemcpyHostToDevice, d.st));
-  CHASE_TRY(split_grouped_prepare_h(d, dsl, static_cast<int>(hs.size()), rows));
+  CHASE_TRY(rns_grouped_prepare_h(d, nmod, dsl, static_cast<int>(hs.size()), rows));
   // the host array must outlive the copy
-  return d.sync_check("grouped slices of H");
+  return d.sync_check("grouped residues of H");
 }
 
-int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, bool split, int tile,
-                          GroupedFilterTimes* times) {
+namespace {
+// The whole of `in` at once; prepared for residue products where nmod > 0.
+int filter_part(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int tile,
+                GroupedFilterTimes* times) {
+  const bool rns = nmod > 0;
   const long long launches0 = chase_kernel_launches();
   GroupedFilterTimes tt;
   // active problems, longest tiles first: the block scheduler then balances the tail
@@ -187,7 +260,7 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
     return CHASE_OK;
   }
   EventPool evp;
-  const int nmaps = split ? 2 : 3;
+  const int nmaps = rns ? 1 + 8 : 3;  // residues: H and a block map per tile width
   CUtensorMap* dmaps = nullptr;
   CHASE_TRY(d.alloc_bytes(reinterpret_cast<void**>(&dmaps), sizeof(CUtensorMap) * nmaps * Q));
   GroupedProblem* dprobs = nullptr;
@@ -206,24 +279,19 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
     g.ld1 = pi.ldw;
     g.mapA = dmaps + nmaps * k;
     g.mapB0 = dmaps + nmaps * k + 1;
-    g.mapB1 = split ? nullptr : dmaps + nmaps * k + 2;
-    if (split) {
+    g.mapB1 = rns ? nullptr : dmaps + nmaps * k + 2;
+    if (rns) {
       if (!pi.A || !pi.Bsl || pi.bcap < pi.b) {
-        set_error("grouped filter: slice workspace missing or too small");
+        set_error("grouped filter: residue workspace missing or too small");
         return CHASE_INVALID_ARG;
       }
-      const int64_t Kp = split_k_padded(pi.n);
-      g.Kp = Kp;
+      g.Kp = rns_k_padded(pi.n);
       g.E = pi.E;
       g.F = pi.F;
       g.Dg = pi.Dg;
       g.Bsl = pi.Bsl;
+      g.G = pi.G;
       g.bcap = pi.bcap;
-      CHASE_TRY(make_tmap_bf16_3d(&maps[nmaps * k], pi.A, 2LL * pi.n, pi.n, kSplitSlices, Kp * 2,
-                                  Kp * 2 * pi.n, kSplitStageK, kSplitTileRows, kSplitSlices));
-      CHASE_TRY(make_tmap_bf16_3d(&maps[nmaps * k + 1], pi.Bsl, 2LL * pi.n, 2LL * pi.b, kSplitSlices,
-                                  Kp * 2, Kp * 2 * 2 * pi.bcap, kSplitStageK, kSplitTileRealCols,
-                                  kSplitSlices));
     }
   }
   CHASE_CUDA(cudaMemcpyAsync(dprobs, probs.data(), sizeof(GroupedProblem) * Q, cudaMemcpyHostToDevice,
@@ -246,7 +314,20 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
   };
 
   int cfg = -1;
-  if (split) {
+  std::vector<int> width(maxdeg + 1, 0);  // residues: tile width of each step
+  if (rns) {
+    bool used[8] = {};
+    for (int i = 1; i <= maxdeg; ++i) {
+      width[i] = residue_tile_width(in, co, i, nmod);
+      used[width[i] / 32 - 1] = true;
+    }
+    for (int k = 0; k < Q; ++k) {
+      const GroupedFilterInput& pi = in[co[k].q];
+      for (int w = 0; w < 8; ++w)
+        if (used[w])
+          CHASE_TRY(rns_grouped_maps(&maps[nmaps * k], &maps[nmaps * k + 1 + w], nmod, 32 * (w + 1),
+                                     pi.A, pi.Bsl, pi.n, pi.b, pi.bcap));
+    }
     CHASE_CUDA(cudaMemcpyAsync(dmaps, maps.data(), sizeof(CUtensorMap) * maps.size(),
                                cudaMemcpyHostToDevice, d.st));
   } else if (tile != CHASE_TILE_AUTO) {
@@ -274,8 +355,8 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
         int bm = 0, bn = 0;
         grouped_fp64_tile(c, &bm, &bn);
         std::vector<GroupedStep> one;
-        int nt = 0, nc = 0;
-        build_step(in, co, 1, bm, bn, 1, sigma0, one, &nt, &nc);
+        StepTotals tot;
+        build_step(in, co, 1, bm, bn, 0, sigma0, one, &tot);
         GroupedStep* dst1 = nullptr;
         CHASE_TRY(d.alloc(&dst1, one.size()));
         CHASE_CUDA(cudaMemcpyAsync(dst1, one.data(), sizeof(GroupedStep) * one.size(),
@@ -288,9 +369,9 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
         }
         const int na = static_cast<int>(one.size()) - 1;
         // one untimed launch, then the timed one
-        CHASE_TRY(zgemm_grouped_fp64(d, c, dprobs, dst1, na, nt, 0));
+        CHASE_TRY(zgemm_grouped_fp64(d, c, dprobs, dst1, na, tot.tiles, 0));
         CHASE_CUDA(cudaEventRecord(ea, d.st));
-        CHASE_TRY(zgemm_grouped_fp64(d, c, dprobs, dst1, na, nt, 0));
+        CHASE_TRY(zgemm_grouped_fp64(d, c, dprobs, dst1, na, tot.tiles, 0));
         CHASE_CUDA(cudaEventRecord(eb, d.st));
         CHASE_TRY(d.sync_check("grouped filter autotune"));
         const float ms = elapsed_ms(ea, eb);
@@ -304,20 +385,19 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
       g_tune_cache[key] = cfg;
     }
   }
-  int bm = kSplitTileRows, bn = kSplitTileRealCols, realc = 2;
-  if (!split) {
+  int bm = 0, bn = 0;
+  if (!rns) {
     grouped_fp64_tile(cfg, &bm, &bn);
-    realc = 1;
     CHASE_TRY(encode_fp64_maps(cfg));
   }
   // ---- every step's list, uploaded once ----
   std::vector<GroupedStep> all, one;
-  std::vector<int> first(maxdeg + 1, 0), nact(maxdeg + 1, 0), ntiles(maxdeg + 1, 0),
-      ncols(maxdeg + 1, 0);
+  std::vector<int> first(maxdeg + 1, 0), nact(maxdeg + 1, 0);
+  std::vector<StepTotals> tot(maxdeg + 1);
   {
     std::vector<double> sigma(Q, 0.0);
     for (int i = 1; i <= maxdeg; ++i) {
-      build_step(in, co, i, bm, bn, realc, sigma, one, &ntiles[i], &ncols[i]);
+      build_step(in, co, i, bm, rns ? width[i] : bn, nmod, sigma, one, &tot[i]);
       first[i] = static_cast<int>(all.size());
       nact[i] = static_cast<int>(one.size()) - 1;
       all.insert(all.end(), one.begin(), one.end());
@@ -335,13 +415,13 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
                              cudaMemcpyHostToDevice, d.st));
 
   // ---- the degree steps, captured into one graph ----
-  CHASE_TRY(split ? zgemm_split_grouped_prepare() : zgemm_grouped_fp64_prepare(cfg));
+  CHASE_TRY(rns ? rns_grouped_ready() : zgemm_grouped_fp64_prepare(cfg));
   const double tg = now_s();
   GraphGuard gg;
   CHASE_CUDA(cudaStreamCreateWithFlags(&gg.cs, cudaStreamNonBlocking));
   std::vector<cudaEvent_t> pev;  // product start / end per step, inside the graph
   for (int i = 1; i <= maxdeg; ++i) {
-    if (ntiles[i] == 0) continue;
+    if (tot[i].tiles == 0) continue;
     cudaEvent_t a = evp.get(), z = evp.get();
     if (!a || !z) {
       set_error("grouped filter: event creation failed");
@@ -366,21 +446,23 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
     }
     size_t k = 0;
     for (int i = 1; i <= maxdeg && st == CHASE_OK; ++i) {
-      if (ntiles[i] == 0) continue;
+      if (tot[i].tiles == 0) continue;
       const int parity = (i - 1) & 1;
       const GroupedStep* sp = dsteps + first[i];
-      if (split) st = split_grouped_slice_x(d, dprobs, sp, nact[i], ncols[i], parity);
+      if (rns) st = rns_grouped_slice_x(d, nmod, dprobs, sp, nact[i], tot[i].cols, parity);
       if (st != CHASE_OK) break;
       // external records: real event nodes of the graph, so the product
       // launches can be timed apart from the slicing
       if (cudaEventRecordWithFlags(pev[k], gg.cs, cudaEventRecordExternal) != cudaSuccess)
         st = CHASE_CUDA_ERROR;
       if (st == CHASE_OK)
-        st = split ? zgemm_split_grouped(d, dprobs, sp, nact[i], ntiles[i], parity)
-                   : zgemm_grouped_fp64(d, cfg, dprobs, sp, nact[i], ntiles[i], parity);
+        st = rns ? rns_grouped_gemm(d, nmod, width[i], dprobs, sp, tot[i].tiles)
+                 : zgemm_grouped_fp64(d, cfg, dprobs, sp, nact[i], tot[i].tiles, parity);
       if (st == CHASE_OK &&
           cudaEventRecordWithFlags(pev[k + 1], gg.cs, cudaEventRecordExternal) != cudaSuccess)
         st = CHASE_CUDA_ERROR;
+      if (st == CHASE_OK && rns)
+        st = rns_grouped_crt(d, nmod, dprobs, sp, nact[i], tot[i].blocks, parity);
       k += 2;
     }
     const cudaError_t ec = cudaStreamEndCapture(gg.cs, &gg.g);
@@ -413,6 +495,55 @@ int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, boo
   tt.steps = maxdeg;
   tt.launches = static_cast<int>(chase_kernel_launches() - launches0);
   if (times) *times = tt;
+  return CHASE_OK;
+}
+
+void add_times(GroupedFilterTimes& to, const GroupedFilterTimes& t) {
+  to.tile_config = t.tile_config;
+  to.steps = std::max(to.steps, t.steps);
+  to.launches += t.launches;
+  to.matvecs += t.matvecs;
+  to.flops += t.flops;
+  to.t_autotune += t.t_autotune;
+  to.t_graph_build += t.t_graph_build;
+  to.t_steps += t.t_steps;
+  to.t_product += t.t_product;
+}
+
+// Residue planes for `in`, made and given back here; halves of the batch in
+// turn where they do not all fit, and FP64 tiles for a problem whose own do not.
+int filter_parts(Dev& d, std::vector<GroupedFilterInput> in, int nmod, int tile,
+                 GroupedFilterTimes& times) {
+  std::vector<int> bcap;
+  for (const GroupedFilterInput& g : in) bcap.push_back(g.b);
+  GroupedFilterTimes t;
+  int st = grouped_rns_prepare(d, in, bcap, nmod);
+  if (st == CHASE_OK) {
+    st = filter_part(d, in, nmod, tile, &t);
+    grouped_rns_release(d, in);
+    add_times(times, t);
+    return st;
+  }
+  if (st != CHASE_OUT_OF_MEMORY) return st;
+  if (in.size() > 1) {
+    const auto mid = in.begin() + static_cast<std::ptrdiff_t>(in.size() / 2);
+    CHASE_TRY(filter_parts(d, std::vector<GroupedFilterInput>(in.begin(), mid), nmod, tile, times));
+    return filter_parts(d, std::vector<GroupedFilterInput>(mid, in.end()), nmod, tile, times);
+  }
+  CHASE_TRY(filter_part(d, in, 0, CHASE_TILE_AUTO, &t));
+  add_times(times, t);
+  return CHASE_OK;
+}
+}  // namespace
+
+int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int tile,
+                          GroupedFilterTimes* times) {
+  bool ready = true;
+  for (const GroupedFilterInput& g : in) ready = ready && (g.n == 0 || g.b == 0 || g.A);
+  if (nmod == 0 || ready) return filter_part(d, in, nmod, tile, times);
+  GroupedFilterTimes t;
+  CHASE_TRY(filter_parts(d, in, nmod, tile, t));
+  if (times) *times = t;
   return CHASE_OK;
 }
 
@@ -515,7 +646,6 @@ extern "C" int chase_filter_batched(int P, const chase_c64* const* H, const int6
   hperm.reserve(totperm);
   std::vector<GroupedPermute> gat(Q), sca(Q);
   std::vector<GroupedFilterInput> in(Q);
-  std::vector<int> bcap(Q);
   int total_cols = 0;
   for (int q = 0; q < Q; ++q) {
     const int p = idx[q];
@@ -549,7 +679,6 @@ extern "C" int chase_filter_batched(int P, const chase_c64* const* H, const int6
     f.b_sup = b_sup[p];
     f.mu1 = mu1[p];
     f.mu_nn = mu_nevnex[p];
-    bcap[q] = b[p];
   }
   CHASE_CUDA(cudaMemcpyAsync(dperm, hperm.data(), sizeof(int) * hperm.size(), cudaMemcpyHostToDevice,
                              d.st));
@@ -558,9 +687,8 @@ extern "C" int chase_filter_batched(int P, const chase_c64* const* H, const int6
   CHASE_CUDA(cudaMemcpyAsync(dscatter, sca.data(), sizeof(GroupedPermute) * Q,
                              cudaMemcpyHostToDevice, d.st));
   CHASE_TRY(launch_grouped_permute(d, dgather, Q, total_cols, false));
-  if (split) CHASE_TRY(grouped_split_prepare(d, in, bcap));
   GroupedFilterTimes tt;
-  CHASE_TRY(grouped_filter_sorted(d, in, split, tile, &tt));
+  CHASE_TRY(grouped_filter_sorted(d, in, grouped_moduli(in, split, tile), tile, &tt));
   // every result is in the sorted copy (even degrees): back to the caller's order
   CHASE_TRY(launch_grouped_permute(d, dscatter, Q, total_cols, true));
   CHASE_TRY(d.sync_check("chase_filter_batched"));

@@ -460,27 +460,33 @@ int rr_alloc(Dev& d, int64_t N, int b, RRWork<T>& w) {
   return CHASE_OK;
 }
 
-// Alg. 2 in three parts: rr_pre forms H Q (FP64, or the split product for
-// CHASE_SPLIT_BF16_RR) and the lower triangle of G = Q^H (H Q) mirrored to
-// the upper one; the eigensolve of G follows (one problem: eigh_device, a
+// Alg. 2 in three parts: rr_pre forms H Q (with the residue planes of H in rs,
+// those it makes for this product alone, or on the FP64 pipe) and the lower
+// triangle of G = Q^H (H Q) mirrored to the upper one; the eigensolve of G follows (one problem: eigh_device, a
 // batch: eigh_batched); rr_post forms Q W, the residuals from (H Q) W, and
 // copies Q W into Q.
 template <class T>
 int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, int b,
-           RRWork<T>& w, const SplitH* sh = nullptr, SplitX* sx = nullptr,
-           double* t_hq = nullptr, const RnsSet* rs = nullptr) {
+           RRWork<T>& w, double* t_hq = nullptr, const RnsSet* rs = nullptr) {
   const int64_t lN = ld_pad<T>(N), lg = ld_pad<T>(b);
   PhaseTimer tq(d.st);  // the product alone (synchronises only when timed)
   if (t_hq) tq.begin(t_hq);
-  bool on_split = false;
+  bool done = false;
   if constexpr (!is_single<T>) {
-    if (sh) {  // H Q on the split product (CHASE_SPLIT_BF16_RR)
-      CHASE_TRY(zgemm_split(d, *sh, *sx, Q, ldq, 0, b, w.HQ, lN, 1.0, 0.0, 0.0));
-      on_split = true;
+    if (!rs && rns_pays(N, b)) {
+      RnsH h;
+      RnsX x;
+      int st = rns_alloc_x(d, N, b, kRnsFp64, is_cplx<T>, x);
+      if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, kRnsFp64, rns_reserve(N, b), h);
+      if (st == CHASE_OK) st = rns_product(d, h, x, Q, ldq, 0, b, w.HQ, lN, 1.0, 0.0, 0.0);
+      for (void* p : {h.A, static_cast<void*>(h.E), static_cast<void*>(h.Dg), x.B,
+                      static_cast<void*>(x.G), static_cast<void*>(x.F)})
+        if (p) d.release(p);
+      if (st != CHASE_OK && st != CHASE_OUT_OF_MEMORY) return st;
+      done = st == CHASE_OK;
     }
   }
-  if (!on_split)
-    CHASE_TRY(filter_product(d, H, N, ldh, rs, Q, ldq, b, w.HQ, lN, 0, 1.0, 0.0, 0.0));
+  if (!done) CHASE_TRY(filter_product(d, H, N, ldh, rs, Q, ldq, b, w.HQ, lN, 0, 1.0, 0.0, 0.0));
   if (t_hq) tq.end();
   // G = Q^H H Q is Hermitian up to rounding: form its lower triangle (the one
   // the eigensolver reads) and take the upper one from it
@@ -509,7 +515,7 @@ int rr_core(Dev& d, const T* H, int64_t N, int64_t ldh, T* Q, int64_t ldq, int b
             double* t_hq = nullptr, const RnsSet* rs = nullptr) {
   if (b == 0) return CHASE_OK;
   const int64_t lg = ld_pad<T>(b);
-  CHASE_TRY(rr_pre<T>(d, H, N, ldh, Q, ldq, b, w, nullptr, nullptr, t_hq, rs));
+  CHASE_TRY(rr_pre<T>(d, H, N, ldh, Q, ldq, b, w, t_hq, rs));
   PhaseTimer tm(d.st);
   tm.begin(t_eigh);
   CHASE_TRY(eigh_device(d, w.G, lg, b, w_dev));  // (W, Lambda) = TSOLVE(G)
@@ -710,8 +716,6 @@ struct Solver {
   int64_t lh = 0, lv = 0, ls = 0, lw = 0;
   OrthWork<T> ow;
   RRWork<T> rw;
-  SplitH sh;  // digit slices of the batched solve's split filter
-  SplitX sx;
   // H in residue planes: FP64 accuracy (FP64 filter, Rayleigh-Ritz), the split
   // filter's, and its reduced precisions / single precision
   RnsH h64, hsplit, hlow;
@@ -724,9 +728,10 @@ struct Solver {
   Wide *Dv = nullptr, *Dw = nullptr;
   int64_t lD = 0;
   bool split = false;
-  bool split_rr = false;              // H Q of Rayleigh-Ritz on the split product too
-  const SplitH* rr_slices = nullptr;  // batched solve: the slices of H used there
-  SplitX* rr_sx = nullptr;
+  bool split_rr = false;  // H Q of Rayleigh-Ritz on the split product too
+  // batched solve: rr_set holds the planes of its grouped filter where they
+  // have the precision that Rayleigh-Ritz asks for
+  bool rr_ready = false;
   double *dw = nullptr, *dres = nullptr;
   int* dperm = nullptr;
   // host state
@@ -1837,8 +1842,8 @@ int batched_after_filter(Dev& d, std::vector<Solver<chase_c64>*>& act,
   for (int i = 0; i < P; ++i) {
     Solver<T>& s = *act[i];
     const int nb = s.b();
-    CHASE_TRY(rr_pre(*view[i], s.dH, s.N, s.lh, s.Va(), s.lv, nb, s.rw,
-                     s.split_rr ? s.rr_slices : nullptr, s.split_rr ? s.rr_sx : nullptr));
+    CHASE_TRY(rr_pre(*view[i], s.dH, s.N, s.lh, s.Va(), s.lv, nb, s.rw, nullptr,
+                     s.rr_ready ? &s.rr_set : nullptr));
     items[i] = EighItem{s.rw.G, ld_pad<T>(nb), nb, wres + off[i]};
   }
   CHASE_TRY(join());
@@ -1973,28 +1978,38 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
                    });
   // Alg. 1 lines 1-2 of every problem
   CHASE_TRY(pool.run(all, [&](Dev& w, int p) { return sv[p].setup(w, true); }));
-  std::vector<GroupedFilterInput> slices(P);  // split: slices of every H, made once
-  if (split) {
-    std::vector<int> bcap(P);
-    for (int p = 0; p < P; ++p) {
-      slices[p].H = sv[p].dH;
-      slices[p].ldh = sv[p].lh;
-      slices[p].n = static_cast<int>(sv[p].N);
-      bcap[p] = sv[p].nx;
-    }
-    CHASE_TRY(grouped_split_prepare(d, slices, bcap));
-    for (int p = 0; p < P; ++p) {  // the same slices serve Rayleigh-Ritz's H Q
+  // residue planes of every H, made once where the memory holds them all
+  // (otherwise the filter makes them for parts of the batch in turn)
+  std::vector<GroupedFilterInput> planes(P);
+  std::vector<int> bcap(P);
+  for (int p = 0; p < P; ++p) {
+    planes[p].H = sv[p].dH;
+    planes[p].ldh = sv[p].lh;
+    planes[p].n = static_cast<int>(sv[p].N);
+    planes[p].b = bcap[p] = sv[p].nx;
+  }
+  const int nmod = grouped_moduli(planes, split, CHASE_TILE_AUTO);
+  if (nmod > 0) {
+    const int st = grouped_rns_prepare(d, planes, bcap, nmod);
+    if (st != CHASE_OK && st != CHASE_OUT_OF_MEMORY) return st;
+    for (int p = 0; p < P && st == CHASE_OK; ++p) {
       Solver<chase_c64>& s = sv[p];
-      s.sh.A = slices[p].A;
-      s.sh.E = slices[p].E;
-      s.sh.Dg = slices[p].Dg;
-      s.sh.N = s.N;
-      s.sh.Kp = split_k_padded(s.N);
-      s.sx.B = slices[p].Bsl;
-      s.sx.F = slices[p].F;
-      s.sx.cap_cols = slices[p].bcap;
-      s.rr_slices = &s.sh;
-      s.rr_sx = &s.sx;
+      RnsH& h = s.h64;
+      h.A = planes[p].A;
+      h.E = planes[p].E;
+      h.Dg = planes[p].Dg;
+      h.N = s.N;
+      h.Kp = s.rx.Kp = s.rx.ldg = rns_k_padded(s.N);
+      h.cplx = 1;
+      h.nmod = h.resident = nmod;
+      s.rx.B = planes[p].Bsl;
+      s.rx.G = static_cast<int16_t*>(planes[p].G);
+      s.rx.F = planes[p].F;
+      s.rx.cap_cols = planes[p].bcap;
+      s.rx.planes = 2 * nmod;
+      s.rr_set.full = &h;
+      s.rr_set.x = &s.rx;
+      s.rr_ready = s.split_rr || nmod == kRnsFp64;
     }
   }
   chase_batch_stats bs{};
@@ -2008,18 +2023,17 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
     in.reserve(act.size());
     for (int p : act) {
       GroupedFilterInput g = sv[p].filter_input();
-      if (split) {
-        g.A = slices[p].A;
-        g.E = slices[p].E;
-        g.Dg = slices[p].Dg;
-        g.Bsl = slices[p].Bsl;
-        g.F = slices[p].F;
-        g.bcap = slices[p].bcap;
-      }
+      g.A = planes[p].A;
+      g.E = planes[p].E;
+      g.Dg = planes[p].Dg;
+      g.Bsl = planes[p].Bsl;
+      g.G = planes[p].G;
+      g.F = planes[p].F;
+      g.bcap = planes[p].bcap;
       in.push_back(g);
     }
     GroupedFilterTimes tt;
-    CHASE_TRY(grouped_filter_sorted(d, in, split, CHASE_TILE_AUTO, &tt));  // line 4, grouped
+    CHASE_TRY(grouped_filter_sorted(d, in, nmod, CHASE_TILE_AUTO, &tt));  // line 4, grouped
     bs.steps += tt.steps;
     bs.tile_config = tt.tile_config;
     bs.matvecs += tt.matvecs;

@@ -157,40 +157,6 @@ inline int gram(Dev& d, int64_t N, const float* X, int64_t ldx, int p, const flo
   return sgram(d, N, X, ldx, p, Y, ldy, q, C, ldc, lower);
 }
 
-// ---- zgemm_split.cu: split-BF16 filter product on the tensor cores --------
-// Slices of H (S planes of N x Kp bf16) and row exponents: complex H gives
-// Ht = [Re H | Im H] (Kp >= 2N), real symmetric H itself (Kp >= N).
-struct SplitH {
-  void* A = nullptr;
-  int* E = nullptr;
-  double* Dg = nullptr;  // real diagonal of H, applied in FP64 by the epilogue
-  int64_t N = 0, Kp = 0;
-  int cplx = 1;
-};
-// Slice workspace for up to max_cols columns of the filter block.
-struct SplitX {
-  void* B = nullptr;
-  int* F = nullptr;
-  int cap_cols = 0;
-  int cplx = 1;
-  void* P = nullptr;  // FP64 partial products of K segments (grow-only)
-  size_t P_cap = 0;   // in units of 16 bytes
-};
-int split_prepare_h(Dev& d, const chase_c64* H, int64_t N, int64_t ldh, SplitH& out);
-int split_prepare_h(Dev& d, const double* H, int64_t N, int64_t ldh, SplitH& out);
-// The same slices from a complex64 / float32 H (entries widened exactly).
-int split_prepare_h(Dev& d, const chase_c32* H, int64_t N, int64_t ldh, SplitH& out);
-int split_prepare_h(Dev& d, const float* H, int64_t N, int64_t ldh, SplitH& out);
-int split_alloc_x(Dev& d, int64_t N, int max_cols, SplitX& out, bool cplx = true);
-// C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1]
-// with the leading `nslices` slices of each operand (7: full accuracy, about
-// 2^-49 relative; 4: about 2^-28; 3: about 2^-21).
-int zgemm_split(Dev& d, const SplitH& h, SplitX& x, const chase_c64* X, int64_t ldx, int j0, int j1,
-                chase_c64* C, int64_t ldc, double alpha, double beta, double shift,
-                int nslices = 7);
-int zgemm_split(Dev& d, const SplitH& h, SplitX& x, const double* X, int64_t ldx, int j0, int j1,
-                double* C, int64_t ldc, double alpha, double beta, double shift, int nslices = 7);
-
 // ---- rns.cu: products with H in residue arithmetic on the tensor cores -----
 // Moduli per accuracy: kRnsFp64 stands in for FP64 GEMMs (operands rounded to
 // 2^-60 of a row's or column's 2-norm), rns_split_moduli(N) for the split
@@ -251,32 +217,44 @@ template <class T>
 int rns_dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, T* C, int64_t ldc,
               double alpha, double beta);
 
+// alpha P, beta and shift of one residue product, prepared on the host.
+struct RnsScale {
+  double alpha, beta, shift;
+  double ap, ap_lo;  // 2^-64 alpha P as the sum of two doubles
+  int plain;         // |alpha| within [2^-100, 2^100]: alpha P 2^e may be formed first
+  int has_beta;
+};
+
 // ---- grouped filter: many independent problems per launch ----------------
 // One problem of a grouped filter, in device memory.  buf0 holds the block
 // sorted by degree (the filter's input and final output), buf1 is the second
-// buffer of the three-term recurrence; their tensor maps (FP64 path) or the
-// slice planes and maps (split path) live in device memory too.
+// buffer of the three-term recurrence.  Tensor maps live in device memory too:
+// of H and both buffers for FP64 tiles, of the residue planes of H and of the
+// active block for residue products.
 struct GroupedProblem {
-  const CUtensorMap* mapA;   // H (FP64) or the slice planes of H (split)
-  const CUtensorMap* mapB0;  // FP64: buf0; split: the slices of the active block
+  const CUtensorMap* mapA;   // H, or the residue planes of H
+  const CUtensorMap* mapB0;  // FP64: buf0; residues: the block's planes, a map per tile width
   const CUtensorMap* mapB1;  // FP64: buf1
   double2* buf0;
   double2* buf1;
   long long ld0, ld1;
-  const int* E;       // split: row exponents of H
-  int* F;             // split: column exponents of the active block
-  const double* Dg;   // split: real diagonal of H
-  void* Bsl;          // split: slice planes of the block [S][2 bcap][Kp]
-  long long Kp;       // split: padded K = 2N rounded up to 16
-  int n, b, bcap;     // rows, columns of the block, column capacity of Bsl
+  const int* E;       // residues: row exponents of H
+  int* F;             // residues: column exponents of the active block
+  const double* Dg;   // residues: real diagonal of H
+  void* Bsl;          // residue planes of the block [plane][bcap][Kp] (bf16)
+  void* G;            // residues of the product, the same shape (int16)
+  long long Kp;       // residues: n rounded up to 64
+  int n, b, bcap;     // rows, columns of the block, column capacity of Bsl and G
 };
 // One active problem of one degree step: columns [s, b) of problem `prob`
-// are filtered; its output tiles are CTAs [tile0, next.tile0) and its
-// columns [col0, next.col0) of the step's column range.  A step's list ends
-// with a sentinel entry holding the totals.
+// are filtered; its output tiles are [tile0, next.tile0), its columns
+// [col0, next.col0) of the step's column range and its reconstruction blocks
+// [blk0, next.blk0).  A step's list ends with a sentinel entry holding the
+// totals.
 struct GroupedStep {
-  int prob, s, tile0, col0;
+  int prob, s, tile0, col0, blk0;
   double alpha, beta, shift;
+  RnsScale sc;
 };
 // FP64 tile shapes of the grouped product (rows x complex columns per CTA).
 constexpr int kGroupedFp64Cfgs = 4;
@@ -287,20 +265,8 @@ int zgemm_grouped_fp64(Dev& d, int cfg, const GroupedProblem* probs, const Group
                        int nact, int ntiles, int parity);
 // Kernel attributes (shared memory size) set outside any stream capture.
 int zgemm_grouped_fp64_prepare(int cfg);
-int zgemm_split_grouped_prepare();
-// Split path: slice the active columns of every active problem (one CTA per
-// column), then the grouped tensor-core product (one CTA per output tile).
-int split_grouped_slice_x(Dev& d, const GroupedProblem* probs, const GroupedStep* steps, int nact,
-                          int ncols, int parity);
-int zgemm_split_grouped(Dev& d, const GroupedProblem* probs, const GroupedStep* steps, int nact,
-                        int ntiles, int parity);
-constexpr int kSplitTileRows = 128;      // rows of H per split tile
-constexpr int kSplitTileRealCols = 64;   // real columns (32 complex) per split tile
-constexpr int kSplitSlices = 7;
-constexpr int kSplitStageK = 32;         // K per TMA stage box (64-byte swizzled rows)
-int64_t split_k_padded(int64_t N);
-// Slices of every problem's H: one CTA per row over all problems; row_prob
-// holds the first global row of each problem (P + 1 entries).
+// Residue planes of every problem's H: one CTA per row over all problems;
+// row0 is the first global row of each problem.
 struct GroupedSliceH {
   const double2* H;
   long long ldh;
@@ -310,12 +276,30 @@ struct GroupedSliceH {
   long long Kp;
   int n, row0;
 };
-int split_grouped_prepare_h(Dev& d, const GroupedSliceH* probs, int P, int total_rows);
-// One problem of grouped_filter_sorted: the block X (b columns, sorted by
+int64_t rns_k_padded(int64_t N);
+int rns_grouped_prepare_h(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows);
+int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, const void* A,
+                     const void* B, int64_t n, int64_t b, int64_t bcap);
+RnsScale rns_scale(int nmod, double alpha, double beta, double shift);  // complex problems
+// Tiles (of width bn) and reconstruction blocks of one problem's step, and the
+// relative time of a 64-wide K step of a tile.
+int rns_grouped_tiles(int nmod, int bn, int n, int cols);
+int rns_grouped_crt_blocks(int n, int cols);
+double rns_stage_cost(int bn);
+// One degree step on residue products: slice the active columns of every
+// active problem, multiply, put the products together.
+int rns_grouped_ready();  // kernel attributes, set outside any stream capture
+int rns_grouped_slice_x(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
+                        int nact, int ncols, int parity);
+int rns_grouped_gemm(Dev& d, int nmod, int bn, const GroupedProblem* probs,
+                     const GroupedStep* steps, int ntiles);
+int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
+                    int nact, int nblocks, int parity);
+// One problem of a grouped filter: the block X (b columns, sorted by
 // ascending degree) is filtered in place with W as the second buffer;
 // start[i] (host, i = 0 .. maxdeg + 1) counts the columns of degree < i.
-// Split path: the slices of H (A, E, Dg) and a slice workspace of bcap >= b
-// columns (Bsl, F), as made by grouped_split_prepare.
+// Residue products: the planes of H (A, E, Dg) and the workspace of bcap >= b
+// columns (Bsl, G, F), as made by grouped_rns_prepare.
 struct GroupedFilterInput {
   const chase_c64* H = nullptr;
   int64_t ldh = 0;
@@ -332,6 +316,7 @@ struct GroupedFilterInput {
   int* E = nullptr;
   double* Dg = nullptr;
   void* Bsl = nullptr;
+  void* G = nullptr;
   int* F = nullptr;
   int bcap = 0;
 };
@@ -340,13 +325,22 @@ struct GroupedFilterTimes {
   long long matvecs = 0;
   double flops = 0, t_autotune = 0, t_graph_build = 0, t_steps = 0, t_product = 0;
 };
-// Slices of every problem's H and the slice workspace for bcap[q] columns
-// (one grouped slicing launch); fills the split fields of `in`.
-int grouped_split_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap);
+// Moduli of a batch's residue products: of the split filter's accuracy, or
+// FP64's; 0 where a batch this small stays on the FP64 tiles.
+int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile);
+// Residue planes of every problem's H and the workspace for bcap[q] columns
+// (one grouped slicing launch); fills the residue fields of `in`.
+// CHASE_OUT_OF_MEMORY leaves nothing behind.
+int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
+                        int nmod);
+void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in);
 // Alg. 4 on every problem of `in` (problems with b == 0 are skipped), one
-// grouped launch per degree step, all steps in one CUDA graph.  tile:
-// CHASE_TILE_AUTO or a fixed FP64 tile shape.  Synchronises the stream.
-int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, bool split, int tile,
+// grouped launch per degree step and part, all steps in one CUDA graph.
+// nmod: residue products with that many moduli (prepared inputs are used as
+// they are; others are prepared here, a part of the batch at a time where the
+// memory does not hold all), 0: FP64 tiles of shape `tile` or, with
+// CHASE_TILE_AUTO, the fastest.  Synchronises the stream.
+int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int tile,
                           GroupedFilterTimes* times);
 
 // Column gather / scatter for many problems: one CTA per column.

@@ -234,7 +234,7 @@ struct Tile {
 };
 
 template <int BN, class TileFn>
-__device__ __forceinline__ void gemm_body(const TileFn& tile, int ntiles, const GemmTab& tab,
+__device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTab& tab,
                                           int maps_in_global, int* __restrict__ err) {
   using C = Cfg<BN>;
   constexpr int NSTAGE = C::NSTAGE;
@@ -940,14 +940,6 @@ struct Out<float> {
   using S = float;
 };
 
-// alpha P and beta of one product, prepared on the host.
-struct CrtScale {
-  double alpha, beta, shift;
-  double ap, ap_lo;  // 2^-64 alpha P as the sum of two doubles
-  int plain;         // |alpha| within [2^-100, 2^100]: alpha P 2^e may be formed first
-  int has_beta;
-};
-
 // Two rows (r, r + 1) per thread, columns blockIdx.y, + gridDim.y, ...
 //
 // The FP64 pipe bounds this kernel (two FMAs a cycle and SM), so it does as
@@ -963,18 +955,17 @@ struct CrtScale {
 // rounding would be the same in every degree step and so add up over the
 // recurrence, where the roundings of an FP64 GEMM average out.
 template <int NM, class E>
-__global__ void __launch_bounds__(128)
-    rns_crt_kernel(const int16_t* __restrict__ G, long long ldg, long long gplane,
-                   const __grid_constant__ CrtTab tab, const int* __restrict__ Ex,
-                   const int* __restrict__ Fx, const double* __restrict__ Dg, int M, int ncols,
-                   int j0, const E* __restrict__ X, long long ldx, E* __restrict__ C, long long ldc,
-                   const __grid_constant__ CrtScale sc) {
+__device__ __forceinline__ void crt_rows(int r0, int c0, int c1, int cstep,
+                                         const int16_t* __restrict__ G, long long ldg,
+                                         long long gplane, const CrtTab& tab,
+                                         const int* __restrict__ Ex, const int* __restrict__ Fx,
+                                         const double* __restrict__ Dg, int M, int j0,
+                                         const E* __restrict__ X, long long ldx,
+                                         E* __restrict__ C, long long ldc, const RnsScale& sc) {
   constexpr bool CP = is_complex<E>;
   constexpr int W = CP ? 2 : 1;
   constexpr bool ACC = NM == kRnsFp64;
   using S = typename Out<E>::S;
-  const int r0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  if (r0 >= M) return;
   int er[2];
   double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (ACC: two doubles)
   bool diag[2];
@@ -995,7 +986,7 @@ __global__ void __launch_bounds__(128)
     dh[h] = d;
     dl[h] = l;
   }
-  for (int c = blockIdx.y; c < ncols; c += gridDim.y) {
+  for (int c = c0; c < c1; c += cstep) {
     const int16_t* g = G + static_cast<long long>(c) * ldg + r0;
     unsigned long long hi[2][W] = {};
     int lo[2][W] = {};
@@ -1073,6 +1064,118 @@ __global__ void __launch_bounds__(128)
         *cp = static_cast<S>(v[0]);
     }
   }
+}
+
+template <int NM, class E>
+__global__ void __launch_bounds__(128)
+    rns_crt_kernel(const int16_t* __restrict__ G, long long ldg, long long gplane,
+                   const __grid_constant__ CrtTab tab, const int* __restrict__ Ex,
+                   const int* __restrict__ Fx, const double* __restrict__ Dg, int M, int ncols,
+                   int j0, const E* __restrict__ X, long long ldx, E* __restrict__ C, long long ldc,
+                   const __grid_constant__ RnsScale sc) {
+  const int r0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+  if (r0 >= M) return;
+  crt_rows<NM, E>(r0, blockIdx.y, ncols, gridDim.y, G, ldg, gplane, tab, Ex, Fx, Dg, M, j0, X, ldx,
+                  C, ldc, sc);
+}
+
+// ---------------------------------------------------------------------------
+// Many problems per launch (the batched filter): one degree step slices the
+// active columns of every problem, multiplies, and puts the products together
+// in three launches.  A launch's work is listed in the step's entries; blocks
+// find theirs by binary search, the persistent GEMM pairs by walking on from
+// their last tile.
+// ---------------------------------------------------------------------------
+// Last entry whose prefix (a member of the entries) is not above g.
+template <class S>
+__device__ __forceinline__ int find_entry(const S* s, int n, int S::*prefix, int g) {
+  int lo = 0, hi = n;
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (s[mid].*prefix <= g) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+template <int NM, int NL>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_grouped_slice_h_kernel(const GroupedSliceH* __restrict__ probs, int P,
+                               const __grid_constant__ SliceTab tab) {
+  const GroupedSliceH& q = probs[find_entry(probs, P, &GroupedSliceH::row0, blockIdx.x)];
+  const int r = blockIdx.x - q.row0;
+  const double2* col = q.H + static_cast<long long>(r) * q.ldh;
+  if (threadIdx.x == 0) q.Dg[r] = col[r].x;
+  slice_vector<NM, NL, double2>(col, q.n, true, r, static_cast<__nv_bfloat16*>(q.A) + r * q.Kp,
+                                q.n * q.Kp, q.E + r, tab, 0, NM);
+}
+
+template <int NM, int NL>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_grouped_slice_x_kernel(const GroupedProblem* __restrict__ probs,
+                               const GroupedStep* __restrict__ steps, int nact, int parity,
+                               const __grid_constant__ SliceTab tab) {
+  const GroupedStep& st = steps[find_entry(steps, nact, &GroupedStep::col0, blockIdx.x)];
+  const GroupedProblem& q = probs[st.prob];
+  const int c = blockIdx.x - st.col0;
+  const double2* x = (parity ? q.buf1 : q.buf0) + (st.s + c) * (parity ? q.ld1 : q.ld0);
+  slice_vector<NM, NL, double2>(x, q.n, false, -1, static_cast<__nv_bfloat16*>(q.Bsl) + c * q.Kp,
+                                q.bcap * q.Kp, q.F + c, tab, 0, NM);
+}
+
+// Tiles of a step: per problem the column tile runs fastest, then row tiles,
+// then planes.
+struct GroupedTiles {
+  const GroupedProblem* probs;
+  const GroupedStep* steps;
+  int bn, at;  // at: entry of the last tile (each thread walks forward)
+  __device__ __forceinline__ void operator()(int t, Tile& T) {
+    while (steps[at + 1].tile0 <= t) ++at;
+    const GroupedStep& st = steps[at];
+    const GroupedProblem& q = probs[st.prob];
+    const int rtiles = (q.n + 2 * BM - 1) / (2 * BM), ctiles = (q.b - st.s + bn - 1) / bn;
+    const int u = t - st.tile0;
+    const int ct = u % ctiles, rest = u / ctiles;
+    const int rt = rest % rtiles, pl = rest / rtiles;
+    T.mapA = q.mapA;
+    T.mapB = q.mapB0 + (bn / 32 - 1);  // one map per tile width
+    T.row0 = rt * 2 * BM;
+    T.col0 = ct * bn;
+    T.planeA = pl;
+    T.planeB = pl;
+    T.modulus = pl / 2;
+    T.nst = (q.n + BK - 1) / BK;
+    T.M = q.n;
+    T.ncols = q.b - st.s;
+    T.ldg = q.Kp;
+    T.G = static_cast<int16_t*>(q.G) + static_cast<long long>(pl) * q.bcap * q.Kp;
+  }
+};
+
+template <int BN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+    rns_grouped_gemm_kernel(const GroupedProblem* __restrict__ probs,
+                            const GroupedStep* __restrict__ steps, int ntiles,
+                            const __grid_constant__ GemmTab tab, int* __restrict__ err) {
+  GroupedTiles g{probs, steps, BN, 0};
+  gemm_body<BN>(g, ntiles, tab, 1, err);
+}
+
+constexpr int kCrtCols = 4;  // columns per block of the grouped reconstruction
+
+template <int NM>
+__global__ void __launch_bounds__(128)
+    rns_grouped_crt_kernel(const GroupedProblem* __restrict__ probs,
+                           const GroupedStep* __restrict__ steps, int nact, int parity,
+                           const __grid_constant__ CrtTab tab) {
+  const GroupedStep& st = steps[find_entry(steps, nact, &GroupedStep::blk0, blockIdx.x)];
+  const GroupedProblem& q = probs[st.prob];
+  const int rchunks = (q.n + 255) / 256, u = blockIdx.x - st.blk0;
+  const int r0 = 2 * (u % rchunks * 128 + threadIdx.x), c0 = u / rchunks * kCrtCols;
+  if (r0 >= q.n) return;
+  crt_rows<NM, double2>(r0, c0, min(c0 + kCrtCols, q.b - st.s), 1, static_cast<int16_t*>(q.G), q.Kp,
+                        static_cast<long long>(q.bcap) * q.Kp, tab, q.E, q.F, q.Dg, q.n, st.s,
+                        parity ? q.buf1 : q.buf0, parity ? q.ld1 : q.ld0,
+                        parity ? q.buf0 : q.buf1, parity ? q.ld0 : q.ld1, st.sc);
 }
 
 // ---------------------------------------------------------------------------
@@ -1169,8 +1272,8 @@ const Tables& tables(int nm, bool cplx) {
   return nm == 7 ? t7r : nm == 8 ? t8r : nm == 11 ? t11r : nm == 12 ? t12r : t14r;
 }
 
-CrtScale crt_scale(const CrtTab& t, double alpha, double beta, double shift) {
-  CrtScale s{};
+RnsScale crt_scale(const CrtTab& t, double alpha, double beta, double shift) {
+  RnsScale s{};
   s.alpha = alpha;
   s.beta = beta;
   s.shift = shift;
@@ -1249,10 +1352,12 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
   return CHASE_OK;
 }
 
+// A 64-wide K step of a pair streams 256 + BN operand rows and multiplies BN
+// columns; narrow tiles are bound by the streaming.
+double stage_cost(int bn) { return std::max(1.0 * bn, 0.5 * (256 + bn)); }
+
 // Columns per tile: the width whose busiest pair (of the 76 that the 152 SMs
-// make) has the least to do.  A 64-wide K step of a pair streams 256 + BN
-// operand rows and multiplies BN columns; narrow tiles are bound by the
-// streaming.
+// make) has the least to do.
 int choose_bn(int64_t M, int ncols, int nplanes) {
   const int64_t rt = (M + 2 * BM - 1) / (2 * BM);
   int best = 32;
@@ -1260,7 +1365,7 @@ int choose_bn(int64_t M, int ncols, int nplanes) {
   for (int bn = 32; bn <= 256; bn += 32) {
     const int64_t tiles = rt * ((ncols + bn - 1) / bn) * nplanes;
     const int64_t per = (tiles + 75) / 76;
-    const double cost = static_cast<double>(per) * std::max(1.0 * bn, 0.5 * (256 + bn));
+    const double cost = static_cast<double>(per) * stage_cost(bn);
     if (best_cost == 0.0 || cost < 0.995 * best_cost) {
       best_cost = cost;
       best = bn;
@@ -1453,6 +1558,46 @@ int dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, E* C, int64
   d.release(G);
   return CHASE_OK;
 }
+
+template <int BN>
+int grouped_pairs() {
+  static const int v = [] {
+    using C = Cfg<BN>;
+    if (cudaFuncSetAttribute(rns_grouped_gemm_kernel<BN>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return pairs_on_device<BN>();
+  }();
+  return v;
+}
+template <int BN>
+int launch_grouped_gemm(Dev& d, const GroupedProblem* probs, const GroupedStep* steps, int ntiles,
+                        const GemmTab& tab) {
+  const int pairs = grouped_pairs<BN>();
+  if (pairs < 1) {
+    set_error("residue GEMM: no CTA pair fits this device");
+    return CHASE_CUDA_ERROR;
+  }
+  rns_grouped_gemm_kernel<BN><<<2 * std::min(ntiles, pairs), kThreads, Cfg<BN>::SMEM, d.st>>>(
+      probs, steps, ntiles, tab, d.err);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+
+// One of the three moduli counts of the batched filter.
+template <class F>
+int with_moduli(int nmod, F&& f) {
+  switch (nmod) {
+    case 11: return f(std::integral_constant<int, 11>());
+    case 12: return f(std::integral_constant<int, 12>());
+    case kRnsFp64: return f(std::integral_constant<int, kRnsFp64>());
+  }
+  set_error("grouped residue product: %d moduli", nmod);
+  return CHASE_INVALID_ARG;
+}
 }  // namespace
 }  // namespace rns
 
@@ -1598,6 +1743,85 @@ int rns_dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, T* C, i
 CHASE_INSTANTIATE_DENSE(chase_c64)
 CHASE_INSTANTIATE_DENSE(double)
 #undef CHASE_INSTANTIATE_DENSE
+
+int64_t rns_k_padded(int64_t N) { return (N + rns::BK - 1) / rns::BK * rns::BK; }
+
+RnsScale rns_scale(int nmod, double alpha, double beta, double shift) {
+  return rns::crt_scale(rns::tables(nmod, true).crt, alpha, beta, shift);
+}
+
+int rns_grouped_prepare_h(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows) {
+  return rns::with_moduli(nmod, [&](auto nm) -> int {
+    constexpr int NM = decltype(nm)::value;
+    rns::rns_grouped_slice_h_kernel<NM, rns::limbs_of(NM)>
+        <<<static_cast<unsigned>(total_rows), rns::kSliceThreads, 0, d.st>>>(
+            probs, P, rns::tables(NM, true).slice);
+    note_launch();
+    CHASE_CUDA(cudaGetLastError());
+    return CHASE_OK;
+  });
+}
+
+int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, const void* A,
+                     const void* B, int64_t n, int64_t b, int64_t bcap) {
+  const int64_t Kp = rns_k_padded(n);
+  CHASE_TRY(make_tmap_bf16_3d(mapA, A, n, n, 2 * nmod, Kp * 2, Kp * 2 * n, rns::BK, rns::BM, 1));
+  return make_tmap_bf16_3d(mapB, B, n, b, 2 * nmod, Kp * 2, Kp * 2 * bcap, rns::BK, bn / 2, 1);
+}
+
+int rns_grouped_tiles(int nmod, int bn, int n, int cols) {
+  return (n + 2 * rns::BM - 1) / (2 * rns::BM) * ((cols + bn - 1) / bn) * 2 * nmod;
+}
+int rns_grouped_crt_blocks(int n, int cols) {
+  return (n + 255) / 256 * ((cols + rns::kCrtCols - 1) / rns::kCrtCols);
+}
+double rns_stage_cost(int bn) { return rns::stage_cost(bn); }
+
+int rns_grouped_slice_x(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
+                        int nact, int ncols, int parity) {
+  return rns::with_moduli(nmod, [&](auto nm) -> int {
+    constexpr int NM = decltype(nm)::value;
+    rns::rns_grouped_slice_x_kernel<NM, rns::limbs_of(NM)>
+        <<<static_cast<unsigned>(ncols), rns::kSliceThreads, 0, d.st>>>(
+            probs, steps, nact, parity, rns::tables(NM, true).slice);
+    note_launch();
+    CHASE_CUDA(cudaGetLastError());
+    return CHASE_OK;
+  });
+}
+int rns_grouped_gemm(Dev& d, int nmod, int bn, const GroupedProblem* probs,
+                     const GroupedStep* steps, int ntiles) {
+  const rns::GemmTab& tab = rns::tables(nmod, true).gemm;
+  switch (bn) {
+    case 32: return rns::launch_grouped_gemm<32>(d, probs, steps, ntiles, tab);
+    case 64: return rns::launch_grouped_gemm<64>(d, probs, steps, ntiles, tab);
+    case 96: return rns::launch_grouped_gemm<96>(d, probs, steps, ntiles, tab);
+    case 128: return rns::launch_grouped_gemm<128>(d, probs, steps, ntiles, tab);
+    case 160: return rns::launch_grouped_gemm<160>(d, probs, steps, ntiles, tab);
+    case 192: return rns::launch_grouped_gemm<192>(d, probs, steps, ntiles, tab);
+    case 224: return rns::launch_grouped_gemm<224>(d, probs, steps, ntiles, tab);
+    default: return rns::launch_grouped_gemm<256>(d, probs, steps, ntiles, tab);
+  }
+}
+int rns_grouped_ready() {
+  return rns::grouped_pairs<32>() > 0 && rns::grouped_pairs<64>() > 0 &&
+                 rns::grouped_pairs<96>() > 0 && rns::grouped_pairs<128>() > 0 &&
+                 rns::grouped_pairs<160>() > 0 && rns::grouped_pairs<192>() > 0 &&
+                 rns::grouped_pairs<224>() > 0 && rns::grouped_pairs<256>() > 0
+             ? CHASE_OK
+             : CHASE_CUDA_ERROR;
+}
+int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
+                    int nact, int nblocks, int parity) {
+  return rns::with_moduli(nmod, [&](auto nm) -> int {
+    constexpr int NM = decltype(nm)::value;
+    rns::rns_grouped_crt_kernel<NM><<<static_cast<unsigned>(nblocks), 128, 0, d.st>>>(
+        probs, steps, nact, parity, rns::tables(NM, true).crt);
+    note_launch();
+    CHASE_CUDA(cudaGetLastError());
+    return CHASE_OK;
+  });
+}
 
 #define CHASE_INSTANTIATE_RNS(T)                                                                 \
   template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, RnsH&);           \
