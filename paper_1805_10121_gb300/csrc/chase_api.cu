@@ -462,7 +462,7 @@ int rr_alloc(Dev& d, int64_t N, int b, RRWork<T>& w) {
 
 // Alg. 2 in three parts: rr_pre forms H Q (with the residue planes of H in rs,
 // those it makes for this product alone, or on the FP64 pipe) and the lower
-// triangle of G = Q^H (H Q) mirrored to the upper one; the eigensolve of G follows (one problem: eigh_device, a
+// triangle of G = Q^H (H Q) mirrored to the upper one; the eigensolve of G follows (one problem: eigh, a
 // batch: eigh_batched); rr_post forms Q W, the residuals from (H Q) W, and
 // copies Q W into Q.
 template <class T>
@@ -518,7 +518,7 @@ int rr_core(Dev& d, const T* H, int64_t N, int64_t ldh, T* Q, int64_t ldq, int b
   CHASE_TRY(rr_pre<T>(d, H, N, ldh, Q, ldq, b, w, t_hq, rs));
   PhaseTimer tm(d.st);
   tm.begin(t_eigh);
-  CHASE_TRY(eigh_device(d, w.G, lg, b, w_dev));  // (W, Lambda) = TSOLVE(G)
+  CHASE_TRY(eigh(d, w.G, lg, b, w_dev));  // (W, Lambda) = TSOLVE(G)
   tm.end();
   return rr_post(d, N, Q, ldq, b, w_dev, res_dev, w, flops);
 }

@@ -353,7 +353,15 @@ struct GroupedPermute {
 };
 int launch_grouped_permute(Dev& d, const GroupedPermute* probs, int P, int total_cols, bool scatter);
 
-// ---- eigh (cuSOLVER, the small projected eigensolve of Alg. 2 line 3) -----
+// ---- eigh_refine.cu: the projected eigensolve of Alg. 2 line 3 ------------
+// G (p x p, Hermitian, both triangles) becomes its eigenvectors, w_dev its
+// eigenvalues ascending: FP64 problems by refining an FP32 solve, or where
+// that does not serve with eigh_device; single precision with eigh_device.
+int eigh(Dev& d, chase_c64* G, int64_t ldg, int p, double* w_dev);
+int eigh(Dev& d, double* G, int64_t ldg, int p, double* w_dev);
+int eigh(Dev& d, chase_c32* G, int64_t ldg, int p, double* w_dev);
+int eigh(Dev& d, float* G, int64_t ldg, int p, double* w_dev);
+// ---- the same by cuSOLVER alone -------------------------------------------
 int eigh_device(Dev& d, chase_c64* G, int64_t ldg, int p, double* w_dev);
 int eigh_device(Dev& d, double* G, int64_t ldg, int p, double* w_dev);
 // Single precision (cheevd / ssyevd); eigenvalues returned in double.
