@@ -279,6 +279,8 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
   cluster_sync();
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  // the set-up above overlaps the kernel before; its results are read below
+  pdl_wait();
 
   // Warps 0 and 1 run their loops with all lanes, and one elected lane issues:
   // with only lane 0 in the loop the operands of every TMA and MMA went
@@ -452,6 +454,9 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
       }
     }
   }
+  // not earlier: blocks of the next kernel would gather, waiting, on the SMs
+  // whose pairs end first, and run there alone
+  pdl_next();
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
   cluster_sync();
@@ -798,6 +803,8 @@ __global__ void __launch_bounds__(kSliceThreads)
     rns_slice_x_kernel(const E* __restrict__ X, long long ldx, int N, int j0,
                        const __grid_constant__ SliceTab tab, __nv_bfloat16* __restrict__ B,
                        long long Kp, long long plane, int* __restrict__ Fx) {
+  pdl_next();
+  pdl_wait();
   const int c = blockIdx.x;
   slice_vector<NM, NL, E>(X + static_cast<long long>(j0 + c) * ldx, N, false, -1, B + c * Kp, plane,
                           Fx + c, tab, 0, NM);
@@ -819,6 +826,8 @@ __global__ void __launch_bounds__(kSliceThreads)
   __shared__ float sf[G][kRowBlock];
   __shared__ uint32_t su[G][kRowBlock];
   __shared__ long long tile[W][kRowBlock][65];
+  pdl_next();
+  pdl_wait();
   const int row = threadIdx.x % kRowBlock, grp = threadIdx.x / kRowBlock;
   const int r0 = blockIdx.x * kRowBlock;
   const bool in = r0 + row < M;
@@ -1073,10 +1082,12 @@ __global__ void __launch_bounds__(128)
                    const int* __restrict__ Fx, const double* __restrict__ Dg, int M, int ncols,
                    int j0, const E* __restrict__ X, long long ldx, E* __restrict__ C, long long ldc,
                    const __grid_constant__ RnsScale sc) {
+  pdl_wait();
   const int r0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  if (r0 >= M) return;
-  crt_rows<NM, E>(r0, blockIdx.y, ncols, gridDim.y, G, ldg, gplane, tab, Ex, Fx, Dg, M, j0, X, ldx,
-                  C, ldc, sc);
+  if (r0 < M)
+    crt_rows<NM, E>(r0, blockIdx.y, ncols, gridDim.y, G, ldg, gplane, tab, Ex, Fx, Dg, M, j0, X,
+                    ldx, C, ldc, sc);
+  pdl_next();  // late, for the reason the GEMM gives
 }
 
 // ---------------------------------------------------------------------------
@@ -1343,12 +1354,11 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
   const int ct = (a.ncols + BN - 1) / BN;
   const int64_t tiles = static_cast<int64_t>(rt) * ct * a.nplanes;
   const unsigned grid = 2 * static_cast<unsigned>(std::min<int64_t>(tiles, pairs));
-  rns_gemm_kernel<BN><<<grid, kThreads, C::SMEM, d.st>>>(
-      tmA, tmB, *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a,
-      static_cast<int>((a.K + BK - 1) / BK), static_cast<int>(a.M), a.ncols, a.G, a.ldg, a.gplane,
-      d.err);
+  CHASE_CUDA(launch_pdl(rns_gemm_kernel<BN>, dim3(grid), dim3(kThreads), C::SMEM, d.st, tmA, tmB,
+                        *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a,
+                        static_cast<int>((a.K + BK - 1) / BK), static_cast<int>(a.M), a.ncols, a.G,
+                        a.ldg, a.gplane, d.err));
   note_launch();
-  CHASE_CUDA(cudaGetLastError());
   return CHASE_OK;
 }
 
@@ -1435,10 +1445,10 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
   const int64_t gplane = static_cast<int64_t>(x.cap_cols) * x.ldg;
   for (int c0 = j0; c0 < j1; c0 += x.cap_cols) {
     const int w = std::min(x.cap_cols, j1 - c0);
-    rns_slice_x_kernel<NM, limbs_of(NM), E><<<static_cast<unsigned>(w), kSliceThreads, 0, d.st>>>(
-        X, ldx, N, c0, t.slice, static_cast<__nv_bfloat16*>(x.B), x.Kp, bplane, x.F);
+    CHASE_CUDA(launch_pdl(rns_slice_x_kernel<NM, limbs_of(NM), E>, dim3(w), dim3(kSliceThreads), 0,
+                          d.st, X, ldx, N, c0, t.slice, static_cast<__nv_bfloat16*>(x.B), x.Kp,
+                          bplane, x.F));
     note_launch();
-    CHASE_CUDA(cudaGetLastError());
     const double alg = (CP ? 8.0 : 2.0) * N * static_cast<double>(N) * w;
     KernelTimer kt(d.st, NM == kRnsFp64 ? CHASE_TIMED_FP64_PRODUCT : CHASE_TIMED_SPLIT_PRODUCT);
     int launched = 0;
@@ -1471,11 +1481,10 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
     const int gx = (N + 255) / 256;
     const dim3 grid(static_cast<unsigned>(gx),
                     static_cast<unsigned>(std::min(w, std::max(1, 16 * 152 / gx))));
-    rns_crt_kernel<NM, E><<<grid, 128, 0, d.st>>>(x.G, x.ldg, gplane, t.crt, h.E, x.F, h.Dg, N, w,
-                                                  c0, X, ldx, C, ldc,
-                                                  crt_scale(t.crt, alpha, beta, shift));
+    CHASE_CUDA(launch_pdl(rns_crt_kernel<NM, E>, grid, dim3(128), 0, d.st, x.G, x.ldg, gplane,
+                          t.crt, h.E, x.F, h.Dg, N, w, c0, X, ldx, C, ldc,
+                          crt_scale(t.crt, alpha, beta, shift)));
     note_launch();
-    CHASE_CUDA(cudaGetLastError());
   }
   return CHASE_OK;
 }
@@ -1500,23 +1509,21 @@ int product_any(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0,
 
 template <class E>
 int slice_columns(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
-  rns_slice_x_kernel<kRnsFp64, limbs_of(kRnsFp64), E>
-      <<<static_cast<unsigned>(b.n), kSliceThreads, 0, d.st>>>(
-          X, ldx, static_cast<int>(b.K), 0, tables(kRnsFp64, is_complex<E>).slice,
-          static_cast<__nv_bfloat16*>(b.P), b.Kp, b.n * b.Kp, b.E);
+  CHASE_CUDA(launch_pdl(rns_slice_x_kernel<kRnsFp64, limbs_of(kRnsFp64), E>,
+                        dim3(static_cast<unsigned>(b.n)), dim3(kSliceThreads), 0, d.st, X, ldx,
+                        static_cast<int>(b.K), 0, tables(kRnsFp64, is_complex<E>).slice,
+                        static_cast<__nv_bfloat16*>(b.P), b.Kp, b.n * b.Kp, b.E));
   note_launch();
-  CHASE_CUDA(cudaGetLastError());
   return CHASE_OK;
 }
 template <class E>
 int slice_rows(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
-  rns_slice_rows_kernel<kRnsFp64, limbs_of(kRnsFp64), E>
-      <<<static_cast<unsigned>((b.n + kRowBlock - 1) / kRowBlock), kSliceThreads, 0, d.st>>>(
-          X, ldx, static_cast<int>(b.n), static_cast<int>(b.K),
-          tables(kRnsFp64, is_complex<E>).slice, static_cast<__nv_bfloat16*>(b.P), b.Kp,
-          b.n * b.Kp, b.E);
+  CHASE_CUDA(launch_pdl(rns_slice_rows_kernel<kRnsFp64, limbs_of(kRnsFp64), E>,
+                        dim3(static_cast<unsigned>((b.n + kRowBlock - 1) / kRowBlock)),
+                        dim3(kSliceThreads), 0, d.st, X, ldx, static_cast<int>(b.n),
+                        static_cast<int>(b.K), tables(kRnsFp64, is_complex<E>).slice,
+                        static_cast<__nv_bfloat16*>(b.P), b.Kp, b.n * b.Kp, b.E));
   note_launch();
-  CHASE_CUDA(cudaGetLastError());
   return CHASE_OK;
 }
 template <class E>
@@ -1550,11 +1557,10 @@ int dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, E* C, int64
   const int gx = static_cast<int>((a.n + 255) / 256);
   const dim3 grid(static_cast<unsigned>(gx),
                   static_cast<unsigned>(std::min<int64_t>(b.n, std::max(1, 16 * 152 / gx))));
-  rns_crt_kernel<kRnsFp64, E><<<grid, 128, 0, d.st>>>(
-      G, ldg, gplane, t.crt, a.E, b.E, nullptr, static_cast<int>(a.n), static_cast<int>(b.n), 0,
-      nullptr, 0, C, ldc, crt_scale(t.crt, alpha, beta, 0.0));
+  CHASE_CUDA(launch_pdl(rns_crt_kernel<kRnsFp64, E>, grid, dim3(128), 0, d.st, G, ldg, gplane,
+                        t.crt, a.E, b.E, nullptr, static_cast<int>(a.n), static_cast<int>(b.n), 0,
+                        nullptr, 0, C, ldc, crt_scale(t.crt, alpha, beta, 0.0)));
   note_launch();
-  CHASE_CUDA(cudaGetLastError());
   d.release(G);
   return CHASE_OK;
 }
