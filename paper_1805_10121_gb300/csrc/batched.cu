@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <chrono>
 #include <cmath>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <numeric>
@@ -179,16 +180,15 @@ void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in) {
     g.A = g.Bsl = g.G = nullptr;
     g.E = g.F = nullptr;
     g.Dg = nullptr;
-    g.bcap = 0;
+    g.bcap = g.sym = 0;
   }
 }
 
 namespace {
-int alloc_planes(Dev& d, GroupedFilterInput& g, int bcap, int nmod) {
+int alloc_block_planes(Dev& d, GroupedFilterInput& g, int bcap, int nmod) {
   const int64_t Kp = rns_k_padded(g.n);
   g.bcap = std::max(bcap, 1);
   const size_t block = static_cast<size_t>(2 * nmod) * g.bcap * Kp * 2;
-  CHASE_TRY(d.alloc_bytes(&g.A, static_cast<size_t>(2 * nmod) * g.n * Kp * 2));
   CHASE_TRY(d.alloc(&g.E, static_cast<size_t>(g.n)));
   CHASE_TRY(d.alloc(&g.Dg, static_cast<size_t>(g.n)));
   CHASE_TRY(d.alloc_bytes(&g.Bsl, block));
@@ -199,35 +199,95 @@ int alloc_planes(Dev& d, GroupedFilterInput& g, int bcap, int nmod) {
 
 int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
                         int nmod) {
-  std::vector<GroupedSliceH> hs;
+  auto give_back = [&](int st) {
+    grouped_rns_release(d, in);
+    return st;
+  };
+  std::vector<GroupedSliceH> all;
+  std::vector<size_t> owner;
   int rows = 0;
+  double entries = 0.0;
   for (size_t q = 0; q < in.size(); ++q) {
     GroupedFilterInput& g = in[q];
     if (g.n == 0) continue;
-    const int st = alloc_planes(d, g, bcap[q], nmod);
-    if (st != CHASE_OK) {
-      grouped_rns_release(d, in);
-      return st;
-    }
-    GroupedSliceH sh;
+    entries += static_cast<double>(g.n) * rns_k_padded(g.n);
+    const int st = alloc_block_planes(d, g, bcap[q], nmod);
+    if (st != CHASE_OK) return give_back(st);
+    GroupedSliceH sh{};
     sh.H = reinterpret_cast<const double2*>(g.H);
     sh.ldh = g.ldh;
-    sh.A = g.A;
     sh.E = g.E;
     sh.Dg = g.Dg;
     sh.Kp = rns_k_padded(g.n);
     sh.n = g.n;
     sh.row0 = rows;
-    hs.push_back(sh);
+    all.push_back(sh);
+    owner.push_back(q);
     rows += g.n;
   }
-  if (hs.empty()) return CHASE_OK;
-  GroupedSliceH* dsl = nullptr;
-  CHASE_TRY(d.alloc(&dsl, hs.size()));
-  CHASE_CUDA(cudaMemcpyAsync(dsl, hs.data(), sizeof(GroupedSliceH) * hs.size(),
-                             cudaMemcpyHostToDevice, d.st));
-  CHASE_TRY(rns_grouped_prepare_h(d, nmod, dsl, static_cast<int>(hs.size()), rows));
-  // the host array must outlive the copy
+  if (all.empty()) return CHASE_OK;
+  const int P = static_cast<int>(all.size());
+  // one list on the device per launch: all problems, then those with one
+  // scale, then the others
+  GroupedSliceH* dl = nullptr;
+  int* mm = nullptr;
+  CHASE_TRY(d.alloc(&dl, 3 * all.size()));
+  CHASE_TRY(d.alloc(&mm, 2 * all.size()));
+  std::vector<int> hmm(2 * all.size());
+  for (int p = 0; p < P; ++p) {
+    hmm[2 * p] = std::numeric_limits<int>::max();
+    hmm[2 * p + 1] = -std::numeric_limits<int>::max();
+  }
+  auto upload = [&](GroupedSliceH* to, const std::vector<GroupedSliceH>& v) -> int {
+    CHASE_CUDA(cudaMemcpyAsync(to, v.data(), sizeof(GroupedSliceH) * v.size(),
+                               cudaMemcpyHostToDevice, d.st));
+    return CHASE_OK;
+  };
+  if (rns_sym_pays(nmod, entries)) {
+    CHASE_TRY(upload(dl, all));
+    CHASE_CUDA(cudaMemcpyAsync(mm, hmm.data(), sizeof(int) * hmm.size(), cudaMemcpyHostToDevice,
+                               d.st));
+    CHASE_TRY(rns_grouped_row_exponents(d, nmod, dl, P, rows, mm));
+    CHASE_CUDA(cudaMemcpyAsync(hmm.data(), mm, sizeof(int) * hmm.size(), cudaMemcpyDeviceToHost,
+                               d.st));
+    CHASE_TRY(d.sync_check("grouped row scales of H"));
+  }
+  std::vector<GroupedSliceH> one, each;
+  int tiles = 0, erows = 0;
+  for (int p = 0; p < P; ++p) {
+    GroupedFilterInput& g = in[owner[p]];
+    GroupedSliceH sh = all[p];
+    g.sym = rns_same_scale(hmm[2 * p], hmm[2 * p + 1]) ? 1 : 0;
+    const int st = d.alloc_bytes(
+        &g.A, static_cast<size_t>(g.sym ? nmod : 2 * nmod) * g.n * rns_k_padded(g.n) * 2);
+    if (st != CHASE_OK) {
+      d.release(dl);
+      d.release(mm);
+      return give_back(st);
+    }
+    sh.A = g.A;
+    sh.s = hmm[2 * p];
+    if (g.sym) {
+      sh.tile0 = tiles;
+      tiles += rns_sym_tiles(g.n);
+      one.push_back(sh);
+    } else {
+      sh.row0 = erows;
+      erows += g.n;
+      each.push_back(sh);
+    }
+  }
+  if (!one.empty()) {
+    CHASE_TRY(upload(dl + P, one));
+    CHASE_TRY(rns_grouped_prepare_sym(d, nmod, dl + P, static_cast<int>(one.size()), tiles));
+  }
+  if (!each.empty()) {
+    CHASE_TRY(upload(dl + 2 * P, each));
+    CHASE_TRY(rns_grouped_prepare_h(d, nmod, dl + 2 * P, static_cast<int>(each.size()), erows));
+  }
+  d.release(mm);
+  d.release(dl);
+  // the host arrays must outlive the copies
   return d.sync_check("grouped residues of H");
 }
 
@@ -292,6 +352,7 @@ int filter_part(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int
       g.Bsl = pi.Bsl;
       g.G = pi.G;
       g.bcap = pi.bcap;
+      g.sym = pi.sym;
     }
   }
   CHASE_CUDA(cudaMemcpyAsync(dprobs, probs.data(), sizeof(GroupedProblem) * Q, cudaMemcpyHostToDevice,
@@ -326,7 +387,7 @@ int filter_part(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int
       for (int w = 0; w < 8; ++w)
         if (used[w])
           CHASE_TRY(rns_grouped_maps(&maps[nmaps * k], &maps[nmaps * k + 1 + w], nmod, 32 * (w + 1),
-                                     pi.A, pi.Bsl, pi.n, pi.b, pi.bcap));
+                                     pi.sym != 0, pi.A, pi.Bsl, pi.n, pi.b, pi.bcap));
     }
     CHASE_CUDA(cudaMemcpyAsync(dmaps, maps.data(), sizeof(CUtensorMap) * maps.size(),
                                cudaMemcpyHostToDevice, d.st));

@@ -477,7 +477,7 @@ int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, 
       RnsH h;
       RnsX x;
       int st = rns_alloc_x(d, N, b, kRnsFp64, is_cplx<T>, x);
-      if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, kRnsFp64, rns_reserve(N, b), h);
+      if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, kRnsFp64, rns_reserve(N, b), false, h);
       if (st == CHASE_OK) st = rns_product(d, h, x, Q, ldq, 0, b, w.HQ, lN, 1.0, 0.0, 0.0);
       for (void* p : {h.A, static_cast<void*>(h.E), static_cast<void*>(h.Dg), x.B,
                       static_cast<void*>(x.G), static_cast<void*>(x.F)})
@@ -854,9 +854,9 @@ struct Solver {
         CHASE_TRY(d.alloc(&Dw, static_cast<size_t>(lD) * nx));
       }
     }
-    if (want_split) CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), reserve, hsplit));
-    if (want_low) CHASE_TRY(rns_prepare_h(d, dH, N, lh, low, reserve, hlow));
-    if (want64) CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, reserve, h64));
+    if (want_split) CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), reserve, true, hsplit));
+    if (want_low) CHASE_TRY(rns_prepare_h(d, dH, N, lh, low, reserve, true, hlow));
+    if (want64) CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, reserve, true, h64));
     filter_set.full = want_split ? &hsplit : want64 ? &h64 : nullptr;
     filter_set.low = want_low ? &hlow : nullptr;
     filter_set.x = &rx;
@@ -1320,7 +1320,7 @@ int filter_impl(const T* H, int64_t N, int64_t ldh, T* V, int64_t ldv, int b, co
                          ? rns_low_moduli(N)
                          : precision == CHASE_FP64 ? kRnsFp64 : rns_split_moduli(N);
     CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), rh));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), true, rh));
     rs.full = &rh;
     rs.x = &rx;
   }
@@ -1448,11 +1448,11 @@ extern "C" int chase_filter_mixed(const chase_c64* H, int64_t N, int64_t ldh, ch
   const int nlow = rns_low_moduli(N);
   CHASE_TRY(rns_alloc_x(d, N, b, any_full ? rns_split_moduli(N) : nlow, true, rx));
   if (any_full) {
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), rns_reserve(N, b), full));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), rns_reserve(N, b), true, full));
     rs.full = &full;
   }
   if (any_low) {
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nlow, rns_reserve(N, b), low));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nlow, rns_reserve(N, b), true, low));
     rs.low = &low;
   }
   CHASE_TRY(launch_permute_cols(d, dV, lv, wk, lw, N, b, dperm, false));
@@ -1560,7 +1560,7 @@ extern "C" int chase_rayleigh_ritz(const chase_c64* H, int64_t N, int64_t ldh, c
   const bool rns = rns_pays(N, b);
   if (rns) {
     CHASE_TRY(rns_alloc_x(d, N, b, kRnsFp64, true, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, rns_reserve(N, b), rh));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, rns_reserve(N, b), false, rh));
     rs.full = &rh;
     rs.x = &rx;
   }
@@ -1605,7 +1605,7 @@ int residuals_impl(const T* H, int64_t N, int64_t ldh, const T* V, int64_t ldv, 
     RnsX rx;
     const int nmod = is_single<T> ? rns_low_moduli(N) : kRnsFp64;
     CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), rh));
+    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), false, rh));
     CHASE_TRY(rns_product(d, rh, rx, dV, lv, 0, b, HV, lw, 1.0, 0.0, 0.0));
   } else {
     CHASE_TRY(gemm(d, N, N, dH, lh, dV, lv, b, HV, lw, 0, b, 1.0, 0.0, 0.0));
@@ -2002,6 +2002,7 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
       h.Kp = s.rx.Kp = s.rx.ldg = rns_k_padded(s.N);
       h.cplx = 1;
       h.nmod = h.resident = nmod;
+      h.sym = planes[p].sym;
       s.rx.B = planes[p].Bsl;
       s.rx.G = static_cast<int16_t*>(planes[p].G);
       s.rx.F = planes[p].F;
@@ -2030,6 +2031,7 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
       g.G = planes[p].G;
       g.F = planes[p].F;
       g.bcap = planes[p].bcap;
+      g.sym = planes[p].sym;
       in.push_back(g);
     }
     GroupedFilterTimes tt;

@@ -168,7 +168,8 @@ int rns_split_moduli(int64_t N);
 int rns_low_moduli(int64_t N);
 // Residue planes of H (per modulus two planes of N x Kp bf16 for complex H,
 // one for real), row exponents and the real diagonal, which the epilogue
-// applies in FP64.  resident < nmod: memory holds only that many moduli at a
+// applies in FP64.  sym: all rows share one scale, 2^exponent, and complex H
+// has one plane per modulus too, the other being its transpose.  resident < nmod: memory holds only that many moduli at a
 // time, and every product slices H anew (src, lds) for each group of them.
 struct RnsH {
   void* A = nullptr;
@@ -179,6 +180,7 @@ struct RnsH {
   const void* src = nullptr;
   int64_t lds = 0;
   int src_kind = 0;  // 0 complex128, 1 float64, 2 complex64, 3 float32
+  int sym = 0, exponent = 0;
 };
 // Workspace for up to cap_cols columns at a time: residue planes of the block
 // (B), of the product (G), column exponents.
@@ -189,9 +191,13 @@ struct RnsX {
   int cap_cols = 0, planes = 0;
   int64_t Kp = 0, ldg = 0;
 };
-// reserve: bytes to leave free when the planes are large
+// reserve: bytes to leave free when the planes are large.  many: the planes
+// serve many products, which pays for looking whether one scale fits all rows
+// (a pass over H and a synchronisation).
+bool rns_sym_pays(int nmod, double entries);  // of H's, or of a whole batch's
 template <class T>
-int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, RnsH& out);
+int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
+                  RnsH& out);
 int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX& out);
 // C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1]
 template <class T>
@@ -245,6 +251,7 @@ struct GroupedProblem {
   void* G;            // residues of the product, the same shape (int16)
   long long Kp;       // residues: n rounded up to 64
   int n, b, bcap;     // rows, columns of the block, column capacity of Bsl and G
+  int sym;            // residues: as RnsH
 };
 // One active problem of one degree step: columns [s, b) of problem `prob`
 // are filtered; its output tiles are [tile0, next.tile0), its columns
@@ -274,11 +281,20 @@ struct GroupedSliceH {
   int* E;
   double* Dg;
   long long Kp;
-  int n, row0;
+  int n, row0, tile0;  // first global row, first global 64 x 64 tile
+  int s;               // the rows' common exponent (sym)
 };
 int64_t rns_k_padded(int64_t N);
+// Row exponents of every H, and their least and largest in minmax (per problem);
+// rns_same_scale says whether these allow one scale for all rows.
+int rns_grouped_row_exponents(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows,
+                              int* minmax);
+bool rns_same_scale(int lo, int hi);
+int rns_sym_tiles(int64_t n);
+// Planes of the problems with a scale per row, and of those with one scale.
 int rns_grouped_prepare_h(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows);
-int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, const void* A,
+int rns_grouped_prepare_sym(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_tiles);
+int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, bool sym, const void* A,
                      const void* B, int64_t n, int64_t b, int64_t bcap);
 RnsScale rns_scale(int nmod, double alpha, double beta, double shift);  // complex problems
 // Tiles (of width bn) and reconstruction blocks of one problem's step, and the
@@ -318,7 +334,7 @@ struct GroupedFilterInput {
   void* Bsl = nullptr;
   void* G = nullptr;
   int* F = nullptr;
-  int bcap = 0;
+  int bcap = 0, sym = 0;
 };
 struct GroupedFilterTimes {
   int tile_config = -1, steps = 0, launches = 0;

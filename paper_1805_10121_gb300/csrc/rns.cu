@@ -155,6 +155,18 @@ __device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
   return d;
 }
 
+// MN-major operand: 128-byte swizzled rows along M, one per K, in 8-row atoms
+// of 1024 bytes; the next 64 of M come 8192 bytes on.
+__device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(8192 >> 4) << 16;   // LBO: the next 64 of M
+  d |= (uint64_t)(1024 >> 4) << 32;   // SBO: the next 8 of K
+  d |= (uint64_t)1 << 46;             // version
+  d |= (uint64_t)2 << 61;             // SWIZZLE_128B
+  return d;
+}
+
 // 8 columns of this thread's row of an accumulator, as 4 column pairs.  The
 // loads are complete after tmem_wait_ld, through which their registers pass so
 // that no use of them can be scheduled before it.
@@ -226,6 +238,7 @@ struct Tile {
   const CUtensorMap* mapB;
   int row0, col0;      // first row, first column of the tile
   int planeA, planeB;  // plane of A and of B
+  bool trans;          // the tile of A is a transposed one of its plane
   int modulus;         // index of the plane's modulus
   int nst;             // stages (K / 64, rounded up)
   int M, ncols;        // rows, columns of the product
@@ -321,7 +334,12 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
           const uint32_t bar = map_to_rank(&full[st], 0);
           if (leader) {
             if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * C::STAGE);
-            tma_load_pair(smem_u32(sA + st * C::A_BYTES), T.mapA, ks * BK, ra, T.planeA, bar);
+            // two boxes of 64 x 64: 64 rows each, or 64 of M each when transposed
+            const uint32_t a = smem_u32(sA + st * C::A_BYTES);
+            const int x = T.trans ? ra : ks * BK, y = T.trans ? ks * BK : ra;
+            tma_load_pair(a, T.mapA, x, y, T.planeA, bar);
+            tma_load_pair(a + C::A_BYTES / 2, T.mapA, T.trans ? x + 64 : x, T.trans ? y : y + 64,
+                          T.planeA, bar);
             tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
           }
           __syncwarp();
@@ -337,9 +355,9 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
     }
   } else if (warp == 1) {
     if (rank == 0) {  // ---------------- MMA issuer
-      // kind::f16: FP32 D, BF16 A and B, K-major, M = 256, N = BN
-      constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                                 ((uint32_t)(2 * BM >> 4) << 24);
+      // kind::f16: FP32 D, BF16 A and B, K-major (bit 15: A MN-major), M = 256, N = BN
+      constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) |
+                                  ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
       bool ok = true;
       long long g = 0;   // stages consumed
       long long c = -1;  // current chunk (accumulator c & 1)
@@ -347,6 +365,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
         Tile T;
         tile(t, T);
         const int cs = tab.m[T.modulus].chunk;
+        const uint32_t idesc = T.trans ? idesc0 | (1u << 15) : idesc0;
         int in = 0;  // stage within the chunk
         for (int ks = 0; ks < T.nst; ++ks, ++g) {
           if (in == 0) {
@@ -367,11 +386,13 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           const uint32_t a0 = smem_u32(sA + st * C::A_BYTES), b0 = smem_u32(sB + st * C::B_BYTES);
           const uint32_t d = tmem + static_cast<uint32_t>(c & 1) * C::BUF;
+          const uint64_t da = T.trans ? desc_sw128_mn(a0) : desc_sw128(a0);
+          const uint64_t step = (T.trans ? 16 * 128 : 32) >> 4;  // 16 of K
           const bool last = in + 1 == cs || ks == T.nst - 1;
           if (leader) {
 #pragma unroll
             for (int k = 0; k < BK / 16; ++k)
-              umma_pair(d, desc_sw128(a0 + k * 32), desc_sw128(b0 + k * 32), idesc,
+              umma_pair(d, da + k * step, desc_sw128(b0 + k * 32), idesc,
                         (in == 0 && k == 0) ? 0u : 1u);
             commit_pair(&empty[st]);
             if (last) commit_pair(&acc_full[c & 1]);
@@ -470,7 +491,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
 struct OneProduct {
   const CUtensorMap* mapA;
   const CUtensorMap* mapB;
-  int rtiles, ctiles, plane0, per_modulus, swap_a, bn, nst, M, ncols;
+  int rtiles, ctiles, plane0, per_modulus, swap_a, sym, bn, nst, M, ncols;
   int16_t* G;
   long long ldg, gplane;
   __device__ __forceinline__ void operator()(int t, Tile& T) const {
@@ -480,7 +501,8 @@ struct OneProduct {
     T.mapB = mapB;
     T.row0 = rt * 2 * BM;
     T.col0 = ct * bn;
-    T.planeA = pl ^ swap_a;
+    T.planeA = sym ? pl >> 1 : pl ^ swap_a;
+    T.trans = sym && (pl & 1);
     T.planeB = plane0 + pl;
     T.modulus = T.planeB / per_modulus;
     T.nst = nst;
@@ -495,10 +517,10 @@ template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmTab tab, int rtiles, int ctiles, int nplanes,
-                    int plane0, int per_modulus, int swap_a, int nst, int M, int ncols,
+                    int plane0, int per_modulus, int swap_a, int sym, int nst, int M, int ncols,
                     int16_t* __restrict__ G,
                     long long ldg, long long gplane, int* __restrict__ err) {
-  OneProduct p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, BN, nst, M, ncols,
+  OneProduct p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, sym, BN, nst, M, ncols,
                G, ldg, gplane};
   gemm_body<BN>(p, rtiles * ctiles * nplanes, tab, 0, err);
 }
@@ -675,7 +697,8 @@ __device__ __forceinline__ int scale_exponent(float ss, uint32_t mb, int off, fl
 }
 
 // Residues in planes [m0, m1) of two neighbouring integers (xr + i xi).
-template <int NM, int NL, bool CP>
+// With BOTH the plane of re - j im follows that of re + j im.
+template <int NM, int NL, bool CP, bool BOTH = CP>
 __device__ __forceinline__ void store_residues(const long long (&xr)[2], const long long (&xi)[2],
                                                __nv_bfloat16* __restrict__ o, long long stride,
                                                const SliceTab& tab, int m0, int m1) {
@@ -703,9 +726,10 @@ __device__ __forceinline__ void store_residues(const long long (&xr)[2], const l
 #pragma unroll
       for (int i = 1; i < NL; ++i) ni = fma_f32x2(pi[i], t.jc[i], ni);
       *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(add_f32x2(nr, ni), t));
-      *reinterpret_cast<uint32_t*>(o + stride) =
-          pack2(reduce2(fma_f32x2(ni, pack_f32x2(-1.f, -1.f), nr), t));
-      o += 2 * stride;
+      if constexpr (BOTH)
+        *reinterpret_cast<uint32_t*>(o + stride) =
+            pack2(reduce2(fma_f32x2(ni, pack_f32x2(-1.f, -1.f), nr), t));
+      o += BOTH ? 2 * stride : stride;
     } else {
       *reinterpret_cast<uint32_t*>(o) = pack2(reduce2(nr, t));
       o += stride;
@@ -713,17 +737,11 @@ __device__ __forceinline__ void store_residues(const long long (&xr)[2], const l
   }
 }
 
-// One vector of n entries (a column of X, or column r of the Hermitian H as
-// row r conjugated) to its residues in planes [m0, m1): element k of plane
-// (m - m0) goes to out[plane * stride + k].  skip: index left out (set to
-// zero), -1 for none.  Integer and packed FP32 arithmetic only, two entries at
-// a time; the norm that sets the scale is summed in FP32 from truncated bits,
-// with a margin for what that loses.
-template <int NM, int NL, class E>
-__device__ __forceinline__ void slice_vector(const E* __restrict__ v, int n, bool conj, int skip,
-                                             __nv_bfloat16* __restrict__ out, long long stride,
-                                             int* __restrict__ exponent, const SliceTab& tab, int m0,
-                                             int m1) {
+// Exponent (scale_exponent) of a vector of n entries, the one at `skip` left
+// out; *nonzero: whether any other is not zero.  Block-wide.
+template <class E>
+__device__ __forceinline__ int vector_exponent(const E* __restrict__ v, int n, int skip, float L,
+                                               bool* nonzero) {
   constexpr bool CP = is_complex<E>;
   __shared__ float sf[kSliceThreads / 32];
   __shared__ uint32_t su[kSliceThreads / 32];
@@ -760,7 +778,24 @@ __device__ __forceinline__ void slice_vector(const E* __restrict__ v, int n, boo
     uint32_t same = mb;
     reduce_block(ss, same, sf, su);
   }
-  const int s = scale_exponent(ss, mb, off, (CP ? 2.f : 1.f) * n, tab.log2_norm);
+  *nonzero = mb != 0;
+  return scale_exponent(ss, mb, off, (CP ? 2.f : 1.f) * n, L);
+}
+
+// One vector of n entries (a column of X, or column r of the Hermitian H as
+// row r conjugated) to its residues in planes [m0, m1): element k of plane
+// (m - m0) goes to out[plane * stride + k].  skip: index left out (set to
+// zero), -1 for none.  Integer and packed FP32 arithmetic only, two entries at
+// a time; the norm that sets the scale is summed in FP32 from truncated bits,
+// with a margin for what that loses.
+template <int NM, int NL, class E>
+__device__ __forceinline__ void slice_vector(const E* __restrict__ v, int n, bool conj, int skip,
+                                             __nv_bfloat16* __restrict__ out, long long stride,
+                                             int* __restrict__ exponent, const SliceTab& tab, int m0,
+                                             int m1) {
+  constexpr bool CP = is_complex<E>;
+  bool nonzero;
+  const int s = vector_exponent(v, n, skip, tab.log2_norm, &nonzero);
   if (threadIdx.x == 0) *exponent = s;
   const bool zero = s == kNonFinite;
   for (int k = 2 * threadIdx.x; k < n; k += 2 * kSliceThreads) {
@@ -795,6 +830,97 @@ __global__ void __launch_bounds__(kSliceThreads)
   if (threadIdx.x == 0) Dg[r] = re_of(col[r]);
   slice_vector<NM, NL, E>(col, N, true, r, A + r * Kp, static_cast<long long>(N) * Kp, Ex + r, tab,
                           m0, m1);
+}
+
+// Exponent of every row of the Hermitian H (from its column, without the
+// diagonal), and the least and the largest over the rows that are not zero.
+template <class E>
+__device__ __forceinline__ void row_exponent(const E* __restrict__ H, long long ldh, int N, int r,
+                                             float L, int* __restrict__ Ex,
+                                             int* __restrict__ minmax) {
+  bool nonzero;
+  const int s = vector_exponent(H + r * ldh, N, r, L, &nonzero);
+  if (threadIdx.x == 0) {
+    Ex[r] = s;
+    if (nonzero) {
+      atomicMin(&minmax[0], s);
+      atomicMax(&minmax[1], s);
+    }
+  }
+}
+template <class E>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_row_exponent_kernel(const E* __restrict__ H, long long ldh, int N, float L,
+                            int* __restrict__ Ex, int* __restrict__ minmax) {
+  row_exponent(H, ldh, N, blockIdx.x, L, Ex, minmax);
+}
+
+// One 64 x 64 tile of the lower triangle of a complex Hermitian H, scaled by
+// 2^s, to one residue plane per modulus: re + j im at (r, k) and, its
+// conjugate's, re - j im at (k, r).  The second plane of the modulus is the
+// transpose of the first.  Only the lower triangle is read, so the plane is
+// exactly that of a Hermitian matrix whatever rounding left in H.
+constexpr int kSymTile = 64;
+constexpr int kSymSmem = 2 * kSymTile * (kSymTile + 1) * 8;
+template <int NM, int NL, class E>
+__device__ __forceinline__ void slice_sym_tile(const E* __restrict__ H, long long ldh, int N, int idx,
+                                               int s, const SliceTab& tab, int m0, int m1,
+                                               __nv_bfloat16* __restrict__ A, long long Kp,
+                                               int* __restrict__ Ex, double* __restrict__ Dg) {
+  extern __shared__ long long sym_smem[];
+  auto re_t = reinterpret_cast<long long (*)[kSymTile + 1]>(sym_smem);
+  auto im_t = re_t + kSymTile;
+  int R = static_cast<int>((sqrtf(8.f * idx + 1.f) - 1.f) * 0.5f);
+  while ((R + 1) * (R + 2) / 2 <= idx) ++R;
+  while (R * (R + 1) / 2 > idx) --R;
+  const int K = idx - R * (R + 1) / 2, r0 = R * kSymTile, k0 = K * kSymTile;
+  const bool diag = R == K;
+  for (int e = threadIdx.x; e < kSymTile * kSymTile; e += kSliceThreads) {
+    const int r = e % kSymTile, k = e / kSymTile;
+    if (diag && r < k) continue;
+    long long xr = 0, xi = 0;
+    if (r0 + r < N && k0 + k < N) {
+      const E v = H[(k0 + k) * ldh + r0 + r];
+      if (diag && r == k) {
+        Dg[r0 + r] = re_of(v);
+        Ex[r0 + r] = s;
+      } else {
+        xr = scaled_int(re_in(v), s);
+        xi = scaled_int(im_in(v), s);
+      }
+    }
+    re_t[r][k] = xr;
+    im_t[r][k] = xi;
+    if (diag && r > k) {
+      re_t[k][r] = xr;
+      im_t[k][r] = -xi;
+    }
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long plane = N * Kp;
+  for (int q = warp; q < kSymTile; q += kSliceThreads / 32) {
+    if (r0 + q < N) {
+      const long long xr[2] = {re_t[q][2 * lane], re_t[q][2 * lane + 1]};
+      const long long xi[2] = {im_t[q][2 * lane], im_t[q][2 * lane + 1]};
+      store_residues<NM, NL, true, false>(xr, xi, A + (r0 + q) * Kp + k0 + 2 * lane, plane, tab, m0,
+                                          m1);
+    }
+    if (!diag && k0 + q < N) {
+      const long long xr[2] = {re_t[2 * lane][q], re_t[2 * lane + 1][q]};
+      const long long xi[2] = {-im_t[2 * lane][q], -im_t[2 * lane + 1][q]};
+      store_residues<NM, NL, true, false>(xr, xi, A + (k0 + q) * Kp + r0 + 2 * lane, plane, tab, m0,
+                                          m1);
+    }
+  }
+}
+template <int NM, int NL, class E>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_slice_sym_kernel(const E* __restrict__ H, long long ldh, int N, int s,
+                         const __grid_constant__ SliceTab tab, int m0, int m1,
+                         __nv_bfloat16* __restrict__ A, long long Kp, int* __restrict__ Ex,
+                         double* __restrict__ Dg) {
+  slice_sym_tile<NM, NL, E>(H, ldh, N, blockIdx.x, s, tab, m0, m1, A, Kp, Ex, Dg);
 }
 
 // Columns [j0, j0 + gridDim.x) of X.
@@ -1108,6 +1234,21 @@ __device__ __forceinline__ int find_entry(const S* s, int n, int S::*prefix, int
   return lo;
 }
 
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_grouped_row_exponent_kernel(const GroupedSliceH* __restrict__ probs, int P, float L,
+                                    int* __restrict__ minmax) {
+  const int p = find_entry(probs, P, &GroupedSliceH::row0, blockIdx.x);
+  const GroupedSliceH& q = probs[p];
+  row_exponent(q.H, q.ldh, q.n, blockIdx.x - q.row0, L, q.E, minmax + 2 * p);
+}
+template <int NM, int NL>
+__global__ void __launch_bounds__(kSliceThreads)
+    rns_grouped_slice_sym_kernel(const GroupedSliceH* __restrict__ probs, int P,
+                                 const __grid_constant__ SliceTab tab) {
+  const GroupedSliceH& q = probs[find_entry(probs, P, &GroupedSliceH::tile0, blockIdx.x)];
+  slice_sym_tile<NM, NL, double2>(q.H, q.ldh, q.n, blockIdx.x - q.tile0, q.s, tab, 0, NM,
+                                  static_cast<__nv_bfloat16*>(q.A), q.Kp, q.E, q.Dg);
+}
 template <int NM, int NL>
 __global__ void __launch_bounds__(kSliceThreads)
     rns_grouped_slice_h_kernel(const GroupedSliceH* __restrict__ probs, int P,
@@ -1151,8 +1292,9 @@ struct GroupedTiles {
     T.mapB = q.mapB0 + (bn / 32 - 1);  // one map per tile width
     T.row0 = rt * 2 * BM;
     T.col0 = ct * bn;
-    T.planeA = pl;
+    T.planeA = q.sym ? pl >> 1 : pl;
     T.planeB = pl;
+    T.trans = q.sym && (pl & 1);
     T.modulus = pl / 2;
     T.nst = (q.n + BK - 1) / BK;
     T.M = q.n;
@@ -1333,6 +1475,7 @@ struct GemmArgs {
   int64_t b_rows, b_planes;  // B: b_planes of b_rows x Kp (plane stride), ncols rows used
   int ncols, nplanes, plane0, per_modulus;
   int swap_a = 0;  // 1: A conjugated (the two planes of a modulus change places)
+  int sym = 0;     // 1: A has one plane per modulus, the other is its transpose
   int16_t* G;
   int64_t ldg, gplane;
   const GemmTab* tab;
@@ -1347,7 +1490,7 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
     return CHASE_CUDA_ERROR;
   }
   CUtensorMap tmA, tmB;
-  CHASE_TRY(make_tmap_bf16_3d(&tmA, a.A, a.K, a.M, a.a_planes, a.Kp * 2, a.Kp * 2 * a.M, BK, BM, 1));
+  CHASE_TRY(make_tmap_bf16_3d(&tmA, a.A, a.K, a.M, a.a_planes, a.Kp * 2, a.Kp * 2 * a.M, BK, 64, 1));
   CHASE_TRY(make_tmap_bf16_3d(&tmB, a.B, a.K, a.ncols, a.b_planes, a.Kp * 2, a.Kp * 2 * a.b_rows,
                               BK, BN / 2, 1));
   const int rt = static_cast<int>((a.M + 2 * BM - 1) / (2 * BM));
@@ -1355,7 +1498,7 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
   const int64_t tiles = static_cast<int64_t>(rt) * ct * a.nplanes;
   const unsigned grid = 2 * static_cast<unsigned>(std::min<int64_t>(tiles, pairs));
   CHASE_CUDA(launch_pdl(rns_gemm_kernel<BN>, dim3(grid), dim3(kThreads), C::SMEM, d.st, tmA, tmB,
-                        *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a,
+                        *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a, a.sym,
                         static_cast<int>((a.K + BK - 1) / BK), static_cast<int>(a.M), a.ncols, a.G,
                         a.ldg, a.gplane, d.err));
   note_launch();
@@ -1397,16 +1540,57 @@ int run_gemm(Dev& d, const GemmArgs& a) {
   }
 }
 
+bool same_scale(int lo, int hi) {
+  return lo <= hi && hi != kNonFinite && static_cast<long long>(hi) - lo <= 1;
+}
+
 // Limbs of an operand scaled to 2^L: 13 bits each, the top one up to 14.
 constexpr int limbs_of(int nm) { return nm <= 8 ? 3 : nm <= 12 ? 4 : 5; }
 
+int sym_tiles(int64_t n) {
+  const int64_t t = (n + kSymTile - 1) / kSymTile;
+  return static_cast<int>(t * (t + 1) / 2);
+}
 template <int NM, class E>
 int slice_h(Dev& d, const RnsH& h, int m0, int m1) {
+  const SliceTab& tab = tables(NM, is_complex<E>).slice;
+  if constexpr (is_complex<E>) {
+    if (h.sym) {
+      auto kernel = rns_slice_sym_kernel<NM, limbs_of(NM), E>;
+      static const cudaError_t ready = cudaFuncSetAttribute(
+          kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSymSmem);
+      CHASE_CUDA(ready);
+      kernel<<<sym_tiles(h.N), kSliceThreads, kSymSmem, d.st>>>(
+          static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N), h.exponent, tab, m0, m1,
+          static_cast<__nv_bfloat16*>(h.A), h.Kp, h.E, h.Dg);
+      note_launch();
+      CHASE_CUDA(cudaGetLastError());
+      return CHASE_OK;
+    }
+  }
   rns_slice_h_kernel<NM, limbs_of(NM), E><<<static_cast<unsigned>(h.N), kSliceThreads, 0, d.st>>>(
-      static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N),
-      tables(NM, is_complex<E>).slice, m0, m1, static_cast<__nv_bfloat16*>(h.A), h.Kp, h.E, h.Dg);
+      static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N), tab, m0, m1,
+      static_cast<__nv_bfloat16*>(h.A), h.Kp, h.E, h.Dg);
   note_launch();
   CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+// Whether all rows of H want the same scale, give or take one bit, and which.
+template <class E>
+int row_scales(Dev& d, const E* H, int64_t ldh, RnsH& h) {
+  int* mm = nullptr;
+  CHASE_TRY(d.alloc(&mm, 2));
+  int host[2] = {kNonFinite, -kNonFinite};
+  CHASE_CUDA(cudaMemcpyAsync(mm, host, sizeof(host), cudaMemcpyHostToDevice, d.st));
+  rns_row_exponent_kernel<E><<<static_cast<unsigned>(h.N), kSliceThreads, 0, d.st>>>(
+      H, ldh, static_cast<int>(h.N), tables(h.nmod, true).slice.log2_norm, h.E, mm);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  CHASE_CUDA(cudaMemcpyAsync(host, mm, sizeof(host), cudaMemcpyDeviceToHost, d.st));
+  CHASE_TRY(d.sync_check("residues of H"));
+  d.release(mm);
+  h.sym = same_scale(host[0], host[1]);
+  h.exponent = host[0];
   return CHASE_OK;
 }
 template <class E>
@@ -1460,7 +1644,8 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
       a.K = N;
       a.M = N;
       a.Kp = h.Kp;
-      a.a_planes = static_cast<int64_t>(h.resident) * PP;
+      a.a_planes = static_cast<int64_t>(h.resident) * (h.sym ? 1 : PP);
+      a.sym = h.sym;
       a.B = x.B;
       a.b_rows = x.cap_cols;
       a.b_planes = NM * PP;
@@ -1639,8 +1824,15 @@ struct Kind<float> {
 int rns_split_moduli(int64_t N) { return N <= 32768 ? 11 : 12; }
 int rns_low_moduli(int64_t N) { return N <= 8192 ? 7 : 8; }
 
+// One plane per modulus instead of two halves what a product streams, once the
+// planes outgrow about half of the L2; below, the pass over H that looks for a
+// common scale costs more (filter N = 1000, 57 MB: 1150 us with two planes,
+// 1170 with one; complex64 N = 2000, 115 MB: 1876 and 1722; split N = 2048, 185
+// MB: 2167 and 1889; N = 4096, 940 MB: 5210 and 4541).
+bool rns_sym_pays(int nmod, double entries) { return 4.0 * nmod * entries > 64e6; }
+
 template <class T>
-int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve,
+int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
                   RnsH& out) {
   out.N = N;
   out.Kp = (N + rns::BK - 1) / rns::BK * rns::BK;
@@ -1649,7 +1841,11 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
   out.nmod = nmod;
   out.src = H;
   out.lds = ldh;
-  const size_t per = static_cast<size_t>(out.cplx ? 2 : 1) * N * out.Kp * 2;  // bytes per modulus
+  CHASE_TRY(d.alloc(&out.E, static_cast<size_t>(N)));
+  CHASE_TRY(d.alloc(&out.Dg, static_cast<size_t>(N)));
+  if constexpr (rns::is_complex<typename Kind<T>::D>)
+    if (many && rns_sym_pays(nmod, static_cast<double>(N) * out.Kp)) CHASE_TRY(rns::row_scales(d, reinterpret_cast<const typename Kind<T>::D*>(H), ldh, out));
+  const size_t per = static_cast<size_t>(out.cplx && !out.sym ? 2 : 1) * N * out.Kp * 2;  // bytes per modulus
   // all moduli resident where the memory allows it; else fewer, sliced anew
   // for every product
   out.resident = nmod;
@@ -1665,8 +1861,6 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
     if (st != CHASE_OUT_OF_MEMORY) break;
   }
   CHASE_TRY(st);
-  CHASE_TRY(d.alloc(&out.E, static_cast<size_t>(N)));
-  CHASE_TRY(d.alloc(&out.Dg, static_cast<size_t>(N)));
   if (out.resident == nmod) return rns::slice_h_moduli(d, out, 0, nmod);
   return CHASE_OK;
 }
@@ -1756,6 +1950,18 @@ RnsScale rns_scale(int nmod, double alpha, double beta, double shift) {
   return rns::crt_scale(rns::tables(nmod, true).crt, alpha, beta, shift);
 }
 
+int rns_grouped_row_exponents(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows,
+                              int* minmax) {
+  rns::rns_grouped_row_exponent_kernel<<<static_cast<unsigned>(total_rows), rns::kSliceThreads, 0,
+                                         d.st>>>(
+      probs, P, rns::tables(nmod, true).slice.log2_norm, minmax);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+bool rns_same_scale(int lo, int hi) { return rns::same_scale(lo, hi); }
+int rns_sym_tiles(int64_t n) { return rns::sym_tiles(n); }
+
 int rns_grouped_prepare_h(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_rows) {
   return rns::with_moduli(nmod, [&](auto nm) -> int {
     constexpr int NM = decltype(nm)::value;
@@ -1767,11 +1973,25 @@ int rns_grouped_prepare_h(Dev& d, int nmod, const GroupedSliceH* probs, int P, i
     return CHASE_OK;
   });
 }
+int rns_grouped_prepare_sym(Dev& d, int nmod, const GroupedSliceH* probs, int P, int total_tiles) {
+  return rns::with_moduli(nmod, [&](auto nm) -> int {
+    constexpr int NM = decltype(nm)::value;
+    auto kernel = rns::rns_grouped_slice_sym_kernel<NM, rns::limbs_of(NM)>;
+    static const cudaError_t ready = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rns::kSymSmem);
+    CHASE_CUDA(ready);
+    kernel<<<static_cast<unsigned>(total_tiles), rns::kSliceThreads, rns::kSymSmem, d.st>>>(
+        probs, P, rns::tables(NM, true).slice);
+    note_launch();
+    CHASE_CUDA(cudaGetLastError());
+    return CHASE_OK;
+  });
+}
 
-int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, const void* A,
+int rns_grouped_maps(CUtensorMap* mapA, CUtensorMap* mapB, int nmod, int bn, bool sym, const void* A,
                      const void* B, int64_t n, int64_t b, int64_t bcap) {
   const int64_t Kp = rns_k_padded(n);
-  CHASE_TRY(make_tmap_bf16_3d(mapA, A, n, n, 2 * nmod, Kp * 2, Kp * 2 * n, rns::BK, rns::BM, 1));
+  CHASE_TRY(make_tmap_bf16_3d(mapA, A, n, n, sym ? nmod : 2 * nmod, Kp * 2, Kp * 2 * n, rns::BK, 64, 1));
   return make_tmap_bf16_3d(mapB, B, n, b, 2 * nmod, Kp * 2, Kp * 2 * bcap, rns::BK, bn / 2, 1);
 }
 
@@ -1830,7 +2050,7 @@ int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const Grouped
 }
 
 #define CHASE_INSTANTIATE_RNS(T)                                                                 \
-  template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, RnsH&);           \
+  template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, bool, RnsH&);     \
   template int rns_product<T>(Dev&, const RnsH&, RnsX&, const T*, int64_t, int, int, T*, int64_t, \
                               double, double, double);
 CHASE_INSTANTIATE_RNS(chase_c64)
