@@ -861,7 +861,8 @@ struct Solver {
     filter_set.low = want_low ? &hlow : nullptr;
     filter_set.x = &rx;
     rr_set.full = want64 ? &h64 : split_rr ? &hsplit : nullptr;
-    rr_set.low = want_low ? &hlow : nullptr;
+    // Rayleigh-Ritz keeps FP64 accuracy whatever the filter's precision is
+    rr_set.low = is_single<T> ? filter_set.low : nullptr;
     rr_set.x = &rx;
     return CHASE_OK;
   }
