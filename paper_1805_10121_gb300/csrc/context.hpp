@@ -106,6 +106,10 @@ int launch_fill_upper_hermitian(Dev& d, T* G, int64_t ldg, int p);
 template <class T>
 int cholesky_inverse(Dev& d, T* G, int64_t ldg, int p, double rel_tol, double shift,
                      double* diag_ref);
+// R (p x p) = L^-H up to ||E||^2 for G = I + E (its lower triangle) = L L^H;
+// e2[j]: the squared norm of column j of E's lower triangle.
+template <class T>
+int launch_near_identity(Dev& d, const T* G, int64_t ldg, int p, T* R, int64_t ldr, double* e2);
 // One Lanczos three-term step on r independent runs (one CTA per run, run c
 // in column c of each N x r block, leading dimension ld):
 // alpha = Re(v^H w); w -= alpha v + beta_prev v_prev; beta = ||w||;

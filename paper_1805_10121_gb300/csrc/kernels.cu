@@ -60,8 +60,8 @@ struct Sc<double2> {
   static __device__ __forceinline__ double2 conj(double2 a) { return make_double2(a.x, -a.y); }
   // acc - a conj(b)
   static __device__ __forceinline__ double2 sub_mul_conj(double2 acc, double2 a, double2 b) {
-    acc.x -= a.x * b.x + a.y * b.y;
-    acc.y -= a.y * b.x - a.x * b.y;
+    acc.x = fma(-a.x, b.x, fma(-a.y, b.y, acc.x));  // four FMAs, not six instructions
+    acc.y = fma(-a.y, b.x, fma(a.x, b.y, acc.y));
     return acc;
   }
   // Re(conj(a) b)
@@ -619,6 +619,32 @@ __global__ void __launch_bounds__(256)
     *g = acc;
 }
 
+// G = I + E (lower triangle) near the identity: column j of I - Phi(E)^H, with
+// Phi the lower triangle and half the diagonal, which is L^-H up to ||E||^2.
+// out[j] = the squared norm of column j of E's lower triangle.
+template <class T>
+__global__ void __launch_bounds__(kRed)
+    near_identity_kernel(const T* __restrict__ G, long long ldg, int p, T* __restrict__ R,
+                         long long ldr, double* __restrict__ out) {
+  __shared__ double scratch[33];
+  const int j = blockIdx.x;
+  double s = 0.0;
+  for (int i = threadIdx.x; i < p; i += kRed) {
+    T v = Sc<T>::zero();
+    if (i < j) {
+      v = Sc<T>::scale(Sc<T>::conj(G[static_cast<long long>(i) * ldg + j]), -1.0);
+      s += Sc<T>::abs2(v);
+    } else if (i == j) {
+      const double e = Sc<T>::re(G[static_cast<long long>(j) * ldg + j]) - 1.0;
+      v = Sc<T>::real(1.0 - 0.5 * e);
+      s += e * e;
+    }
+    R[static_cast<long long>(j) * ldr + i] = v;
+  }
+  s = block_sum(s, scratch);
+  if (threadIdx.x == 0) out[j] = s;
+}
+
 template <class T>
 __global__ void copy_diag_kernel(const T* __restrict__ G, long long ld, int p,
                                  double* __restrict__ out, double shift) {
@@ -922,6 +948,15 @@ int launch_zero_triangle(Dev& d, T* A, int64_t lda, int p, bool lower) {
 }
 
 template <class T>
+int launch_near_identity(Dev& d, const T* G, int64_t ldg, int p, T* R, int64_t ldr, double* e2) {
+  if (p == 0) return CHASE_OK;
+  near_identity_kernel<<<p, kRed, 0, d.st>>>(dp(G), ldg, p, dp(R), ldr, e2);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+
+template <class T>
 int cholesky_inverse(Dev& d, T* G, int64_t ldg, int p, double rel_tol, double shift,
                      double* diag_ref) {
   if (p == 0) return CHASE_OK;
@@ -983,6 +1018,7 @@ int launch_normalize_cols(Dev& d, T* X, int64_t ldx, int64_t N, int r) {
   template int launch_zero_triangle<T>(Dev&, T*, int64_t, int, bool);                              \
   template int launch_hermitian_from_lower<T>(Dev&, const T*, int64_t, T*, int64_t, int64_t);      \
   template int cholesky_inverse<T>(Dev&, T*, int64_t, int, double, double, double*);               \
+  template int launch_near_identity<T>(Dev&, const T*, int64_t, int, T*, int64_t, double*);         \
   template int launch_lanczos_step<T>(Dev&, int64_t, int64_t, int, int, const T*, const T*, T*,    \
                                       T*, double*, double*, double);                               \
   template int launch_normalize_cols<T>(Dev&, T*, int64_t, int64_t, int);

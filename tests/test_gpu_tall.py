@@ -86,3 +86,17 @@ def test_rayleigh_ritz(n, b):
     assert np.max(np.abs(resid - res)) <= 50 * (b + n ** 0.5) * U / max(np.min(np.diff(lam)), 1e-6)
     x = qd.cpu().numpy()
     assert np.linalg.norm(x.conj().T @ x - np.eye(b)) <= 20 * (b + n ** 0.5) * U
+
+
+@pytest.mark.parametrize("n,b", [(300, 33), (700, 129)])
+@pytest.mark.parametrize("decades", [0, 2, 4, 5])
+def test_second_pass_near_and_far_from_the_identity(n, b, decades):
+    # the first pass leaves cond(V)^2 u: below 1e-8 the second factor is its
+    # first-order form, above it the whole elimination
+    rng = np.random.default_rng(n + decades)
+    w = np.linalg.qr(rng.standard_normal((b, b)) + 1j * rng.standard_normal((b, b)))[0]
+    v = (householder(gauss(n, b, n).numpy())[0] * np.logspace(0.0, -decades, b)[None, :]) @ w
+    ref, cond = householder(v)
+    q = chase.chase_orthonormalize(None, on_device(torch.from_numpy(v))).cpu().numpy()
+    assert np.linalg.norm(q.conj().T @ q - np.eye(b)) <= 20 * (b + n ** 0.5) * U
+    assert np.linalg.norm(q - ref) <= 20 * cond * (b + n ** 0.5) * U
