@@ -158,10 +158,10 @@ size_t rns_reserve(int64_t N, int b) {
 template <class T>
 int filter_product(Dev& d, const T* H, int64_t N, int64_t ldh, const RnsSet* rs, const T* X,
                    int64_t ldx, int b, T* Y, int64_t ldy, int j0, double alpha, double beta,
-                   double shift, int nslices = 7) {
+                   double shift, int nslices = 7, bool sliced = false, int next0 = -1) {
   if (rs) {
     const RnsH* h = nslices < 7 || !rs->full ? rs->low : rs->full;
-    return rns_product(d, *h, *rs->x, X, ldx, j0, b, Y, ldy, alpha, beta, shift);
+    return rns_product(d, *h, *rs->x, X, ldx, j0, b, Y, ldy, alpha, beta, shift, sliced, next0);
   }
   return timed_h_product(d, H, N, ldh, X, ldx, b, Y, ldy, j0, alpha, beta, shift);
 }
@@ -191,18 +191,23 @@ int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx,
   const double e = 0.5 * (b_sup - mu_nn);
   const double sigma1 = e / (mu1 - c);     // line 3
   long long mv = 0, low = 0;
-  auto product = [&](const FilterGroup& g, int s, const T* src, int64_t lds, T* dst, int64_t ldd,
+  // a single run of columns: each product leaves the residues of its result
+  // for the next one
+  const bool chain = rs && groups.size() == 1 &&
+                     rns_chains(rs->full ? *rs->full : *rs->low, groups[0].ncols, *rs->x);
+  auto product = [&](const FilterGroup& g, int i, const T* src, int64_t lds, T* dst, int64_t ldd,
                      double alpha, double beta) -> int {
-    const int j0 = g.col0 + s, j1 = g.col0 + g.ncols;
+    const int j0 = g.col0 + (i > 1 ? g.start[i] : 0), j1 = g.col0 + g.ncols;
     if (j0 >= j1) return CHASE_OK;
     CHASE_TRY(filter_product(d, H, N, ldh, rs, src, lds, j1, dst, ldd, j0, alpha, beta, c,
-                             g.nslices));
+                             g.nslices, chain && i > 1,
+                             chain && i < maxdeg ? g.col0 + g.start[i + 1] : -1));
     mv += j1 - j0;
     if (rs && g.nslices < 7) low += j1 - j0;
     return CHASE_OK;
   };
   // line 4: W = (sigma_1 / e) (H - c I) V
-  for (const FilterGroup& g : groups) CHASE_TRY(product(g, 0, X, ldx, Wk, ldw, sigma1 / e, 0.0));
+  for (const FilterGroup& g : groups) CHASE_TRY(product(g, 1, X, ldx, Wk, ldw, sigma1 / e, 0.0));
   double sigma = sigma1;  // line 5
   T* Vb = X;
   T* Wb = Wk;
@@ -212,7 +217,7 @@ int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx,
     // line 9: V[:, s:] = 2 (tau / e) (H - c I) W[:, s:] - tau sigma V[:, s:],
     // s = the first column of each run with degree >= i (lines 12-14)
     for (const FilterGroup& g : groups)
-      CHASE_TRY(product(g, g.start[i], Wb, ldW, Vb, ldV, 2.0 * tau / e, -tau * sigma));
+      CHASE_TRY(product(g, i, Wb, ldW, Vb, ldV, 2.0 * tau / e, -tau * sigma));
     std::swap(Vb, Wb);  // line 10
     std::swap(ldV, ldW);
     sigma = tau;  // line 11

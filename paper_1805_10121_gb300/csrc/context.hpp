@@ -194,6 +194,7 @@ struct RnsX {
   int* F = nullptr;
   int cap_cols = 0, planes = 0;
   int64_t Kp = 0, ldg = 0;
+  int flip = 0;  // which half of F (2 cap_cols) the residues in B belong to
 };
 // reserve: bytes to leave free when the planes are large.  many: the planes
 // serve many products, which pays for looking whether one scale fits all rows
@@ -203,10 +204,15 @@ template <class T>
 int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
                   RnsH& out);
 int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX& out);
-// C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1]
+// C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1].
+// Chained products (where rns_chains allows it for the widest): next0 >= 0
+// leaves the residues of C[:, next0:j1] in x, and a product with sliced takes
+// those as X[:, j0:j1] for its j0 = next0.
+bool rns_chains(const RnsH& h, int b, const RnsX& x);
 template <class T>
 int rns_product(Dev& d, const RnsH& h, RnsX& x, const T* X, int64_t ldx, int j0, int j1, T* C,
-                int64_t ldc, double alpha, double beta, double shift);
+                int64_t ldc, double alpha, double beta, double shift, bool sliced = false,
+                int next0 = -1);
 
 // Products of tall blocks (orthogonalisation, Rayleigh-Ritz) at FP64 accuracy.
 // n vectors of K entries in residue planes: the columns of a block, or its rows.

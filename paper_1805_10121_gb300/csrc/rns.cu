@@ -1089,6 +1089,125 @@ struct Out<float> {
 // shares, alpha P and alpha (H_rr - shift), carry a second double: their
 // rounding would be the same in every degree step and so add up over the
 // recurrence, where the roundings of an FP64 GEMM average out.
+// What two rows of a product share over its columns.
+struct CrtRows {
+  int er[2];
+  double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (as two doubles)
+  bool diag[2];
+};
+__device__ __forceinline__ void crt_constants(CrtRows& k, int r0, int M, const int* __restrict__ Ex,
+                                              const double* __restrict__ Dg, const RnsScale& sc) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const bool in = r0 + h < M;
+    k.er[h] = in ? Ex[r0 + h] : 0;
+    const double a = in && Dg ? Dg[r0 + h] : 0.0, b = -sc.shift;
+    double d = a + b;
+    const double t = d - a;
+    double l = (a - (d - t)) + (b - t);
+    k.diag[h] = d != 0.0;
+    if (sc.plain) {
+      const double p = sc.alpha * d;
+      l = fma(sc.alpha, d, -p) + sc.alpha * l;
+      d = p;
+    }
+    k.dh[h] = d;
+    k.dl[h] = l;
+  }
+}
+
+// Rows r0, r0 + 1 of column j0 + c of the product: written to C and returned.
+template <int NM, class E>
+__device__ __forceinline__ void crt_pair(const CrtRows& k, int r0, int c,
+                                         const int16_t* __restrict__ G, long long ldg,
+                                         long long gplane, const CrtTab& tab,
+                                         const int* __restrict__ Fx, int M, int j0,
+                                         const E* __restrict__ X, long long ldx,
+                                         E* __restrict__ C, long long ldc, const RnsScale& sc,
+                                         E (&out)[2]) {
+  constexpr bool CP = is_complex<E>;
+  constexpr int W = CP ? 2 : 1;
+  constexpr bool ACC = NM == kRnsFp64;
+  using S = typename Out<E>::S;
+  const int16_t* g = G + static_cast<long long>(c) * ldg + r0;
+  unsigned long long hi[2][W] = {};
+  int lo[2][W] = {};
+#pragma unroll
+  for (int m = 0; m < NM; ++m) {
+    const CrtMod& t = tab.m[m];
+    if constexpr (CP) {
+      const uint32_t u = *reinterpret_cast<const uint32_t*>(g + (2 * m) * gplane);
+      const uint32_t w = *reinterpret_cast<const uint32_t*>(g + (2 * m + 1) * gplane);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int a = static_cast<int16_t>(u >> (16 * h)), b = static_cast<int16_t>(w >> (16 * h));
+        const int s = a + b, d = a - b;
+        hi[h][0] += static_cast<unsigned long long>(static_cast<long long>(s)) * t.re_hi;
+        hi[h][1] += static_cast<unsigned long long>(static_cast<long long>(d)) * t.im_hi;
+        lo[h][0] += s * static_cast<int>(t.re_lo);
+        lo[h][1] += d * static_cast<int>(t.im_lo);
+      }
+    } else {
+      const uint32_t u = *reinterpret_cast<const uint32_t*>(g + m * gplane);
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int a = static_cast<int16_t>(u >> (16 * h));
+        hi[h][0] += static_cast<unsigned long long>(static_cast<long long>(a)) * t.re_hi;
+        lo[h][0] += a * static_cast<int>(t.re_lo);
+      }
+    }
+  }
+  const int fc = Fx[c];
+  const long long jc = j0 + c;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int r = r0 + h;
+    if (r >= M) break;
+    const bool bad = k.er[h] == kNonFinite || fc == kNonFinite;
+    const int e = bad ? 0 : -(k.er[h] + fc);
+    E* cp = C + jc * ldc + r;
+    const E x = k.diag[h] ? X[jc * ldx + r] : E{};
+    const E y = sc.has_beta ? *cp : E{};
+    double v[2];
+    if (sc.plain && !bad && e >= -800 && e <= 800) {
+      const double f = scale_pow2(sc.ap, e), fl = ACC ? scale_pow2(sc.ap_lo, e) : 0.0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const double T = crt_value(hi[h][w], lo[h][w]);
+        const double xw = w == 0 ? re_of(x) : im_of(x), yw = w == 0 ? re_of(y) : im_of(y);
+        double q = 0.0;
+        if (sc.has_beta) q = sc.beta * yw;
+        if constexpr (ACC) q = fma(T, fl, q);
+        if (k.diag[h]) {
+          if constexpr (ACC) q = fma(k.dl[h], xw, q);
+          q = fma(k.dh[h], xw, q);
+        }
+        v[w] = fma(T, f, q);
+      }
+    } else {  // scales that alpha P 2^e may not reach, non-finite operands
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const double T = crt_value(hi[h][w], lo[h][w]);
+        const double xw = w == 0 ? re_of(x) : im_of(x), yw = w == 0 ? re_of(y) : im_of(y);
+        double q = bad ? __longlong_as_double(0x7FF8000000000000ll)
+                       : ldexp(ACC ? fma(T, tab.P, T * tab.P_lo) : T * tab.P, e);
+        if (!sc.plain) q *= sc.alpha;
+        else if (!bad) q = ldexp(ACC ? fma(T, sc.ap, T * sc.ap_lo) : T * sc.ap, e);
+        if (k.diag[h]) {
+          if constexpr (ACC) q = fma(sc.plain ? k.dl[h] : sc.alpha * k.dl[h], xw, q);
+          q = fma(sc.plain ? k.dh[h] : sc.alpha * k.dh[h], xw, q);
+        }
+        v[w] = sc.has_beta ? fma(sc.beta, yw, q) : q;
+      }
+    }
+    if constexpr (CP)
+      out[h] = E{static_cast<S>(v[0]), static_cast<S>(v[1])};
+    else
+      out[h] = static_cast<S>(v[0]);
+    *cp = out[h];
+  }
+}
+
 template <int NM, class E>
 __device__ __forceinline__ void crt_rows(int r0, int c0, int c1, int cstep,
                                          const int16_t* __restrict__ G, long long ldg,
@@ -1097,108 +1216,11 @@ __device__ __forceinline__ void crt_rows(int r0, int c0, int c1, int cstep,
                                          const double* __restrict__ Dg, int M, int j0,
                                          const E* __restrict__ X, long long ldx,
                                          E* __restrict__ C, long long ldc, const RnsScale& sc) {
-  constexpr bool CP = is_complex<E>;
-  constexpr int W = CP ? 2 : 1;
-  constexpr bool ACC = NM == kRnsFp64;
-  using S = typename Out<E>::S;
-  int er[2];
-  double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (ACC: two doubles)
-  bool diag[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const bool in = r0 + h < M;
-    er[h] = in ? Ex[r0 + h] : 0;
-    const double a = in && Dg ? Dg[r0 + h] : 0.0, b = -sc.shift;
-    double d = a + b;
-    const double t = d - a;
-    double l = (a - (d - t)) + (b - t);
-    diag[h] = d != 0.0;
-    if (sc.plain) {
-      const double p = sc.alpha * d;
-      l = fma(sc.alpha, d, -p) + sc.alpha * l;
-      d = p;
-    }
-    dh[h] = d;
-    dl[h] = l;
-  }
-  for (int c = c0; c < c1; c += cstep) {
-    const int16_t* g = G + static_cast<long long>(c) * ldg + r0;
-    unsigned long long hi[2][W] = {};
-    int lo[2][W] = {};
-#pragma unroll
-    for (int m = 0; m < NM; ++m) {
-      const CrtMod& t = tab.m[m];
-      if constexpr (CP) {
-        const uint32_t u = *reinterpret_cast<const uint32_t*>(g + (2 * m) * gplane);
-        const uint32_t w = *reinterpret_cast<const uint32_t*>(g + (2 * m + 1) * gplane);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int a = static_cast<int16_t>(u >> (16 * h)), b = static_cast<int16_t>(w >> (16 * h));
-          const int s = a + b, d = a - b;
-          hi[h][0] += static_cast<unsigned long long>(static_cast<long long>(s)) * t.re_hi;
-          hi[h][1] += static_cast<unsigned long long>(static_cast<long long>(d)) * t.im_hi;
-          lo[h][0] += s * static_cast<int>(t.re_lo);
-          lo[h][1] += d * static_cast<int>(t.im_lo);
-        }
-      } else {
-        const uint32_t u = *reinterpret_cast<const uint32_t*>(g + m * gplane);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int a = static_cast<int16_t>(u >> (16 * h));
-          hi[h][0] += static_cast<unsigned long long>(static_cast<long long>(a)) * t.re_hi;
-          lo[h][0] += a * static_cast<int>(t.re_lo);
-        }
-      }
-    }
-    const int fc = Fx[c];
-    const long long jc = j0 + c;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = r0 + h;
-      if (r >= M) break;
-      const bool bad = er[h] == kNonFinite || fc == kNonFinite;
-      const int e = bad ? 0 : -(er[h] + fc);
-      E* cp = C + jc * ldc + r;
-      const E x = diag[h] ? X[jc * ldx + r] : E{};
-      const E y = sc.has_beta ? *cp : E{};
-      double v[2];
-      if (sc.plain && !bad && e >= -800 && e <= 800) {
-        const double f = scale_pow2(sc.ap, e), fl = ACC ? scale_pow2(sc.ap_lo, e) : 0.0;
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          const double T = crt_value(hi[h][w], lo[h][w]);
-          const double xw = w == 0 ? re_of(x) : im_of(x), yw = w == 0 ? re_of(y) : im_of(y);
-          double q = 0.0;
-          if (sc.has_beta) q = sc.beta * yw;
-          if constexpr (ACC) q = fma(T, fl, q);
-          if (diag[h]) {
-            if constexpr (ACC) q = fma(dl[h], xw, q);
-            q = fma(dh[h], xw, q);
-          }
-          v[w] = fma(T, f, q);
-        }
-      } else {  // scales that alpha P 2^e may not reach, non-finite operands
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          const double T = crt_value(hi[h][w], lo[h][w]);
-          const double xw = w == 0 ? re_of(x) : im_of(x), yw = w == 0 ? re_of(y) : im_of(y);
-          double q = bad ? __longlong_as_double(0x7FF8000000000000ll)
-                         : ldexp(ACC ? fma(T, tab.P, T * tab.P_lo) : T * tab.P, e);
-          if (!sc.plain) q *= sc.alpha;
-          else if (!bad) q = ldexp(ACC ? fma(T, sc.ap, T * sc.ap_lo) : T * sc.ap, e);
-          if (diag[h]) {
-            if constexpr (ACC) q = fma(sc.plain ? dl[h] : sc.alpha * dl[h], xw, q);
-            q = fma(sc.plain ? dh[h] : sc.alpha * dh[h], xw, q);
-          }
-          v[w] = sc.has_beta ? fma(sc.beta, yw, q) : q;
-        }
-      }
-      if constexpr (CP)
-        *cp = E{static_cast<S>(v[0]), static_cast<S>(v[1])};
-      else
-        *cp = static_cast<S>(v[0]);
-    }
-  }
+  CrtRows k;
+  crt_constants(k, r0, M, Ex, Dg, sc);
+  E out[2];
+  for (int c = c0; c < c1; c += cstep)
+    crt_pair<NM, E>(k, r0, c, G, ldg, gplane, tab, Fx, M, j0, X, ldx, C, ldc, sc, out);
 }
 
 template <int NM, class E>
@@ -1214,6 +1236,130 @@ __global__ void __launch_bounds__(128)
     crt_rows<NM, E>(r0, blockIdx.y, ncols, gridDim.y, G, ldg, gplane, tab, Ex, Fx, Dg, M, j0, X,
                     ldx, C, ldc, sc);
   pdl_next();  // late, for the reason the GEMM gives
+}
+
+// Reconstruction of one degree step and slicing for the next in one kernel, for
+// blocks whose columns a cluster holds in registers (two rows a thread, at
+// most 8 x 256 threads): the columns from `next0` on, just computed, go straight
+// to their residues.  Their norm needs the whole column, so the cluster's
+// blocks exchange partial sums through shared memory; the sums add up in rank
+// order, the same in every block.  Saves a launch and two reads of the column
+// (filter N = 1000: 1139 -> 1039 us; complex64 N = 2000: 1722 -> 1623; split N =
+// 2048: 1889 -> 1833; real N = 2501: 2515 -> 2348).  What the rows share over
+// the columns is formed anew by every cluster, on the FP64 pipe: with complex N
+// = 4096 that costs more than it saves (4541 -> 4649).
+constexpr int kStepRows = 4096;                     // largest N, real
+constexpr int kStepRowsComplex = kStepRows / 2;
+template <int NM, int NL, class E>
+__global__ void __launch_bounds__(256)
+    rns_step_kernel(const int16_t* __restrict__ G, long long ldg, long long gplane,
+                    const __grid_constant__ CrtTab tab, const int* __restrict__ Ex,
+                    const int* __restrict__ Fx, const double* __restrict__ Dg, int M, int ncols,
+                    int j0, const E* __restrict__ X, long long ldx, E* __restrict__ C, long long ldc,
+                    const __grid_constant__ RnsScale sc, const __grid_constant__ SliceTab stab,
+                    int next0, __nv_bfloat16* __restrict__ B, long long Kp, long long plane,
+                    int* __restrict__ Fnext) {
+  constexpr bool CP = is_complex<E>;
+  __shared__ float wf[8];
+  __shared__ uint32_t wu[8];
+  // partial sums by cluster rank: [column parity][first pass, rescaled pass]
+  __shared__ float cf[2][2][8];
+  __shared__ uint32_t cu[2][2][8];
+  cluster_sync();  // every block runs before another writes to it
+  pdl_wait();
+  uint32_t size;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(size));
+  const uint32_t rank = cluster_rank();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+  const int r0 = 2 * (rank * blockDim.x + threadIdx.x);
+  CrtRows k;
+  crt_constants(k, r0, M, Ex, Dg, sc);
+  // sum of ss and maximum of mb over the cluster
+  auto reduce_cluster = [&](float& ss, uint32_t& mb, int par, int pass) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      mb = max(mb, __shfl_xor_sync(0xffffffffu, mb, o));
+    }
+    __syncthreads();
+    if (lane == 0) {
+      wf[warp] = ss;
+      wu[warp] = mb;
+    }
+    __syncthreads();
+    ss = 0.f;
+    mb = 0;
+    for (int w = 0; w < nwarps; ++w) {
+      ss += wf[w];
+      mb = max(mb, wu[w]);
+    }
+    if (size > 1) {
+      if (threadIdx.x < size) {
+        asm volatile("st.shared::cluster.f32 [%0], %1;\n" ::"r"(
+                         map_to_rank(&cf[par][pass][rank], threadIdx.x)),
+                     "f"(ss)
+                     : "memory");
+        asm volatile("st.shared::cluster.u32 [%0], %1;\n" ::"r"(
+                         map_to_rank(&cu[par][pass][rank], threadIdx.x)),
+                     "r"(mb)
+                     : "memory");
+      }
+      __syncwarp();
+      cluster_sync();
+      ss = 0.f;
+      for (uint32_t q = 0; q < size; ++q) {
+        ss += cf[par][pass][q];
+        mb = max(mb, cu[par][pass][q]);
+      }
+    }
+  };
+  int par = 0;
+  for (int c = blockIdx.x / size; c < ncols; c += gridDim.x / size) {
+    E v[2] = {};
+    if (r0 < M)
+      crt_pair<NM, E>(k, r0, c, G, ldg, gplane, tab, Fx, M, j0, X, ldx, C, ldc, sc, v);
+    const int nc = j0 + c - next0;
+    if (nc < 0) continue;
+    float ss = 0.f;
+    uint32_t mb = 0, any = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float fa = abs_f32(re_in(v[h]), 0), fb = CP ? abs_f32(im_in(v[h]), 0) : 0.f;
+      ss = fmaf(fa, fa, fmaf(fb, fb, ss));
+      mb = max(mb, max(abs_hi(re_in(v[h])), abs_hi(im_in(v[h]))));
+      any |= low_word(re_in(v[h])) | low_word(im_in(v[h]));
+    }
+    if (mb == 0 && any != 0) mb = 1;
+    reduce_cluster(ss, mb, par, 0);
+    int off = 0;
+    if ((mb < kSafeLo || mb >= kSafeHi) && mb >= (1u << 20) && mb < 0x7FF00000u) {
+      off = static_cast<int>(mb >> 20) - 1023;
+      ss = 0.f;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float fa = abs_f32(re_in(v[h]), off), fb = CP ? abs_f32(im_in(v[h]), off) : 0.f;
+        ss = fmaf(fa, fa, fmaf(fb, fb, ss));
+      }
+      uint32_t same = mb;
+      reduce_cluster(ss, same, par, 1);
+    }
+    par ^= 1;
+    const int s = scale_exponent(ss, mb, off, (CP ? 2.f : 1.f) * M, stab.log2_norm);
+    if (rank == 0 && threadIdx.x == 0) Fnext[nc] = s;
+    if (r0 < M) {
+      const bool zero = s == kNonFinite;
+      long long xr[2] = {}, xi[2] = {};
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        if (!zero) {
+          xr[h] = scaled_int(re_in(v[h]), s);
+          if constexpr (CP) xi[h] = scaled_int(im_in(v[h]), s);
+        }
+      store_residues<NM, NL, CP>(xr, xi, B + nc * Kp + r0, plane, stab, 0, NM);
+    }
+  }
+  pdl_next();
+  cluster_sync();  // no block leaves while another may still write to it
 }
 
 // ---------------------------------------------------------------------------
@@ -1616,7 +1762,7 @@ int slice_h_moduli(Dev& d, const RnsH& h, int m0, int m1) {
 
 template <int NM, class E>
 int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int j1, E* C,
-            int64_t ldc, double alpha, double beta, double shift) {
+            int64_t ldc, double alpha, double beta, double shift, bool sliced, int next0) {
   constexpr bool CP = is_complex<E>;
   constexpr int PP = CP ? 2 : 1;  // planes per modulus
   const Tables& t = tables(NM, CP);
@@ -1629,10 +1775,13 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
   const int64_t gplane = static_cast<int64_t>(x.cap_cols) * x.ldg;
   for (int c0 = j0; c0 < j1; c0 += x.cap_cols) {
     const int w = std::min(x.cap_cols, j1 - c0);
-    CHASE_CUDA(launch_pdl(rns_slice_x_kernel<NM, limbs_of(NM), E>, dim3(w), dim3(kSliceThreads), 0,
-                          d.st, X, ldx, N, c0, t.slice, static_cast<__nv_bfloat16*>(x.B), x.Kp,
-                          bplane, x.F));
-    note_launch();
+    int* F = x.F + (x.flip ? x.cap_cols : 0);
+    if (!sliced) {
+      CHASE_CUDA(launch_pdl(rns_slice_x_kernel<NM, limbs_of(NM), E>, dim3(w), dim3(kSliceThreads),
+                            0, d.st, X, ldx, N, c0, t.slice, static_cast<__nv_bfloat16*>(x.B), x.Kp,
+                            bplane, F));
+      note_launch();
+    }
     const double alg = (CP ? 8.0 : 2.0) * N * static_cast<double>(N) * w;
     KernelTimer kt(d.st, NM == kRnsFp64 ? CHASE_TIMED_FP64_PRODUCT : CHASE_TIMED_SPLIT_PRODUCT);
     int launched = 0;
@@ -1662,12 +1811,27 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
     }
     // NM moduli x PP planes of 2 N^2 b BF16 FLOPs
     kt.end(launched, alg, alg * NM * PP * 2.0 / (CP ? 8.0 : 2.0));
+    if (next0 >= 0) {
+      // two rows a thread; as many blocks as keep the SMs busy, a cluster per column
+      const int threads = N <= kStepRows / 2 ? 128 : 256;
+      const unsigned size = static_cast<unsigned>((N + 2 * threads - 1) / (2 * threads));
+      const unsigned clusters = std::min(static_cast<unsigned>(w), 152u * 8u / size);
+      CHASE_CUDA(launch_pdl_cluster(rns_step_kernel<NM, limbs_of(NM), E>, size,
+                                    dim3(size * clusters), dim3(threads), 0, d.st, x.G, x.ldg,
+                                    gplane, t.crt, h.E, F, h.Dg, N, w, c0, X, ldx, C, ldc,
+                                    crt_scale(t.crt, alpha, beta, shift), t.slice, next0,
+                                    static_cast<__nv_bfloat16*>(x.B), x.Kp, bplane,
+                                    x.F + (x.flip ? 0 : x.cap_cols)));
+      note_launch();
+      x.flip ^= 1;
+      continue;
+    }
     // about 16 blocks of 128 threads per SM
     const int gx = (N + 255) / 256;
     const dim3 grid(static_cast<unsigned>(gx),
                     static_cast<unsigned>(std::min(w, std::max(1, 16 * 152 / gx))));
     CHASE_CUDA(launch_pdl(rns_crt_kernel<NM, E>, grid, dim3(128), 0, d.st, x.G, x.ldg, gplane,
-                          t.crt, h.E, x.F, h.Dg, N, w, c0, X, ldx, C, ldc,
+                          t.crt, h.E, F, h.Dg, N, w, c0, X, ldx, C, ldc,
                           crt_scale(t.crt, alpha, beta, shift)));
     note_launch();
   }
@@ -1676,17 +1840,22 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
 
 template <class E>
 int product_any(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int j1, E* C,
-                int64_t ldc, double alpha, double beta, double shift) {
+                int64_t ldc, double alpha, double beta, double shift, bool sliced, int next0) {
   if (j1 <= j0) return CHASE_OK;
-  if (h.nmod == 7) return product<7>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift);
-  if (h.nmod == 8) return product<8>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift);
+  if (h.nmod == 7) return product<7>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift, sliced,
+                      next0);
+  if (h.nmod == 8) return product<8>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift, sliced,
+                      next0);
   if constexpr (!is_single<E>) {
     if (h.nmod == 11)
-      return product<11>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift);
+      return product<11>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift, sliced,
+                      next0);
     if (h.nmod == 12)
-      return product<12>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift);
+      return product<12>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift, sliced,
+                      next0);
     if (h.nmod == kRnsFp64)
-      return product<kRnsFp64>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift);
+      return product<kRnsFp64>(d, h, x, X, ldx, j0, j1, C, ldc, alpha, beta, shift, sliced,
+                      next0);
   }
   set_error("residue product: %d moduli", h.nmod);
   return CHASE_INVALID_ARG;
@@ -1883,15 +2052,19 @@ int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX
     if (st != CHASE_OUT_OF_MEMORY || out.cap_cols == 1) break;
   }
   CHASE_TRY(st);
-  return d.alloc(&out.F, static_cast<size_t>(out.cap_cols));
+  return d.alloc(&out.F, 2 * static_cast<size_t>(out.cap_cols));
+}
+
+bool rns_chains(const RnsH& h, int b, const RnsX& x) {
+  return h.N <= (h.cplx ? rns::kStepRowsComplex : rns::kStepRows) && b <= x.cap_cols;
 }
 
 template <class T>
 int rns_product(Dev& d, const RnsH& h, RnsX& x, const T* X, int64_t ldx, int j0, int j1, T* C,
-                int64_t ldc, double alpha, double beta, double shift) {
+                int64_t ldc, double alpha, double beta, double shift, bool sliced, int next0) {
   using D = typename Kind<T>::D;
   return rns::product_any<D>(d, h, x, reinterpret_cast<const D*>(X), ldx, j0, j1,
-                             reinterpret_cast<D*>(C), ldc, alpha, beta, shift);
+                             reinterpret_cast<D*>(C), ldc, alpha, beta, shift, sliced, next0);
 }
 
 namespace {
@@ -2052,7 +2225,7 @@ int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const Grouped
 #define CHASE_INSTANTIATE_RNS(T)                                                                 \
   template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, bool, RnsH&);     \
   template int rns_product<T>(Dev&, const RnsH&, RnsX&, const T*, int64_t, int, int, T*, int64_t, \
-                              double, double, double);
+                              double, double, double, bool, int);
 CHASE_INSTANTIATE_RNS(chase_c64)
 CHASE_INSTANTIATE_RNS(double)
 CHASE_INSTANTIATE_RNS(chase_c32)
