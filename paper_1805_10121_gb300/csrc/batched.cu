@@ -243,7 +243,7 @@ int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::
                                cudaMemcpyHostToDevice, d.st));
     return CHASE_OK;
   };
-  if (rns_sym_pays(nmod, entries)) {
+  if (rns_sym_pays(2 * nmod, entries)) {
     CHASE_TRY(upload(dl, all));
     CHASE_CUDA(cudaMemcpyAsync(mm, hmm.data(), sizeof(int) * hmm.size(), cudaMemcpyHostToDevice,
                                d.st));

@@ -172,8 +172,9 @@ int rns_split_moduli(int64_t N);
 int rns_low_moduli(int64_t N);
 // Residue planes of H (per modulus two planes of N x Kp bf16 for complex H,
 // one for real), row exponents and the real diagonal, which the epilogue
-// applies in FP64.  sym: all rows share one scale, 2^exponent, and complex H
-// has one plane per modulus too, the other being its transpose.  resident < nmod: memory holds only that many moduli at a
+// applies in FP64.  sym: all rows share one scale, 2^exponent; complex H has one
+// plane per modulus too, the other being its transpose, and real H's planes
+// hold the lower triangle and the 256 x 256 blocks on the diagonal.  resident < nmod: memory holds only that many moduli at a
 // time, and every product slices H anew (src, lds) for each group of them.
 struct RnsH {
   void* A = nullptr;
@@ -199,7 +200,7 @@ struct RnsX {
 // reserve: bytes to leave free when the planes are large.  many: the planes
 // serve many products, which pays for looking whether one scale fits all rows
 // (a pass over H and a synchronisation).
-bool rns_sym_pays(int nmod, double entries);  // of H's, or of a whole batch's
+bool rns_sym_pays(int planes, double entries);  // of H's, or of a whole batch's
 template <class T>
 int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
                   RnsH& out);

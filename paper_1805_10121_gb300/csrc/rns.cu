@@ -239,6 +239,11 @@ struct Tile {
   int row0, col0;      // first row, first column of the tile
   int planeA, planeB;  // plane of A and of B
   bool trans;          // the tile of A is a transposed one of its plane
+  bool tri;            // ... is that right of the diagonal's 256 x 256 block only
+  // whether the stage at k does load a transposed tile
+  __device__ __forceinline__ bool transposed(int k) const {
+    return trans || (tri && k >= row0 + 2 * BM);
+  }
   int modulus;         // index of the plane's modulus
   int nst;             // stages (K / 64, rounded up)
   int M, ncols;        // rows, columns of the product
@@ -336,10 +341,11 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
             if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * C::STAGE);
             // two boxes of 64 x 64: 64 rows each, or 64 of M each when transposed
             const uint32_t a = smem_u32(sA + st * C::A_BYTES);
-            const int x = T.trans ? ra : ks * BK, y = T.trans ? ks * BK : ra;
+            const bool tr = T.transposed(ks * BK);
+            const int x = tr ? ra : ks * BK, y = tr ? ks * BK : ra;
             tma_load_pair(a, T.mapA, x, y, T.planeA, bar);
-            tma_load_pair(a + C::A_BYTES / 2, T.mapA, T.trans ? x + 64 : x, T.trans ? y : y + 64,
-                          T.planeA, bar);
+            tma_load_pair(a + C::A_BYTES / 2, T.mapA, tr ? x + 64 : x, tr ? y : y + 64, T.planeA,
+                          bar);
             tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
           }
           __syncwarp();
@@ -365,7 +371,6 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
         Tile T;
         tile(t, T);
         const int cs = tab.m[T.modulus].chunk;
-        const uint32_t idesc = T.trans ? idesc0 | (1u << 15) : idesc0;
         int in = 0;  // stage within the chunk
         for (int ks = 0; ks < T.nst; ++ks, ++g) {
           if (in == 0) {
@@ -386,8 +391,10 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           const uint32_t a0 = smem_u32(sA + st * C::A_BYTES), b0 = smem_u32(sB + st * C::B_BYTES);
           const uint32_t d = tmem + static_cast<uint32_t>(c & 1) * C::BUF;
-          const uint64_t da = T.trans ? desc_sw128_mn(a0) : desc_sw128(a0);
-          const uint64_t step = (T.trans ? 16 * 128 : 32) >> 4;  // 16 of K
+          const bool tr = T.transposed(ks * BK);
+          const uint32_t idesc = tr ? idesc0 | (1u << 15) : idesc0;
+          const uint64_t da = tr ? desc_sw128_mn(a0) : desc_sw128(a0);
+          const uint64_t step = (tr ? 16 * 128 : 32) >> 4;  // 16 of K
           const bool last = in + 1 == cs || ks == T.nst - 1;
           if (leader) {
 #pragma unroll
@@ -501,8 +508,9 @@ struct OneProduct {
     T.mapB = mapB;
     T.row0 = rt * 2 * BM;
     T.col0 = ct * bn;
-    T.planeA = sym ? pl >> 1 : pl ^ swap_a;
-    T.trans = sym && (pl & 1);
+    T.planeA = sym == 1 ? pl >> 1 : pl ^ swap_a;
+    T.trans = sym == 1 && (pl & 1);
+    T.tri = sym == 2;
     T.planeB = plane0 + pl;
     T.modulus = T.planeB / per_modulus;
     T.nst = nst;
@@ -855,11 +863,13 @@ __global__ void __launch_bounds__(kSliceThreads)
   row_exponent(H, ldh, N, blockIdx.x, L, Ex, minmax);
 }
 
-// One 64 x 64 tile of the lower triangle of a complex Hermitian H, scaled by
-// 2^s, to one residue plane per modulus: re + j im at (r, k) and, its
-// conjugate's, re - j im at (k, r).  The second plane of the modulus is the
-// transpose of the first.  Only the lower triangle is read, so the plane is
-// exactly that of a Hermitian matrix whatever rounding left in H.
+// One 64 x 64 tile of the lower triangle of a Hermitian H, scaled by 2^s, to
+// one residue plane per modulus.  Complex: re + j im at (r, k) and, its
+// conjugate's, re - j im at (k, r); the second plane of the modulus is the
+// transpose of the first.  Real: the lower triangle, with the 256 x 256 blocks
+// on the diagonal whole; products load the rest transposed.  Only the lower
+// triangle is read, so the plane is exactly that of a Hermitian matrix
+// whatever rounding left in H.
 constexpr int kSymTile = 64;
 constexpr int kSymSmem = 2 * kSymTile * (kSymTile + 1) * 8;
 template <int NM, int NL, class E>
@@ -867,6 +877,7 @@ __device__ __forceinline__ void slice_sym_tile(const E* __restrict__ H, long lon
                                                int s, const SliceTab& tab, int m0, int m1,
                                                __nv_bfloat16* __restrict__ A, long long Kp,
                                                int* __restrict__ Ex, double* __restrict__ Dg) {
+  constexpr bool CP = is_complex<E>;
   extern __shared__ long long sym_smem[];
   auto re_t = reinterpret_cast<long long (*)[kSymTile + 1]>(sym_smem);
   auto im_t = re_t + kSymTile;
@@ -886,14 +897,14 @@ __device__ __forceinline__ void slice_sym_tile(const E* __restrict__ H, long lon
         Ex[r0 + r] = s;
       } else {
         xr = scaled_int(re_in(v), s);
-        xi = scaled_int(im_in(v), s);
+        if constexpr (CP) xi = scaled_int(im_in(v), s);
       }
     }
     re_t[r][k] = xr;
-    im_t[r][k] = xi;
+    if constexpr (CP) im_t[r][k] = xi;
     if (diag && r > k) {
       re_t[k][r] = xr;
-      im_t[k][r] = -xi;
+      if constexpr (CP) im_t[k][r] = -xi;
     }
   }
   __syncthreads();
@@ -902,15 +913,24 @@ __device__ __forceinline__ void slice_sym_tile(const E* __restrict__ H, long lon
   for (int q = warp; q < kSymTile; q += kSliceThreads / 32) {
     if (r0 + q < N) {
       const long long xr[2] = {re_t[q][2 * lane], re_t[q][2 * lane + 1]};
-      const long long xi[2] = {im_t[q][2 * lane], im_t[q][2 * lane + 1]};
-      store_residues<NM, NL, true, false>(xr, xi, A + (r0 + q) * Kp + k0 + 2 * lane, plane, tab, m0,
-                                          m1);
+      long long xi[2] = {};
+      if constexpr (CP) {
+        xi[0] = im_t[q][2 * lane];
+        xi[1] = im_t[q][2 * lane + 1];
+      }
+      store_residues<NM, NL, CP, false>(xr, xi, A + (r0 + q) * Kp + k0 + 2 * lane, plane, tab, m0,
+                                        m1);
     }
-    if (!diag && k0 + q < N) {
+    constexpr int kBlock = 2 * BM / kSymTile;
+    if ((CP ? !diag : !diag && R / kBlock == K / kBlock) && k0 + q < N) {
       const long long xr[2] = {re_t[2 * lane][q], re_t[2 * lane + 1][q]};
-      const long long xi[2] = {-im_t[2 * lane][q], -im_t[2 * lane + 1][q]};
-      store_residues<NM, NL, true, false>(xr, xi, A + (k0 + q) * Kp + r0 + 2 * lane, plane, tab, m0,
-                                          m1);
+      long long xi[2] = {};
+      if constexpr (CP) {
+        xi[0] = -im_t[2 * lane][q];
+        xi[1] = -im_t[2 * lane + 1][q];
+      }
+      store_residues<NM, NL, CP, false>(xr, xi, A + (k0 + q) * Kp + r0 + 2 * lane, plane, tab, m0,
+                                        m1);
     }
   }
 }
@@ -1441,6 +1461,7 @@ struct GroupedTiles {
     T.planeA = q.sym ? pl >> 1 : pl;
     T.planeB = pl;
     T.trans = q.sym && (pl & 1);
+    T.tri = false;
     T.modulus = pl / 2;
     T.nst = (q.n + BK - 1) / BK;
     T.M = q.n;
@@ -1621,7 +1642,8 @@ struct GemmArgs {
   int64_t b_rows, b_planes;  // B: b_planes of b_rows x Kp (plane stride), ncols rows used
   int ncols, nplanes, plane0, per_modulus;
   int swap_a = 0;  // 1: A conjugated (the two planes of a modulus change places)
-  int sym = 0;     // 1: A has one plane per modulus, the other is its transpose
+  int sym = 0;     // 1: A has one plane per modulus, the other is its transpose; 2: A's
+                   // planes are symmetric and hold the lower triangle
   int16_t* G;
   int64_t ldg, gplane;
   const GemmTab* tab;
@@ -1700,19 +1722,17 @@ int sym_tiles(int64_t n) {
 template <int NM, class E>
 int slice_h(Dev& d, const RnsH& h, int m0, int m1) {
   const SliceTab& tab = tables(NM, is_complex<E>).slice;
-  if constexpr (is_complex<E>) {
-    if (h.sym) {
-      auto kernel = rns_slice_sym_kernel<NM, limbs_of(NM), E>;
-      static const cudaError_t ready = cudaFuncSetAttribute(
-          kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSymSmem);
-      CHASE_CUDA(ready);
-      kernel<<<sym_tiles(h.N), kSliceThreads, kSymSmem, d.st>>>(
-          static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N), h.exponent, tab, m0, m1,
-          static_cast<__nv_bfloat16*>(h.A), h.Kp, h.E, h.Dg);
-      note_launch();
-      CHASE_CUDA(cudaGetLastError());
-      return CHASE_OK;
-    }
+  if (h.sym) {
+    auto kernel = rns_slice_sym_kernel<NM, limbs_of(NM), E>;
+    static const cudaError_t ready = cudaFuncSetAttribute(
+        kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSymSmem);
+    CHASE_CUDA(ready);
+    kernel<<<sym_tiles(h.N), kSliceThreads, kSymSmem, d.st>>>(
+        static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N), h.exponent, tab, m0, m1,
+        static_cast<__nv_bfloat16*>(h.A), h.Kp, h.E, h.Dg);
+    note_launch();
+    CHASE_CUDA(cudaGetLastError());
+    return CHASE_OK;
   }
   rns_slice_h_kernel<NM, limbs_of(NM), E><<<static_cast<unsigned>(h.N), kSliceThreads, 0, d.st>>>(
       static_cast<const E*>(h.src), h.lds, static_cast<int>(h.N), tab, m0, m1,
@@ -1794,7 +1814,7 @@ int product(Dev& d, const RnsH& h, RnsX& x, const E* X, int64_t ldx, int j0, int
       a.M = N;
       a.Kp = h.Kp;
       a.a_planes = static_cast<int64_t>(h.resident) * (h.sym ? 1 : PP);
-      a.sym = h.sym;
+      a.sym = h.sym ? (CP ? 1 : 2) : 0;
       a.B = x.B;
       a.b_rows = x.cap_cols;
       a.b_planes = NM * PP;
@@ -1993,12 +2013,13 @@ struct Kind<float> {
 int rns_split_moduli(int64_t N) { return N <= 32768 ? 11 : 12; }
 int rns_low_moduli(int64_t N) { return N <= 8192 ? 7 : 8; }
 
-// One plane per modulus instead of two halves what a product streams, once the
-// planes outgrow about half of the L2; below, the pass over H that looks for a
+// One plane per modulus instead of two (real: one triangle of it) halves what a
+// product streams, once the planes outgrow about half of the L2; below, the pass over H that looks for a
 // common scale costs more (filter N = 1000, 57 MB: 1150 us with two planes,
 // 1170 with one; complex64 N = 2000, 115 MB: 1876 and 1722; split N = 2048, 185
-// MB: 2167 and 1889; N = 4096, 940 MB: 5210 and 4541).
-bool rns_sym_pays(int nmod, double entries) { return 4.0 * nmod * entries > 64e6; }
+// MB: 2167 and 1889; N = 4096, 940 MB: 5210 and 4541; real N = 2501, 179 MB:
+// 2362 and 2232).
+bool rns_sym_pays(int planes, double entries) { return 2.0 * planes * entries > 64e6; }
 
 template <class T>
 int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
@@ -2012,8 +2033,8 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
   out.lds = ldh;
   CHASE_TRY(d.alloc(&out.E, static_cast<size_t>(N)));
   CHASE_TRY(d.alloc(&out.Dg, static_cast<size_t>(N)));
-  if constexpr (rns::is_complex<typename Kind<T>::D>)
-    if (many && rns_sym_pays(nmod, static_cast<double>(N) * out.Kp)) CHASE_TRY(rns::row_scales(d, reinterpret_cast<const typename Kind<T>::D*>(H), ldh, out));
+  if (many && rns_sym_pays(out.cplx ? 2 * nmod : nmod, static_cast<double>(N) * out.Kp))
+    CHASE_TRY(rns::row_scales(d, reinterpret_cast<const typename Kind<T>::D*>(H), ldh, out));
   const size_t per = static_cast<size_t>(out.cplx && !out.sym ? 2 : 1) * N * out.Kp * 2;  // bytes per modulus
   // all moduli resident where the memory allows it; else fewer, sliced anew
   // for every product

@@ -88,3 +88,26 @@ def test_batch_of_both_kinds(split):
                                precision=chase.CHASE_SPLIT_BF16 if split else chase.CHASE_FP64)
     for (n, b), v, ref, d in zip(shapes, vs, refs, degs):
         assert err(v, ref) <= bar(max(n, 64), int(d[0]), split)
+
+
+# real H holds one triangle from N = 1537 (FP64), 1728 (split) and 2150 (FP32) on
+@pytest.mark.parametrize("n,b", [(1100, 30), (1537, 33), (1791, 65), (1793, 9), (2047, 17), (2305, 130)])
+@pytest.mark.parametrize("kind", ["plain", "graded", "rounded"])
+@pytest.mark.parametrize("field,split", [("f64", False), ("f64", True), ("f32", False)])
+def test_real_filter(n, b, kind, field, split):
+    g = hermitian(n, n + b, True).clone()
+    if kind == "graded":
+        d = torch.logspace(0.0, -1.5, n, dtype=torch.float64, device=DEV)
+        g = d[:, None] * g * d[None, :]
+    elif kind == "rounded":
+        g = g * (1.0 + U * torch.randn(n, n, dtype=torch.float64, device=DEV))
+    dt = torch.float64 if field == "f64" else torch.float32
+    h, v = (x.to(dt).t().contiguous().t() for x in (g, gauss(n, b, n - b, True)))
+    ref = reference(h.double(), v.double(), 6, 1.6, -1.5, -0.9)
+    if field == "f64":
+        chase.chase_filter_real(h, v, [6] * b, 1.6, -1.5, -0.9,
+                                precision=chase.CHASE_SPLIT_BF16 if split else chase.CHASE_FP64)
+        assert err(v, ref) <= bar(n, 6, split)
+    else:
+        chase.chase_filter_f32(h, v, [6] * b, 1.6, -1.5, -0.9)
+        assert err(v.double(), ref) <= 16 * 6 * ((2 * n) ** 0.5 * 2.0 ** -30 + 8 * 2.0 ** -24)
