@@ -715,13 +715,20 @@ bool ld_ok(int64_t ld, int64_t n) { return ld >= std::max<int64_t>(1, n); }
 // finish (ascending output).
 // Inputs must be finite: a NaN or Inf in H or a block would otherwise run
 // through every step and surface, if at all, as a breakdown far from its
-// cause.  One pass of the column-norm kernel per array (a norm that
-// overflows, |entries| above about 1e154, is rejected too); `what` names
-// the array in the message.
+// cause.  A norm that overflows, |entries| above about 1e154, is rejected too:
+// one pass for the largest magnitude, and only where that is in doubt (2^480
+// and above; FP32: not finite) the column norms; `what` names the array in the
+// message.  (H with N = 4096: 60 us of norms, 45 of magnitudes.)
 template <class T>
 int check_finite(Dev& d, const T* X, int64_t ld, int64_t rows, int64_t cols, const char* where,
                  const char* what) {
   if (rows == 0 || cols == 0) return CHASE_OK;
+  unsigned *most = nullptr, top = 0;
+  CHASE_TRY(d.alloc(&most, 1));
+  CHASE_TRY(launch_max_magnitude(d, X, ld, rows, cols, most));
+  CHASE_CUDA(cudaMemcpyAsync(&top, most, sizeof(top), cudaMemcpyDeviceToHost, d.st));
+  CHASE_TRY(d.sync_check(where));
+  if (top < (is_single<T> ? 0x7F800000u : (1023u + 480u) << 20)) return CHASE_OK;
   double* nrm = nullptr;
   CHASE_TRY(d.alloc(&nrm, static_cast<size_t>(cols)));
   CHASE_TRY(launch_col_norms(d, X, ld, rows, static_cast<int>(cols), nrm));

@@ -88,6 +88,10 @@ int launch_permute_cols(Dev& d, const T* X, int64_t ldx, T* Y, int64_t ldy, int6
 // out[j] = ||X[:, j]||_2
 template <class T>
 int launch_col_norms(Dev& d, const T* X, int64_t ldx, int64_t N, int b, double* out);
+// out[0] = the largest magnitude of X as bits: the high word of a double's, an
+// FP32 value's own; infinities and NaN above every finite one.
+template <class T>
+int launch_max_magnitude(Dev& d, const T* X, int64_t ldx, int64_t rows, int64_t cols, unsigned* out);
 // X[:, j] *= 1 / s[j]   (s[j] == 0 leaves the column)
 template <class T>
 int launch_col_inv_scale(Dev& d, T* X, int64_t ldx, int64_t N, int b, const double* s);

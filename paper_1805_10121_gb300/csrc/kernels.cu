@@ -433,6 +433,39 @@ __global__ void __launch_bounds__(kRed) col_norms_kernel(const T* __restrict__ X
   if (threadIdx.x == 0) out[blockIdx.x] = sqrt(s);
 }
 
+// Largest magnitude of X as bits, the high word of a double or an FP32 value:
+// ordered like the magnitudes, infinities and NaN above all.  Integers only, so
+// it runs at the memory's rate where the norms are bound by the FP64 pipe.
+__device__ __forceinline__ uint32_t magnitude(double v) {
+  return static_cast<uint32_t>(__double2hiint(v)) & 0x7FFFFFFFu;
+}
+__device__ __forceinline__ uint32_t magnitude(float v) { return __float_as_uint(v) & 0x7FFFFFFFu; }
+__device__ __forceinline__ uint32_t magnitude(double2 v) {
+  return max(magnitude(v.x), magnitude(v.y));
+}
+__device__ __forceinline__ uint32_t magnitude(float2 v) {
+  return max(magnitude(v.x), magnitude(v.y));
+}
+template <class T>
+__global__ void __launch_bounds__(kRed)
+    max_magnitude_kernel(const T* __restrict__ X, long long ldx, long long rows, long long cols,
+                         unsigned* __restrict__ out) {
+  uint32_t m = 0;
+  for (long long j = blockIdx.y; j < cols; j += gridDim.y) {
+    const T* x = X + j * ldx;
+    const long long step = static_cast<long long>(gridDim.x) * kRed;
+    long long i = static_cast<long long>(blockIdx.x) * kRed + threadIdx.x;
+    for (; i + 3 * step < rows; i += 4 * step) {  // four loads in flight
+      const T a = x[i], b = x[i + step], c = x[i + 2 * step], e = x[i + 3 * step];
+      m = max(max(m, max(magnitude(a), magnitude(b))), max(magnitude(c), magnitude(e)));
+    }
+    for (; i < rows; i += step) m = max(m, magnitude(x[i]));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+}
+
 template <class T>
 __global__ void col_inv_scale_kernel(T* __restrict__ X, long long ldx, long long N,
                                      const double* __restrict__ s) {
@@ -830,6 +863,21 @@ int launch_col_norms(Dev& d, const T* X, int64_t ldx, int64_t N, int b, double* 
 }
 
 template <class T>
+int launch_max_magnitude(Dev& d, const T* X, int64_t ldx, int64_t rows, int64_t cols,
+                         unsigned* out) {
+  CHASE_CUDA(cudaMemsetAsync(out, 0, sizeof(unsigned), d.st));
+  if (rows == 0 || cols == 0) return CHASE_OK;
+  // a block takes about 1024 entries of a column at a time, eight blocks an SM
+  const unsigned gx = static_cast<unsigned>(std::min<int64_t>((rows + 4 * kRed - 1) / (4 * kRed), 64));
+  const unsigned gy = static_cast<unsigned>(
+      std::min<int64_t>(cols, std::max<int64_t>(1, 152 * 8 / gx)));
+  max_magnitude_kernel<<<dim3(gx, gy), kRed, 0, d.st>>>(dp(X), ldx, rows, cols, out);
+  note_launch();
+  CHASE_CUDA(cudaGetLastError());
+  return CHASE_OK;
+}
+
+template <class T>
 int launch_col_inv_scale(Dev& d, T* X, int64_t ldx, int64_t N, int b, const double* s) {
   if (b == 0 || N == 0) return CHASE_OK;
   if (b > 65535) {
@@ -1011,6 +1059,7 @@ int launch_normalize_cols(Dev& d, T* X, int64_t ldx, int64_t N, int r) {
   template int launch_permute_cols<T>(Dev&, const T*, int64_t, T*, int64_t, int64_t, int,         \
                                       const int*, bool);                                           \
   template int launch_col_norms<T>(Dev&, const T*, int64_t, int64_t, int, double*);                \
+  template int launch_max_magnitude<T>(Dev&, const T*, int64_t, int64_t, int64_t, unsigned*);      \
   template int launch_col_inv_scale<T>(Dev&, T*, int64_t, int64_t, int, const double*);            \
   template int launch_resid_norms<T>(Dev&, const T*, int64_t, const T*, int64_t, int64_t, int,     \
                                      const double*, double*);                                      \
