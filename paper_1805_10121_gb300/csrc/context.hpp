@@ -244,6 +244,8 @@ struct RnsScale {
   double ap, ap_lo;  // 2^-64 alpha P as the sum of two doubles
   int plain;         // |alpha| within [2^-100, 2^100]: alpha P 2^e may be formed first
   int has_beta;
+  float apf, apf_lo, bf, bf_lo;  // ap and beta as sums of two floats
+  int single;                    // those are in FP32's range
 };
 
 // ---- grouped filter: many independent problems per launch ----------------

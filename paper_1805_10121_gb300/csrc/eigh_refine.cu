@@ -162,10 +162,9 @@ __global__ void __launch_bounds__(kThreads)
 // columns of B = A' J orthogonal turn J into eigenvectors and each column of B
 // into a multiple of one, so J itself is not needed.  A warp holds a pair of
 // columns in registers; the p / 2 pairs of a round are disjoint, and p - 1
-// rounds meet every pair (round robin).  Issue slots bound it, 1.5 us a round
-// at p = 64.  The library's solver, hundreds of launches of a few microseconds,
-// takes 1.3 ms at p = 70 whatever G is; the rotations stop early when G is nearly
-// diagonal, as it is from the second iteration of a solve on.
+// rounds meet every pair (round robin).  Latency of dot product and rotation
+// bounds it, 0.4 us a round; the library's solver, launches of a few
+// microseconds each, takes 1.3 ms at p = 70 (JACFIG).
 // ---------------------------------------------------------------------------
 constexpr int kJacobiMax = 96, kJacobiRows = kJacobiMax / 32, kJacobiThreads = 1024;
 constexpr int kJacobiSweeps = 14;

@@ -1063,10 +1063,13 @@ struct CrtTab {
   double P, P_lo;  // 2^-64 times the product of the moduli, as the sum of two doubles
 };
 
-// X / P 2^64, rounded to a double.
+// X / P 2^64
+__device__ __forceinline__ long long crt_fraction(unsigned long long hi, int lo) {
+  return static_cast<long long>(hi +
+                                static_cast<unsigned long long>(static_cast<long long>(lo >> 16)));
+}
 __device__ __forceinline__ double crt_value(unsigned long long hi, int lo) {
-  return static_cast<double>(
-      static_cast<long long>(hi + static_cast<unsigned long long>(static_cast<long long>(lo >> 16))));
+  return static_cast<double>(crt_fraction(hi, lo));
 }
 // v 2^e for v 2^e below overflow; 0 for 0 and where it would be denormal
 __device__ __forceinline__ double scale_pow2(double v, int e) {
@@ -1111,6 +1114,7 @@ struct Out<float> {
 // recurrence, where the roundings of an FP64 GEMM average out.
 // What two rows of a product share over its columns.
 struct CrtRows {
+  float df[2], dfl[2];  // single precision: alpha (H_rr - shift) as two floats
   int er[2];
   double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (as two doubles)
   bool diag[2];
@@ -1133,7 +1137,15 @@ __device__ __forceinline__ void crt_constants(CrtRows& k, int r0, int M, const i
     }
     k.dh[h] = d;
     k.dl[h] = l;
+    k.df[h] = static_cast<float>(d);
+    k.dfl[h] = static_cast<float>(d - k.df[h]);
   }
+}
+
+// v 2^e for a normal float whose result is one too; 0 where it would not be
+__device__ __forceinline__ float scale_pow2f(float v, int e) {
+  const int u = __float_as_int(v), x = ((u >> 23) & 0xFF) + e;
+  return x > 0 && (u & 0x7F800000) != 0 ? __int_as_float(u + e * (1 << 23)) : 0.f;
 }
 
 // Rows r0, r0 + 1 of column j0 + c of the product: written to C and returned.
@@ -1189,6 +1201,32 @@ __device__ __forceinline__ void crt_pair(const CrtRows& k, int r0, int c,
     const E x = k.diag[h] ? X[jc * ldx + r] : E{};
     const E y = sc.has_beta ? *cp : E{};
     double v[2];
+    if constexpr (is_single<E>) {
+      // results are stored in FP32: each constant as two floats, so what the
+      // steps share is not rounded to one, and one FP32 FMA per term
+      const int x0 = ((__float_as_int(sc.apf) >> 23) & 0xFF) + e;
+      if (sc.single && !bad && x0 >= 27 && x0 <= 190) {
+        const float f = scale_pow2f(sc.apf, e), fl = scale_pow2f(sc.apf_lo, e);
+        float q[2] = {};
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          const float T = static_cast<float>(crt_fraction(hi[h][w], lo[h][w]));
+          const float xw = w == 0 ? re_in(x) : im_in(x), yw = w == 0 ? re_in(y) : im_in(y);
+          float a = T * fl;
+          if (sc.has_beta) a = fmaf(sc.bf_lo, yw, a);
+          if (k.diag[h]) a = fmaf(k.dfl[h], xw, a);
+          if (sc.has_beta) a = fmaf(sc.bf, yw, a);
+          if (k.diag[h]) a = fmaf(k.df[h], xw, a);
+          q[w] = fmaf(T, f, a);
+        }
+        if constexpr (CP)
+          out[h] = E{q[0], q[1]};
+        else
+          out[h] = q[0];
+        *cp = out[h];
+        continue;
+      }
+    }
     if (sc.plain && !bad && e >= -800 && e <= 800) {
       const double f = scale_pow2(sc.ap, e), fl = ACC ? scale_pow2(sc.ap_lo, e) : 0.0;
 #pragma unroll
@@ -1285,15 +1323,15 @@ __global__ void __launch_bounds__(256)
   // partial sums by cluster rank: [column parity][first pass, rescaled pass]
   __shared__ float cf[2][2][8];
   __shared__ uint32_t cu[2][2][8];
-  cluster_sync();  // every block runs before another writes to it
-  pdl_wait();
   uint32_t size;
   asm volatile("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(size));
   const uint32_t rank = cluster_rank();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
   const int r0 = 2 * (rank * blockDim.x + threadIdx.x);
   CrtRows k;
-  crt_constants(k, r0, M, Ex, Dg, sc);
+  crt_constants(k, r0, M, Ex, Dg, sc);  // H's own, not of the kernel before
+  cluster_sync();  // every block runs before another writes to it
+  pdl_wait();
   // sum of ss and maximum of mb over the cluster
   auto reduce_cluster = [&](float& ss, uint32_t& mb, int par, int pass) {
 #pragma unroll
@@ -1601,6 +1639,12 @@ RnsScale crt_scale(const CrtTab& t, double alpha, double beta, double shift) {
   s.ap_lo = std::fma(alpha, t.P, -s.ap) + alpha * t.P_lo;
   s.plain = std::fabs(alpha) >= std::ldexp(1.0, -100) && std::fabs(alpha) <= std::ldexp(1.0, 100);
   s.has_beta = beta != 0.0;
+  s.apf = static_cast<float>(s.ap);
+  s.apf_lo = static_cast<float>(s.ap - s.apf);
+  s.bf = static_cast<float>(beta);
+  s.bf_lo = static_cast<float>(beta - s.bf);
+  s.single = s.plain && std::fabs(s.ap) >= std::ldexp(1.0, -100) &&
+             std::fabs(s.ap) <= std::ldexp(1.0, 100) && std::fabs(beta) <= std::ldexp(1.0, 100);
   return s;
 }
 
