@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kThreads)
 // bounds it, 0.4 us a round; the library's solver, launches of a few
 // microseconds each, takes 1.3 ms at p = 70 (JACFIG).
 // ---------------------------------------------------------------------------
-constexpr int kJacobiMax = 96, kJacobiRows = kJacobiMax / 32, kJacobiThreads = 1024;
+constexpr int kJacobiMax = 96, kJacobiThreads = 1024;
 constexpr int kJacobiSweeps = 14;
 
 __device__ __forceinline__ void add_diag(float2& a, float v) { a.x += v; }
@@ -189,31 +189,36 @@ __device__ __forceinline__ float2 combine(float2 a, float c, float2 b, float s) 
 __device__ __forceinline__ float combine(float a, float c, float b, float s) {
   return fmaf(c, a, s * b);
 }
-__device__ __forceinline__ float2 warp_add(float2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
-    v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
-  }
-  return v;
-}
 __device__ __forceinline__ float warp_add(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+// The two parts in the two halves of the warp after the first exchange: seven
+// shuffles instead of ten.
+__device__ __forceinline__ float2 warp_add(float2 v) {
+  const bool upper = threadIdx.x & 16;
+  float a = upper ? v.y : v.x;
+  a += __shfl_xor_sync(0xffffffffu, upper ? v.x : v.y, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  const float b = __shfl_xor_sync(0xffffffffu, a, 16);
+  return upper ? make_float2(b, a) : make_float2(a, b);
 }
 __device__ __forceinline__ double2 widen(float2 a, float f) {
   return make_double2(static_cast<double>(a.x) * f, static_cast<double>(a.y) * f);
 }
 __device__ __forceinline__ double widen(float a, float f) { return static_cast<double>(a) * f; }
 
-template <class D, class F>
+// R: rows of a column per lane, p <= 32 R.
+template <int R, class D, class F>
 __global__ void __launch_bounds__(kJacobiThreads, 1)
     jacobi_kernel(const D* __restrict__ A, long long lda, int p, const double* __restrict__ norm,
                   D* __restrict__ X, long long ldx) {
   extern __shared__ double jacobi_smem[];
   F* B = reinterpret_cast<F*>(jacobi_smem);  // p x p, column-major
   __shared__ int s_rotated[2];
+  __shared__ float s_norm[kJacobiMax];  // squared column norms
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   constexpr int kWarps = kJacobiThreads / 32;
   __shared__ double s_f;
@@ -239,36 +244,47 @@ __global__ void __launch_bounds__(kJacobiThreads, 1)
   __syncthreads();
   const int n = (p + 1) & ~1;
   for (int sweep = 0; sweep < kJacobiSweeps; ++sweep) {
+    // afresh in each sweep; a rotation moves t |g| between the two
+    for (int j = warp; j < p; j += kWarps) {
+      float v = 0.f;
+      for (int i = lane; i < p; i += 32) v += norm2(B[j * p + i]);
+      v = warp_add(v);
+      if (lane == 0) s_norm[j] = v;
+    }
+    __syncthreads();
     for (int round = 0; round < n - 1; ++round) {
       for (int k = warp; k < n / 2; k += kWarps) {
         const int k2 = n - 1 - k;
         const int i = k == 0 ? 0 : 1 + (k - 1 + round) % (n - 1);
         const int j = 1 + (k2 - 1 + round) % (n - 1);
         if (i >= p || j >= p) continue;
-        F a[kJacobiRows], b[kJacobiRows], g = F{};
-        float na = 0.f, nb = 0.f;
+        F a[R], b[R], g = F{};
 #pragma unroll
-        for (int r = 0; r < kJacobiRows; ++r) {
+        for (int r = 0; r < R; ++r) {
           const int row = lane + 32 * r;
           a[r] = row < p ? B[i * p + row] : F{};
           b[r] = row < p ? B[j * p + row] : F{};
           g = conj_dot(g, a[r], b[r]);
-          na += norm2(a[r]);
-          nb += norm2(b[r]);
         }
+        const float na = s_norm[i], nb = s_norm[j];
         g = warp_add(g);
-        const float2 nn = warp_add(make_float2(na, nb));
         const float g2 = norm2(g);
         // cosine below FP32's resolution: orthogonal
-        if (!(g2 > 4e-14f * nn.x * nn.y)) continue;
-        if (lane == 0 && g2 > 1e-12f * nn.x * nn.y) s_rotated[sweep & 1] = 1;
+        if (!(g2 > 4e-14f * na * nb)) continue;
         const float ig = rsqrtf(g2);
         const F ph = scale_f(g, ig);
-        const float zeta = 0.5f * (nn.y - nn.x) * ig;
-        const float t = copysignf(1.f, zeta) / (fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f)));
+        const float zeta = 0.5f * (nb - na) * ig;
+        const float t =
+            copysignf(__fdividef(1.f, fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f))), zeta);
         const float c = rsqrtf(fmaf(t, t, 1.f)), s = t * c;
+        if (lane == 0) {
+          const float move = t * g2 * ig;
+          s_norm[i] = na - move;
+          s_norm[j] = nb + move;
+          if (g2 > 1e-12f * na * nb) s_rotated[sweep & 1] = 1;
+        }
 #pragma unroll
-        for (int r = 0; r < kJacobiRows; ++r) {
+        for (int r = 0; r < R; ++r) {
           const int row = lane + 32 * r;
           const F h = cmul_conj(b[r], ph);
           if (row < p) {
@@ -424,14 +440,21 @@ int refine(Dev& d, T* G, int64_t ldg, int p, double* w_dev, bool* done) {
   centre_kernel<D><<<p, kThreads, 0, d.st>>>(dp(G), ldg, p, dp(w.A), ld, w.norm, w.rep);
   note_launch();
   if (p <= kJacobiMax) {
-    static const cudaError_t ready =
-        cudaFuncSetAttribute(jacobi_kernel<D, F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             kJacobiMax * kJacobiMax * static_cast<int>(sizeof(F)));
-    CHASE_CUDA(ready);
-    jacobi_kernel<D, F><<<1, kJacobiThreads, sizeof(F) * n, d.st>>>(dp(w.A), ld, p, w.norm, dp(w.X),
-                                                                    ld);
-    note_launch();
-    CHASE_CUDA(cudaGetLastError());
+    auto launch = [&](auto rows) -> int {
+      constexpr int R = decltype(rows)::value;
+      auto kernel = jacobi_kernel<R, D, F>;
+      static const cudaError_t ready =
+          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               32 * R * 32 * R * static_cast<int>(sizeof(F)));
+      CHASE_CUDA(ready);
+      kernel<<<1, kJacobiThreads, sizeof(F) * n, d.st>>>(dp(w.A), ld, p, w.norm, dp(w.X), ld);
+      note_launch();
+      CHASE_CUDA(cudaGetLastError());
+      return CHASE_OK;
+    };
+    CHASE_TRY(p <= 32   ? launch(std::integral_constant<int, 1>())
+              : p <= 64 ? launch(std::integral_constant<int, 2>())
+                        : launch(std::integral_constant<int, 3>()));
   } else {
     CHASE_TRY(d.alloc(&w.F, n));
     narrow_kernel<D, F><<<p, kThreads, 0, d.st>>>(dp(w.A), ld, p, w.norm,
