@@ -957,25 +957,26 @@ __global__ void __launch_bounds__(kSliceThreads)
 }
 
 // Rows of a column-major X (M x K) as vectors: row r of plane q goes to
-// out[q * plane + r * Kp]. A block takes 32 rows; reads are coalesced along
-// the rows, and a 32 x 64 tile of scaled integers in shared memory turns them
-// into stores along K.  Bound by the 2 bytes per plane and entry it writes.
-constexpr int kRowBlock = 32;
-template <int NM, int NL, class E>
+// out[q * plane + r * Kp]. A block takes RB rows; reads are coalesced along
+// the rows, and an RB x 64 tile of scaled integers in shared memory turns them
+// into stores along K.  Bound by the 2 bytes per plane and entry it writes
+// when there are rows for all SMs; with fewer, blocks of 8 rows instead of 32
+// (M = K = 197: 33 -> 15 us; M = 1000, K = 70: 16 -> 7 us).
+template <int RB, int NM, int NL, class E>
 __global__ void __launch_bounds__(kSliceThreads)
     rns_slice_rows_kernel(const E* __restrict__ X, long long ldx, int M, int K,
                           const __grid_constant__ SliceTab tab, __nv_bfloat16* __restrict__ out,
                           long long Kp, long long plane, int* __restrict__ Ex) {
   constexpr bool CP = is_complex<E>;
   constexpr int W = CP ? 2 : 1;
-  constexpr int G = kSliceThreads / kRowBlock;  // threads per row
-  __shared__ float sf[G][kRowBlock];
-  __shared__ uint32_t su[G][kRowBlock];
-  __shared__ long long tile[W][kRowBlock][65];
+  constexpr int G = kSliceThreads / RB;  // threads per row
+  __shared__ float sf[G][RB];
+  __shared__ uint32_t su[G][RB];
+  __shared__ long long tile[W][RB][65];
   pdl_next();
   pdl_wait();
-  const int row = threadIdx.x % kRowBlock, grp = threadIdx.x / kRowBlock;
-  const int r0 = blockIdx.x * kRowBlock;
+  const int row = threadIdx.x % RB, grp = threadIdx.x / RB;
+  const int r0 = blockIdx.x * RB;
   const bool in = r0 + row < M;
   const E* x = X + r0 + row;
   float ss = 0.f;
@@ -1035,7 +1036,7 @@ __global__ void __launch_bounds__(kSliceThreads)
       if constexpr (CP) tile[W - 1][row][kk] = b;
     }
     __syncthreads();
-    for (int q = warp; q < kRowBlock && r0 + q < M; q += kSliceThreads / 32) {
+    for (int q = warp; q < RB && r0 + q < M; q += kSliceThreads / 32) {
       long long xr[2], xi[2] = {};
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -1934,15 +1935,19 @@ int slice_columns(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
   note_launch();
   return CHASE_OK;
 }
-template <class E>
-int slice_rows(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
-  CHASE_CUDA(launch_pdl(rns_slice_rows_kernel<kRnsFp64, limbs_of(kRnsFp64), E>,
-                        dim3(static_cast<unsigned>((b.n + kRowBlock - 1) / kRowBlock)),
-                        dim3(kSliceThreads), 0, d.st, X, ldx, static_cast<int>(b.n),
-                        static_cast<int>(b.K), tables(kRnsFp64, is_complex<E>).slice,
-                        static_cast<__nv_bfloat16*>(b.P), b.Kp, b.n * b.Kp, b.E));
+template <int RB, class E>
+int slice_rows_by(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
+  CHASE_CUDA(launch_pdl(rns_slice_rows_kernel<RB, kRnsFp64, limbs_of(kRnsFp64), E>,
+                        dim3(static_cast<unsigned>((b.n + RB - 1) / RB)), dim3(kSliceThreads), 0,
+                        d.st, X, ldx, static_cast<int>(b.n), static_cast<int>(b.K),
+                        tables(kRnsFp64, is_complex<E>).slice, static_cast<__nv_bfloat16*>(b.P),
+                        b.Kp, b.n * b.Kp, b.E));
   note_launch();
   return CHASE_OK;
+}
+template <class E>
+int slice_rows(Dev& d, const E* X, int64_t ldx, RnsBlock& b) {
+  return b.n < 32 * 152 ? slice_rows_by<8>(d, X, ldx, b) : slice_rows_by<32>(d, X, ldx, b);
 }
 template <class E>
 int dense(Dev& d, const RnsBlock& a, bool conj_a, const RnsBlock& b, E* C, int64_t ldc,
