@@ -239,10 +239,11 @@ struct Tile {
   int row0, col0;      // first row, first column of the tile
   int planeA, planeB;  // plane of A and of B
   bool trans;          // the tile of A is a transposed one of its plane
-  bool tri;            // ... is that right of the diagonal's 256 x 256 block only
-  // whether the stage at k does load a transposed tile
+  // whether the stage at k loads a transposed tile: with TRI, right of the
+  // diagonal's 256 x 256 block
+  template <bool TRI>
   __device__ __forceinline__ bool transposed(int k) const {
-    return trans || (tri && k >= row0 + 2 * BM);
+    return TRI ? k >= row0 + 2 * BM : trans;
   }
   int modulus;         // index of the plane's modulus
   int nst;             // stages (K / 64, rounded up)
@@ -341,7 +342,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
             if (rank == 0) mbar_arrive_expect_tx(&full[st], 2 * C::STAGE);
             // two boxes of 64 x 64: 64 rows each, or 64 of M each when transposed
             const uint32_t a = smem_u32(sA + st * C::A_BYTES);
-            const bool tr = T.transposed(ks * BK);
+            const bool tr = T.template transposed<TileFn::kTri>(ks * BK);
             const int x = tr ? ra : ks * BK, y = tr ? ks * BK : ra;
             tma_load_pair(a, T.mapA, x, y, T.planeA, bar);
             tma_load_pair(a + C::A_BYTES / 2, T.mapA, tr ? x + 64 : x, tr ? y : y + 64, T.planeA,
@@ -391,7 +392,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
           asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
           const uint32_t a0 = smem_u32(sA + st * C::A_BYTES), b0 = smem_u32(sB + st * C::B_BYTES);
           const uint32_t d = tmem + static_cast<uint32_t>(c & 1) * C::BUF;
-          const bool tr = T.transposed(ks * BK);
+          const bool tr = T.template transposed<TileFn::kTri>(ks * BK);
           const uint32_t idesc = tr ? idesc0 | (1u << 15) : idesc0;
           const uint64_t da = tr ? desc_sw128_mn(a0) : desc_sw128(a0);
           const uint64_t step = (tr ? 16 * 128 : 32) >> 4;  // 16 of K
@@ -495,7 +496,9 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
 // Tiles of one product: the column tile runs fastest, so the pairs working at
 // one time share rows of A and the B plane stays in L2; then row tiles, then
 // planes.
+template <bool TRI>
 struct OneProduct {
+  static constexpr bool kTri = TRI;
   const CUtensorMap* mapA;
   const CUtensorMap* mapB;
   int rtiles, ctiles, plane0, per_modulus, swap_a, sym, bn, nst, M, ncols;
@@ -508,9 +511,8 @@ struct OneProduct {
     T.mapB = mapB;
     T.row0 = rt * 2 * BM;
     T.col0 = ct * bn;
-    T.planeA = sym == 1 ? pl >> 1 : pl ^ swap_a;
-    T.trans = sym == 1 && (pl & 1);
-    T.tri = sym == 2;
+    T.planeA = sym ? pl >> 1 : pl ^ swap_a;
+    T.trans = sym && (pl & 1);
     T.planeB = plane0 + pl;
     T.modulus = T.planeB / per_modulus;
     T.nst = nst;
@@ -521,14 +523,16 @@ struct OneProduct {
   }
 };
 
-template <int BN>
+// TRI is a template parameter: its test in every stage, where no stage needs it,
+// made a warm split solve's filter at N = 4095 6 % slower.
+template <int BN, bool TRI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     rns_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                     const __grid_constant__ GemmTab tab, int rtiles, int ctiles, int nplanes,
                     int plane0, int per_modulus, int swap_a, int sym, int nst, int M, int ncols,
                     int16_t* __restrict__ G,
                     long long ldg, long long gplane, int* __restrict__ err) {
-  OneProduct p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, sym, BN, nst, M, ncols,
+  OneProduct<TRI> p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, sym, BN, nst, M, ncols,
                G, ldg, gplane};
   gemm_body<BN>(p, rtiles * ctiles * nplanes, tab, 0, err);
 }
@@ -1482,6 +1486,7 @@ __global__ void __launch_bounds__(kSliceThreads)
 // Tiles of a step: per problem the column tile runs fastest, then row tiles,
 // then planes.
 struct GroupedTiles {
+  static constexpr bool kTri = false;
   const GroupedProblem* probs;
   const GroupedStep* steps;
   int bn, at;  // at: entry of the last tile (each thread walks forward)
@@ -1500,7 +1505,6 @@ struct GroupedTiles {
     T.planeA = q.sym ? pl >> 1 : pl;
     T.planeB = pl;
     T.trans = q.sym && (pl & 1);
-    T.tri = false;
     T.modulus = pl / 2;
     T.nst = (q.n + BK - 1) / BK;
     T.M = q.n;
@@ -1654,8 +1658,10 @@ template <int BN>
 int pairs_on_device() {
   static const int v = [] {
     using C = Cfg<BN>;
-    if (cudaFuncSetAttribute(rns_gemm_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             C::SMEM) != cudaSuccess) {
+    if (cudaFuncSetAttribute(rns_gemm_kernel<BN, false>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess ||
+        cudaFuncSetAttribute(rns_gemm_kernel<BN, true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess) {
       cudaGetLastError();
       return 0;
     }
@@ -1671,7 +1677,7 @@ int pairs_on_device() {
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, rns_gemm_kernel<BN>, &cfg) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveClusters(&n, rns_gemm_kernel<BN, false>, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
       return 0;
     }
@@ -1710,8 +1716,9 @@ int launch_gemm(Dev& d, const GemmArgs& a) {
   const int ct = (a.ncols + BN - 1) / BN;
   const int64_t tiles = static_cast<int64_t>(rt) * ct * a.nplanes;
   const unsigned grid = 2 * static_cast<unsigned>(std::min<int64_t>(tiles, pairs));
-  CHASE_CUDA(launch_pdl(rns_gemm_kernel<BN>, dim3(grid), dim3(kThreads), C::SMEM, d.st, tmA, tmB,
-                        *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a, a.sym,
+  const auto kernel = a.sym == 2 ? rns_gemm_kernel<BN, true> : rns_gemm_kernel<BN, false>;
+  CHASE_CUDA(launch_pdl(kernel, dim3(grid), dim3(kThreads), C::SMEM, d.st, tmA, tmB,
+                        *a.tab, rt, ct, a.nplanes, a.plane0, a.per_modulus, a.swap_a, a.sym == 1 ? 1 : 0,
                         static_cast<int>((a.K + BK - 1) / BK), static_cast<int>(a.M), a.ncols, a.G,
                         a.ldg, a.gplane, d.err));
   note_launch();
