@@ -308,7 +308,13 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
   const bool leader = elect_one();
   if (warp == 0) {
     {  // ---------------- TMA producer (both CTAs)
+      // Stage and parity are counted along: these loops have a few hundred
+      // cycles per stage, and 64-bit divisions for them took 4 to 5 % of every
+      // product.  A wait for
+      // the phase before a barrier's first returns at once.
       long long g = 0;  // stages issued by this CTA
+      int st = 0;
+      uint32_t ph = 1;
       bool ok = true;
       const CUtensorMap* last = nullptr;
       for (int t = pair; t < ntiles && ok; t += npairs) {
@@ -330,9 +336,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
         const int ra = T.row0 + static_cast<int>(rank) * BM;
         const int cb = T.col0 + static_cast<int>(rank) * (BN / 2);
         for (int ks = 0; ks < T.nst; ++ks, ++g) {
-          const int st = static_cast<int>(g % NSTAGE);
-          if (g >= NSTAGE &&
-              !wait_cluster_bounded(&empty[st], static_cast<uint32_t>((g / NSTAGE) & 1) ^ 1u)) {
+          if (!wait_cluster_bounded(&empty[st], ph)) {
             if (leader) atomicOr(err, KERR_TIMEOUT_EMPTY);
             ok = false;
             break;
@@ -350,6 +354,10 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
             tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
           }
           __syncwarp();
+          if (++st == NSTAGE) {
+            st = 0;
+            ph ^= 1u;
+          }
         }
       }
       // no copy may be in flight when the pair ends (the even CTA's barriers
@@ -365,48 +373,51 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
       // kind::f16: FP32 D, BF16 A and B, K-major (bit 15: A MN-major), M = 256, N = BN
       constexpr uint32_t idesc0 = (1u << 4) | (1u << 7) | (1u << 10) |
                                   ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(2 * BM >> 4) << 24);
+      const uint64_t ak = desc_sw128(smem_u32(sA)), amn = desc_sw128_mn(smem_u32(sA));
+      const uint64_t b0 = desc_sw128(smem_u32(sB));
       bool ok = true;
-      long long g = 0;   // stages consumed
-      long long c = -1;  // current chunk (accumulator c & 1)
+      int st = 0, buf = 0;               // stage, accumulator
+      uint32_t ph = 0, acc_ph = 1;
       for (int t = pair; t < ntiles && ok; t += npairs) {
         Tile T;
         tile(t, T);
         const int cs = tab.m[T.modulus].chunk;
-        int in = 0;  // stage within the chunk
-        for (int ks = 0; ks < T.nst; ++ks, ++g) {
-          if (in == 0) {
-            ++c;
-            if (c >= 2 && !wait_cluster_bounded(&acc_empty[c & 1],
-                                                static_cast<uint32_t>((c >> 1) & 1) ^ 1u)) {
-              if (leader) atomicOr(err, KERR_TIMEOUT_FULL);
-              ok = false;
-              break;
-            }
-          }
-          const int st = static_cast<int>(g % NSTAGE);
-          if (!wait_cluster_bounded(&full[st], static_cast<uint32_t>((g / NSTAGE) & 1))) {
+        for (int k0 = 0; k0 < T.nst && ok; k0 += cs) {  // a chunk per accumulator
+          if (!wait_cluster_bounded(&acc_empty[buf], acc_ph)) {
             if (leader) atomicOr(err, KERR_TIMEOUT_FULL);
             ok = false;
             break;
           }
-          asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-          const uint32_t a0 = smem_u32(sA + st * C::A_BYTES), b0 = smem_u32(sB + st * C::B_BYTES);
-          const uint32_t d = tmem + static_cast<uint32_t>(c & 1) * C::BUF;
-          const bool tr = T.template transposed<TileFn::kTri>(ks * BK);
-          const uint32_t idesc = tr ? idesc0 | (1u << 15) : idesc0;
-          const uint64_t da = tr ? desc_sw128_mn(a0) : desc_sw128(a0);
-          const uint64_t step = (tr ? 16 * 128 : 32) >> 4;  // 16 of K
-          const bool last = in + 1 == cs || ks == T.nst - 1;
-          if (leader) {
+          const int k1 = min(k0 + cs, T.nst);
+          const uint32_t d = tmem + static_cast<uint32_t>(buf) * C::BUF;
+          for (int ks = k0; ks < k1; ++ks) {
+            if (!wait_cluster_bounded(&full[st], ph)) {
+              if (leader) atomicOr(err, KERR_TIMEOUT_FULL);
+              ok = false;
+              break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const bool tr = T.template transposed<TileFn::kTri>(ks * BK);
+            const uint32_t idesc = tr ? idesc0 | (1u << 15) : idesc0;
+            const uint64_t da = (tr ? amn : ak) + static_cast<uint64_t>(st * (C::A_BYTES >> 4));
+            const uint64_t db = b0 + static_cast<uint64_t>(st * (C::B_BYTES >> 4));
+            const uint64_t step = (tr ? 16 * 128 : 32) >> 4;  // 16 of K
+            if (leader) {
 #pragma unroll
-            for (int k = 0; k < BK / 16; ++k)
-              umma_pair(d, da + k * step, desc_sw128(b0 + k * 32), idesc,
-                        (in == 0 && k == 0) ? 0u : 1u);
-            commit_pair(&empty[st]);
-            if (last) commit_pair(&acc_full[c & 1]);
+              for (int k = 0; k < BK / 16; ++k)
+                umma_pair(d, da + k * step, db + k * (32 >> 4), idesc,
+                          (ks == k0 && k == 0) ? 0u : 1u);
+              commit_pair(&empty[st]);
+              if (ks == k1 - 1) commit_pair(&acc_full[buf]);
+            }
+            __syncwarp();
+            if (++st == NSTAGE) {
+              st = 0;
+              ph ^= 1u;
+            }
           }
-          __syncwarp();
-          in = last ? 0 : in + 1;
+          buf ^= 1;
+          if (buf == 0) acc_ph ^= 1u;
         }
       }
       // every MMA of this pair has completed when this fires
@@ -422,7 +433,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
     const int rit = static_cast<int>(rank) * BM + q * 32 + lane;  // row in the tile
     const uint32_t tbase = tmem + (static_cast<uint32_t>(q * 32) << 16) + hf * C::HC;
     const uint32_t bar_e0 = map_to_rank(&acc_empty[0], 0), bar_e1 = map_to_rank(&acc_empty[1], 0);
-    long long c = 0;
+    unsigned c = 0;  // chunk: accumulator c & 1, its phase c >> 1
     bool ok = true;
     for (int t = pair; t < ntiles && ok; t += npairs) {
       Tile T;
