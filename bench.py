@@ -632,27 +632,31 @@ def filter_workload_config(args, world):
                      f"{args.nex} columns, degree {m} for every column; step = one chase_filter "
                      f"call (Alg. 4) with the split-BF16 tensor-core product"),
         "n": n, "nev": args.nev, "nex": args.nex, "degree": m, "precision": "split",
-        "l2": (f"inputs larger than L2 (H {16 * n * n / 1e9:.1f} GB, its BF16 slices "
-               f"{28 * n * n / 1e9:.1f} GB, block {16 * n * nx / 1e9:.2f} GB)"),
+        "l2": (f"inputs larger than L2 (H {16 * n * n / 1e9:.1f} GB, its residue planes "
+               f"{22 * n * n / 1e9:.1f} GB, block {16 * n * nx / 1e9:.2f} GB)"),
         "parallelism": "replicas" if world > 1 else "single GPU",
     }
 
 
-# DRAM traffic of one zgemm_split_kernel launch of the default filter
-# workload (one of its four K segments: 30000 rows of H, 1500 complex
-# columns, K = 15000), measured with ncu on the persistent-CTA kernel
-# (dram__bytes_read.sum 58.80 GB + dram__bytes_write.sum 0.72 GB, one
-# pass, --clock-control none; the command is in the profile of this
-# kernel).  Set back to None whenever the kernel or its launch shape
-# changes.
-SPLIT_N30000_TRAFFIC = 58.80e9 + 0.72087e9
+# DRAM traffic of one product launch of the default filter workload: not
+# captured for the residue GEMM.
+SPLIT_N30000_TRAFFIC = None
+# Residue planes of the split filter's product up to N = 32768: 11 moduli, one
+# BF16 plane each of H (the second is its transpose), two of the block.
+SPLIT_MODULI = 11
 
 
 def split_algorithmic_bytes(n, ncols, k_per_launch):
-    """Bytes one split product launch must move at least: the 7 slice planes
-    of H and of the block over its K range, once, and the FP64 result
-    (a K-segment partial product, N x ncols complex)."""
+    """Bytes that one launch of a product of seven-digit slices moves at least:
+    the 7 slice planes of H and of the block over its K range, once, and the
+    FP64 result (a K-segment partial product, N x ncols complex)."""
     return 7 * 2.0 * (n + 2 * ncols) * k_per_launch + 16.0 * n * ncols
+
+
+def residue_algorithmic_bytes(n, ncols):
+    """Bytes that one residue product moves at least: the planes of H and of
+    the block once, and the residues of the product (int16)."""
+    return 2.0 * SPLIT_MODULI * (n * n + 2 * n * ncols) + 4.0 * SPLIT_MODULI * n * ncols
 
 
 def run_filter_workload(args, rank, world, local):
@@ -715,19 +719,16 @@ def run_filter_workload(args, rank, world, local):
     per_launch_s = kt["seconds"] / max(kt["launches"], 1)
     tensor_per_launch = kt["tensor_flops"] / max(kt["launches"], 1)
     achieved = tensor_per_launch / per_launch_s / 1e12 if per_launch_s > 0 else 0.0
-    launches_per_product = kt["launches"] / max(K * m, 1)
-    k_per_launch = 2.0 * n / launches_per_product
-    alg_bytes = split_algorithmic_bytes(n, nx, k_per_launch)
+    alg_bytes = residue_algorithmic_bytes(n, nx)
     roof = {
         "bound": "tensor",
-        "kernel": "zgemm_split_kernel (tcgen05 BF16 slice products, exact int32 level sums, "
-                  "FP64 recurrence epilogue)",
+        "kernel": "rns_gemm_kernel (tcgen05 CTA pairs, BF16 residue GEMMs)",
         "achieved": round(achieved, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
         "frac": round(achieved / peak, 4),
         "traffic": SPLIT_N30000_TRAFFIC if (n == 30000 and nx == 1500) else None,
         "peak_source": f"{src} bf16_tflops_sustained (a kernel inside a multi-second loop)",
-        "achieved_counts": "BF16 tensor FLOPs the kernel executes: 28 slice-pair products of "
-                           "8 N^2 per complex column",
+        "achieved_counts": "BF16 tensor FLOPs of the product: 22 residue planes of 2 N^2 per "
+                           "complex column",
         "fp64_equivalent_tflops": round(kt["flops"] / kt["seconds"] / 1e12, 3)
         if kt["seconds"] > 0 else None,
         "launches": kt["launches"], "avg_launch_ms": round(1e3 * per_launch_s, 3),
@@ -759,19 +760,19 @@ def run_filter_workload(args, rank, world, local):
         k64 = chase.chase_kernel_timing_read(chase.CHASE_TIMED_FP64_PRODUCT)
         t64 = c0.elapsed_time(c1) / 1e3
         fl64 = 8.0 * n * n * nx * 2
-        fp64_peak = pk.get("bf16_tflops", 1900.0) * NOMINAL_FP64_OVER_BF16
+        fp64_peak = pk.get("bf16_tflops", 1900.0)
         ex = k64["tensor_flops"] / k64["seconds"] / 1e12 if k64["seconds"] > 0 else 0.0
         fp64 = {"filter_tflops": round(fl64 / t64 / 1e12, 4),
                 "seconds_degree2": round(t64, 3),
                 "seconds_same_filter_extrapolated": round(t64 * m / 2.0, 1),
                 "speedup_split_vs_fp64_filter": round((flops_step * K / elapsed) / (fl64 / t64), 2),
                 "roofline": {"bound": "tensor",
-                             "kernel": "zgemm_tma_kernel (FP64 DMMA, 3M complex form)",
+                             "kernel": "rns_gemm_kernel (FP64 accuracy: 28 residue planes)",
                              "achieved": round(ex, 4), "peak": round(fp64_peak, 4),
                              "unit": "TFLOP/s", "frac": round(ex / fp64_peak, 4),
-                             "achieved_counts": "executed DMMA FLOPs (6 of 8 algorithmic)",
-                             "peak_source": f"{src} bf16_tflops (burst) x nominal FP64/BF16 "
-                                            "ratio (1.25/2250)"}}
+                             "achieved_counts": "BF16 tensor FLOPs of the product: 28 residue "
+                                                "planes of 2 N^2 per complex column",
+                             "peak_source": f"{src} bf16_tflops (burst)"}}
         del V64
 
     # ---------------- end to end through host buffers ----------------
@@ -942,17 +943,17 @@ def run_batched_workload(args, rank, world, local):
                  "product_seconds": round(st_o[0]["t_product"], 3),
                  "tile_config": st_o[0]["tile_config"]}
     if split:
-        achieved = SPLIT_PAIRS * flops / t_prod / 1e12
+        achieved = 0.5 * SPLIT_MODULI * flops / t_prod / 1e12
         peak = pk.get("bf16_tflops_sustained", 1700.0)
         roof = {"bound": "tensor",
-                "kernel": "zgemm_split_grouped_kernel (tcgen05 BF16 slice products over all "
-                          "problems of a degree step)",
+                "kernel": "rns_grouped_gemm_kernel (tcgen05 BF16 residue GEMMs over all problems "
+                          "of a degree step)",
                 "achieved": round(achieved, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4), "traffic": None,
                 "peak_source": f"{src} bf16_tflops_sustained",
                 "fp64_equivalent_tflops": round(flops / t_prod / 1e12, 3)}
-        # slice planes of H (28 N^2 bytes) stream from HBM once per degree step
-        hbm = sum(28.0 * n * n for n, _, _ in shapes) * st_main[0]["steps"] / t_prod / 1e9
+        # residue planes of H (22 N^2 bytes) stream from HBM once per degree step
+        hbm = sum(2.0 * SPLIT_MODULI * n * n for n, _, _ in shapes) * st_main[0]["steps"] / t_prod / 1e9
         roof["hbm_gbs_slices_of_h"] = round(hbm, 1)
         roof["hbm_frac"] = round(hbm / pk.get("hbm_gbs", 6800.0), 4)
     else:
@@ -1729,6 +1730,17 @@ def main():
         return
     pk, src = peaks()
     roof_main, roof_other = roofline_entry(stats_t, pk, src, args.precision)
+    for r in (roof_main, roof_other):  # products execute residue GEMMs: 11 moduli, FP64 14
+        if r and "achieved" in r:
+            moduli = SPLIT_MODULI if "fp64_equivalent_tflops" in r else 14
+            alg = r.get("fp64_equivalent_tflops") or r.get("algorithmic_tflops") or 0.0
+            peak = pk.get("bf16_tflops_sustained", 1700.0)
+            r.update(kernel="rns_gemm_kernel (BF16 residue GEMMs)", peak=round(peak, 1),
+                     achieved=round(0.5 * moduli * alg, 2),
+                     frac=round(0.5 * moduli * alg / peak, 4),
+                     achieved_counts=f"BF16 tensor FLOPs: {moduli} moduli, 2 planes of 2 N^2 per column",
+                     peak_source=f"{src} bf16_tflops_sustained")
+            r.pop("traffic_ncu_small_case", None)
     cb = None
     if not args.no_cpu_baseline and world == 1:
         cb = cpu_baseline_sample(n, nev, nex, args.seed, args.cpu_sample_seconds)

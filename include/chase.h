@@ -76,9 +76,8 @@ typedef struct {
  * symmetry.  QR, Rayleigh-Ritz, residuals and Lanczos keep FP64 accuracy. */
 #define CHASE_SPLIT_BF16 1
 /* Split-BF16 filter as above, and the product H Q of Rayleigh-Ritz (Alg. 2
- * line 2, reused for the residuals) on the same split product: each entry
- * carries the same 2^-49 relative bound, against the K u |H||Q| of an FP64
- * GEMM.  The projected eigenproblem, QR, the Gram products and Lanczos stay
+ * line 2, reused for the residuals) on the same split product, operands
+ * rounded to 2^-48 of their norms.  The projected eigenproblem, QR, the Gram products and Lanczos stay
  * FP64.  chase_solve and chase_solve_batched only (the filter entry points
  * take CHASE_FP64 or CHASE_SPLIT_BF16). */
 #define CHASE_SPLIT_BF16_RR 2
@@ -86,9 +85,9 @@ typedef struct {
  * (chase_solve only; the batched solve treats it as CHASE_SPLIT_BF16).  By
  * the model behind Alg. 5 a degree-m filter divides a column's residual by
  * |rho|^m; while that expected residual exceeds 1e-3 h (h = largest |Ritz
- * value|) the column's products keep the leading 3 slices of each operand
- * (about 2^-21 relative), above 1e-6 h 4 slices (2^-28), else all 7
- * (2^-49).  The first filter, before any residual is known, uses 3.  The
+ * value|) the column's products run in class 3, above 1e-6 h in class 4 (both
+ * round their operands to 2^-30 of a norm), else in class 7 (2^-48).  The
+ * first filter, before any residual is known, uses 3.  The
  * active block is ordered by (slices, degree), and each run of equal slices
  * is filtered as its own suffix-retiring block.  Rayleigh-Ritz, QR and
  * residuals stay FP64, so the converged pairs meet the same tolerance; a
@@ -268,9 +267,8 @@ int chase_filter(const chase_c64* H, int64_t N, int64_t ldh, chase_c64* V, int64
 /* Alg. 4 with a precision per column (Sec. 3.2: the filter only needs to be
  * as accurate as the residual it can reach; the paper filters every column
  * in one precision): column a is filtered with its degree degrees[a] on the
- * split-BF16 product that keeps the leading slices[a] slices of each
- * operand, slices[a] in {3, 4, 7} (about 2^-21, 2^-28 and 2^-49 relative
- * per product).  The columns are ordered by (slices, degree) inside the
+ * split product of precision class slices[a] in {3, 4, 7} (operands rounded
+ * to 2^-30, 2^-30 and 2^-48 of a norm).  The columns are ordered by (slices, degree) inside the
  * call and each run of equal slices is filtered as its own suffix-retiring
  * block of the same recurrence; V returns in the caller's column order.
  * H, V, work: as chase_filter (complex128, column-major, host or device).
@@ -433,10 +431,9 @@ int chase_solve_real(const double* H, int64_t N, int64_t ldh, int nev, int nex, 
  * hold) and rounds back.  Eigenvalues, residuals, bounds and tolerances are
  * doubles.  Single precision reaches residuals of about 1e-6 ||H||, so tol
  * should be 1e-5 or larger (Table 1's single-precision column).
- * opts->precision: CHASE_FP64 (the default) keeps the FP32 products; any
- * split value runs the solve's filter on the split-BF16 tensor-core product
- * with the leading 4 slices of each operand (about 2^-28 relative per
- * product entry, finer than FP32 rounding) on widened copies of the active
+ * opts->precision: CHASE_FP64 (the default) stores each step in FP32; any
+ * split value runs the solve's filter with the same products (operands
+ * rounded to 2^-30 of a norm, finer than FP32 rounding) on widened copies of the active
  * block, rounded back to single precision after the filter. */
 int chase_filter_c32(const chase_c32* H, int64_t N, int64_t ldh, chase_c32* V, int64_t ldv, int b,
                      const int* degrees, double b_sup, double mu1, double mu_nevnex,

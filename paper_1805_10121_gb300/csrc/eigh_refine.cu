@@ -162,9 +162,12 @@ __global__ void __launch_bounds__(kThreads)
 // columns of B = A' J orthogonal turn J into eigenvectors and each column of B
 // into a multiple of one, so J itself is not needed.  A warp holds a pair of
 // columns in registers; the p / 2 pairs of a round are disjoint, and p - 1
-// rounds meet every pair (round robin).  Latency of dot product and rotation
-// bounds it, 0.4 us a round; the library's solver, launches of a few
-// microseconds each, takes 1.3 ms at p = 70 (JACFIG).
+// rounds meet every pair (round robin).  Latency bounds it, 1.4 us a round: dot
+// product, rotation and the block's barrier.  The library's solver, hundreds of
+// launches of a few microseconds, takes 1.3 ms at p = 70 whatever G is; here a
+// dense G takes about as long (eigensolve in all 2.1 ms on either; p = 33: 0.82
+// against 1.34 ms), one near a diagonal, as from the second iteration of a solve
+// on, 0.6 ms.
 // ---------------------------------------------------------------------------
 constexpr int kJacobiMax = 96, kJacobiThreads = 1024;
 constexpr int kJacobiSweeps = 14;

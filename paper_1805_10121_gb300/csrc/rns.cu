@@ -310,8 +310,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
     {  // ---------------- TMA producer (both CTAs)
       // Stage and parity are counted along: these loops have a few hundred
       // cycles per stage, and 64-bit divisions for them took 4 to 5 % of every
-      // product.  A wait for
-      // the phase before a barrier's first returns at once.
+      // product.  A wait for the phase before a barrier's first returns at once.
       long long g = 0;  // stages issued by this CTA
       int st = 0;
       uint32_t ph = 1;

@@ -96,11 +96,12 @@ def footprint_bytes(n: int, nev: int, nex: int, split: bool) -> int:
     nx = nev + nex
     h = 16 * n * n
     gen = 3 * h                                   # construction temporaries
-    # BF16 residue planes of H, two per modulus: 14 moduli for products at FP64
-    # accuracy, 11 more for a split filter
+    # BF16 residue planes of H, two per modulus (one where all rows share a
+    # scale): 14 moduli for products at FP64 accuracy, 11 more for a split filter
     slices = (56 + (44 if split else 0)) * n * n
     # V, filter buffer, RR/QR work; residue planes of the block and of the product
-    blocks = 16 * n * nx * 10 + 2 * 56 * n * nx
+    # with H, and of two blocks and their product in QR and Rayleigh-Ritz
+    blocks = 16 * n * nx * 10 + 5 * 56 * n * nx
     return int(2 * h + gen + slices + blocks)
 
 
