@@ -1119,17 +1119,22 @@ struct Out<float> {
 // little as the recurrence allows: one conversion and, per real component,
 // T (alpha P 2^e) + (alpha (H_rr - shift)) x + beta y, with powers of two
 // applied to exponent bits and every test on integers (about 19 FP64
-// instructions a component before, 6 with the FP64 moduli, 4 otherwise).  With
-// the slicing likewise moved off that pipe, a product with N = 4096 and 788
-// columns (11 moduli) takes 115 us less outside its GEMM (205 us before).
+// instructions a component before, 4 now).  With the slicing likewise moved off
+// that pipe, a product with N = 4096 and 788 columns (11 moduli) takes 115 us
+// less outside its GEMM (205 us before).
 //
 // With the FP64 moduli (ACC) the constants that every product of a filter
-// shares, alpha P and alpha (H_rr - shift), carry a second double: their
-// rounding would be the same in every degree step and so add up over the
-// recurrence, where the roundings of an FP64 GEMM average out.
+// shares, alpha P and alpha (H_rr - shift), carry a second part, 2^-53 of the
+// first: their rounding would be the same in every degree step and so add up
+// over the recurrence, where the roundings of an FP64 GEMM average out.  Its
+// terms are formed in FP32 from truncated operands (24 bits of a 2^-53 part),
+// and in FP64 where they leave FP32's range (FP64 filter N = 4096: 4420 -> 4346
+// us, N = 1000: 932 -> 909 us, the errors against 64 bits as before).
+
 // What two rows of a product share over its columns.
 struct CrtRows {
   float df[2], dfl[2];  // single precision: alpha (H_rr - shift) as two floats
+  float dl32[2];        // dl in FP32
   int er[2];
   double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (as two doubles)
   bool diag[2];
@@ -1154,7 +1159,19 @@ __device__ __forceinline__ void crt_constants(CrtRows& k, int r0, int M, const i
     k.dl[h] = l;
     k.df[h] = static_cast<float>(d);
     k.dfl[h] = static_cast<float>(d - k.df[h]);
+    k.dl32[h] = static_cast<float>(l);
   }
+}
+
+// v as FP32, truncated, by its bits, for |v| < 2^100; 0 below FP32's range
+__device__ __forceinline__ float truncate_f32(double v) {
+  return copysignf(abs_f32(v, 0), __int_as_float(__double2hiint(v)));
+}
+// v as a double, by its bits; 0 for a denormal
+__device__ __forceinline__ double extend_f64(float v) {
+  const int u = __float_as_int(v), m = u & 0x7FFFFFFF;
+  const int h = (u & static_cast<int>(0x80000000u)) | ((m >> 3) + (896 << 20));
+  return m >= (1 << 23) ? __hiloint2double(h, m << 29) : 0.0;
 }
 
 // v 2^e for a normal float whose result is one too; 0 where it would not be
@@ -1244,6 +1261,33 @@ __device__ __forceinline__ void crt_pair(const CrtRows& k, int r0, int c,
     }
     if (sc.plain && !bad && e >= -800 && e <= 800) {
       const double f = scale_pow2(sc.ap, e), fl = ACC ? scale_pow2(sc.ap_lo, e) : 0.0;
+      if constexpr (ACC) {
+        // the low parts of the constants, 2^-53 of the others, in FP32, where
+        // their terms are in its range
+        const int xf = (__double2hiint(f) >> 20) & 0x7FF;
+        uint32_t big = abs_hi(re_in(x));
+        if constexpr (CP) big = max(big, abs_hi(im_in(x)));
+        if (xf >= 1023 - 85 && xf <= 1023 + 60 && big < ((1023u + 60u) << 20)) {
+          const float fl32 = truncate_f32(scale_pow2(sc.ap_lo, e + 32));
+#pragma unroll
+          for (int w = 0; w < W; ++w) {
+            const long long t = crt_fraction(hi[h][w], lo[h][w]);
+            const double xw = w == 0 ? re_of(x) : im_of(x), yw = w == 0 ? re_of(y) : im_of(y);
+            float a = static_cast<float>(static_cast<int>(t >> 32)) * fl32;
+            if (k.diag[h]) a = fmaf(k.dl32[h], truncate_f32(xw), a);
+            double q = extend_f64(a);
+            if (sc.has_beta) q = fma(sc.beta, yw, q);
+            if (k.diag[h]) q = fma(k.dh[h], xw, q);
+            v[w] = fma(static_cast<double>(t), f, q);
+          }
+          if constexpr (CP)
+            out[h] = E{static_cast<S>(v[0]), static_cast<S>(v[1])};
+          else
+            out[h] = static_cast<S>(v[0]);
+          *cp = out[h];
+          continue;
+        }
+      }
 #pragma unroll
       for (int w = 0; w < W; ++w) {
         const double T = crt_value(hi[h][w], lo[h][w]);
