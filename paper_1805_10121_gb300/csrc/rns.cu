@@ -167,28 +167,26 @@ __device__ __forceinline__ uint64_t desc_sw128_mn(uint32_t saddr) {
   return d;
 }
 
-// 8 columns of this thread's row of an accumulator, as 4 column pairs.  The
-// loads are complete after tmem_wait_ld, through which their registers pass so
-// that no use of them can be scheduled before it.
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, unsigned long long (&r)[4]) {
-  uint32_t u[8];
+// 8 columns of this thread's row of an accumulator.  The load is asynchronous:
+// its registers may not be read, and so not packed in pairs either, before
+// tmem_wait_ld, through which they pass so that no use can be scheduled earlier.
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&u)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
                : "=r"(u[0]), "=r"(u[1]), "=r"(u[2]), "=r"(u[3]), "=r"(u[4]), "=r"(u[5]), "=r"(u[6]),
                  "=r"(u[7])
                : "r"(taddr));
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    r[i] = static_cast<unsigned long long>(u[2 * i]) |
-           static_cast<unsigned long long>(u[2 * i + 1]) << 32;
 }
-__device__ __forceinline__ void tmem_wait_ld(unsigned long long (&r)[4]) {
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&u)[8]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+l"(r[0]), "+l"(r[1]), "+l"(r[2]), "+l"(r[3])::"memory");
+               : "+r"(u[0]), "+r"(u[1]), "+r"(u[2]), "+r"(u[3]), "+r"(u[4]), "+r"(u[5]), "+r"(u[6]),
+                 "+r"(u[7])::"memory");
 }
 // Two FP32 operations in one instruction, each rounded as its scalar form.
+__device__ __forceinline__ unsigned long long pack_b32x2(uint32_t lo, uint32_t hi) {
+  return static_cast<unsigned long long>(lo) | static_cast<unsigned long long>(hi) << 32;
+}
 __device__ __forceinline__ unsigned long long pack_f32x2(float lo, float hi) {
-  return static_cast<unsigned long long>(__float_as_uint(lo)) |
-         static_cast<unsigned long long>(__float_as_uint(hi)) << 32;
+  return pack_b32x2(__float_as_uint(lo), __float_as_uint(hi));
 }
 __device__ __forceinline__ unsigned long long fma_f32x2(unsigned long long a, unsigned long long b,
                                                         unsigned long long c) {
@@ -456,7 +454,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const uint32_t tb = tbase + static_cast<uint32_t>(c & 1) * C::BUF;
         // the load of the next 8 columns is in flight while these are reduced
-        unsigned long long r[2][4];
+        uint32_t r[2][8];
         tmem_ld8(tb, r[0]);
 #pragma unroll
         for (int j0 = 0; j0 < C::HC; j0 += 8) {
@@ -465,7 +463,8 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             // |v| <= 2^24, an integer; v - p rint(v / p), exact
-            const unsigned long long v = r[(j0 / 8) & 1][j];
+            const unsigned long long v =
+                pack_b32x2(r[(j0 / 8) & 1][2 * j], r[(j0 / 8) & 1][2 * j + 1]);
             const unsigned long long k = add_f32x2(fma_f32x2(v, invp2, rnd2), mrnd2);
             acc[j0 / 2 + j] = add_f32x2(acc[j0 / 2 + j], fma_f32x2(k, mp2, v));
           }
