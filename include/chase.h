@@ -205,6 +205,14 @@ long long chase_device_allocations(void);
  * calling program has synchronised; a call in flight keeps what it uses). */
 int chase_release_workspace(void);
 
+/* Bounds the device workspace that each later call of the calling thread may
+ * hold at a time, in bytes (0 or less: no bound, the default).  Calls behave as
+ * if the device had no more: with fewer residue planes of H resident, fewer
+ * columns at a time, parts of a batch in turn, FP64 products without planes,
+ * and CHASE_OUT_OF_MEMORY where the least of these does not fit.  The host
+ * threads of chase_solve_batched count the bound each on its own. */
+int chase_workspace_limit(long long bytes);
+
 /* Kernel timing, for benchmarks (the paper has no counterpart).  While
  * timing is on, the library records a pair of CUDA events on the launching
  * stream around the launches of its products with H:

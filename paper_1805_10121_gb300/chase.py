@@ -21,7 +21,7 @@ import torch
 __all__ = [
     "ChaseError", "ChaseOpts", "ChaseStats", "lib", "lib_path", "declared_symbols",
     "chase_opts_default", "chase_last_error", "chase_filter_mixed", "chase_kernel_launches", "chase_device_allocations",
-    "chase_release_workspace",
+    "chase_release_workspace", "chase_workspace_limit",
     "chase_kernel_timing",
     "chase_kernel_timing_read", "chase_wait_selftest", "CHASE_TIMED_SPLIT_PRODUCT", "CHASE_TIMED_FP64_PRODUCT", "chase_filter", "chase_lanczos",
     "chase_degrees", "chase_lock", "chase_tridiag_eigh", "chase_dos_estimate", "chase_orthonormalize",
@@ -122,6 +122,7 @@ _SIGNATURES = {
     "chase_kernel_launches": (ctypes.c_longlong, []),
     "chase_device_allocations": (ctypes.c_longlong, []),
     "chase_release_workspace": (_int, []),
+    "chase_workspace_limit": (_int, [ctypes.c_longlong]),
     "chase_kernel_timing": (_int, [_int]),
     "chase_wait_selftest": (_int, [ctypes.c_longlong, _c_p]),
     "chase_kernel_timing_read": (_int, [_int, _dp, ctypes.POINTER(ctypes.c_longlong), _dp, _dp]),
@@ -204,6 +205,11 @@ def chase_device_allocations() -> int:
 def chase_release_workspace() -> None:
     """Hand the workspace that the library keeps between calls back to the driver."""
     _check(lib().chase_release_workspace(), "chase_release_workspace")
+
+
+def chase_workspace_limit(nbytes: int) -> None:
+    """Bound the workspace of each later call of this thread (0: no bound)."""
+    _check(lib().chase_workspace_limit(int(nbytes)), "chase_workspace_limit")
 
 
 CHASE_TIMED_SPLIT_PRODUCT = 0

@@ -148,9 +148,48 @@ struct RnsSet {
 // columns or rows, the FP64 kernels are done sooner than its three launches.
 bool rns_pays(int64_t N, int b) { return N >= 128 && b > kFewColMax; }
 
-// Bytes that a call may still allocate after the residue planes of H.
+// Bytes that a call may still allocate after the residue planes of H: the
+// Lanczos vectors, row panels and the projected eigenproblem (the planes of
+// tall products are left out: those fall back).
 size_t rns_reserve(int64_t N, int b) {
-  return (size_t(2) << 30) + static_cast<size_t>(N) * b * 16 * 4;
+  const size_t n = static_cast<size_t>(N), w = static_cast<size_t>(b);
+  return 16 * (n * 128 + w * (4096 + 16 * w)) + std::min(size_t(1) << 30, 4 * n * n);
+}
+
+// Residue planes of H (h with nmod moduli, one set or several) and the
+// workspace x for b columns.  Where they do not all fit beside the reserve, with
+// fewer moduli resident and fewer columns at a time; where one modulus of each
+// and one column do not, CHASE_OUT_OF_MEMORY with nothing held if the caller has
+// another way (optional), else the same again with less in reserve.
+struct PlaneSet {
+  int nmod;
+  RnsH* h;
+};
+template <class T>
+int prepare_products(Dev& d, const T* H, int64_t N, int64_t ldh, int b, bool many, bool optional,
+                     const std::vector<PlaneSet>& sets, RnsX& x) {
+  int widest = 0;
+  for (const PlaneSet& s : sets) widest = std::max(widest, s.nmod);
+  size_t reserve = rns_reserve(N, b);
+  int cols = b, most = kRnsMaxModuli;
+  for (;;) {
+    int st = rns_alloc_x(d, N, cols, widest, is_cplx<T>, x);
+    for (const PlaneSet& s : sets)
+      if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, s.nmod, most, reserve, many, *s.h);
+    if (st != CHASE_OUT_OF_MEMORY) return st;
+    rns_release(d, x);
+    for (const PlaneSet& s : sets) rns_release(d, *s.h);
+    if (cols > 1 || most > 1) {
+      cols = (cols + 1) / 2;
+      most = (most + 1) / 2;
+    } else if (!optional && reserve > 0) {
+      cols = b;
+      most = kRnsMaxModuli;
+      reserve = reserve > (size_t(1) << 20) ? reserve / 2 : 0;
+    } else {
+      return st;
+    }
+  }
 }
 
 // One filter product: in residue arithmetic when H is prepared for it, else
@@ -509,12 +548,10 @@ int rr_pre(Dev& d, const T* H, int64_t N, int64_t ldh, const T* Q, int64_t ldq, 
     if (!rs && rns_pays(N, b)) {
       RnsH h;
       RnsX x;
-      int st = rns_alloc_x(d, N, b, kRnsFp64, is_cplx<T>, x);
-      if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, kRnsFp64, rns_reserve(N, b), false, h);
+      int st = prepare_products(d, H, N, ldh, b, false, true, {{kRnsFp64, &h}}, x);
       if (st == CHASE_OK) st = rns_product(d, h, x, Q, ldq, 0, b, w.HQ, lN, 1.0, 0.0, 0.0);
-      for (void* p : {h.A, static_cast<void*>(h.E), static_cast<void*>(h.Dg), x.B,
-                      static_cast<void*>(x.G), static_cast<void*>(x.F)})
-        if (p) d.release(p);
+      rns_release(d, h);
+      rns_release(d, x);
       if (st != CHASE_OK && st != CHASE_OUT_OF_MEMORY) return st;
       done = st == CHASE_OK;
     }
@@ -885,15 +922,14 @@ struct Solver {
   // solver's filter and Rayleigh-Ritz share one set; a split filter has its
   // own (with CHASE_SPLIT_BF16_ADAPT a second one for its reduced precisions)
   // beside Rayleigh-Ritz's FP64 one; single precision needs the low set only.
+  // Where the memory does not hold them, products at FP64 accuracy and those
+  // of the single-precision solver run on the FP64 and FP32 pipes.
   int prepare_rns(Dev& d) {
     rns = split || rns_pays(N, nx);
     if (!rns) return CHASE_OK;
-    const bool want64 = !is_single<T> && !split_rr && rns_pays(N, nx);
+    bool want64 = !is_single<T> && !split_rr && rns_pays(N, nx);
     const bool want_split = !is_single<T> && split;
     const bool want_low = is_single<T> || o.precision == CHASE_SPLIT_BF16_ADAPT;
-    const int low = rns_low_moduli(N);
-    const size_t reserve = rns_reserve(N, nx);
-    CHASE_TRY(rns_alloc_x(d, N, nx, want64 ? kRnsFp64 : want_split ? rns_split_moduli(N) : low, is_cplx<T>, rx));
     if constexpr (is_single<T>) {
       if (split) {
         lD = ld_pad<Wide>(N);
@@ -901,9 +937,21 @@ struct Solver {
         CHASE_TRY(d.alloc(&Dw, static_cast<size_t>(lD) * nx));
       }
     }
-    if (want_split) CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), reserve, true, hsplit));
-    if (want_low) CHASE_TRY(rns_prepare_h(d, dH, N, lh, low, reserve, true, hlow));
-    if (want64) CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, reserve, true, h64));
+    std::vector<PlaneSet> sets;
+    if (want_split) sets.push_back({rns_split_moduli(N), &hsplit});
+    if (want_low) sets.push_back({rns_low_moduli(N), &hlow});
+    if (want64) sets.push_back({kRnsFp64, &h64});
+    int st = prepare_products(d, dH, N, lh, nx, true, want64 || !split, sets, rx);
+    if (st == CHASE_OUT_OF_MEMORY && !split) {
+      rns = false;
+      return CHASE_OK;
+    }
+    if (st == CHASE_OUT_OF_MEMORY && want64) {  // the filter's alone
+      want64 = false;
+      sets.pop_back();
+      st = prepare_products(d, dH, N, lh, nx, true, false, sets, rx);
+    }
+    CHASE_TRY(st);
     filter_set.full = want_split ? &hsplit : want64 ? &h64 : nullptr;
     filter_set.low = want_low ? &hlow : nullptr;
     filter_set.x = &rx;
@@ -1359,7 +1407,7 @@ int filter_impl(const T* H, int64_t N, int64_t ldh, T* V, int64_t ldv, int b, co
   CHASE_CUDA(cudaMemcpyAsync(start.data(), dstart, sizeof(int) * start.size(), cudaMemcpyDeviceToHost, d.st));
   CHASE_CUDA(cudaMemcpyAsync(&maxdeg, dinfo, sizeof(int), cudaMemcpyDeviceToHost, d.st));
   CHASE_TRY(d.sync_check("chase_filter plan"));
-  const bool rns = precision != CHASE_FP64 || rns_pays(N, b);
+  bool rns = precision != CHASE_FP64 || rns_pays(N, b);
   RnsH rh;
   RnsX rx;
   RnsSet rs;
@@ -1367,8 +1415,11 @@ int filter_impl(const T* H, int64_t N, int64_t ldh, T* V, int64_t ldv, int b, co
     const int nmod = is_single<T> || precision == CHASE_SPLIT_BF16_4 || precision == CHASE_SPLIT_BF16_3
                          ? rns_low_moduli(N)
                          : precision == CHASE_FP64 ? kRnsFp64 : rns_split_moduli(N);
-    CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), true, rh));
+    const int st = prepare_products(d, dH, N, lh, b, true, precision == CHASE_FP64, {{nmod, &rh}}, rx);
+    if (st == CHASE_OUT_OF_MEMORY && precision == CHASE_FP64)
+      rns = false;  // on the FP64 pipe (FP32 in single precision)
+    else
+      CHASE_TRY(st);
     rs.full = &rh;
     rs.x = &rx;
   }
@@ -1493,16 +1544,12 @@ extern "C" int chase_filter_mixed(const chase_c64* H, int64_t N, int64_t ldh, ch
   rs.x = &rx;
   const bool any_low = *std::min_element(ns.begin(), ns.end()) < 7;
   const bool any_full = *std::max_element(ns.begin(), ns.end()) == 7;
-  const int nlow = rns_low_moduli(N);
-  CHASE_TRY(rns_alloc_x(d, N, b, any_full ? rns_split_moduli(N) : nlow, true, rx));
-  if (any_full) {
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, rns_split_moduli(N), rns_reserve(N, b), true, full));
-    rs.full = &full;
-  }
-  if (any_low) {
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nlow, rns_reserve(N, b), true, low));
-    rs.low = &low;
-  }
+  std::vector<PlaneSet> sets;
+  if (any_full) sets.push_back({rns_split_moduli(N), &full});
+  if (any_low) sets.push_back({rns_low_moduli(N), &low});
+  CHASE_TRY(prepare_products(d, dH, N, lh, b, true, false, sets, rx));
+  rs.full = any_full ? &full : nullptr;
+  rs.low = any_low ? &low : nullptr;
   CHASE_TRY(launch_permute_cols(d, dV, lv, wk, lw, N, b, dperm, false));
   CHASE_TRY(filter_groups(d, dH, N, lh, wk, lw, dV, lv, groups, maxdeg, b_sup, mu1, mu_nevnex,
                           nullptr, &rs));
@@ -1602,18 +1649,9 @@ extern "C" int chase_rayleigh_ritz(const chase_c64* H, int64_t N, int64_t ldh, c
   double *dw = nullptr, *dr = nullptr;
   CHASE_TRY(d.alloc(&dw, b));
   if (resid) CHASE_TRY(d.alloc(&dr, b));
-  RnsH rh;
-  RnsX rx;
-  RnsSet rs;
-  const bool rns = rns_pays(N, b);
-  if (rns) {
-    CHASE_TRY(rns_alloc_x(d, N, b, kRnsFp64, true, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, kRnsFp64, rns_reserve(N, b), false, rh));
-    rs.full = &rh;
-    rs.x = &rx;
-  }
+  // the product with H is made, or falls back, inside
   double te = 0.0, fl = 0.0;
-  CHASE_TRY(rr_core(d, dH, N, lh, dQ, lq, b, dw, dr, w, &te, &fl, nullptr, rns ? &rs : nullptr));
+  CHASE_TRY(rr_core(d, dH, N, lh, dQ, lq, b, dw, dr, w, &te, &fl));
   if (!dev) CHASE_TRY(copy_block(d, Q, ldq, dQ, lq, N, b, cudaMemcpyDeviceToHost));
   CHASE_CUDA(cudaMemcpyAsync(ritz, dw, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
   if (resid) CHASE_CUDA(cudaMemcpyAsync(resid, dr, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
@@ -1648,16 +1686,17 @@ int residuals_impl(const T* H, int64_t N, int64_t ldh, const T* V, int64_t ldv, 
   CHASE_TRY(d.alloc(&dl, b));
   CHASE_TRY(d.alloc(&dr, b));
   CHASE_CUDA(cudaMemcpyAsync(dl, lambda, sizeof(double) * b, cudaMemcpyHostToDevice, d.st));
-  if (rns_pays(N, b)) {
-    RnsH rh;
-    RnsX rx;
-    const int nmod = is_single<T> ? rns_low_moduli(N) : kRnsFp64;
-    CHASE_TRY(rns_alloc_x(d, N, b, nmod, is_cplx<T>, rx));
-    CHASE_TRY(rns_prepare_h(d, dH, N, lh, nmod, rns_reserve(N, b), false, rh));
-    CHASE_TRY(rns_product(d, rh, rx, dV, lv, 0, b, HV, lw, 1.0, 0.0, 0.0));
-  } else {
-    CHASE_TRY(gemm(d, N, N, dH, lh, dV, lv, b, HV, lw, 0, b, 1.0, 0.0, 0.0));
-  }
+  RnsH rh;
+  RnsX rx;
+  int st = CHASE_OUT_OF_MEMORY;
+  if (rns_pays(N, b))
+    st = prepare_products(d, dH, N, lh, b, false, true,
+                          {{is_single<T> ? rns_low_moduli(N) : kRnsFp64, &rh}}, rx);
+  if (st == CHASE_OK)
+    st = rns_product(d, rh, rx, dV, lv, 0, b, HV, lw, 1.0, 0.0, 0.0);
+  else if (st == CHASE_OUT_OF_MEMORY)
+    st = gemm(d, N, N, dH, lh, dV, lv, b, HV, lw, 0, b, 1.0, 0.0, 0.0);
+  CHASE_TRY(st);
   CHASE_TRY(launch_resid_norms(d, HV, lw, dV, lv, N, b, dl, dr));
   CHASE_CUDA(cudaMemcpyAsync(resid, dr, sizeof(double) * b, cudaMemcpyDeviceToHost, d.st));
   return d.sync_check("chase_residuals");

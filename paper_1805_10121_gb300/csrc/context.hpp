@@ -15,13 +15,19 @@ namespace chase {
 struct Dev {
   cudaStream_t st = nullptr;
   int* err = nullptr;  // device int, bit field of KERR_* codes
-  std::vector<void*> bufs;
+  struct Block {
+    void* p;
+    size_t bytes;
+  };
+  std::vector<Block> bufs;
+  size_t held = 0;   // bytes of bufs
+  size_t limit;      // chase_workspace_limit of the thread that made the context
   // A view on another context's stream with a flag slot of its own (the
   // per-problem flags of a batch): err is borrowed, and leaving the view
   // does not synchronise (its workspace is released stream-ordered).
   bool own_err = true, sync_on_exit = true;
 
-  explicit Dev(void* stream) : st(static_cast<cudaStream_t>(stream)) {}
+  explicit Dev(void* stream);
   Dev(const Dev&) = delete;
   Dev& operator=(const Dev&) = delete;
   ~Dev();
@@ -34,15 +40,13 @@ struct Dev {
   }
   // Give an allocation of this context back before the context ends.
   void release(void* p);
+  // Bytes that this context can still allocate.
+  int free_bytes(size_t* bytes);
   // Synchronise the stream and turn the device error flag into a status.
   int sync_check(const char* where);
 };
 
 bool is_device_ptr(const void* p);
-
-// Bytes that the library's pool on the current device holds but does not use:
-// free memory to the library although cudaMemGetInfo counts it as taken.
-size_t pool_idle_bytes();
 
 // Records a CUDA event pair on stream `s` around product launches while
 // chase_kernel_timing is on (a no-op otherwise).  end() gives the launches
@@ -201,14 +205,17 @@ struct RnsX {
   int64_t Kp = 0, ldg = 0;
   int flip = 0;  // which half of F (2 cap_cols) the residues in B belong to
 };
-// reserve: bytes to leave free when the planes are large.  many: the planes
+// most: moduli resident at most.  reserve: bytes to leave free.  many: the planes
 // serve many products, which pays for looking whether one scale fits all rows
-// (a pass over H and a synchronisation).
+// (a pass over H and a synchronisation).  CHASE_OUT_OF_MEMORY leaves nothing
+// behind, of the workspace (rns_alloc_x) either.
 bool rns_sym_pays(int planes, double entries);  // of H's, or of a whole batch's
 template <class T>
-int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
-                  RnsH& out);
+int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, int most, size_t reserve,
+                  bool many, RnsH& out);
 int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX& out);
+void rns_release(Dev& d, RnsH& h);
+void rns_release(Dev& d, RnsX& x);
 // C[:, j0:j1] = alpha (H X[:, j0:j1] - shift X[:, j0:j1]) + beta C[:, j0:j1].
 // Chained products (where rns_chains allows it for the widest): next0 >= 0
 // leaves the residues of C[:, next0:j1] in x, and a product with sliced takes

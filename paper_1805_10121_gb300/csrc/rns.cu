@@ -44,6 +44,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <limits>
 #include <type_traits>
 
 #include "common.cuh"
@@ -2130,11 +2131,18 @@ int rns_low_moduli(int64_t N) { return N <= 8192 ? 7 : 8; }
 // 2362 and 2232).
 bool rns_sym_pays(int planes, double entries) { return 2.0 * planes * entries > 64e6; }
 
+namespace rns {
+namespace {
+// From here on (bytes of planes) the driver is asked what is free, about 3 us,
+// so that the planes leave `reserve`; below, only an allocation that fails makes
+// fewer moduli resident.
+constexpr size_t kLargePlanes = size_t(1) << 25;
+
 template <class T>
-int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t reserve, bool many,
-                  RnsH& out) {
+int prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, int most, size_t reserve,
+              bool many, RnsH& out) {
   out.N = N;
-  out.Kp = (N + rns::BK - 1) / rns::BK * rns::BK;
+  out.Kp = (N + BK - 1) / BK * BK;
   out.src_kind = Kind<T>::k;
   out.cplx = out.src_kind % 2 == 0 ? 1 : 0;
   out.nmod = nmod;
@@ -2143,16 +2151,19 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
   CHASE_TRY(d.alloc(&out.E, static_cast<size_t>(N)));
   CHASE_TRY(d.alloc(&out.Dg, static_cast<size_t>(N)));
   if (many && rns_sym_pays(out.cplx ? 2 * nmod : nmod, static_cast<double>(N) * out.Kp))
-    CHASE_TRY(rns::row_scales(d, reinterpret_cast<const typename Kind<T>::D*>(H), ldh, out));
+    CHASE_TRY(row_scales(d, reinterpret_cast<const typename Kind<T>::D*>(H), ldh, out));
   const size_t per = static_cast<size_t>(out.cplx && !out.sym ? 2 : 1) * N * out.Kp * 2;  // bytes per modulus
   // all moduli resident where the memory allows it; else fewer, sliced anew
   // for every product
-  out.resident = nmod;
-  if (per * nmod > (size_t(16) << 30)) {
-    size_t free_b = 0, total_b = 0;
-    CHASE_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    free_b += pool_idle_bytes();
+  out.resident = std::min(nmod, std::max(most, 1));
+  if (per * nmod > kLargePlanes || d.limit != std::numeric_limits<size_t>::max()) {
+    size_t free_b = 0;
+    CHASE_TRY(d.free_bytes(&free_b));
     while (out.resident > 1 && per * out.resident + reserve > free_b) out.resident /= 2;
+    if (per * out.resident + reserve > free_b) {
+      set_error("residue planes of H: %zu bytes a modulus do not fit the memory", per);
+      return CHASE_OUT_OF_MEMORY;
+    }
   }
   int st = CHASE_OUT_OF_MEMORY;
   for (; out.resident >= 1; out.resident /= 2) {
@@ -2160,8 +2171,28 @@ int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, size_t r
     if (st != CHASE_OUT_OF_MEMORY) break;
   }
   CHASE_TRY(st);
-  if (out.resident == nmod) return rns::slice_h_moduli(d, out, 0, nmod);
-  return CHASE_OK;
+  return out.resident == nmod ? slice_h_moduli(d, out, 0, nmod) : CHASE_OK;
+}
+}  // namespace
+}  // namespace rns
+
+void rns_release(Dev& d, RnsH& h) {
+  for (void* p : {h.A, static_cast<void*>(h.E), static_cast<void*>(h.Dg)})
+    if (p) d.release(p);
+  h = RnsH{};
+}
+void rns_release(Dev& d, RnsX& x) {
+  for (void* p : {x.B, static_cast<void*>(x.G), static_cast<void*>(x.F)})
+    if (p) d.release(p);
+  x = RnsX{};
+}
+
+template <class T>
+int rns_prepare_h(Dev& d, const T* H, int64_t N, int64_t ldh, int nmod, int most, size_t reserve,
+                  bool many, RnsH& out) {
+  const int st = rns::prepare_h(d, H, N, ldh, nmod, most, reserve, many, out);
+  if (st == CHASE_OUT_OF_MEMORY) rns_release(d, out);
+  return st;
 }
 
 int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX& out) {
@@ -2177,12 +2208,16 @@ int rns_alloc_x(Dev& d, int64_t N, int max_cols, int max_moduli, bool cplx, RnsX
       void* g = nullptr;
       st = d.alloc_bytes(&g, bytes);
       out.G = static_cast<int16_t*>(g);
-      if (st != CHASE_OK) d.release(out.B);
+      if (st != CHASE_OK) {
+        d.release(out.B);
+        out.B = nullptr;
+      }
     }
     if (st != CHASE_OUT_OF_MEMORY || out.cap_cols == 1) break;
   }
-  CHASE_TRY(st);
-  return d.alloc(&out.F, 2 * static_cast<size_t>(out.cap_cols));
+  if (st == CHASE_OK) st = d.alloc(&out.F, 2 * static_cast<size_t>(out.cap_cols));
+  if (st == CHASE_OUT_OF_MEMORY) rns_release(d, out);
+  return st;
 }
 
 bool rns_chains(const RnsH& h, int b, const RnsX& x) {
@@ -2353,7 +2388,7 @@ int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const Grouped
 }
 
 #define CHASE_INSTANTIATE_RNS(T)                                                                 \
-  template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, size_t, bool, RnsH&);     \
+  template int rns_prepare_h<T>(Dev&, const T*, int64_t, int64_t, int, int, size_t, bool, RnsH&); \
   template int rns_product<T>(Dev&, const RnsH&, RnsX&, const T*, int64_t, int, int, T*, int64_t, \
                               double, double, double, bool, int);
 CHASE_INSTANTIATE_RNS(chase_c64)

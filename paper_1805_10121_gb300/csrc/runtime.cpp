@@ -138,8 +138,14 @@ int make_tmap_bf16_3d(CUtensorMap* map, const void* base, int64_t d0, int64_t d1
 // ---------------------------------------------------------------------------
 // Device context
 // ---------------------------------------------------------------------------
+namespace {
+thread_local size_t t_workspace_limit = std::numeric_limits<size_t>::max();
+}
+
+Dev::Dev(void* stream) : st(static_cast<cudaStream_t>(stream)), limit(t_workspace_limit) {}
+
 Dev::~Dev() {
-  for (void* p : bufs) cudaFreeAsync(p, st);
+  for (const Block& b : bufs) cudaFreeAsync(b.p, st);
   if (err && own_err) cudaFreeAsync(err, st);
   if (sync_on_exit) cudaStreamSynchronize(st);
 }
@@ -203,16 +209,20 @@ cudaError_t pool_malloc(void** p, size_t bytes, cudaStream_t st) {
 }
 }  // namespace
 
-size_t pool_idle_bytes() {
+int Dev::free_bytes(size_t* bytes) {
+  size_t free_b = 0, total_b = 0;
+  CHASE_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  // what the library's pool holds but does not use is free to the library
   cudaMemPool_t pool = device_pool();
   uint64_t reserved = 0, used = 0;
-  if (!pool ||
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess ||
-      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return reserved > used ? static_cast<size_t>(reserved - used) : 0;
+  if (pool &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) == cudaSuccess &&
+      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess &&
+      reserved > used)
+    free_b += static_cast<size_t>(reserved - used);
+  cudaGetLastError();
+  *bytes = std::min(free_b, limit - std::min(limit, held));
+  return CHASE_OK;
 }
 
 int Dev::init() {
@@ -227,6 +237,10 @@ int Dev::init() {
 int Dev::alloc_bytes(void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return CHASE_OK;
+  if (held > limit || bytes > limit - held) {
+    set_error("device workspace allocation of %zu bytes is beyond the workspace limit", bytes);
+    return CHASE_OUT_OF_MEMORY;
+  }
   g_allocs.fetch_add(1, std::memory_order_relaxed);
   cudaError_t e = pool_malloc(p, bytes, st);
   if (e != cudaSuccess) {
@@ -235,13 +249,15 @@ int Dev::alloc_bytes(void** p, size_t bytes) {
     *p = nullptr;
     return CHASE_OUT_OF_MEMORY;
   }
-  bufs.push_back(*p);
+  bufs.push_back(Block{*p, bytes});
+  held += bytes;
   return CHASE_OK;
 }
 
 void Dev::release(void* p) {
   for (auto it = bufs.begin(); it != bufs.end(); ++it)
-    if (*it == p) {
+    if (it->p == p) {
+      held -= it->bytes;
       bufs.erase(it);
       cudaFreeAsync(p, st);
       return;
@@ -406,6 +422,12 @@ extern "C" int chase_release_workspace(void) {
       const cudaError_t e = cudaMemPoolTrimTo(p, 0);
       if (e != cudaSuccess) return chase::cuda_status(e, "chase_release_workspace");
     }
+  return CHASE_OK;
+}
+
+extern "C" int chase_workspace_limit(long long bytes) {
+  chase::t_workspace_limit =
+      bytes > 0 ? static_cast<size_t>(bytes) : std::numeric_limits<size_t>::max();
   return CHASE_OK;
 }
 
