@@ -172,11 +172,11 @@ int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int ti
   return tile == CHASE_TILE_AUTO && step >= 2e7 ? kRnsFp64 : 0;
 }
 
-void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in) {
+void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in, GroupedWork& w) {
+  for (void* p : {w.block, w.planes})
+    if (p) d.release(p);
+  w = GroupedWork{};
   for (GroupedFilterInput& g : in) {
-    for (void* p : {g.A, static_cast<void*>(g.E), static_cast<void*>(g.Dg), g.Bsl, g.G,
-                    static_cast<void*>(g.F)})
-      if (p) d.release(p);
     g.A = g.Bsl = g.G = nullptr;
     g.E = g.F = nullptr;
     g.Dg = nullptr;
@@ -185,39 +185,56 @@ void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in) {
 }
 
 namespace {
-int alloc_block_planes(Dev& d, GroupedFilterInput& g, int bcap, int nmod) {
-  const int64_t Kp = rns_k_padded(g.n);
-  g.bcap = std::max(bcap, 1);
-  const size_t block = static_cast<size_t>(2 * nmod) * g.bcap * Kp * 2;
-  CHASE_TRY(d.alloc(&g.E, static_cast<size_t>(g.n)));
-  CHASE_TRY(d.alloc(&g.Dg, static_cast<size_t>(g.n)));
-  CHASE_TRY(d.alloc_bytes(&g.Bsl, block));
-  CHASE_TRY(d.alloc_bytes(&g.G, block));
-  return d.alloc(&g.F, static_cast<size_t>(g.bcap));
-}
-}  // namespace
+// Parts of one allocation, each on a 256-byte boundary: an allocation (and its
+// release) per part cost about 5 us a problem on the host.
+struct Parts {
+  unsigned char* base = nullptr;
+  size_t at = 0;
+  void* take(size_t bytes) {
+    void* p = base ? base + at : nullptr;
+    at += (bytes + 255) / 256 * 256;
+    return p;
+  }
+};
 
-int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
-                        int nmod) {
-  auto give_back = [&](int st) {
-    grouped_rns_release(d, in);
-    return st;
-  };
+// Exponents, diagonals and the planes of the blocks of every problem; without a
+// base only their sum is formed.
+void block_parts(std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap, int nmod,
+                 Parts& parts) {
+  for (size_t q = 0; q < in.size(); ++q) {
+    GroupedFilterInput& g = in[q];
+    if (g.n == 0) continue;
+    g.bcap = std::max(bcap[q], 1);
+    const size_t block = static_cast<size_t>(2 * nmod) * g.bcap * rns_k_padded(g.n) * 2;
+    g.E = static_cast<int*>(parts.take(sizeof(int) * g.n));
+    g.Dg = static_cast<double*>(parts.take(sizeof(double) * g.n));
+    g.Bsl = parts.take(block);
+    g.G = parts.take(block);
+    g.F = static_cast<int*>(parts.take(sizeof(int) * g.bcap));
+  }
+}
+void plane_parts(std::vector<GroupedFilterInput>& in, int nmod, Parts& parts) {
+  for (GroupedFilterInput& g : in)
+    if (g.n > 0)
+      g.A = parts.take(static_cast<size_t>(g.sym ? nmod : 2 * nmod) * g.n * rns_k_padded(g.n) * 2);
+}
+
+int prepare_planes(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
+                   int nmod, size_t reserve, GroupedWork& w) {
   std::vector<GroupedSliceH> all;
   std::vector<size_t> owner;
   int rows = 0;
   double entries = 0.0;
+  Parts parts;
+  block_parts(in, bcap, nmod, parts);
+  const size_t block_bytes = parts.at;
   for (size_t q = 0; q < in.size(); ++q) {
     GroupedFilterInput& g = in[q];
     if (g.n == 0) continue;
     entries += static_cast<double>(g.n) * rns_k_padded(g.n);
-    const int st = alloc_block_planes(d, g, bcap[q], nmod);
-    if (st != CHASE_OK) return give_back(st);
     GroupedSliceH sh{};
     sh.H = reinterpret_cast<const double2*>(g.H);
     sh.ldh = g.ldh;
-    sh.E = g.E;
-    sh.Dg = g.Dg;
     sh.Kp = rns_k_padded(g.n);
     sh.n = g.n;
     sh.row0 = rows;
@@ -227,12 +244,28 @@ int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::
   }
   if (all.empty()) return CHASE_OK;
   const int P = static_cast<int>(all.size());
+  CHASE_TRY(d.alloc_bytes(&w.block, block_bytes));
+  parts = Parts{static_cast<unsigned char*>(w.block)};
+  block_parts(in, bcap, nmod, parts);
+  for (int p = 0; p < P; ++p) {
+    all[p].E = in[owner[p]].E;
+    all[p].Dg = in[owner[p]].Dg;
+  }
   // one list on the device per launch: all problems, then those with one
   // scale, then the others
-  GroupedSliceH* dl = nullptr;
-  int* mm = nullptr;
-  CHASE_TRY(d.alloc(&dl, 3 * all.size()));
-  CHASE_TRY(d.alloc(&mm, 2 * all.size()));
+  struct Lists {
+    Dev& d;
+    GroupedSliceH* problems = nullptr;
+    int* minmax = nullptr;
+    ~Lists() {
+      if (problems) d.release(problems);
+      if (minmax) d.release(minmax);
+    }
+  } lists{d};
+  CHASE_TRY(d.alloc(&lists.problems, 3 * all.size()));
+  CHASE_TRY(d.alloc(&lists.minmax, 2 * all.size()));
+  GroupedSliceH* const dl = lists.problems;
+  int* const mm = lists.minmax;
   std::vector<int> hmm(2 * all.size());
   for (int p = 0; p < P; ++p) {
     hmm[2 * p] = std::numeric_limits<int>::max();
@@ -252,19 +285,24 @@ int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::
                                d.st));
     CHASE_TRY(d.sync_check("grouped row scales of H"));
   }
+  for (int p = 0; p < P; ++p)
+    in[owner[p]].sym = rns_same_scale(hmm[2 * p], hmm[2 * p + 1]) ? 1 : 0;
+  parts = Parts{};
+  plane_parts(in, nmod, parts);
+  size_t free_b = 0;
+  CHASE_TRY(d.free_bytes(&free_b));
+  if (parts.at + reserve > free_b) {
+    set_error("residue planes of a batch: %zu bytes do not fit the memory", parts.at);
+    return CHASE_OUT_OF_MEMORY;
+  }
+  CHASE_TRY(d.alloc_bytes(&w.planes, parts.at));
+  parts = Parts{static_cast<unsigned char*>(w.planes)};
+  plane_parts(in, nmod, parts);
   std::vector<GroupedSliceH> one, each;
   int tiles = 0, erows = 0;
   for (int p = 0; p < P; ++p) {
-    GroupedFilterInput& g = in[owner[p]];
+    const GroupedFilterInput& g = in[owner[p]];
     GroupedSliceH sh = all[p];
-    g.sym = rns_same_scale(hmm[2 * p], hmm[2 * p + 1]) ? 1 : 0;
-    const int st = d.alloc_bytes(
-        &g.A, static_cast<size_t>(g.sym ? nmod : 2 * nmod) * g.n * rns_k_padded(g.n) * 2);
-    if (st != CHASE_OK) {
-      d.release(dl);
-      d.release(mm);
-      return give_back(st);
-    }
     sh.A = g.A;
     sh.s = hmm[2 * p];
     if (g.sym) {
@@ -285,10 +323,16 @@ int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::
     CHASE_TRY(upload(dl + 2 * P, each));
     CHASE_TRY(rns_grouped_prepare_h(d, nmod, dl + 2 * P, static_cast<int>(each.size()), erows));
   }
-  d.release(mm);
-  d.release(dl);
   // the host arrays must outlive the copies
   return d.sync_check("grouped residues of H");
+}
+}  // namespace
+
+int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
+                        int nmod, size_t reserve, GroupedWork& w) {
+  const int st = prepare_planes(d, in, bcap, nmod, reserve, w);
+  if (st != CHASE_OK) grouped_rns_release(d, in, w);
+  return st;
 }
 
 namespace {
@@ -571,29 +615,39 @@ void add_times(GroupedFilterTimes& to, const GroupedFilterTimes& t) {
   to.t_product += t.t_product;
 }
 
+// What filter_part allocates for `in` (maps, problems, step lists).
+size_t list_bytes(const std::vector<GroupedFilterInput>& in) {
+  size_t bytes = size_t(1) << 20;
+  for (const GroupedFilterInput& g : in)
+    bytes += 9 * sizeof(CUtensorMap) + sizeof(GroupedProblem) + (g.maxdeg + 1) * 2 * sizeof(GroupedStep);
+  return bytes;
+}
+
 // Residue planes for `in`, made and given back here; halves of the batch in
-// turn where they do not all fit, and FP64 tiles for a problem whose own do not.
+// turn where they do not all fit (filter_part runs out of memory only before it
+// touches a block), and FP64 tiles for a problem whose own do not.
 int filter_parts(Dev& d, std::vector<GroupedFilterInput> in, int nmod, int tile,
                  GroupedFilterTimes& times) {
   std::vector<int> bcap;
   for (const GroupedFilterInput& g : in) bcap.push_back(g.b);
   GroupedFilterTimes t;
-  int st = grouped_rns_prepare(d, in, bcap, nmod);
+  GroupedWork w;
+  int st = grouped_rns_prepare(d, in, bcap, nmod, list_bytes(in), w);
   if (st == CHASE_OK) {
     st = filter_part(d, in, nmod, tile, &t);
-    grouped_rns_release(d, in);
-    add_times(times, t);
-    return st;
+    grouped_rns_release(d, in, w);
   }
-  if (st != CHASE_OUT_OF_MEMORY) return st;
-  if (in.size() > 1) {
-    const auto mid = in.begin() + static_cast<std::ptrdiff_t>(in.size() / 2);
-    CHASE_TRY(filter_parts(d, std::vector<GroupedFilterInput>(in.begin(), mid), nmod, tile, times));
-    return filter_parts(d, std::vector<GroupedFilterInput>(mid, in.end()), nmod, tile, times);
+  if (st == CHASE_OUT_OF_MEMORY) {
+    if (in.size() > 1) {
+      const auto mid = in.begin() + static_cast<std::ptrdiff_t>(in.size() / 2);
+      CHASE_TRY(filter_parts(d, std::vector<GroupedFilterInput>(in.begin(), mid), nmod, tile, times));
+      return filter_parts(d, std::vector<GroupedFilterInput>(mid, in.end()), nmod, tile, times);
+    }
+    t = GroupedFilterTimes{};
+    st = filter_part(d, in, 0, CHASE_TILE_AUTO, &t);
   }
-  CHASE_TRY(filter_part(d, in, 0, CHASE_TILE_AUTO, &t));
-  add_times(times, t);
-  return CHASE_OK;
+  if (st == CHASE_OK) add_times(times, t);
+  return st;
 }
 }  // namespace
 

@@ -2076,10 +2076,19 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
     planes[p].b = bcap[p] = sv[p].nx;
   }
   const int nmod = grouped_moduli(planes, split, CHASE_TILE_AUTO);
+  GroupedWork work;
+  bool resident = false;
   if (nmod > 0) {
-    const int st = grouped_rns_prepare(d, planes, bcap, nmod);
+    // beside what the iterations allocate: step lists, row panels, the batched
+    // eigensolver's copies and workspace
+    size_t reserve = size_t(64) << 20;
+    for (int p = 0; p < P; ++p)
+      reserve += 16 * static_cast<size_t>(bcap[p]) * (4096 + 16 * static_cast<size_t>(bcap[p])) +
+                 2 * sizeof(GroupedStep) * (o.deg_max + 1);
+    const int st = grouped_rns_prepare(d, planes, bcap, nmod, reserve, work);
     if (st != CHASE_OK && st != CHASE_OUT_OF_MEMORY) return st;
-    for (int p = 0; p < P && st == CHASE_OK; ++p) {
+    resident = st == CHASE_OK;
+    for (int p = 0; p < P && resident; ++p) {
       Solver<chase_c64>& s = sv[p];
       RnsH& h = s.h64;
       h.A = planes[p].A;
@@ -2122,7 +2131,18 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
       in.push_back(g);
     }
     GroupedFilterTimes tt;
-    CHASE_TRY(grouped_filter_sorted(d, in, nmod, CHASE_TILE_AUTO, &tt));  // line 4, grouped
+    int st = grouped_filter_sorted(d, in, nmod, CHASE_TILE_AUTO, &tt);  // line 4, grouped
+    if (st == CHASE_OUT_OF_MEMORY && resident) {  // without planes that stay
+      resident = false;
+      grouped_rns_release(d, planes, work);
+      for (int p = 0; p < P; ++p) sv[p].rr_ready = false;
+      for (GroupedFilterInput& g : in) {
+        g.A = nullptr;
+        g.bcap = 0;
+      }
+      st = grouped_filter_sorted(d, in, nmod, CHASE_TILE_AUTO, &tt);
+    }
+    CHASE_TRY(st);
     bs.steps += tt.steps;
     bs.tile_config = tt.tile_config;
     bs.matvecs += tt.matvecs;

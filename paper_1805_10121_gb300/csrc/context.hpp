@@ -369,17 +369,21 @@ struct GroupedFilterTimes {
 // FP64's; 0 where a batch this small stays on the FP64 tiles.
 int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile);
 // Residue planes of every problem's H and the workspace for bcap[q] columns
-// (one grouped slicing launch); fills the residue fields of `in`.
-// CHASE_OUT_OF_MEMORY leaves nothing behind.
+// (one grouped slicing launch), which leave `reserve` bytes free; fills the
+// residue fields of `in`.  A status other than CHASE_OK leaves nothing behind.
+struct GroupedWork {  // of all problems: their planes of H, and the rest
+  void *block = nullptr, *planes = nullptr;
+};
 int grouped_rns_prepare(Dev& d, std::vector<GroupedFilterInput>& in, const std::vector<int>& bcap,
-                        int nmod);
-void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in);
+                        int nmod, size_t reserve, GroupedWork& w);
+void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in, GroupedWork& w);
 // Alg. 4 on every problem of `in` (problems with b == 0 are skipped), one
 // grouped launch per degree step and part, all steps in one CUDA graph.
 // nmod: residue products with that many moduli (prepared inputs are used as
 // they are; others are prepared here, a part of the batch at a time where the
 // memory does not hold all), 0: FP64 tiles of shape `tile` or, with
-// CHASE_TILE_AUTO, the fastest.  Synchronises the stream.
+// CHASE_TILE_AUTO, the fastest.  Synchronises the stream.  With prepared inputs
+// CHASE_OUT_OF_MEMORY leaves every block as it was.
 int grouped_filter_sorted(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int tile,
                           GroupedFilterTimes* times);
 

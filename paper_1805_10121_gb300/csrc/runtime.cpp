@@ -255,10 +255,11 @@ int Dev::alloc_bytes(void** p, size_t bytes) {
 }
 
 void Dev::release(void* p) {
-  for (auto it = bufs.begin(); it != bufs.end(); ++it)
+  for (auto it = bufs.rbegin(); it != bufs.rend(); ++it)  // mostly one of the last
     if (it->p == p) {
       held -= it->bytes;
-      bufs.erase(it);
+      *it = bufs.back();
+      bufs.pop_back();
       cudaFreeAsync(p, st);
       return;
     }

@@ -146,3 +146,44 @@ def test_single_precision_solve(mb):
         st, ritz, _, _ = chase.chase_solve_c32(h, nev, nex, 1e-5, v, s)
     assert st == chase.CHASE_OK
     assert np.max(np.abs(ritz[:nev] - lam.cpu().numpy()[:nev])) <= 1e-5 * float(lam.abs().max())
+
+
+SHAPES = [(500, 30), (300, 20), (257, 9), (300, 40), (129, 12), (400, 24)]
+
+
+# H of the batch: 13 MB; its planes 27 to 53 MB, of the blocks 9 MB
+@pytest.mark.parametrize("split", [False, True])
+def test_batched_filter(split):
+    m = 6
+    hs = [hermitian(n, 20 + i, False) for i, (n, b) in enumerate(SHAPES)]
+    vs = [gauss(n, b, 30 + i, False) for i, (n, b) in enumerate(SHAPES)]
+    refs = [reference(h, v, m, 1.6, -1.5, -0.9) for h, v in zip(hs, vs)]
+    ways = set()
+    for mb in (4, 6, 12, 24, 48, 0):
+        got = [v.clone() for v in vs]
+        with limit(mb * MB):
+            st = chase.chase_filter_batched(hs, got, [np.full(b, m, dtype=np.int32) for _, b in SHAPES],
+                                            [1.6] * 6, [-1.5] * 6, [-0.9] * 6,
+                                            precision=chase.CHASE_SPLIT_BF16 if split else chase.CHASE_FP64)
+        ways.add((st["launches"], st["tile_config"] < 0))
+        assert st["matvecs"] == m * sum(b for _, b in SHAPES)
+        for (n, b), v, ref in zip(SHAPES, got, refs):
+            assert err(v, ref) <= bar(n, m, "c128", split)
+    assert len({k for k, rns in ways if rns}) > 1  # the batch at once, and in parts
+    assert not all(rns for _, rns in ways)  # and FP64 tiles for what does not fit alone
+
+
+@pytest.mark.parametrize("precision", [chase.CHASE_FP64, chase.CHASE_SPLIT_BF16, chase.CHASE_SPLIT_BF16_RR])
+@pytest.mark.parametrize("mb", [48, 160, 0])
+def test_batched_solve(precision, mb):
+    shapes = [(500, 20, 10), (300, 12, 6), (400, 16, 8)]
+    lam = [synth.spectrum_uniform(n, 40 + n, device=DEV) for n, _, _ in shapes]
+    hs = [synth.hermitian_dft(x, 41) for x in lam]
+    vs = [synth.gaussian_block(n, nev + nex, 42, device=DEV) for n, nev, nex in shapes]
+    ss = [synth.gaussian_block(n, 5, 43, device=DEV) for n, _, _ in shapes]
+    with limit(mb * MB):
+        out = chase.chase_solve_batched(hs, [s[1] for s in shapes], [s[2] for s in shapes], [1e-10] * 3, vs, ss,
+                                        opts=chase.chase_opts_default(precision=precision))
+    assert out[0] == chase.CHASE_OK
+    for x, ritz, (n, nev, nex) in zip(lam, out[2], shapes):
+        assert np.max(np.abs(ritz[:nev] - x.cpu().numpy()[:nev])) <= 1e-10 * float(x.abs().max())
