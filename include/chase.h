@@ -68,7 +68,8 @@ typedef struct {
  * rounded to 2^-60 of the 2-norm of a row of H or a column of the block, put
  * together and finished in FP64: no further from the exact product than an
  * FP64 GEMM); smaller ones on the FP64 pipes.  The batched entry points do the
- * same for batches of 2e7 FLOPs and more per degree step. */
+ * same for batches of 2e7 FLOPs and more per degree step, unless they are of so
+ * many small problems that the FP64 pipe is done sooner. */
 #define CHASE_FP64 0
 /* Split: the same residue products with the operands rounded to 2^-48 of
  * those norms.  The diagonal of H and the recurrence's shift/scale/axpby are
@@ -151,8 +152,9 @@ typedef struct {
 } chase_stats;
 
 /* Tile choice of the grouped FP64 filter: residue products for batches of 2e7
- * FLOPs and more per degree step, below that the candidates timed on the first
- * degree step (result cached per batch shape); or 0..3 for a fixed shape
+ * FLOPs and more per degree step where the FP64 pipe is not sooner done (many
+ * small problems), else the candidates timed on the first degree step (result
+ * cached per batch shape); or 0..3 for a fixed shape
  * (0: 64 x 16, 1: 64 x 32, 2: 128 x 16, 3: 64 x 8 rows x complex columns). */
 #define CHASE_TILE_AUTO (-1)
 
@@ -162,7 +164,7 @@ typedef struct {
   int steps;               /* degree steps (the largest degree of the batch; summed over
                               the iterations of chase_solve_batched) */
   int tile_config;         /* FP64 tile shape used (see CHASE_TILE_AUTO); -1 for residue
-                              products (split, and FP64 batches of some size) */
+                              products (split and FP64 batches of some size) */
   int launches;            /* kernel launches of the call (graph nodes counted once) */
   long long matvecs;       /* column products with H over all problems (sum of the degrees) */
   double flops;            /* 8 N^2 per column product, summed over problems */

@@ -159,8 +159,37 @@ float elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
 
 }  // namespace
 
-// Residue products from 2e7 FLOPs a degree step on: below that the FP64 tiles
-// take less time than the three launches (about 20 us).
+namespace {
+// Estimates of one degree step in microseconds, where all columns are active.
+// FP64 tiles of 64 x 8: the longest tile, or what the SMs get through (32
+// problems of N = 256, 19 columns: 368 us; 300 of N = 64, 8: 73; 2000 of N = 16,
+// 8: 134).  Residue products of small problems: three launches and 1.27 us a
+// tile and pair (8 of N = 256: 31; 300 of N = 64: 160 with 14 moduli, 134 with
+// 11; 2000 of N = 16: 947 and 777); larger tiles take longer, but there the FP64
+// tiles are far behind.
+double fp64_step_us(const std::vector<GroupedFilterInput>& in) {
+  double longest = 0.0, sum = 0.0;
+  for (const GroupedFilterInput& g : in) {
+    if (g.n == 0 || g.b == 0) continue;
+    longest = std::max(longest, 8.0 + 0.5 * g.n);
+    sum += ((g.n + 63) / 64) * ((g.b + 7) / 8) * static_cast<double>(g.n) / 260.0;
+  }
+  return std::max(longest, sum);
+}
+double residue_step_us(const std::vector<GroupedFilterInput>& in, int nmod) {
+  double tiles = 0.0;
+  for (const GroupedFilterInput& g : in)
+    if (g.n > 0 && g.b > 0)
+      tiles += rns_grouped_tiles(nmod, std::min(256, (g.b + 31) / 32 * 32), g.n, g.b);
+  return 25.0 + 1.27 * tiles / 76.0;
+}
+}  // namespace
+
+// Residue products, for an FP64 batch from 2e7 FLOPs a degree step on, unless
+// the FP64 tiles are done sooner: many problems of few rows each fill the device
+// with FP64 tiles, where each of their residue planes pads a tile of 256 rows.
+// 2000 problems of N = 16, ten steps in all: 11.2 ms on the FP64 tiles, 20.4 and
+// 18.8 ms as residues (14 and 11 moduli); 200 of N = 100: 3.0, 2.8 and 2.5 ms.
 int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile) {
   int64_t most = 0;
   double step = 0.0;
@@ -168,8 +197,9 @@ int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int ti
     most = std::max<int64_t>(most, g.n);
     step += 8.0 * g.n * static_cast<double>(g.n) * g.b;
   }
-  if (split) return rns_split_moduli(most);
-  return tile == CHASE_TILE_AUTO && step >= 2e7 ? kRnsFp64 : 0;
+  const int nmod = split ? rns_split_moduli(most) : kRnsFp64;
+  if (!split && (tile != CHASE_TILE_AUTO || step < 2e7)) return 0;
+  return residue_step_us(in, nmod) < fp64_step_us(in) ? nmod : 0;
 }
 
 void grouped_rns_release(Dev& d, std::vector<GroupedFilterInput>& in, GroupedWork& w) {
@@ -519,6 +549,12 @@ int filter_part(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int
   CHASE_CUDA(cudaMemcpyAsync(dsteps, all.data(), sizeof(GroupedStep) * all.size(),
                              cudaMemcpyHostToDevice, d.st));
 
+  // Small problems: a pair takes tiles that follow one another, mostly planes of
+  // one problem, whose description it then finds in L1 and whose tensor maps it
+  // acquires once (200 problems of N = 100: 134 -> 99 us a step).  Larger ones
+  // differ in length and share H's rows, so the pairs take turns.
+  const bool in_row = in[co[0].q].n <= 256;
+
   // ---- the degree steps, captured into one graph ----
   CHASE_TRY(rns ? rns_grouped_ready() : zgemm_grouped_fp64_prepare(cfg));
   const double tg = now_s();
@@ -561,7 +597,7 @@ int filter_part(Dev& d, const std::vector<GroupedFilterInput>& in, int nmod, int
       if (cudaEventRecordWithFlags(pev[k], gg.cs, cudaEventRecordExternal) != cudaSuccess)
         st = CHASE_CUDA_ERROR;
       if (st == CHASE_OK)
-        st = rns ? rns_grouped_gemm(d, nmod, width[i], dprobs, sp, tot[i].tiles)
+        st = rns ? rns_grouped_gemm(d, nmod, width[i], dprobs, sp, nact[i], tot[i].tiles, in_row)
                  : zgemm_grouped_fp64(d, cfg, dprobs, sp, nact[i], tot[i].tiles, parity);
       if (st == CHASE_OK &&
           cudaEventRecordWithFlags(pev[k + 1], gg.cs, cudaEventRecordExternal) != cudaSuccess)
@@ -803,7 +839,7 @@ extern "C" int chase_filter_batched(int P, const chase_c64* const* H, const int6
                              cudaMemcpyHostToDevice, d.st));
   CHASE_TRY(launch_grouped_permute(d, dgather, Q, total_cols, false));
   GroupedFilterTimes tt;
-  CHASE_TRY(grouped_filter_sorted(d, in, grouped_moduli(in, split, tile), tile, &tt));
+  CHASE_TRY(grouped_filter_sorted(d, in, grouped_moduli(in, split, tile), split ? CHASE_TILE_AUTO : tile, &tt));
   // every result is in the sorted copy (even degrees): back to the caller's order
   CHASE_TRY(launch_grouped_permute(d, dscatter, Q, total_cols, true));
   CHASE_TRY(d.sync_check("chase_filter_batched"));

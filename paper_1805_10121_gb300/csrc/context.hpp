@@ -331,8 +331,9 @@ double rns_stage_cost(int bn);
 int rns_grouped_ready();  // kernel attributes, set outside any stream capture
 int rns_grouped_slice_x(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
                         int nact, int ncols, int parity);
+// in_row: each pair takes tiles that follow one another, else they take turns
 int rns_grouped_gemm(Dev& d, int nmod, int bn, const GroupedProblem* probs,
-                     const GroupedStep* steps, int ntiles);
+                     const GroupedStep* steps, int nact, int ntiles, bool in_row);
 int rns_grouped_crt(Dev& d, int nmod, const GroupedProblem* probs, const GroupedStep* steps,
                     int nact, int nblocks, int parity);
 // One problem of a grouped filter: the block X (b columns, sorted by
@@ -366,7 +367,7 @@ struct GroupedFilterTimes {
   double flops = 0, t_autotune = 0, t_graph_build = 0, t_steps = 0, t_product = 0;
 };
 // Moduli of a batch's residue products: of the split filter's accuracy, or
-// FP64's; 0 where a batch this small stays on the FP64 tiles.
+// FP64's; 0 where the FP64 tiles take less time.
 int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile);
 // Residue planes of every problem's H and the workspace for bcap[q] columns
 // (one grouped slicing launch), which leave `reserve` bytes free; fills the

@@ -251,8 +251,12 @@ struct Tile {
   long long ldg;
 };
 
+// The pair's tiles: first, first + step, ... below last.
+struct Walk {
+  int first, last, step;
+};
 template <int BN, class TileFn>
-__device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTab& tab,
+__device__ __forceinline__ void gemm_body(TileFn& tile, const Walk w, const GemmTab& tab,
                                           int maps_in_global, int* __restrict__ err) {
   using C = Cfg<BN>;
   constexpr int NSTAGE = C::NSTAGE;
@@ -270,7 +274,6 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
-  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NSTAGE; ++s) {
@@ -315,7 +318,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
       uint32_t ph = 1;
       bool ok = true;
       const CUtensorMap* last = nullptr;
-      for (int t = pair; t < ntiles && ok; t += npairs) {
+      for (int t = w.first; t < w.last && ok; t += w.step) {
         Tile T;
         tile(t, T);
         if (T.mapA != last) {
@@ -376,7 +379,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
       bool ok = true;
       int st = 0, buf = 0;               // stage, accumulator
       uint32_t ph = 0, acc_ph = 1;
-      for (int t = pair; t < ntiles && ok; t += npairs) {
+      for (int t = w.first; t < w.last && ok; t += w.step) {
         Tile T;
         tile(t, T);
         const int cs = tab.m[T.modulus].chunk;
@@ -433,7 +436,7 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, int ntiles, const GemmTa
     const uint32_t bar_e0 = map_to_rank(&acc_empty[0], 0), bar_e1 = map_to_rank(&acc_empty[1], 0);
     unsigned c = 0;  // chunk: accumulator c & 1, its phase c >> 1
     bool ok = true;
-    for (int t = pair; t < ntiles && ok; t += npairs) {
+    for (int t = w.first; t < w.last && ok; t += w.step) {
       Tile T;
       tile(t, T);
       const Modulus m = tab.m[T.modulus];
@@ -544,7 +547,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                     long long ldg, long long gplane, int* __restrict__ err) {
   OneProduct<TRI> p{&tmA, &tmB, rtiles, ctiles, plane0, per_modulus, swap_a, sym, BN, nst, M, ncols,
                G, ldg, gplane};
-  gemm_body<BN>(p, rtiles * ctiles * nplanes, tab, 0, err);
+  gemm_body<BN>(p, Walk{static_cast<int>(blockIdx.x >> 1), rtiles * ctiles * nplanes,
+                        static_cast<int>(gridDim.x >> 1)},
+                tab, 0, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -1543,8 +1548,10 @@ struct GroupedTiles {
   static constexpr bool kTri = false;
   const GroupedProblem* probs;
   const GroupedStep* steps;
-  int bn, at;  // at: entry of the last tile (each thread walks forward)
+  int bn, nact, at;  // at: entry of the last tile
   __device__ __forceinline__ void operator()(int t, Tile& T) {
+    // the first tile's entry by binary search, then a walk forward
+    if (at < 0) at = find_entry(steps, nact, &GroupedStep::tile0, t);
     while (steps[at + 1].tile0 <= t) ++at;
     const GroupedStep& st = steps[at];
     const GroupedProblem& q = probs[st.prob];
@@ -1571,13 +1578,19 @@ struct GroupedTiles {
 template <int BN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     rns_grouped_gemm_kernel(const GroupedProblem* __restrict__ probs,
-                            const GroupedStep* __restrict__ steps, int ntiles,
+                            const GroupedStep* __restrict__ steps, int nact, int ntiles, int in_row,
                             const __grid_constant__ GemmTab tab, int* __restrict__ err) {
-  GroupedTiles g{probs, steps, BN, 0};
-  gemm_body<BN>(g, ntiles, tab, 1, err);
+  GroupedTiles g{probs, steps, BN, nact, -1};
+  const int pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int per = (ntiles + npairs - 1) / npairs;
+  const Walk w = in_row ? Walk{min(pair * per, ntiles), min((pair + 1) * per, ntiles), 1}
+                        : Walk{pair, ntiles, npairs};
+  gemm_body<BN>(g, w, tab, 1, err);
 }
 
-constexpr int kCrtCols = 4;  // columns per block of the grouped reconstruction
+// Columns per block of the grouped reconstruction: a block of a small problem has
+// few rows, and one column after the other only lengthens its chain.
+__host__ __device__ constexpr int crt_cols(int n) { return n <= 256 ? 1 : 4; }
 
 template <int NM>
 __global__ void __launch_bounds__(128)
@@ -1587,9 +1600,10 @@ __global__ void __launch_bounds__(128)
   const GroupedStep& st = steps[find_entry(steps, nact, &GroupedStep::blk0, blockIdx.x)];
   const GroupedProblem& q = probs[st.prob];
   const int rchunks = (q.n + 255) / 256, u = blockIdx.x - st.blk0;
-  const int r0 = 2 * (u % rchunks * 128 + threadIdx.x), c0 = u / rchunks * kCrtCols;
+  const int cols = crt_cols(q.n);
+  const int r0 = 2 * (u % rchunks * 128 + threadIdx.x), c0 = u / rchunks * cols;
   if (r0 >= q.n) return;
-  crt_rows<NM, double2>(r0, c0, min(c0 + kCrtCols, q.b - st.s), 1, static_cast<int16_t*>(q.G), q.Kp,
+  crt_rows<NM, double2>(r0, c0, min(c0 + cols, q.b - st.s), 1, static_cast<int16_t*>(q.G), q.Kp,
                         static_cast<long long>(q.bcap) * q.Kp, tab, q.E, q.F, q.Dg, q.n, st.s,
                         parity ? q.buf1 : q.buf0, parity ? q.ld1 : q.ld0,
                         parity ? q.buf0 : q.buf1, parity ? q.ld0 : q.ld1, st.sc);
@@ -2063,15 +2077,15 @@ int grouped_pairs() {
   return v;
 }
 template <int BN>
-int launch_grouped_gemm(Dev& d, const GroupedProblem* probs, const GroupedStep* steps, int ntiles,
-                        const GemmTab& tab) {
+int launch_grouped_gemm(Dev& d, const GroupedProblem* probs, const GroupedStep* steps, int nact,
+                        int ntiles, bool in_row, const GemmTab& tab) {
   const int pairs = grouped_pairs<BN>();
   if (pairs < 1) {
     set_error("residue GEMM: no CTA pair fits this device");
     return CHASE_CUDA_ERROR;
   }
   rns_grouped_gemm_kernel<BN><<<2 * std::min(ntiles, pairs), kThreads, Cfg<BN>::SMEM, d.st>>>(
-      probs, steps, ntiles, tab, d.err);
+      probs, steps, nact, ntiles, in_row ? 1 : 0, tab, d.err);
   note_launch();
   CHASE_CUDA(cudaGetLastError());
   return CHASE_OK;
@@ -2337,7 +2351,7 @@ int rns_grouped_tiles(int nmod, int bn, int n, int cols) {
   return (n + 2 * rns::BM - 1) / (2 * rns::BM) * ((cols + bn - 1) / bn) * 2 * nmod;
 }
 int rns_grouped_crt_blocks(int n, int cols) {
-  return (n + 255) / 256 * ((cols + rns::kCrtCols - 1) / rns::kCrtCols);
+  return (n + 255) / 256 * ((cols + rns::crt_cols(n) - 1) / rns::crt_cols(n));
 }
 double rns_stage_cost(int bn) { return rns::stage_cost(bn); }
 
@@ -2354,17 +2368,17 @@ int rns_grouped_slice_x(Dev& d, int nmod, const GroupedProblem* probs, const Gro
   });
 }
 int rns_grouped_gemm(Dev& d, int nmod, int bn, const GroupedProblem* probs,
-                     const GroupedStep* steps, int ntiles) {
+                     const GroupedStep* steps, int nact, int ntiles, bool in_row) {
   const rns::GemmTab& tab = rns::tables(nmod, true).gemm;
   switch (bn) {
-    case 32: return rns::launch_grouped_gemm<32>(d, probs, steps, ntiles, tab);
-    case 64: return rns::launch_grouped_gemm<64>(d, probs, steps, ntiles, tab);
-    case 96: return rns::launch_grouped_gemm<96>(d, probs, steps, ntiles, tab);
-    case 128: return rns::launch_grouped_gemm<128>(d, probs, steps, ntiles, tab);
-    case 160: return rns::launch_grouped_gemm<160>(d, probs, steps, ntiles, tab);
-    case 192: return rns::launch_grouped_gemm<192>(d, probs, steps, ntiles, tab);
-    case 224: return rns::launch_grouped_gemm<224>(d, probs, steps, ntiles, tab);
-    default: return rns::launch_grouped_gemm<256>(d, probs, steps, ntiles, tab);
+    case 32: return rns::launch_grouped_gemm<32>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 64: return rns::launch_grouped_gemm<64>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 96: return rns::launch_grouped_gemm<96>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 128: return rns::launch_grouped_gemm<128>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 160: return rns::launch_grouped_gemm<160>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 192: return rns::launch_grouped_gemm<192>(d, probs, steps, nact, ntiles, in_row, tab);
+    case 224: return rns::launch_grouped_gemm<224>(d, probs, steps, nact, ntiles, in_row, tab);
+    default: return rns::launch_grouped_gemm<256>(d, probs, steps, nact, ntiles, in_row, tab);
   }
 }
 int rns_grouped_ready() {

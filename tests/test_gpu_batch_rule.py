@@ -1,0 +1,43 @@
+"""Batches on both sides of the rule that chooses between residue products and
+FP64 tiles (many problems of few rows take the FP64 tiles, in either precision),
+and products whose tiles each pair of blocks takes one after the other (all
+problems up to N = 256) or in turn, with one large problem among small ones.
+
+Tolerance: as in test_gpu_scales.py."""
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1805_10121_gb300 import chase
+from tests.test_gpu_rns import gauss, hermitian, reference
+from tests.test_gpu_scales import bar, err
+
+pytestmark = pytest.mark.gpu
+
+TINY = [(16, 4)] * 60 + [(40, 9)] * 200
+SMALL = [(256, 19), (129, 7), (200, 33), (64, 5), (255, 1), (130, 40)] * 3
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    from paper_1805_10121_gb300 import build
+    build.build()
+    chase.lib()
+
+
+@pytest.mark.parametrize("shapes,rns", [(TINY, False), (SMALL, True), (SMALL + [(257, 12)], True),
+                                        (TINY + [(700, 40)], True)])
+@pytest.mark.parametrize("split", [False, True])
+def test_batch(shapes, rns, split):
+    hs = [hermitian(n, i, False) for i, (n, b) in enumerate(shapes)]
+    vs = [gauss(n, b, 100 + i, False).clone() for i, (n, b) in enumerate(shapes)]
+    # degrees that retire columns, so that later steps hold fewer tiles
+    degs = [2 * (1 + np.arange(b, dtype=np.int32) % 3) for n, b in shapes]
+    refs = [[reference(h, v, m, 1.6, -1.5, -0.9) for m in (2, 4, 6)] for h, v in zip(hs, vs)]
+    st = chase.chase_filter_batched(hs, vs, degs, [1.6] * len(hs), [-1.5] * len(hs), [-0.9] * len(hs),
+                                    precision=chase.CHASE_SPLIT_BF16 if split else chase.CHASE_FP64)
+    assert (st["tile_config"] < 0) == rns
+    for (n, b), v, ref in zip(shapes, vs, refs):
+        for k in range(min(3, b)):
+            assert err(v[:, k::3], ref[k][:, k::3]) <= bar(max(n, 64), 2 * (k + 1), split)
