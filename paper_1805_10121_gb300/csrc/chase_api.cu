@@ -1828,9 +1828,11 @@ namespace {
 // (locking, degrees and the reordering).
 // Problem i's launches go to stream fan[i % fan.size()] (the small kernels
 // of different problems then run side by side); the batch's stream d.st
-// forks to and joins the fan around each phase.
+// forks to and joins the fan around each phase; arenas[k] serves the products
+// on stream fan[k].
 int batched_after_filter(Dev& d, std::vector<Solver<chase_c64>*>& act,
-                         const std::vector<cudaStream_t>& fan, double* t) {
+                         const std::vector<cudaStream_t>& fan, std::vector<Arena>& arenas,
+                         double* t) {
   using T = chase_c64;
   const int P = static_cast<int>(act.size());
   if (P == 0) return CHASE_OK;
@@ -1864,6 +1866,7 @@ int batched_after_filter(Dev& d, std::vector<Solver<chase_c64>*>& act,
     view[i]->err = flags + i;
     view[i]->own_err = false;
     view[i]->sync_on_exit = false;
+    if (!arenas.empty()) view[i]->arena = &arenas[i % arenas.size()];
   }
   std::vector<int> hf(P);
   auto read_flags = [&](const char* where) -> int {
@@ -2065,6 +2068,28 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
                    });
   // Alg. 1 lines 1-2 of every problem
   CHASE_TRY(pool.run(all, [&](Dev& w, int p) { return sv[p].setup(w, true); }));
+  // An arena per stream for the tall products of QR and Rayleigh-Ritz, as large
+  // as the largest problem's: about 40 allocations a problem and iteration took
+  // most of both phases (64 problems of N = 200, in all 198 ms, with arenas 94;
+  // 32 of N = 1000 255 and 196 ms).
+  std::vector<Arena> arenas;
+  {
+    size_t most = 0;
+    for (const Solver<chase_c64>& s : sv) {
+      const size_t n = rns_k_padded(s.N), w = rns_k_padded(s.nx);
+      // 28 planes of two operands and of the product, and their exponents
+      most = std::max(most, 56 * (2 * n * w + std::max(n * w, w * w)) + 16 * (n + w) + 4096);
+    }
+    size_t free_b = 0;
+    CHASE_TRY(d.free_bytes(&free_b));
+    void* p = nullptr;
+    if (most * fan.s.size() <= free_b / 4 && d.alloc_bytes(&p, most * fan.s.size()) == CHASE_OK)
+      for (size_t k = 0; k < fan.s.size(); ++k) {
+        arenas.emplace_back();
+        arenas[k].base = static_cast<unsigned char*>(p) + k * most;
+        arenas[k].size = most;
+      }
+  }
   // residue planes of every H, made once where the memory holds them all
   // (otherwise the filter makes them for parts of the batch in turn)
   std::vector<GroupedFilterInput> planes(P);
@@ -2162,7 +2187,7 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
     std::vector<Solver<chase_c64>*> ap;
     for (int p : act) ap.push_back(&sv[p]);
     double tph[4] = {0.0, 0.0, 0.0, 0.0};
-    CHASE_TRY(batched_after_filter(d, ap, fan.s, tph));
+    CHASE_TRY(batched_after_filter(d, ap, fan.s, arenas, tph));
     bs.t_qr += tph[0];
     bs.t_rr += tph[1];
     bs.t_eigh += tph[2];

@@ -10,6 +10,14 @@
 
 namespace chase {
 
+// A block of workspace for the buffers of one product after the other on one
+// stream: taken in turn, and all of it free again once each has been released.
+struct Arena {
+  unsigned char* base = nullptr;
+  size_t size = 0, at = 0;
+  int live = 0;
+};
+
 // Device context of one ABI call: the stream, a device error flag and the
 // stream-ordered workspace allocations, released when the context ends.
 struct Dev {
@@ -22,6 +30,7 @@ struct Dev {
   std::vector<Block> bufs;
   size_t held = 0;   // bytes of bufs
   size_t limit;      // chase_workspace_limit of the thread that made the context
+  Arena* arena = nullptr;  // where allocations come from while they fit; borrowed
   // A view on another context's stream with a flag slot of its own (the
   // per-problem flags of a batch): err is borrowed, and leaving the view
   // does not synchronise (its workspace is released stream-ordered).

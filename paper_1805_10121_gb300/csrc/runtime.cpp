@@ -237,6 +237,13 @@ int Dev::init() {
 int Dev::alloc_bytes(void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) return CHASE_OK;
+  const size_t rounded = (bytes + 255) / 256 * 256;
+  if (arena && rounded <= arena->size - arena->at) {
+    *p = arena->base + arena->at;
+    arena->at += rounded;
+    ++arena->live;
+    return CHASE_OK;
+  }
   if (held > limit || bytes > limit - held) {
     set_error("device workspace allocation of %zu bytes is beyond the workspace limit", bytes);
     return CHASE_OUT_OF_MEMORY;
@@ -255,6 +262,10 @@ int Dev::alloc_bytes(void** p, size_t bytes) {
 }
 
 void Dev::release(void* p) {
+  if (arena && p >= arena->base && p < arena->base + arena->size) {
+    if (--arena->live == 0) arena->at = 0;
+    return;
+  }
   for (auto it = bufs.rbegin(); it != bufs.rend(); ++it)  // mostly one of the last
     if (it->p == p) {
       held -= it->bytes;

@@ -9,7 +9,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_1805_10121_gb300 import chase
+from paper_1805_10121_gb300 import chase, synth
 from tests.test_gpu_rns import gauss, hermitian, reference
 from tests.test_gpu_scales import bar, err
 
@@ -41,3 +41,22 @@ def test_batch(shapes, rns, split):
     for (n, b), v, ref in zip(shapes, vs, refs):
         for k in range(min(3, b)):
             assert err(v[:, k::3], ref[k][:, k::3]) <= bar(max(n, 64), 2 * (k + 1), split)
+
+
+@pytest.mark.parametrize("precision", [chase.CHASE_FP64, chase.CHASE_SPLIT_BF16])
+def test_solve_with_more_problems_than_streams(precision):
+    # problems of different sizes follow one another on each stream
+    shapes = [(130 + 37 * ((7 * i) % 20), 6 + i % 9, 3 + i % 4) for i in range(36)]
+    lam = [synth.spectrum_uniform(n, 50 + i, device="cuda") for i, (n, _, _) in enumerate(shapes)]
+    hs = [synth.hermitian_dft(x, 51 + i) for i, x in enumerate(lam)]
+    vs = [synth.gaussian_block(n, a + x, 52 + i, device="cuda") for i, (n, a, x) in enumerate(shapes)]
+    ss = [synth.gaussian_block(n, 5, 53 + i, device="cuda") for i, (n, _, _) in enumerate(shapes)]
+    out = chase.chase_solve_batched(hs, [s[1] for s in shapes], [s[2] for s in shapes], 1e-10, vs, ss,
+                                    opts=chase.chase_opts_default(precision=precision))
+    assert out[0] == chase.CHASE_OK
+    for h, v, x, ritz, (n, nev, nex) in zip(hs, vs, lam, out[2], shapes):
+        top = float(x.abs().max())
+        assert np.max(np.abs(ritz[:nev] - x.cpu().numpy()[:nev])) <= 1e-10 * top
+        y = v[:, :nev]
+        r = torch.linalg.norm(h @ y - y * torch.from_numpy(ritz[:nev]).to(y.device), dim=0)
+        assert float(r.max()) <= 1.05e-10 * top
