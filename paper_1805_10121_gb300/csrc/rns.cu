@@ -1143,6 +1143,7 @@ struct CrtRows {
   int er[2];
   double dh[2], dl[2];  // plain: alpha (H_rr - shift), else H_rr - shift (as two doubles)
   bool diag[2];
+  bool f32[2];          // single precision: df is in FP32's range
 };
 __device__ __forceinline__ void crt_constants(CrtRows& k, int r0, int M, const int* __restrict__ Ex,
                                               const double* __restrict__ Dg, const RnsScale& sc) {
@@ -1164,7 +1165,10 @@ __device__ __forceinline__ void crt_constants(CrtRows& k, int r0, int M, const i
     k.dl[h] = l;
     k.df[h] = static_cast<float>(d);
     k.dfl[h] = static_cast<float>(d - k.df[h]);
-    k.dl32[h] = static_cast<float>(l);
+    // beyond 2^100 the low part, or its product, may leave FP32's range; left out
+    // there, the constant is the rounded one
+    k.f32[h] = abs_hi(d) < ((1023u + 100u) << 20);
+    k.dl32[h] = k.f32[h] ? static_cast<float>(l) : 0.f;
   }
 }
 
@@ -1242,7 +1246,7 @@ __device__ __forceinline__ void crt_pair(const CrtRows& k, int r0, int c,
       // results are stored in FP32: each constant as two floats, so what the
       // steps share is not rounded to one, and one FP32 FMA per term
       const int x0 = ((__float_as_int(sc.apf) >> 23) & 0xFF) + e;
-      if (sc.single && !bad && x0 >= 27 && x0 <= 190) {
+      if (sc.single && k.f32[h] && !bad && x0 >= 27 && x0 <= 190) {
         const float f = scale_pow2f(sc.apf, e), fl = scale_pow2f(sc.apf_lo, e);
         float q[2] = {};
 #pragma unroll
