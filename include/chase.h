@@ -9,8 +9,8 @@
  *   the layout of C99 `double complex` and `std::complex<double>` (the
  *   paper's element type, Listing 1).  Element (i, j) of a matrix with
  *   leading dimension ld sits at index j*ld + i.
- * - H is Hermitian and stored in full (both triangles are read).  It is
- *   never modified: the shift (A - cI) of Alg. 4 is applied inside the
+ * - H is Hermitian and stored in full: which triangle a product reads, or
+ *   both, depends on its size.  It is never modified: the shift (A - cI) of Alg. 4 is applied inside the
  *   product instead of on A (the paper's Shift() kernel, Listing 1).
  * - Array arguments marked "host or device" may point to host memory or to
  *   device memory of the current CUDA device; the library detects which
@@ -19,8 +19,9 @@
  *   arrays of one call must be of the same kind.
  * - The caller owns every array it passes (the paper's ChaseBLAS takes
  *   caller-owned buffers, Listing 2).  Device workspace needed beyond the
- *   caller's arrays is allocated stream-ordered (cudaMallocAsync) on
- *   `stream` and released before the call returns.
+ *   caller's arrays is allocated stream-ordered on `stream` from a memory
+ *   pool of the library's own and given back to that pool before the call
+ *   returns (chase_release_workspace).
  * - `stream` is a cudaStream_t (NULL = the legacy default stream).  Every
  *   call returns after its work on `stream` has completed.
  * - Every entry point returns a CHASE_* status; none aborts or throws.  On a
@@ -64,21 +65,28 @@ typedef struct {
 
 /* ---- arithmetic of the filter products (Alg. 4) ---- */
 /* FP64 accuracy.  Products with H of more than 6 columns and N >= 128 run on
- * the BF16 tensor cores in residue arithmetic (exact products of the operands
- * rounded to 2^-60 of the 2-norm of a row of H or a column of the block, put
- * together and finished in FP64: no further from the exact product than an
- * FP64 GEMM); smaller ones on the FP64 pipes.  The batched entry points do the
+ * the BF16 tensor cores in residue arithmetic: exact products of the operands
+ * rounded to 2^-60 of the 2-norm of a row of H (without its diagonal) or of a
+ * column of the block, put together and finished in FP64.  In norm, column by
+ * column, the result is no further from the exact product than an FP64 GEMM's.
+ * Entry by entry it need not be: of an entry 2^-k of its row's or column's norm
+ * 60 - k bits count, so a product that is small because small entries meet small
+ * ones (H of nearly uncoupled blocks, a column tiny on one of them) keeps fewer
+ * digits than in FP64.  These products read H through its Hermitian symmetry
+ * (column r conjugated, or the lower triangle alone, stands for row r) and take
+ * its diagonal as real.  Smaller products run on the FP64 pipes.  The batched entry points do the
  * same for batches of 2e7 FLOPs and more per degree step, unless they are of so
  * many small problems that the FP64 pipe is done sooner. */
 #define CHASE_FP64 0
 /* Split: the same residue products with the operands rounded to 2^-48 of
- * those norms.  The diagonal of H and the recurrence's shift/scale/axpby are
- * applied in FP64.  Reads H through its Hermitian
- * symmetry.  QR, Rayleigh-Ritz, residuals and Lanczos keep FP64 accuracy. */
+ * those norms (2^-52 for N above 32768, and for filters with a degree below 8 on
+ * sums of more than 16384 real terms).  The diagonal of H and the recurrence's
+ * shift/scale/axpby are applied in FP64.  QR, Rayleigh-Ritz, residuals and
+ * Lanczos keep FP64 accuracy. */
 #define CHASE_SPLIT_BF16 1
 /* Split-BF16 filter as above, and the product H Q of Rayleigh-Ritz (Alg. 2
- * line 2, reused for the residuals) on the same split product, operands
- * rounded to 2^-48 of their norms.  The projected eigenproblem, QR, the Gram products and Lanczos stay
+ * line 2, reused for the residuals) on a split product too, operands of both
+ * rounded to 2^-52 of their norms.  The projected eigenproblem, QR, the Gram products and Lanczos stay
  * FP64.  chase_solve and chase_solve_batched only (the filter entry points
  * take CHASE_FP64 or CHASE_SPLIT_BF16). */
 #define CHASE_SPLIT_BF16_RR 2
@@ -417,8 +425,7 @@ int chase_residuals_noalloc(const chase_c64* H, int64_t N, int64_t ldh, const ch
 /* Real symmetric problems (Sec. 5.1: the library is templated on the field
  * as well as the precision).  Same arguments, layouts, ownership and errors
  * as chase_filter, chase_residuals and chase_solve, with float64 matrices
- * and real symmetric H (both triangles stored; the split-BF16 slices read
- * row r of H from its column r).  Flop counts use 2 N^2 per column product
+ * and real symmetric H (both triangles stored).  Flop counts use 2 N^2 per column product
  * (8 N^2 for complex).  Leading dimensions need not be even: odd ones are
  * staged through padded device buffers inside the call. */
 int chase_filter_real(const double* H, int64_t N, int64_t ldh, double* V, int64_t ldv, int b,
@@ -434,8 +441,10 @@ int chase_solve_real(const double* H, int64_t N, int64_t ldh, int nev, int nex, 
 /* Single precision (Sec. 5.1 templates the library on the precision too):
  * complex64 (`_c32`) and float32 (`_f32`) versions of chase_filter,
  * chase_residuals and chase_solve with the same arguments, layouts and
- * errors.  Every product with H, the Gram products and the projected
- * eigensolve (cheevd / ssyevd) run in FP32 on the CUDA cores; the
+ * errors.  Products with H of more than 6 columns and N >= 128 run on the tensor
+ * cores in residue arithmetic (operands rounded to 2^-30 of a norm, results
+ * stored in FP32); smaller ones, the Gram products and the projected
+ * eigensolve (cheevd / ssyevd) in FP32 on the CUDA cores; the
  * orthogonalisation runs in double on widened copies of the block (Cholesky
  * QR squares the condition number of a filtered block, which FP32 cannot
  * hold) and rounds back.  Eigenvalues, residuals, bounds and tolerances are

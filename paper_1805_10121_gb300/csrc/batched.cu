@@ -190,14 +190,14 @@ double residue_step_us(const std::vector<GroupedFilterInput>& in, int nmod) {
 // with FP64 tiles, where each of their residue planes pads a tile of 256 rows.
 // 2000 problems of N = 16, ten steps in all: 11.2 ms on the FP64 tiles, 20.4 and
 // 18.8 ms as residues (14 and 11 moduli); 200 of N = 100: 3.0, 2.8 and 2.5 ms.
-int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile) {
+int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile, bool rr) {
   int64_t most = 0;
   double step = 0.0;
   for (const GroupedFilterInput& g : in) {
     most = std::max<int64_t>(most, g.n);
     step += 8.0 * g.n * static_cast<double>(g.n) * g.b;
   }
-  const int nmod = split ? rns_split_moduli(most) : kRnsFp64;
+  const int nmod = !split ? kRnsFp64 : rr ? kRnsSplitRR : rns_split_moduli(most, true);
   if (!split && (tile != CHASE_TILE_AUTO || step < 2e7)) return 0;
   return residue_step_us(in, nmod) < fp64_step_us(in) ? nmod : 0;
 }

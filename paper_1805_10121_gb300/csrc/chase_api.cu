@@ -938,7 +938,7 @@ struct Solver {
       }
     }
     std::vector<PlaneSet> sets;
-    if (want_split) sets.push_back({rns_split_moduli(N), &hsplit});
+    if (want_split) sets.push_back({split_rr ? kRnsSplitRR : rns_split_moduli(N, is_cplx<T>), &hsplit});
     if (want_low) sets.push_back({rns_low_moduli(N), &hlow});
     if (want64) sets.push_back({kRnsFp64, &h64});
     int st = prepare_products(d, dH, N, lh, nx, true, want64 || !split, sets, rx);
@@ -1414,7 +1414,9 @@ int filter_impl(const T* H, int64_t N, int64_t ldh, T* V, int64_t ldv, int b, co
   if (rns) {
     const int nmod = is_single<T> || precision == CHASE_SPLIT_BF16_4 || precision == CHASE_SPLIT_BF16_3
                          ? rns_low_moduli(N)
-                         : precision == CHASE_FP64 ? kRnsFp64 : rns_split_moduli(N);
+                         : precision == CHASE_FP64
+                             ? kRnsFp64
+                             : rns_split_moduli(N, is_cplx<T>, start[8] > 0 ? 2 : 8);
     const int st = prepare_products(d, dH, N, lh, b, true, precision == CHASE_FP64, {{nmod, &rh}}, rx);
     if (st == CHASE_OUT_OF_MEMORY && precision == CHASE_FP64)
       rns = false;  // on the FP64 pipe (FP32 in single precision)
@@ -1545,7 +1547,10 @@ extern "C" int chase_filter_mixed(const chase_c64* H, int64_t N, int64_t ldh, ch
   const bool any_low = *std::min_element(ns.begin(), ns.end()) < 7;
   const bool any_full = *std::max_element(ns.begin(), ns.end()) == 7;
   std::vector<PlaneSet> sets;
-  if (any_full) sets.push_back({rns_split_moduli(N), &full});
+  int least = kMaxDegAllowed;  // of the columns in full precision
+  for (int a = 0; a < b; ++a)
+    if (ns[a] == 7) least = std::min(least, deg[a]);
+  if (any_full) sets.push_back({rns_split_moduli(N, true, least), &full});
   if (any_low) sets.push_back({rns_low_moduli(N), &low});
   CHASE_TRY(prepare_products(d, dH, N, lh, b, true, false, sets, rx));
   rs.full = any_full ? &full : nullptr;
@@ -2100,7 +2105,7 @@ extern "C" int chase_solve_batched(int P, const chase_c64* const* H, const int64
     planes[p].n = static_cast<int>(sv[p].N);
     planes[p].b = bcap[p] = sv[p].nx;
   }
-  const int nmod = grouped_moduli(planes, split, CHASE_TILE_AUTO);
+  const int nmod = grouped_moduli(planes, split, CHASE_TILE_AUTO, o.precision == CHASE_SPLIT_BF16_RR);
   GroupedWork work;
   bool resident = false;
   if (nmod > 0) {

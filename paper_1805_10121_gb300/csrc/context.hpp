@@ -180,12 +180,14 @@ inline int gram(Dev& d, int64_t N, const float* X, int64_t ldx, int p, const flo
 
 // ---- rns.cu: products with H in residue arithmetic on the tensor cores -----
 // Moduli per accuracy: kRnsFp64 stands in for FP64 GEMMs (operands rounded to
-// 2^-60 of a row's or column's 2-norm), rns_split_moduli(N) for the split
-// filter (2^-48), rns_low_moduli(N) for its reduced precisions and for single
-// precision (2^-30).
+// 2^-60 of a row's or column's 2-norm), rns_split_moduli for the split filter
+// (2^-48, or 2^-52), kRnsSplitRR for a single product that replaces one at FP64
+// accuracy (H Q of CHASE_SPLIT_BF16_RR; 2^-52), rns_low_moduli(N) for the
+// filter's reduced precisions and for single precision (2^-30).
 constexpr int kRnsMaxModuli = 14;
 constexpr int kRnsFp64 = 14;
-int rns_split_moduli(int64_t N);
+constexpr int kRnsSplitRR = 12;
+int rns_split_moduli(int64_t N, bool cplx, int least_degree = 8);
 int rns_low_moduli(int64_t N);
 // Residue planes of H (per modulus two planes of N x Kp bf16 for complex H,
 // one for real), row exponents and the real diagonal, which the epilogue
@@ -377,7 +379,8 @@ struct GroupedFilterTimes {
 };
 // Moduli of a batch's residue products: of the split filter's accuracy, or
 // FP64's; 0 where the FP64 tiles take less time.
-int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile);
+// rr: the planes serve H Q of CHASE_SPLIT_BF16_RR too.
+int grouped_moduli(const std::vector<GroupedFilterInput>& in, bool split, int tile, bool rr = false);
 // Residue planes of every problem's H and the workspace for bcap[q] columns
 // (one grouped slicing launch), which leave `reserve` bytes free; fills the
 // residue fields of `in`.  A status other than CHASE_OK leaves nothing behind.

@@ -2135,10 +2135,16 @@ struct Kind<float> {
 }  // namespace
 
 // The rounding of the operands, relative to a product, grows like sqrt(N); the
-// splits into 7-bit digits that these stand for had errors independent of N:
-// 2.6e-12 after a filter of degree 20 at N = 8000 (digits: 4.6e-12), 4.6e-12
-// at N = 20000 (6.3e-12).  One modulus more takes over where they would meet.
-int rns_split_moduli(int64_t N) { return N <= 32768 ? 11 : 12; }
+// splits into 7-bit digits that these stand for had errors independent of N, but
+// with a bias that added up over a filter's steps.  Degree 20: 4.4e-12 at N =
+// 20000 (digits 6.5e-12), 4.8e-12 at N = 30000 (7.9e-12), uniform spectrum
+// 3.8e-12 at both (3.5e-12, 4.5e-12).  Degree 2, uniform, sums of K = 2 N: 4.3e-13
+// at N = 8192 (5.0e-13), 5.9e-13 at 16384 (3.6e-13), 8.3e-13 at 30000 (4.7e-13).
+// One modulus more, a sixteenth of the error, takes over where they would meet,
+// and for few steps of long sums before that.
+int rns_split_moduli(int64_t N, bool cplx, int least_degree) {
+  return N > 32768 || ((cplx ? 2 : 1) * N > 16384 && least_degree < 8) ? 12 : 11;
+}
 int rns_low_moduli(int64_t N) { return N <= 8192 ? 7 : 8; }
 
 // One plane per modulus instead of two (real: one triangle of it) halves what a
