@@ -280,6 +280,7 @@ __global__ void __launch_bounds__(kJacobiThreads, 1)
         const float t =
             copysignf(__fdividef(1.f, fabsf(zeta) + sqrtf(fmaf(zeta, zeta, 1.f))), zeta);
         const float c = rsqrtf(fmaf(t, t, 1.f)), s = t * c;
+        __syncwarp();  // every lane has read both norms
         if (lane == 0) {
           const float move = t * g2 * ig;
           s_norm[i] = na - move;
