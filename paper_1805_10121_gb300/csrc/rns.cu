@@ -110,11 +110,13 @@ __device__ __forceinline__ bool try_wait_cluster(uint64_t* bar, uint32_t parity)
       : "memory");
   return done != 0;
 }
+// A whole warp's wait, with one answer for all lanes: lanes that disagreed about
+// a time-out would part and wait for one another in different places.
 __device__ __forceinline__ bool wait_cluster_bounded(uint64_t* bar, uint32_t parity) {
-  if (try_wait_cluster(bar, parity)) return true;
+  if (__all_sync(0xffffffffu, try_wait_cluster(bar, parity))) return true;
   const long long t0 = clock64();
-  while (!try_wait_cluster(bar, parity)) {
-    if (clock64() - t0 > kWaitBudgetCycles) return false;
+  while (!__all_sync(0xffffffffu, try_wait_cluster(bar, parity))) {
+    if (__any_sync(0xffffffffu, clock64() - t0 > kWaitBudgetCycles)) return false;
   }
   return true;
 }
@@ -354,7 +356,6 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, const Walk w, const Gemm
                           bar);
             tma_load_pair(smem_u32(sB + st * C::B_BYTES), T.mapB, ks * BK, cb, T.planeB, bar);
           }
-          __syncwarp();
           if (++st == NSTAGE) {
             st = 0;
             ph ^= 1u;
@@ -411,7 +412,6 @@ __device__ __forceinline__ void gemm_body(TileFn& tile, const Walk w, const Gemm
               commit_pair(&empty[st]);
               if (ks == k1 - 1) commit_pair(&acc_full[buf]);
             }
-            __syncwarp();
             if (++st == NSTAGE) {
               st = 0;
               ph ^= 1u;
