@@ -252,15 +252,65 @@ def prec_code(name):
             "split_adapt": chase.CHASE_SPLIT_BF16_ADAPT, "fp64": chase.CHASE_FP64}[name]
 
 
-# Slice-pair products the split-BF16 kernel executes per FP64-equivalent
-# product: pairs (s, t) of 7 slices with s + t <= 6.
+# Residue planes of a complex product with H: two per modulus, each a BF16 GEMM of
+# 2 N^2 FLOPs per column beside 8 N^2 algorithmic ones.
+FP64_MODULI = 14
+
+
+def split_moduli(n, rr=False):
+    """Moduli of the split filter's products (degrees of 8 and more), or of those
+    of CHASE_SPLIT_BF16_RR, which serve H Q too."""
+    return 12 if rr or n > 32768 else 11
+
+
+def residue_entry(flops, secs, moduli, pk, src, what, timing, peak_key="bf16_tflops_sustained"):
+    """Roofline of residue products: `flops` algorithmic FLOPs in `secs`."""
+    alg = flops / secs / 1e12 if secs > 0 else 0.0
+    peak = pk.get(peak_key, 1700.0)
+    return {
+        "bound": "tensor",
+        "kernel": f"rns_gemm_kernel (tcgen05 CTA pairs, BF16 residue GEMMs): {what}",
+        "achieved": round(0.5 * moduli * alg, 2),
+        "peak": round(peak, 1),
+        "unit": "TFLOP/s",
+        "frac": round(0.5 * moduli * alg / peak, 4),
+        "traffic": None,
+        "peak_source": f"{src} {peak_key}",
+        "achieved_counts": f"BF16 tensor FLOPs of the products: {moduli} moduli, 2 planes of "
+                           "2 N^2 per complex column",
+        "fp64_equivalent_tflops": round(alg, 4),
+        "timing": timing,
+    }
+
+
+def residue_roofline(stats_list, n, pk, src, precision):
+    """(dominant product's roofline, the other's) of a solve: its filters, and H Q
+    of Rayleigh-Ritz, which only CHASE_SPLIT_BF16_RR makes at split precision.
+    The filter phase holds slicing and reconstruction beside the GEMMs."""
+    rr_split = precision == "split_rr"
+    filt = residue_entry(sum(s["flops_filter"] for s in stats_list),
+                         sum(s["t_filter"] for s in stats_list),
+                         FP64_MODULI if precision == "fp64" else split_moduli(n, rr_split), pk, src,
+                         "the filter steps",
+                         "filter phase (slicing, products, reconstruction), CUDA events on the "
+                         "solve's stream")
+    if precision == "split_adapt":
+        filt["achieved_counts"] += " (reduced-precision products execute 7 or 8)"
+    rr_t = sum(s["t_rr_product"] for s in stats_list)
+    rr = residue_entry(sum(s["flops_rr_product"] for s in stats_list), rr_t,
+                       split_moduli(n, True) if rr_split else FP64_MODULI, pk, src,
+                       "Rayleigh-Ritz H Q", "H Q products, CUDA events on the solve's stream")
+    return (rr, filt) if rr_t >= sum(s["t_filter"] for s in stats_list) else (filt, rr)
+
+
+# Slice-pair products the seven-digit split product executed per FP64-equivalent
+# product: pairs (s, t) of 7 slices with s + t <= 6.  That product, the FP64
+# tiles' figures below and roofline_entry describe the kernels before residue
+# products; no bench line reports them any more.
 SPLIT_PAIRS = 28
 
 
-# DRAM traffic of single launches of other shapes, measured with ncu: the
-# sequence workload's own launches (N = 8000, 480 columns; the FP64 H Q on
-# its 64 x 16 tile) have no capture, so its "traffic" stays null and these
-# figures ride along as context.
+# DRAM traffic of single launches of those kernels, measured with ncu.
 NCU_TRAFFIC = {
     "zgemm_split_kernel": {"case": "N=8000, 1500 complex columns, full-width degree step of the "
                                    "persistent kernel (the sequence workload's blocks are narrower)",
@@ -343,11 +393,12 @@ def roofline_entry(stats_list, pk, src, precision):
     return filt, rr
 
 
-def lanczos_entry(stats_list, n, pk, src):
-    """Rate of the Lanczos phase (Alg. 6): its matvecs run on the few-column
+def lanczos_entry(stats_list, n, pk, src, planes=False):
+    """Rate of the Lanczos phase (Alg. 6).  Its matvecs run on the few-column
     product (one vector per step after a warm start), which reads H once per
     step and is bound by the FP64 FMA pipe (2 FLOP/byte against a machine
-    balance of 0.15)."""
+    balance of 0.15), or (planes) as residue products, which stream the planes
+    of H, 28 N^2 bytes where all rows share a scale."""
     mv = sum(s.get("lanczos_matvecs", 0) for s in stats_list)
     t = sum(s["t_lanczos"] for s in stats_list)
     if mv <= 0 or t <= 0:
@@ -356,6 +407,22 @@ def lanczos_entry(stats_list, n, pk, src):
     hbm_bytes = 16.0 * n * n * mv  # warm-started solves: one vector per step
     peak = pk.get("bf16_tflops", 1900.0) * NOMINAL_FP64_OVER_BF16
     tf = flops / t / 1e12
+    if planes:
+        gbs = 2.0 * FP64_MODULI * n * n * mv / t / 1e9
+        return {
+            "kernel": "rns_gemm_kernel (BF16 residue GEMMs): the Lanczos matvecs",
+            "bound": "hbm",
+            "matvecs": int(mv),
+            "seconds": round(t, 4),
+            "achieved": round(gbs, 1),
+            "peak": pk.get("hbm_gbs", 6800.0),
+            "unit": "GB/s",
+            "frac": round(gbs / pk.get("hbm_gbs", 6800.0), 4),
+            "fp64_equivalent_tflops": round(tf, 4),
+            "timing": "whole Lanczos phase (matvecs, three-term steps, host tridiagonal "
+                      "eigensolves), CUDA events on the solve's stream",
+            "peak_source": f"{src} hbm_gbs",
+        }
     return {
         "kernel": "fewcol_kernel (FP64 FMA on the CUDA cores): the Lanczos matvecs",
         "bound": "fp64",
@@ -641,22 +708,21 @@ def filter_workload_config(args, world):
 # DRAM traffic of one product launch of the default filter workload: not
 # captured for the residue GEMM.
 SPLIT_N30000_TRAFFIC = None
-# Residue planes of the split filter's product up to N = 32768: 11 moduli, one
-# BF16 plane each of H (the second is its transpose), two of the block.
-SPLIT_MODULI = 11
 
 
 def split_algorithmic_bytes(n, ncols, k_per_launch):
-    """Bytes that one launch of a product of seven-digit slices moves at least:
-    the 7 slice planes of H and of the block over its K range, once, and the
-    FP64 result (a K-segment partial product, N x ncols complex)."""
+    """Bytes that one launch of the seven-digit split product (see SPLIT_PAIRS)
+    moved at least: the 7 slice planes of H and of the block over its K range,
+    once, and the FP64 result (a K-segment partial product, N x ncols complex)."""
     return 7 * 2.0 * (n + 2 * ncols) * k_per_launch + 16.0 * n * ncols
 
 
 def residue_algorithmic_bytes(n, ncols):
-    """Bytes that one residue product moves at least: the planes of H and of
-    the block once, and the residues of the product (int16)."""
-    return 2.0 * SPLIT_MODULI * (n * n + 2 * n * ncols) + 4.0 * SPLIT_MODULI * n * ncols
+    """Bytes that one residue product of a split filter moves at least: the planes
+    of H (one BF16 plane per modulus, the second is its transpose) and of the
+    block (two) once, and the residues of the product (int16)."""
+    m = split_moduli(n)
+    return 2.0 * m * (n * n + 2 * n * ncols) + 4.0 * m * n * ncols
 
 
 def run_filter_workload(args, rank, world, local):
@@ -942,21 +1008,16 @@ def run_batched_workload(args, rank, world, local):
                  "tflops": round(flops / t_o / 1e12, 4), "seconds": round(t_o, 3),
                  "product_seconds": round(st_o[0]["t_product"], 3),
                  "tile_config": st_o[0]["tile_config"]}
-    if split:
-        achieved = 0.5 * SPLIT_MODULI * flops / t_prod / 1e12
-        peak = pk.get("bf16_tflops_sustained", 1700.0)
-        roof = {"bound": "tensor",
-                "kernel": "rns_grouped_gemm_kernel (tcgen05 BF16 residue GEMMs over all problems "
-                          "of a degree step)",
-                "achieved": round(achieved, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
-                "frac": round(achieved / peak, 4), "traffic": None,
-                "peak_source": f"{src} bf16_tflops_sustained",
-                "fp64_equivalent_tflops": round(flops / t_prod / 1e12, 3)}
-        # residue planes of H (22 N^2 bytes) stream from HBM once per degree step
-        hbm = sum(2.0 * SPLIT_MODULI * n * n for n, _, _ in shapes) * st_main[0]["steps"] / t_prod / 1e9
+    if st_main[0]["tile_config"] < 0:
+        moduli = split_moduli(max(n for n, _, _ in shapes)) if split else FP64_MODULI
+        roof = residue_entry(flops, t_prod, moduli, pk, src, "all problems of a degree step",
+                             "product launches, CUDA events inside the step graph")
+        roof["kernel"] = roof["kernel"].replace("rns_gemm_kernel", "rns_grouped_gemm_kernel")
+        # residue planes of H (2 N^2 bytes a modulus) stream from HBM once per degree step
+        hbm = sum(2.0 * moduli * n * n for n, _, _ in shapes) * st_main[0]["steps"] / t_prod / 1e9
         roof["hbm_gbs_slices_of_h"] = round(hbm, 1)
         roof["hbm_frac"] = round(hbm / pk.get("hbm_gbs", 6800.0), 4)
-    else:
+    else:  # FP64 tiles: batches of little work, or a tile shape named on the command line
         peak = pk.get("bf16_tflops", 1900.0) * NOMINAL_FP64_OVER_BF16
         achieved = FP64_EXECUTED_PER_ALGORITHMIC * flops / t_prod / 1e12
         roof = {"bound": "tensor",
@@ -1221,10 +1282,11 @@ def run_side_workload(args, rank, world, local):
     sequence workload: the Lanczos bound estimate of a warm start (Alg. 6,
     one vector, k = 25 matvecs), the full Lanczos of a cold start (1 + n_vec
     = 5 vectors as one block) and the residual norms of the nev + nex block
-    (one product with H plus the fused norm kernel).  All are FP64; on this
-    GPU the FP64 pipe, not HBM, bounds each of them (the one-vector matvec
-    has 2 FLOP/byte against a machine balance of 0.15), so each line gives
-    the FP64 rate and the HBM rate the pass over H achieved."""
+    (one product with H plus the fused norm kernel).  The Lanczos entry point's
+    products have at most 6 columns and run on the FP64 pipe, which bounds them
+    (the one-vector matvec has 2 FLOP/byte against a machine balance of 0.15);
+    the residuals' product runs on the tensor cores.  Each line gives its share
+    of that unit's rate and the HBM rate the pass over H achieved."""
     from paper_1805_10121_gb300 import build, chase, synth
     build.build()
     chase.lib()
@@ -1266,12 +1328,16 @@ def run_side_workload(args, rank, world, local):
     fp64_peak = pk.get("bf16_tflops", 1900.0) * NOMINAL_FP64_OVER_BF16
     hbm = pk.get("hbm_gbs", 6800.0)
 
-    def entry(what, secs, flops, hbm_bytes, kernel):
+    def entry(what, secs, flops, hbm_bytes, kernel, residues=False):
         tf = flops / secs / 1e12
         gbs = hbm_bytes / secs / 1e9
-        return {"step": what, "kernel": kernel, "seconds": round(secs, 5),
-                "tflops": round(tf, 4), "fp64_frac": round(tf / fp64_peak, 4),
-                "hbm_gbs": round(gbs, 1), "hbm_frac": round(gbs / hbm, 4)}
+        e = {"step": what, "kernel": kernel, "seconds": round(secs, 5),
+             "tflops": round(tf, 4), "hbm_gbs": round(gbs, 1), "hbm_frac": round(gbs / hbm, 4)}
+        if residues:
+            e["bf16_frac"] = round(0.5 * FP64_MODULI * tf / pk.get("bf16_tflops", 1900.0), 4)
+        else:
+            e["fp64_frac"] = round(tf / fp64_peak, 4)
+        return e
 
     h_bytes = 16.0 * n * n
     rows = [
@@ -1280,7 +1346,8 @@ def run_side_workload(args, rank, world, local):
         entry("Lanczos with DoS, cold start (5 vectors, 25 steps)", t_cold, 8.0 * n * n * k * 5,
               h_bytes * k, "fewcol_kernel<5> + lanczos_step_kernel"),
         entry(f"residual norms of {nx} columns", t_res, 8.0 * n * n * nx,
-              h_bytes + 3 * 16.0 * n * nx, "zgemm_tma_kernel + resid_norms_kernel"),
+              h_bytes + 3 * 16.0 * n * nx,
+              "rns_gemm_kernel (planes of H made for this one product) + resid_norms_kernel", True),
     ]
     cfg = workload_config(args, world)
     cfg["workload"] = (f"steps beside the filter on problem 1 of the sequence workload, N={n}, "
@@ -1729,18 +1796,7 @@ def main():
             torch.distributed.destroy_process_group()
         return
     pk, src = peaks()
-    roof_main, roof_other = roofline_entry(stats_t, pk, src, args.precision)
-    for r in (roof_main, roof_other):  # products execute residue GEMMs: 11 moduli, FP64 14
-        if r and "achieved" in r:
-            moduli = SPLIT_MODULI if "fp64_equivalent_tflops" in r else 14
-            alg = r.get("fp64_equivalent_tflops") or r.get("algorithmic_tflops") or 0.0
-            peak = pk.get("bf16_tflops_sustained", 1700.0)
-            r.update(kernel="rns_gemm_kernel (BF16 residue GEMMs)", peak=round(peak, 1),
-                     achieved=round(0.5 * moduli * alg, 2),
-                     frac=round(0.5 * moduli * alg / peak, 4),
-                     achieved_counts=f"BF16 tensor FLOPs: {moduli} moduli, 2 planes of 2 N^2 per column",
-                     peak_source=f"{src} bf16_tflops_sustained")
-            r.pop("traffic_ncu_small_case", None)
+    roof_main, roof_other = residue_roofline(stats_t, n, pk, src, args.precision)
     cb = None
     if not args.no_cpu_baseline and world == 1:
         cb = cpu_baseline_sample(n, nev, nex, args.seed, args.cpu_sample_seconds)
@@ -1774,7 +1830,9 @@ def main():
         "warmup_iterations": [s["iterations"] for _, s in stats_w],
         "roofline": roof_main,
         "roofline_other_kernel": roof_other,
-        "lanczos": lanczos_entry(stats_t, n, pk, src),
+        # a warm start's one vector takes the planes from N^2 = 4e6 on
+        "lanczos": lanczos_entry(stats_t, n, pk, src,
+                                 args.precision != "split_rr" and n * n >= 4e6),
         "fp64_same_problem": fp64,
         "split_rr_same_problem": split_rr,
         "cpu_baseline": cb,
