@@ -30,7 +30,9 @@
  * - Calls may run at the same time from several host threads on different
  *   streams (each thread keeps its own eigensolver handle); their results
  *   are bit-identical to the same calls run one at a time, whatever else
- *   runs on the device.  Calls that share an output array must be ordered
+ *   runs on the device (while its memory lasts: a call that does not get the
+ *   workspace for residue products may go on on the FP64 pipe, which rounds
+ *   differently).  Calls that share an output array must be ordered
  *   by the caller.
  */
 #ifndef CHASE_H_
@@ -97,15 +99,15 @@ typedef struct {
  * value|) the column's products run in class 3, above 1e-6 h in class 4 (both
  * round their operands to 2^-30 of a norm), else in class 7 (2^-48).  The
  * first filter, before any residual is known, uses 3.  The
- * active block is ordered by (slices, degree), and each run of equal slices
+ * active block is ordered by (class, degree), and each run of equal classes
  * is filtered as its own suffix-retiring block.  Rayleigh-Ritz, QR and
- * residuals stay FP64, so the converged pairs meet the same tolerance; a
+ * residuals keep FP64 accuracy, so the converged pairs meet the same tolerance; a
  * low-precision column only limits how far this filter can reduce its
  * residual, which it could not reduce to the tolerance anyway. */
 #define CHASE_SPLIT_BF16_ADAPT 3
-/* chase_filter only: split-BF16 products with the leading 4 or 3 slices of
- * each operand (about 2^-28 or 2^-21 relative per product), the reduced
- * precisions CHASE_SPLIT_BF16_ADAPT switches between. */
+/* chase_filter only: split products of the classes 4 and 3, the reduced
+ * precisions CHASE_SPLIT_BF16_ADAPT switches to (operands of both rounded to
+ * 2^-30 of a norm). */
 #define CHASE_SPLIT_BF16_4 4
 #define CHASE_SPLIT_BF16_3 5
 
@@ -153,10 +155,10 @@ typedef struct {
   double t_rr_product;     /* seconds of Rayleigh-Ritz's H Q products (inside t_rr) */
   double flops_rr_product; /* their algorithmic FLOPs (8 N^2 b complex, 2 N^2 b real) */
   int filter_slices_low;   /* iterations in which some column products of the split
-                              filter kept fewer than 7 slices (CHASE_SPLIT_BF16_ADAPT;
+                              filter ran in a class below 7 (CHASE_SPLIT_BF16_ADAPT;
                               single precision) */
   long long lanczos_matvecs; /* column products with H inside Alg. 6 (k per run) */
-  long long filter_matvecs_low; /* filter column products made with fewer than 7 slices */
+  long long filter_matvecs_low; /* filter column products made in a class below 7 */
 } chase_stats;
 
 /* Tile choice of the grouped FP64 filter: residue products for batches of 2e7
@@ -236,8 +238,9 @@ int chase_workspace_limit(long long bytes);
  * chase_kernel_timing_read waits for the recorded events of one kind and
  * returns their summed duration (seconds), the kernel launches they cover,
  * the algorithmic FLOPs (8 N^2 per complex column, 2 N^2 per real column)
- * and the executed tensor FLOPs (split: slice pairs x algorithmic; FP64: 6
- * of every 8 algorithmic complex FLOPs, the 3M form).  flops and
+ * and the executed tensor FLOPs (residue products: moduli / 2 for complex,
+ * moduli for real columns, per algorithmic FLOP; on the FP64 pipe 6 of every 8
+ * algorithmic complex FLOPs, the 3M form).  flops and
  * tensor_flops are nullable.  Recording adds two event records per product
  * call and no synchronisation.  Errors: CHASE_INVALID_ARG, CHASE_CUDA_ERROR. */
 /* Failure detection (the paper has no counterpart): every wait of the
@@ -286,8 +289,8 @@ int chase_filter(const chase_c64* H, int64_t N, int64_t ldh, chase_c64* V, int64
  * as accurate as the residual it can reach; the paper filters every column
  * in one precision): column a is filtered with its degree degrees[a] on the
  * split product of precision class slices[a] in {3, 4, 7} (operands rounded
- * to 2^-30, 2^-30 and 2^-48 of a norm).  The columns are ordered by (slices, degree) inside the
- * call and each run of equal slices is filtered as its own suffix-retiring
+ * to 2^-30, 2^-30 and 2^-48 of a norm).  The columns are ordered by (class, degree) inside the
+ * call and each run of equal classes is filtered as its own suffix-retiring
  * block of the same recurrence; V returns in the caller's column order.
  * H, V, work: as chase_filter (complex128, column-major, host or device).
  * degrees, slices: b ints each, host or device.

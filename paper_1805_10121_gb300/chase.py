@@ -332,8 +332,8 @@ def chase_filter(H, V, degrees, b_sup, mu1, mu_nevnex, work=None, stream=None,
 
 
 def chase_filter_mixed(H, V, degrees, slices, b_sup, mu1, mu_nevnex, work=None, stream=None):
-    """Alg. 4 with a precision per column: ``slices[a]`` in {3, 4, 7} slices of
-    the split-BF16 product for column a (complex128 tensors, V in place)."""
+    """Alg. 4 with a precision per column: ``slices[a]`` in {3, 4, 7}, the class
+    of the split product for column a (complex128 tensors, V in place)."""
     n = H.shape[0]
     hp, ldh = _mat(H, n, "H")
     vp, ldv = _mat(V, n, "V")

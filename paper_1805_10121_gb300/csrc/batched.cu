@@ -185,8 +185,9 @@ double residue_step_us(const std::vector<GroupedFilterInput>& in, int nmod) {
 }
 }  // namespace
 
-// Residue products, for an FP64 batch from 2e7 FLOPs a degree step on, unless
-// the FP64 tiles are done sooner: many problems of few rows each fill the device
+// Residue products, for an FP64 batch from 2e7 FLOPs a degree step on (a cautious
+// line: 8 problems of N = 128, 10 columns, 1e7, take 70 us a step on the tiles,
+// 28 as 11-moduli residues), unless the FP64 tiles are done sooner: many problems of few rows each fill the device
 // with FP64 tiles, where each of their residue planes pads a tile of 256 rows.
 // 2000 problems of N = 16, ten steps in all: 11.2 ms on the FP64 tiles, 20.4 and
 // 18.8 ms as residues (14 and 11 moduli); 200 of N = 100: 3.0, 2.8 and 2.5 ms.

@@ -144,8 +144,11 @@ struct RnsSet {
   RnsX* x = nullptr;
 };
 
-// Products with H take the residue path from this size on; below it, a few
-// columns or rows, the FP64 kernels are done sooner than its three launches.
+// Products with H take the residue path from this size on.  Below 7 columns the
+// few-column kernel reads H once and needs no planes; below 128 rows a tile of
+// the GEMM would be mostly padding.  The line is a cautious one: degree 20 takes
+// 394 us as residues with N = 128 and 7 columns, and 1465 us on the FP64 pipe
+// with N = 127 and 9 (its K loop runs alone on a few SMs).
 bool rns_pays(int64_t N, int b) { return N >= 128 && b > kFewColMax; }
 
 // Bytes that a call may still allocate after the residue planes of H: the
@@ -220,7 +223,7 @@ struct FilterGroup {
 // columns of the same three-term recurrence (the coefficients of Eq. 7 do
 // not depend on the column), filtered with its own precision and retiring
 // its own finished columns.  Adds the column products to *matvecs and those
-// made with fewer than 7 slices to *matvecs_low.
+// made in a class below 7 to *matvecs_low.
 template <class T>
 int filter_groups(Dev& d, const T* H, int64_t N, int64_t ldh, T* X, int64_t ldx, T* Wk,
                   int64_t ldw, const std::vector<FilterGroup>& groups, int maxdeg, double b_sup,
@@ -807,7 +810,7 @@ struct Solver {
   RnsSet filter_set, rr_set;
   bool rns = false;
   // single precision with CHASE_SPLIT_BF16: the filter runs on widened FP64
-  // copies of the active block (Dv, Dw), the product with 4 slices
+  // copies of the active block (Dv, Dw)
   using Wide = typename std::conditional<is_cplx<T>, chase_c64, double>::type;
   Wide *Dv = nullptr, *Dw = nullptr;
   int64_t lD = 0;
@@ -823,8 +826,8 @@ struct Solver {
   int d0 = 0, nconv = 0, iter = 0, status = CHASE_OK, maxdeg = 0;
   bool grouped = false;  // the batched solve filters through the grouped kernels
   std::vector<int> m, order, perm, start;
-  // slices of the split product per column (7 = full precision; the FP64
-  // filter ignores it), and the runs of equal precision the filter works on
+  // precision class of the split product per column (7: full; the FP64 filter
+  // ignores it), and the runs of equal precision the filter works on
   std::vector<int> cls;
   std::vector<FilterGroup> groups;
   std::vector<double> ritz, res, ra, rr;
@@ -838,7 +841,7 @@ struct Solver {
   T* Va() const { return dV + static_cast<size_t>(nconv) * lv; }
   bool more() const { return status == CHASE_OK && nconv < nev && iter < o.max_iter; }
 
-  // Everything before the loop of Alg. 1; `grouped_split` leaves the slices
+  // Everything before the loop of Alg. 1; `grouped_split` leaves the planes
   // of H to the caller.
   int setup(Dev& d, bool grouped_split) {
     std::memset(&S, 0, sizeof(S));
@@ -863,9 +866,8 @@ struct Solver {
     CHASE_TRY(d.alloc(&Wk, static_cast<size_t>(lw) * nx));  // filter double buffer / permutation scratch
     CHASE_TRY(orth_alloc(d, N, nx, nx, ow));
     CHASE_TRY(rr_alloc(d, N, nx, rw));
-    // single precision: every product in FP32 on the CUDA cores, or with
-    // CHASE_SPLIT_BF16 the filter's products on the split tensor-core
-    // product (4 slices, about 2^-28 relative: finer than FP32 rounding)
+    // single precision: each step stored in FP32, or with a split precision the
+    // filter on widened copies of the block
     split = is_single<T> ? o.precision != CHASE_FP64
                          : (o.precision == CHASE_SPLIT_BF16 || o.precision == CHASE_SPLIT_BF16_RR ||
                             o.precision == CHASE_SPLIT_BF16_ADAPT);
@@ -990,7 +992,7 @@ struct Solver {
     return true;
   }
 
-  // Slices of the split product before any residual is known: 3 with
+  // Class of the split product before any residual is known: 3 with
   // CHASE_SPLIT_BF16_ADAPT (the first filter starts from random vectors),
   // 4 for single precision, else 7.  The batched solve's grouped filter
   // takes one precision for all columns (7).
@@ -1000,15 +1002,15 @@ struct Solver {
     return 7;
   }
 
-  // CHASE_SPLIT_BF16_ADAPT: slices of the split product for one column in the
+  // CHASE_SPLIT_BF16_ADAPT: class of the split product for one column in the
   // next filter (Sec. 3.2: the filter only has to beat the residual it can
   // reach).  By the model behind Alg. 5 a degree-m filter divides the
   // residual by |rho|^m; while that expected residual stays above 1e-3 h the
-  // column's products keep 3 slices (about 2^-21 relative), above 1e-6 h 4
-  // slices (2^-28), else all 7 (2^-49).  Columns whose degree was chosen to
+  // column's products run in class 3, above 1e-6 h in class 4 (operands of both
+  // rounded to 2^-30 of a norm), else in 7 (2^-48).  Columns whose degree was chosen to
   // reach the tolerance therefore run in full precision, and only those
   // that cannot converge in this filter (degree capped at DEGMAX, or a Ritz
-  // value inside the damped interval) run on fewer slices.
+  // value inside the damped interval) run in a lower class.
   int column_slices(double res_a, double ritz_a, int m_a, double c, double e) const {
     if constexpr (is_single<T>) return 4;
     if (o.precision != CHASE_SPLIT_BF16_ADAPT || grouped || !(e > 0.0)) return 7;
@@ -1514,7 +1516,7 @@ extern "C" int chase_filter_mixed(const chase_c64* H, int64_t N, int64_t ldh, ch
   const int64_t lw = ld_pad<chase_c64>(N);
   chase_c64* wk = dev && lw == N ? work : nullptr;
   if (!wk) CHASE_TRY(d.alloc(&wk, static_cast<size_t>(lw) * b));
-  // columns ordered by (slices, degree): runs of equal precision, each sorted
+  // columns ordered by (class, degree): runs of equal precision, each sorted
   // by degree, each filtered as its own suffix-retiring block
   std::vector<int> order(b);
   std::iota(order.begin(), order.end(), 0);

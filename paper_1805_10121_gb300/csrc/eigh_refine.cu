@@ -166,8 +166,9 @@ __global__ void __launch_bounds__(kThreads)
 // product, rotation and the block's barrier.  The library's solver, hundreds of
 // launches of a few microseconds, takes 1.3 ms at p = 70 whatever G is; here a
 // dense G takes about as long (eigensolve in all 2.1 ms on either; p = 33: 0.82
-// against 1.34 ms), one near a diagonal, as from the second iteration of a solve
-// on, 0.6 ms.
+// against 1.34 ms; whole Rayleigh-Ritz call, N = 1000: 2.04 ms at p = 96 here,
+// 2.22 at p = 97 with the library), one near a diagonal, as from the second
+// iteration of a solve on, 0.6 ms.
 // ---------------------------------------------------------------------------
 constexpr int kJacobiMax = 96, kJacobiThreads = 1024;
 constexpr int kJacobiSweeps = 14;
