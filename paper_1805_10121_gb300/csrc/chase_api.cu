@@ -161,9 +161,11 @@ size_t rns_reserve(int64_t N, int b) {
 
 // Residue planes of H (h with nmod moduli, one set or several) and the
 // workspace x for b columns.  Where they do not all fit beside the reserve, with
-// fewer moduli resident and fewer columns at a time; where one modulus of each
-// and one column do not, CHASE_OUT_OF_MEMORY with nothing held if the caller has
-// another way (optional), else the same again with less in reserve.
+// fewer moduli resident and fewer columns at a time.  If the caller has another
+// way (optional), CHASE_OUT_OF_MEMORY with nothing held where one modulus of each
+// and 8 columns do not fit: with fewer the passes over H that slice it anew, 14
+// for each 8 columns, cost more than the FP64 product.  Else down to one column,
+// then the same again with less in reserve.
 struct PlaneSet {
   int nmod;
   RnsH* h;
@@ -174,16 +176,18 @@ int prepare_products(Dev& d, const T* H, int64_t N, int64_t ldh, int b, bool man
   int widest = 0;
   for (const PlaneSet& s : sets) widest = std::max(widest, s.nmod);
   size_t reserve = rns_reserve(N, b);
+  const int least = optional ? std::min(b, 8) : 1;
   int cols = b, most = kRnsMaxModuli;
   for (;;) {
     int st = rns_alloc_x(d, N, cols, widest, is_cplx<T>, x);
+    if (st == CHASE_OK && x.cap_cols < least) st = CHASE_OUT_OF_MEMORY;
     for (const PlaneSet& s : sets)
       if (st == CHASE_OK) st = rns_prepare_h(d, H, N, ldh, s.nmod, most, reserve, many, *s.h);
     if (st != CHASE_OUT_OF_MEMORY) return st;
     rns_release(d, x);
     for (const PlaneSet& s : sets) rns_release(d, *s.h);
-    if (cols > 1 || most > 1) {
-      cols = (cols + 1) / 2;
+    if (cols > least || most > 1) {
+      cols = std::max(least, (cols + 1) / 2);
       most = (most + 1) / 2;
     } else if (!optional && reserve > 0) {
       cols = b;
